@@ -109,32 +109,6 @@ __device__ __forceinline__ T ld_in(const T *p) {
 // T a-edge at c01, L t-edge at c00.
 enum { EB = 0, ER = 1, ET = 2, EL = 3 };
 
-// Segments of a 2D cell from its corner colours (and the face colour on a
-// saddle): returns the count, endpoints as edge codes.
-__device__ __forceinline__ int cell_segs(int c00, int c10, int c01, int c11, int phif, int seg[2][2]) {
-    int mB = c00 != c10, mR = c10 != c11, mT = c01 != c11, mL = c00 != c01;
-    int nm = mB + mR + mT + mL;
-    if (nm == 2) {
-        int k = 0;
-        if (mB) seg[0][k++] = EB;
-        if (mR) seg[0][k++] = ER;
-        if (mT) seg[0][k++] = ET;
-        if (mL) seg[0][k++] = EL;
-        return 1;
-    }
-    if (nm == 4) {
-        if (c00 == phif) {
-            seg[0][0] = EB; seg[0][1] = ER;
-            seg[1][0] = EL; seg[1][1] = ET;
-        } else {
-            seg[0][0] = EB; seg[0][1] = EL;
-            seg[1][0] = ER; seg[1][1] = ET;
-        }
-        return 2;
-    }
-    return 0;
-}
-
 // Circle through A, B, C meeting the grid line x = 0; only roots on the edge
 // (0 <= y <= 1) count, the one nearest ylin is kept (Fig. 2).  rad2 gets the
 // squared radius.
@@ -454,15 +428,44 @@ __global__ void __launch_bounds__(256) advect_list_kernel(SweepArgs a, MarkerLis
 }
 
 // ----------------------------------------------------------- cell context
+// the integers -2 .. 2 as doubles, by bit patterns (an integer conversion would
+// go through the FP64 pipe)
+__device__ __forceinline__ double small_double(int q) {
+    const int hi = (q & 1) ? 0x3FF00000 : (q ? 0x40000000 : 0);
+    return __hiloint2double(hi | (q & 0x80000000), 0);
+}
+
+// Segments of a 2D cell by its markers m (bits EB, ER, ET, EL) and, on a saddle,
+// whether its lower-left colour equals the face colour: the endpoints of segment
+// k in bits 4 k .. 4 k + 3 (first, second), the number of segments in *ns.  The
+// order is the oracle's.
+__device__ __forceinline__ unsigned seg_codes(unsigned m, bool same, int *ns) {
+    if (m == 15u) {
+        *ns = 2;
+        return same ? (EB | ER << 2 | EL << 4 | ET << 6) : (EB | EL << 2 | ER << 4 | ET << 6);
+    }
+    *ns = m ? 1 : 0;
+    return m ? (unsigned)(__ffs(m) - 1) | (unsigned)(31 - __clz(m)) << 2 : 0u;
+}
+
+// A plane of the face family with in-plane transverse axis TT and normal NN
+// through one node, offsets (da, dt) along (A, TT) in da [-2, 2], dt [-1, 2].
+// The window's node and face colours are two bit masks, so that segments,
+// crossings and polyline neighbours are integer selects: every lane of a warp
+// follows one instruction stream whatever its edges, and the marker data is
+// read in two rounds of independent loads (the bins that decide the crossings
+// come with the colours, then the coordinates of the four points).  With
+// branches per edge code and per segment the loads of divergent lanes came one
+// after another, up to twenty rounds of L2 latency: a list of a few hundred
+// edges took 22 us where this form takes 15 (32^3, one sphere), and one of
+// 1.4e5 edges 51 us where it takes 45 (512^3).
 template <int D, bool F = false>
 struct SweepCell {
     static constexpr int A = D, T1 = (D + 1) % 3, T2 = (D + 2) % 3;
     const SweepArgs &a;
     int p[3];
-    // colour bytes of the plane window da in [-2, 2], dt in [-1, 2] of the
-    // family being processed, loaded in one batch (byte (da+2) + 5 (dt+1) of
-    // three 64-bit registers)
-    unsigned long long w0, w1, w2;
+    // bit (da + 2) + 5 (dt + 1): node colour, and the colour of the node's face
+    unsigned col, face;
 
     __device__ SweepCell(const SweepArgs &args, int x, int y, int z) : a(args) {
         p[0] = x;
@@ -476,10 +479,6 @@ struct SweepCell {
         q[T2] = p[T2] + d2;
         return lin3(a.g, q);
     }
-    __device__ __forceinline__ int colid(int id) const { return __ldg(a.cb + id) & 1; }
-
-    // plane of the face family with in-plane transverse axis TT and normal NN
-    // through the cell's node; offsets (da, dt) along (A, TT)
     template <int TT, int NN>
     __device__ __forceinline__ int pid(int da, int dt) const {
         int q[3];
@@ -490,99 +489,96 @@ struct SweepCell {
     }
     template <int TT, int NN>
     __device__ __forceinline__ void loadw() {
-        unsigned long long v[3] = {0ull, 0ull, 0ull};
+        unsigned c = 0, f = 0;
 #pragma unroll
         for (int dt = -1; dt <= 2; dt++)
 #pragma unroll
             for (int da = -2; da <= 2; da++) {
                 const int i = (da + 2) + 5 * (dt + 1);
-                v[i >> 3] |= (unsigned long long)__ldg(a.cb + pid<TT, NN>(da, dt)) << (8 * (i & 7));
+                const unsigned b = __ldg(a.cb + pid<TT, NN>(da, dt));
+                c |= (b & 1u) << i;
+                f |= ((b >> (1 + NN)) & 1u) << i;
             }
-        w0 = v[0];
-        w1 = v[1];
-        w2 = v[2];
+        col = c;
+        face = f;
     }
-    __device__ __forceinline__ int wb(int da, int dt) const {
-        const int i = (da + 2) + 5 * (dt + 1);
-        const unsigned long long v = i < 8 ? w0 : (i < 16 ? w1 : w2);
-        return (int)((v >> (8 * (i & 7))) & 0xFF);
+    __device__ __forceinline__ static int wi(int da, int dt) { return (da + 2) + 5 * (dt + 1); }
+    // markers of cell (da, dt) (bits EB, ER, ET, EL)
+    __device__ __forceinline__ unsigned marks(int i) const {
+        const unsigned w = col >> i;
+        const unsigned c00 = w & 1u, c10 = (w >> 1) & 1u, c01 = (w >> 5) & 1u, c11 = (w >> 6) & 1u;
+        return (c00 ^ c10) | (c10 ^ c11) << ER | (c01 ^ c11) << ET | (c00 ^ c01) << EL;
     }
+    // does the cell's lower-left colour equal its face's?
+    __device__ __forceinline__ bool same(int i) const { return (((col ^ face) >> i) & 1u) == 0u; }
+    __device__ __forceinline__ unsigned segs(int da, int dt, int *ns) const {
+        const int i = wi(da, dt);
+        return seg_codes(marks(i), same(i), ns);
+    }
+
+    // Endpoints left of x = 0 per edge code (bits EB, ER, ET, EL) of the cells
+    // (-1, 0) and (0, 0), in bits 0-3 and 4-7: x = q + adv < 0 <=> bin < -2 q for
+    // the edge's node offset q.  (bins of edges without a marker are read and
+    // not used)
     template <int TT, int NN>
-    __device__ int psegs(int da, int dt, int seg[2][2]) const {
-        int b00 = wb(da, dt);
-        return cell_segs(b00 & 1, wb(da + 1, dt) & 1, wb(da, dt + 1) & 1, wb(da + 1, dt + 1) & 1,
-                         (b00 >> (1 + NN)) & 1, seg);
-    }
-    // bin of the advected a-coordinate of the marker on edge code e of cell
-    // (da, dt), and the integer da' with x = da' + adv
-    template <int TT, int NN>
-    __device__ __forceinline__ int pbin(int e, int da, int dt, int *off) const {
-        if (e == EB || e == ET) {
-            *off = da;
-            return ld_in<F>(a.bin[A] + pid<TT, NN>(da, dt + (e == ET ? 1 : 0)));
-        }
-        int aa = da + (e == ER ? 1 : 0);
-        *off = aa;
-        return ld_in<F>(a.bin[TT] + pid<TT, NN>(aa, dt));
-    }
-    // advected position (x along A, y along TT) relative to the cell's node
-    template <int TT, int NN>
-    __device__ __forceinline__ P2 ppos(int e, int da, int dt) const {
-        P2 r;
-        if (e == EB || e == ET) {
-            int tt = dt + (e == ET ? 1 : 0);
-            r.x = (double)da + ld_in<F>(a.adv[A] + pid<TT, NN>(da, tt));
-            r.y = (double)tt;
-        } else {
-            int aa = da + (e == ER ? 1 : 0);
-            int id = pid<TT, NN>(aa, dt);
-            r.x = (double)aa + ld_in<F>(a.adv[TT] + id);
-            r.y = (double)dt + __ldg(a.s[TT] + id);
-        }
-        return r;
-    }
-    // is the endpoint left of x = 0 (thr = 0) or of x = 1/2 (thr = 1)?
-    template <int TT, int NN>
-    __device__ __forceinline__ bool pleft(int e, int da, int dt, int thr) const {
-        int off;
-        int b = pbin<TT, NN>(e, da, dt, &off);
-        return b < thr - 2 * off;
+    __device__ __forceinline__ unsigned left_bits() const {
+        const int8_t *ba = a.bin[A], *bt = a.bin[TT];
+        const int bB1 = ld_in<F>(ba + pid<TT, NN>(-1, 0)), bT1 = ld_in<F>(ba + pid<TT, NN>(-1, 1));
+        const int bB0 = ld_in<F>(ba + pid<TT, NN>(0, 0)), bT0 = ld_in<F>(ba + pid<TT, NN>(0, 1));
+        const int bL1 = ld_in<F>(bt + pid<TT, NN>(-1, 0)), bL0 = ld_in<F>(bt + pid<TT, NN>(0, 0)),
+                  bR0 = ld_in<F>(bt + pid<TT, NN>(1, 0));
+        const unsigned mid = bL0 < 0;  // the edge between the two cells
+        return (unsigned)(bB1 < 2) | mid << ER | (unsigned)(bT1 < 2) << ET | (unsigned)(bL1 < 2) << EL |
+               ((unsigned)(bB0 < 0) | (unsigned)(bR0 < -2) << ER | (unsigned)(bT0 < 0) << ET | mid << EL) << 4;
     }
     // number of segments of cells (-1, 0) and (0, 0) crossing x = 0
-    template <int TT, int NN>
-    __device__ int count_crossings() const {
+    __device__ __forceinline__ int count_crossings(unsigned left) const {
         int n = 0;
+#pragma unroll
         for (int da = -1; da <= 0; da++) {
-            int seg[2][2];
-            int ns = psegs<TT, NN>(da, 0, seg);
-            for (int k = 0; k < ns; k++)
-                n += pleft<TT, NN>(seg[k][0], da, 0, 0) != pleft<TT, NN>(seg[k][1], da, 0, 0);
+            int ns;
+            const unsigned sg = segs(da, 0, &ns), lc = left >> (4 * (da + 1));
+#pragma unroll
+            for (int k = 0; k < 2; k++)
+                if (k < ns) n += ((lc >> ((sg >> (4 * k)) & 3)) ^ (lc >> ((sg >> (4 * k + 2)) & 3))) & 1;
         }
         return n;
     }
-    // neighbour along the polyline of the marker on edge e of cell (da, dt),
-    // found in the cell across that edge
+
+    // a marker of the window: its node offset (qa, qt) and whether it lies on an
+    // A-edge (EB, ET) or a TT-edge (EL, ER)
+    struct Mark {
+        int qa, qt;
+        bool on_a;
+    };
+    __device__ __forceinline__ static Mark mark(int e, int da, int dt) {
+        return Mark{da + (e == ER), dt + (e == ET), (e & 1) == 0};
+    }
+    // its advected position (x along A, y along TT) relative to the cell's node
     template <int TT, int NN>
-    __device__ bool neighbour(int e, int da, int dt, P2 *out) const {
-        int oda = da, odt = dt, oe;
-        switch (e) {
-        case EB: odt = dt - 1; oe = ET; break;
-        case ET: odt = dt + 1; oe = EB; break;
-        case EL: oda = da - 1; oe = ER; break;
-        default: oda = da + 1; oe = EL; break;
-        }
-        int seg[2][2];
-        int ns = psegs<TT, NN>(oda, odt, seg);
-        for (int k = 0; k < ns; k++) {
-            int other = -1;
-            if (seg[k][0] == oe) other = seg[k][1];
-            else if (seg[k][1] == oe) other = seg[k][0];
-            if (other >= 0) {
-                *out = ppos<TT, NN>(other, oda, odt);
-                return true;
-            }
-        }
-        return false;
+    __device__ __forceinline__ P2 pos(const Mark &m) const {
+        const int id = pid<TT, NN>(m.qa, m.qt);
+        const double *pa = m.on_a ? a.adv[A] : a.adv[TT];
+        const double x = ld_in<F>(pa + id);
+        double s = 0.0;
+        if (!m.on_a) s = __ldg(a.s[TT] + id);
+        P2 r;
+        r.x = small_double(m.qa) + x;
+        r.y = small_double(m.qt) + s;
+        return r;
+    }
+    // the marker next along the polyline beyond edge e of cell (da, dt), in the
+    // cell across that edge; false when that cell has no segment ending on it
+    __device__ __forceinline__ bool next_mark(int e, int da, int dt, Mark *out) const {
+        const int oda = da + (e == ER) - (e == EL), odt = dt + (e == ET) - (e == EB);
+        const int oe = e ^ 2;  // the same edge seen from there: EB <-> ET, EL <-> ER
+        const int i = wi(oda, odt);
+        const unsigned m = marks(i);
+        const unsigned rest = m & ~(1u << oe);
+        // two markers: the other one; a saddle: EB-ER, EL-ET or EB-EL, ER-ET
+        const int other = m == 15u ? (same(i) ? oe ^ 1 : 3 - oe) : __ffs(rest) - 1;
+        *out = mark(other & 3, oda, odt);
+        return ((m >> oe) & 1u) && rest;
     }
 
     // Crossings of the advected polyline of cells (-1, 0) and (0, 0) with the
@@ -593,19 +589,18 @@ struct SweepCell {
         int n;
         int el0, er0, da0, el1, er1, da1, el2, er2, da2;
     };
-    template <int TT, int NN>
-    __device__ __forceinline__ Crossings crossings() const {
+    __device__ __forceinline__ Crossings crossings(unsigned left) const {
         Crossings c{};
 #pragma unroll
         for (int da = -1; da <= 0; da++) {
-            int seg[2][2];
-            const int ns = psegs<TT, NN>(da, 0, seg);
+            int ns;
+            const unsigned sg = segs(da, 0, &ns), lc = left >> (4 * (da + 1));
 #pragma unroll
             for (int k = 0; k < 2; k++) {
-                if (k >= ns) continue;
-                const bool l0 = pleft<TT, NN>(seg[k][0], da, 0, 0), l1 = pleft<TT, NN>(seg[k][1], da, 0, 0);
-                if (l0 == l1) continue;
-                const int el = l0 ? seg[k][0] : seg[k][1], er = l0 ? seg[k][1] : seg[k][0];
+                const int e0 = (sg >> (4 * k)) & 3, e1 = (sg >> (4 * k + 2)) & 3;
+                const bool l0 = (lc >> e0) & 1u, l1 = (lc >> e1) & 1u;
+                if (k >= ns || l0 == l1) continue;
+                const int el = l0 ? e0 : e1, er = l0 ? e1 : e0;
                 if (c.n == 0) { c.el0 = el; c.er0 = er; c.da0 = da; }
                 else if (c.n == 1) { c.el1 = el; c.er1 = er; c.da1 = da; }
                 else if (c.n == 2) { c.el2 = el; c.er2 = er; c.da2 = da; }
@@ -614,13 +609,14 @@ struct SweepCell {
         }
         return c;
     }
-    // the crossing's advected endpoints and its linear crossing height
-    template <int TT, int NN>
-    __device__ __forceinline__ double crossing_line(int el, int er, int cda, P2 &Pa, P2 &Pb) const {
-        Pa = ppos<TT, NN>(el, cda, 0);
-        Pb = ppos<TT, NN>(er, cda, 0);
+    // linear crossing height of the segment Pa Pb with x = 0
+    __device__ __forceinline__ static double crossing_line(const P2 &Pa, const P2 &Pb) {
         const double tt = (0.0 - Pa.x) / (Pb.x - Pa.x);
         return Pa.y + tt * (Pb.y - Pa.y);
+    }
+    template <int TT, int NN>
+    __device__ __forceinline__ double crossing_height(int el, int er, int cda) const {
+        return crossing_line(pos<TT, NN>(mark(el, cda, 0)), pos<TT, NN>(mark(er, cda, 0)));
     }
 
     // Unaligned edge of family (TT, NN) at the cell's node (carries a marker):
@@ -629,8 +625,8 @@ struct SweepCell {
     // half: -1 one lane per edge; 0, 1 the lanes of a pair sharing the edge
     // (the even lane counts and stores).
     template <int TT, int NN>
-    __device__ void unaligned(unsigned ev[C_N], int half = -1) const {
-        const Crossings c = crossings<TT, NN>();
+    __device__ __forceinline__ void unaligned(unsigned left, unsigned ev[C_N], int half = -1) const {
+        const Crossings c = crossings(left);
         const int myid = lin3(a.g, p);
         const bool lead = half <= 0;
         if (lead) ev[C_MARKERS]++;
@@ -642,28 +638,29 @@ struct SweepCell {
             return;
         }
         int el = c.el0, er = c.er0, cda = c.da0;
-        P2 Pa, Pb;
-        double ylin = crossing_line<TT, NN>(el, er, cda, Pa, Pb);
         if (c.n == 3) {
             // a fold of the polyline: the crossing with the median linear
             // height, by the same three compare-exchanges as the oracle
-            P2 A1, B1, A2, B2;
-            const double y1 = crossing_line<TT, NN>(c.el1, c.er1, c.da1, A1, B1);
-            const double y2 = crossing_line<TT, NN>(c.el2, c.er2, c.da2, A2, B2);
             // (v_k tracks yl[o_k], so the comparisons are the oracle's)
-            double v0 = ylin, v1 = y1, v2 = y2, tv;
+            double v0 = crossing_height<TT, NN>(c.el0, c.er0, c.da0), v1 = crossing_height<TT, NN>(c.el1, c.er1, c.da1),
+                   v2 = crossing_height<TT, NN>(c.el2, c.er2, c.da2), tv;
             int o0 = 0, o1 = 1, o2 = 2, tmp;
             if (v0 > v1) { tmp = o0; o0 = o1; o1 = tmp; tv = v0; v0 = v1; v1 = tv; }
             if (v1 > v2) { tmp = o1; o1 = o2; o2 = tmp; tv = v1; v1 = v2; v2 = tv; }
             if (v0 > v1) { tmp = o0; o0 = o1; o1 = tmp; tv = v0; v0 = v1; v1 = tv; }
-            if (o1 == 1) { el = c.el1; er = c.er1; cda = c.da1; Pa = A1; Pb = B1; ylin = y1; }
-            else if (o1 == 2) { el = c.el2; er = c.er2; cda = c.da2; Pa = A2; Pb = B2; ylin = y2; }
+            if (o1 == 1) { el = c.el1; er = c.er1; cda = c.da1; }
+            else if (o1 == 2) { el = c.el2; er = c.er2; cda = c.da2; }
             if (lead) ev[C_MULTI]++;
         }
-        // both neighbours first, then the two circle fits
-        P2 P1 = Pa, P4 = Pb;
-        const bool h1 = neighbour<TT, NN>(el, cda, 0, &P1);
-        const bool h4 = neighbour<TT, NN>(er, cda, 0, &P4);
+        // the crossing segment and its neighbours along the polyline (their own
+        // ends where there is none), all loads together, then the two fits
+        const Mark ma = mark(el, cda, 0), mb = mark(er, cda, 0);
+        Mark m1, m4;
+        const bool h1 = next_mark(el, cda, 0, &m1), h4 = next_mark(er, cda, 0, &m4);
+        if (!h1) m1 = ma;
+        if (!h4) m4 = mb;
+        const P2 Pa = pos<TT, NN>(ma), Pb = pos<TT, NN>(mb), P1 = pos<TT, NN>(m1), P4 = pos<TT, NN>(m4);
+        const double ylin = crossing_line(Pa, Pb);
         if (lead && !h1) ev[C_INCONSISTENT]++;
         if (lead && !h4) ev[C_INCONSISTENT]++;
         if (half < 0) {
@@ -674,6 +671,13 @@ struct SweepCell {
         }
     }
 
+    // is the endpoint on edge e of cell (da, dt) left of x = 1/2?
+    template <int TT, int NN>
+    __device__ __forceinline__ bool left_of_half(int e, int da, int dt) const {
+        const Mark m = mark(e, da, dt);
+        const int b = ld_in<F>((m.on_a ? a.bin[A] : a.bin[TT]) + pid<TT, NN>(m.qa, m.qt));
+        return b < 1 - 2 * m.qa;
+    }
     // Face-centre colour of the family's 2D cell at the node (saddle faces): the
     // phase of the advected polyline at the centre, reached from the node along
     // the a-line to x = 1/2 and then up the line x = 1/2 to y = 1/2.
@@ -681,18 +685,20 @@ struct SweepCell {
     __device__ int face_phase(int ncol0) const {
         int par = ncol0;
         for (int da = -1; da <= 1; da++) {
-            if ((wb(da, 0) & 1) == (wb(da + 1, 0) & 1)) continue;
+            const int i = wi(da, 0);
+            if (((col >> i) & 1u) == ((col >> (i + 1)) & 1u)) continue;
             int b = ld_in<F>(a.bin[A] + pid<TT, NN>(da, 0));
             if (b >= -2 * da && b < 1 - 2 * da) par ^= 1;
         }
         for (int da = -1; da <= 1; da++) {
-            int seg[2][2];
-            int ns = psegs<TT, NN>(da, 0, seg);
+            int ns;
+            const unsigned sg = segs(da, 0, &ns);
             for (int k = 0; k < ns; k++) {
-                bool l0 = pleft<TT, NN>(seg[k][0], da, 0, 1), l1 = pleft<TT, NN>(seg[k][1], da, 0, 1);
+                const int e0 = (sg >> (4 * k)) & 3, e1 = (sg >> (4 * k + 2)) & 3;
+                bool l0 = left_of_half<TT, NN>(e0, da, 0), l1 = left_of_half<TT, NN>(e1, da, 0);
                 if (l0 == l1) continue;
-                P2 L = ppos<TT, NN>(l0 ? seg[k][0] : seg[k][1], da, 0);
-                P2 R = ppos<TT, NN>(l0 ? seg[k][1] : seg[k][0], da, 0);
+                P2 L = pos<TT, NN>(mark(l0 ? e0 : e1, da, 0));
+                P2 R = pos<TT, NN>(mark(l0 ? e1 : e0, da, 0));
                 double tt = (0.5 - L.x) / (R.x - L.x);
                 double yl = L.y + tt * (R.y - L.y);
                 if (yl < 0.5) par ^= 1;
@@ -915,9 +921,11 @@ __device__ __forceinline__ int sweep_tile(const SweepArgs &a, int tile, uint8_t 
                         push[4] = chk1;
                         push[5] = chk2;
                     } else {
-                        if (chk1 && (cell.template loadw<T1, T2>(), cell.template count_crossings<T1, T2>()) >= 2)
+                        if (chk1 && (cell.template loadw<T1, T2>(),
+                                     cell.count_crossings(cell.template left_bits<T1, T2>())) >= 2)
                             ev[C_ANNIHILATE]++;
-                        if (chk2 && (cell.template loadw<T2, T1>(), cell.template count_crossings<T2, T1>()) >= 2)
+                        if (chk2 && (cell.template loadw<T2, T1>(),
+                                     cell.count_crossings(cell.template left_bits<T2, T1>())) >= 2)
                             ev[C_ANNIHILATE]++;
                     }
                     out_marker |= pres1 || pres2;
@@ -1044,17 +1052,22 @@ __device__ __forceinline__ void fp64_item(const SweepArgs &a, int kind, int k, u
     const int id = (int)ld_in<F>(a.work[kind] + k);
     const int x = id % a.g.n[0], y = (id / a.g.n[0]) % a.g.n[1], z = id / (a.g.n[0] * a.g.n[1]);
     SweepCell<D, F> cell(a, x, y, z);
-    if ((kind & 1) == 0) cell.template loadw<T1, T2>();
-    else cell.template loadw<T2, T1>();
+    unsigned left;
+    if ((kind & 1) == 0) {
+        cell.template loadw<T1, T2>();
+        left = cell.template left_bits<T1, T2>();
+    } else {
+        cell.template loadw<T2, T1>();
+        left = cell.template left_bits<T2, T1>();
+    }
     if (kind >= 4) {
         // an even number (>= 2) of advected crossings met on an edge that keeps
         // no marker (Fig. 5)
-        const int nc = (kind == 4) ? cell.template count_crossings<T1, T2>() : cell.template count_crossings<T2, T1>();
-        if (nc >= 2) ev[C_ANNIHILATE]++;
+        if (cell.count_crossings(left) >= 2) ev[C_ANNIHILATE]++;
     } else if (kind == 0) {
-        cell.template unaligned<T1, T2>(ev, half);
+        cell.template unaligned<T1, T2>(left, ev, half);
     } else if (kind == 1) {
-        cell.template unaligned<T2, T1>(ev, half);
+        cell.template unaligned<T2, T1>(left, ev, half);
     } else {
         int ncol0 = ld_in<F>(a.cbo + id) & 1;
         int bit = (kind == 2) ? (cell.template face_phase<T1, T2>(ncol0) << (1 + T2))
