@@ -109,6 +109,32 @@ __device__ __forceinline__ T ld_in(const T *p) {
 // T a-edge at c01, L t-edge at c00.
 enum { EB = 0, ER = 1, ET = 2, EL = 3 };
 
+// Comparisons on the bit patterns: a floating-point comparison goes through
+// the FP64 pipe (2 lanes per clock and SM), which bounds the long lists, and a
+// circle fit has ten of them.  For the values that occur the outcomes are the
+// IEEE ones: -0 equals 0, and a NaN satisfies neither in_unit nor below_zero.
+__device__ __forceinline__ unsigned long long dbits(double v) { return (unsigned long long)__double_as_longlong(v); }
+__device__ __forceinline__ unsigned long long abs_bits(double v) { return dbits(v) & 0x7FFFFFFFFFFFFFFFull; }
+// 0 <= v <= 1
+__device__ __forceinline__ bool in_unit(double v) {
+    const unsigned long long b = dbits(v);
+    return b <= 0x3FF0000000000000ull || b == 0x8000000000000000ull;
+}
+// v < 0
+__device__ __forceinline__ bool below_zero(double v) {
+    return dbits(v) - 0x8000000000000001ull <= 0xFFF0000000000000ull - 0x8000000000000001ull;
+}
+// an offset clamped to [0, 1-]
+__device__ __forceinline__ double clamp_offset(double y) {
+    if (below_zero(y)) return 0.0;
+    return __double_as_longlong(y) > __double_as_longlong(ONE_MINUS) ? ONE_MINUS : y;
+}
+// 2 v: an exponent increment for a normal number
+__device__ __forceinline__ double twice(double v) {
+    const unsigned long long b = dbits(v);
+    return ((b >> 52) & 0x7FF) ? __longlong_as_double((long long)(b + (1ull << 52))) : 2.0 * v;
+}
+
 // Circle through A, B, C meeting the grid line x = 0; only roots on the edge
 // (0 <= y <= 1) count, the one nearest ylin is kept (Fig. 2).  rad2 gets the
 // squared radius.
@@ -117,20 +143,20 @@ __device__ __forceinline__ bool circle_root(P2 A, P2 B, P2 C, double ylin, doubl
     double cx = C.x - A.x, cy = C.y - A.y;
     double b2 = bx * bx + by * by;
     double c2 = cx * cx + cy * cy;
-    double det = 2.0 * (bx * cy - by * cx);
-    if (fabs(det) <= 1e-12 * (b2 + c2)) return false;
+    double det = twice(bx * cy - by * cx);
+    if (abs_bits(det) <= dbits(1e-12 * (b2 + c2))) return false;
     double ux = (cy * b2 - by * c2) / det;
     double uy = (bx * c2 - cx * b2) / det;
     double r2 = ux * ux + uy * uy;
-    double dx = 0.0 - (A.x + ux);
+    double dx = A.x + ux;
     double disc = r2 - dx * dx;
-    if (disc < 0.0) return false;
+    if (below_zero(disc)) return false;
     double sq = sqrt(disc);
     double yc = A.y + uy;
     double yp = yc + sq, ym = yc - sq;
-    bool okp = (yp >= 0.0 && yp <= 1.0), okm = (ym >= 0.0 && ym <= 1.0);
+    bool okp = in_unit(yp), okm = in_unit(ym);
     if (!okp && !okm) return false;
-    if (okp && okm) *root = (fabs(yp - ylin) <= fabs(ym - ylin)) ? yp : ym;
+    if (okp && okm) *root = (abs_bits(yp - ylin) <= abs_bits(ym - ylin)) ? yp : ym;
     else *root = okp ? yp : ym;
     *rad2 = r2;
     return true;
@@ -143,8 +169,8 @@ __device__ __forceinline__ bool circle_root(P2 A, P2 B, P2 C, double ylin, doubl
 // the square roots are taken only within that margin.
 __device__ __forceinline__ bool ratio_above_10(double r2max, double r2min) {
     const double t = 100.0 * r2min;
-    if (r2max > t * (1.0 + 1e-12)) return true;
-    if (r2max < t * (1.0 - 1e-12)) return false;
+    if (dbits(r2max) > dbits(t * (1.0 + 1e-12))) return true;
+    if (dbits(r2max) < dbits(t * (1.0 - 1e-12))) return false;
     return sqrt(r2max) > 10.0 * sqrt(r2min);
 }
 
@@ -165,8 +191,8 @@ static __device__ __noinline__ double circle_pair(P2 P1, P2 Pa, P2 Pb, P2 P4, do
     if (va && vb) {
         // above the ratio the radii differ, so the larger squared radius names
         // the larger circle
-        const double r2max = ra2 > rb2 ? ra2 : rb2, r2min = ra2 > rb2 ? rb2 : ra2;
-        if (ratio_above_10(r2max, r2min)) y = ra2 > rb2 ? ya : yb;
+        const bool a_larger = dbits(ra2) > dbits(rb2);
+        if (ratio_above_10(a_larger ? ra2 : rb2, a_larger ? rb2 : ra2)) y = a_larger ? ya : yb;
         else y = 0.5 * (ya + yb);
     } else if (va) {
         y = ya;
@@ -175,9 +201,7 @@ static __device__ __noinline__ double circle_pair(P2 P1, P2 Pa, P2 Pb, P2 P4, do
     } else {
         y = ylin;
     }
-    if (y < 0.0) y = 0.0;
-    if (y > ONE_MINUS) y = ONE_MINUS;
-    return y;
+    return clamp_offset(y);
 }
 
 // circle_pair with one fit per lane of a lane pair (adjacent lanes of a warp;
@@ -197,8 +221,8 @@ static __device__ __noinline__ double circle_pair_split(P2 P1, P2 Pa, P2 Pb, P2 
     const bool va = half ? vo : v, vb = half ? v : vo;
     double res;
     if (va && vb) {
-        const double r2max = ra2 > rb2 ? ra2 : rb2, r2min = ra2 > rb2 ? rb2 : ra2;
-        if (ratio_above_10(r2max, r2min)) res = ra2 > rb2 ? ya : yb;
+        const bool a_larger = dbits(ra2) > dbits(rb2);
+        if (ratio_above_10(a_larger ? ra2 : rb2, a_larger ? rb2 : ra2)) res = a_larger ? ya : yb;
         else res = 0.5 * (ya + yb);
     } else if (va) {
         res = ya;
@@ -207,9 +231,7 @@ static __device__ __noinline__ double circle_pair_split(P2 P1, P2 Pa, P2 Pb, P2 
     } else {
         res = ylin;
     }
-    if (res < 0.0) res = 0.0;
-    if (res > ONE_MINUS) res = ONE_MINUS;
-    return res;
+    return clamp_offset(res);
 }
 
 // trilinear u_D at node q shifted by s along axis e; lerps in x, y, z order
@@ -448,8 +470,8 @@ __device__ __forceinline__ unsigned seg_codes(unsigned m, bool same, int *ns) {
     return m ? (unsigned)(__ffs(m) - 1) | (unsigned)(31 - __clz(m)) << 2 : 0u;
 }
 
-// A plane of the face family with in-plane transverse axis TT and normal NN
-// through one node, offsets (da, dt) along (A, TT) in da [-2, 2], dt [-1, 2].
+// A plane of one face family through a node, offsets (da, dt) along (A, T) in
+// da [-2, 2], dt [-1, 2], T the family's transverse axis.
 // The window's node and face colours are two bit masks, so that segments,
 // crossings and polyline neighbours are integer selects: every lane of a warp
 // follows one instruction stream whatever its edges, and the marker data is
@@ -457,47 +479,50 @@ __device__ __forceinline__ unsigned seg_codes(unsigned m, bool same, int *ns) {
 // come with the colours, then the coordinates of the four points).  With
 // branches per edge code and per segment the loads of divergent lanes came one
 // after another, up to twenty rounds of L2 latency: a list of a few hundred
-// edges took 22 us where this form takes 15 (32^3, one sphere), and one of
-// 1.4e5 edges 51 us where it takes 45 (512^3).
+// edges took 22 us where this form takes 10 (32^3, one sphere), and one of
+// 1.4e5 edges 51 us where it takes 42 (512^3).
 template <int D, bool F = false>
 struct SweepCell {
     static constexpr int A = D, T1 = (D + 1) % 3, T2 = (D + 2) % 3;
     const SweepArgs &a;
-    int p[3];
+    // the node, and its coordinate, the extent and the stride along A and the
+    // transverse axis (T1 for family 0, T2 for family 1).  The family is a
+    // run-time value: both share one copy of the code (a short list is bound by
+    // instruction fetches as much as by data) and lanes of both run together.
+    const int id, fam;
+    int pa, pt, na, nt, sa, st;
     // bit (da + 2) + 5 (dt + 1): node colour, and the colour of the node's face
     unsigned col, face;
 
-    __device__ SweepCell(const SweepArgs &args, int x, int y, int z) : a(args) {
-        p[0] = x;
-        p[1] = y;
-        p[2] = z;
+    __device__ SweepCell(const SweepArgs &args, int id_, int x, int y, int z, int fam_) : a(args), id(id_), fam(fam_) {
+        const int p[3] = {x, y, z}, s[3] = {1, a.g.n[0], a.g.n[0] * a.g.n[1]};
+        pa = p[A];
+        na = a.g.n[A];
+        sa = s[A];
+        pt = fam ? p[T2] : p[T1];
+        nt = fam ? a.g.n[T2] : a.g.n[T1];
+        st = fam ? s[T2] : s[T1];
     }
-    __device__ __forceinline__ int id3(int da, int d1, int d2) const {
-        int q[3];
-        q[A] = p[A] + da;
-        q[T1] = p[T1] + d1;
-        q[T2] = p[T2] + d2;
-        return lin3(a.g, q);
-    }
-    template <int TT, int NN>
+    // per-family arrays by selects (indexing would copy the arguments to local memory)
+    __device__ __forceinline__ const int8_t *bin_t() const { return fam ? a.bin[T2] : a.bin[T1]; }
+    __device__ __forceinline__ const double *adv_t() const { return fam ? a.adv[T2] : a.adv[T1]; }
+    __device__ __forceinline__ const double *s_t() const { return fam ? a.s[T2] : a.s[T1]; }
+    __device__ __forceinline__ double *so_t() const { return fam ? a.so[T2] : a.so[T1]; }
+    // node at offset (da, dt)
     __device__ __forceinline__ int pid(int da, int dt) const {
-        int q[3];
-        q[A] = p[A] + da;
-        q[TT] = p[TT] + dt;
-        q[NN] = p[NN];
-        return lin3(a.g, q);
+        return id + (wrapc(pa + da, na) - pa) * sa + (wrapc(pt + dt, nt) - pt) * st;
     }
-    template <int TT, int NN>
     __device__ __forceinline__ void loadw() {
         unsigned c = 0, f = 0;
+        const int fb = 1 + (fam ? T1 : T2);
 #pragma unroll
         for (int dt = -1; dt <= 2; dt++)
 #pragma unroll
             for (int da = -2; da <= 2; da++) {
                 const int i = (da + 2) + 5 * (dt + 1);
-                const unsigned b = __ldg(a.cb + pid<TT, NN>(da, dt));
+                const unsigned b = __ldg(a.cb + pid(da, dt));
                 c |= (b & 1u) << i;
-                f |= ((b >> (1 + NN)) & 1u) << i;
+                f |= ((b >> fb) & 1u) << i;
             }
         col = c;
         face = f;
@@ -520,13 +545,12 @@ struct SweepCell {
     // (-1, 0) and (0, 0), in bits 0-3 and 4-7: x = q + adv < 0 <=> bin < -2 q for
     // the edge's node offset q.  (bins of edges without a marker are read and
     // not used)
-    template <int TT, int NN>
     __device__ __forceinline__ unsigned left_bits() const {
-        const int8_t *ba = a.bin[A], *bt = a.bin[TT];
-        const int bB1 = ld_in<F>(ba + pid<TT, NN>(-1, 0)), bT1 = ld_in<F>(ba + pid<TT, NN>(-1, 1));
-        const int bB0 = ld_in<F>(ba + pid<TT, NN>(0, 0)), bT0 = ld_in<F>(ba + pid<TT, NN>(0, 1));
-        const int bL1 = ld_in<F>(bt + pid<TT, NN>(-1, 0)), bL0 = ld_in<F>(bt + pid<TT, NN>(0, 0)),
-                  bR0 = ld_in<F>(bt + pid<TT, NN>(1, 0));
+        const int8_t *ba = a.bin[A], *bt = bin_t();
+        const int bB1 = ld_in<F>(ba + pid(-1, 0)), bT1 = ld_in<F>(ba + pid(-1, 1));
+        const int bB0 = ld_in<F>(ba + pid(0, 0)), bT0 = ld_in<F>(ba + pid(0, 1));
+        const int bL1 = ld_in<F>(bt + pid(-1, 0)), bL0 = ld_in<F>(bt + pid(0, 0)),
+                  bR0 = ld_in<F>(bt + pid(1, 0));
         const unsigned mid = bL0 < 0;  // the edge between the two cells
         return (unsigned)(bB1 < 2) | mid << ER | (unsigned)(bT1 < 2) << ET | (unsigned)(bL1 < 2) << EL |
                ((unsigned)(bB0 < 0) | (unsigned)(bR0 < -2) << ER | (unsigned)(bT0 < 0) << ET | mid << EL) << 4;
@@ -555,13 +579,11 @@ struct SweepCell {
         return Mark{da + (e == ER), dt + (e == ET), (e & 1) == 0};
     }
     // its advected position (x along A, y along TT) relative to the cell's node
-    template <int TT, int NN>
     __device__ __forceinline__ P2 pos(const Mark &m) const {
-        const int id = pid<TT, NN>(m.qa, m.qt);
-        const double *pa = m.on_a ? a.adv[A] : a.adv[TT];
-        const double x = ld_in<F>(pa + id);
+        const int q = pid(m.qa, m.qt);
+        const double x = ld_in<F>((m.on_a ? a.adv[A] : adv_t()) + q);
         double s = 0.0;
-        if (!m.on_a) s = __ldg(a.s[TT] + id);
+        if (!m.on_a) s = __ldg(s_t() + q);
         P2 r;
         r.x = small_double(m.qa) + x;
         r.y = small_double(m.qt) + s;
@@ -614,26 +636,23 @@ struct SweepCell {
         const double tt = (0.0 - Pa.x) / (Pb.x - Pa.x);
         return Pa.y + tt * (Pb.y - Pa.y);
     }
-    template <int TT, int NN>
     __device__ __forceinline__ double crossing_height(int el, int er, int cda) const {
-        return crossing_line(pos<TT, NN>(mark(el, cda, 0)), pos<TT, NN>(mark(er, cda, 0)));
+        return crossing_line(pos(mark(el, cda, 0)), pos(mark(er, cda, 0)));
     }
 
-    // Unaligned edge of family (TT, NN) at the cell's node (carries a marker):
+    // Unaligned edge of the family at the cell's node (carries a marker):
     // crossings of the advected polyline with the grid line x = 0 in strip 0
     // (Fig. 1c), then the two circle fits with the ratio rule (Fig. 2).
     // half: -1 one lane per edge; 0, 1 the lanes of a pair sharing the edge
     // (the even lane counts and stores).
-    template <int TT, int NN>
     __device__ __forceinline__ void unaligned(unsigned left, unsigned ev[C_N], int half = -1) const {
         const Crossings c = crossings(left);
-        const int myid = lin3(a.g, p);
         const bool lead = half <= 0;
         if (lead) ev[C_MARKERS]++;
         if ((c.n & 1) == 0) {
             if (lead) {
                 ev[C_INCONSISTENT]++;
-                a.so[TT][myid] = 0.5;
+                so_t()[id] = 0.5;
             }
             return;
         }
@@ -642,8 +661,8 @@ struct SweepCell {
             // a fold of the polyline: the crossing with the median linear
             // height, by the same three compare-exchanges as the oracle
             // (v_k tracks yl[o_k], so the comparisons are the oracle's)
-            double v0 = crossing_height<TT, NN>(c.el0, c.er0, c.da0), v1 = crossing_height<TT, NN>(c.el1, c.er1, c.da1),
-                   v2 = crossing_height<TT, NN>(c.el2, c.er2, c.da2), tv;
+            double v0 = crossing_height(c.el0, c.er0, c.da0), v1 = crossing_height(c.el1, c.er1, c.da1),
+                   v2 = crossing_height(c.el2, c.er2, c.da2), tv;
             int o0 = 0, o1 = 1, o2 = 2, tmp;
             if (v0 > v1) { tmp = o0; o0 = o1; o1 = tmp; tv = v0; v0 = v1; v1 = tv; }
             if (v1 > v2) { tmp = o1; o1 = o2; o2 = tmp; tv = v1; v1 = v2; v2 = tv; }
@@ -659,35 +678,33 @@ struct SweepCell {
         const bool h1 = next_mark(el, cda, 0, &m1), h4 = next_mark(er, cda, 0, &m4);
         if (!h1) m1 = ma;
         if (!h4) m4 = mb;
-        const P2 Pa = pos<TT, NN>(ma), Pb = pos<TT, NN>(mb), P1 = pos<TT, NN>(m1), P4 = pos<TT, NN>(m4);
+        const P2 Pa = pos(ma), Pb = pos(mb), P1 = pos(m1), P4 = pos(m4);
         const double ylin = crossing_line(Pa, Pb);
         if (lead && !h1) ev[C_INCONSISTENT]++;
         if (lead && !h4) ev[C_INCONSISTENT]++;
         if (half < 0) {
-            a.so[TT][myid] = circle_pair(P1, Pa, Pb, P4, ylin, h1, h4);
+            so_t()[id] = circle_pair(P1, Pa, Pb, P4, ylin, h1, h4);
         } else {
             const double y = circle_pair_split(P1, Pa, Pb, P4, ylin, h1, h4, half);
-            if (lead) a.so[TT][myid] = y;
+            if (lead) so_t()[id] = y;
         }
     }
 
     // is the endpoint on edge e of cell (da, dt) left of x = 1/2?
-    template <int TT, int NN>
     __device__ __forceinline__ bool left_of_half(int e, int da, int dt) const {
         const Mark m = mark(e, da, dt);
-        const int b = ld_in<F>((m.on_a ? a.bin[A] : a.bin[TT]) + pid<TT, NN>(m.qa, m.qt));
+        const int b = ld_in<F>((m.on_a ? a.bin[A] : bin_t()) + pid(m.qa, m.qt));
         return b < 1 - 2 * m.qa;
     }
     // Face-centre colour of the family's 2D cell at the node (saddle faces): the
     // phase of the advected polyline at the centre, reached from the node along
     // the a-line to x = 1/2 and then up the line x = 1/2 to y = 1/2.
-    template <int TT, int NN>
     __device__ int face_phase(int ncol0) const {
         int par = ncol0;
         for (int da = -1; da <= 1; da++) {
             const int i = wi(da, 0);
             if (((col >> i) & 1u) == ((col >> (i + 1)) & 1u)) continue;
-            int b = ld_in<F>(a.bin[A] + pid<TT, NN>(da, 0));
+            int b = ld_in<F>(a.bin[A] + pid(da, 0));
             if (b >= -2 * da && b < 1 - 2 * da) par ^= 1;
         }
         for (int da = -1; da <= 1; da++) {
@@ -695,10 +712,10 @@ struct SweepCell {
             const unsigned sg = segs(da, 0, &ns);
             for (int k = 0; k < ns; k++) {
                 const int e0 = (sg >> (4 * k)) & 3, e1 = (sg >> (4 * k + 2)) & 3;
-                bool l0 = left_of_half<TT, NN>(e0, da, 0), l1 = left_of_half<TT, NN>(e1, da, 0);
+                bool l0 = left_of_half(e0, da, 0), l1 = left_of_half(e1, da, 0);
                 if (l0 == l1) continue;
-                P2 L = pos<TT, NN>(mark(l0 ? e0 : e1, da, 0));
-                P2 R = pos<TT, NN>(mark(l0 ? e1 : e0, da, 0));
+                P2 L = pos(mark(l0 ? e0 : e1, da, 0));
+                P2 R = pos(mark(l0 ? e1 : e0, da, 0));
                 double tt = (0.5 - L.x) / (R.x - L.x);
                 double yl = L.y + tt * (R.y - L.y);
                 if (yl < 0.5) par ^= 1;
@@ -811,7 +828,6 @@ __device__ __forceinline__ int sweep_tile(const SweepArgs &a, int tile, uint8_t 
             bool push_al = false;
             int myid = 0;
             if (valid) {
-                SweepCell<D, F> cell(a, x, y, z);
                 myid = lin(a.g, x, y, z);
                 // staged index of node (da, d1, d2) relative to the cell
                 const int r0 = (l[A] + 1) + RA * (l[T1] + R1 * l[T2]);
@@ -879,7 +895,8 @@ __device__ __forceinline__ int sweep_tile(const SweepArgs &a, int tile, uint8_t 
                             if (nl == 1 || nl == 3) {
                                 double sv[3];
                                 for (int k = 0; k < nl; k++) {
-                                    double xv = ld_in<F>(a.adv[A] + cell.id3(land[k], 0, 0));
+                                    double xv = ld_in<F>(a.adv[A] + lin(a.g, x + (A == 0 ? land[k] : 0), y + (A == 1 ? land[k] : 0),
+                                                                      z + (A == 2 ? land[k] : 0)));
                                     double sn = xv - (double)(-land[k]);
                                     if (sn > ONE_MINUS) sn = ONE_MINUS;
                                     sv[k] = sn;
@@ -921,12 +938,12 @@ __device__ __forceinline__ int sweep_tile(const SweepArgs &a, int tile, uint8_t 
                         push[4] = chk1;
                         push[5] = chk2;
                     } else {
-                        if (chk1 && (cell.template loadw<T1, T2>(),
-                                     cell.count_crossings(cell.template left_bits<T1, T2>())) >= 2)
-                            ev[C_ANNIHILATE]++;
-                        if (chk2 && (cell.template loadw<T2, T1>(),
-                                     cell.count_crossings(cell.template left_bits<T2, T1>())) >= 2)
-                            ev[C_ANNIHILATE]++;
+                        for (int fam = 0; fam < 2; fam++) {
+                            if (!(fam ? chk2 : chk1)) continue;
+                            SweepCell<D, F> cell(a, myid, x, y, z, fam);
+                            cell.loadw();
+                            if (cell.count_crossings(cell.left_bits()) >= 2) ev[C_ANNIHILATE]++;
+                        }
                     }
                     out_marker |= pres1 || pres2;
                     // face colours: family 1 faces are normal to T2, family 2 to T1
@@ -1051,27 +1068,18 @@ __device__ __forceinline__ void fp64_item(const SweepArgs &a, int kind, int k, u
     constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
     const int id = (int)ld_in<F>(a.work[kind] + k);
     const int x = id % a.g.n[0], y = (id / a.g.n[0]) % a.g.n[1], z = id / (a.g.n[0] * a.g.n[1]);
-    SweepCell<D, F> cell(a, x, y, z);
-    unsigned left;
-    if ((kind & 1) == 0) {
-        cell.template loadw<T1, T2>();
-        left = cell.template left_bits<T1, T2>();
-    } else {
-        cell.template loadw<T2, T1>();
-        left = cell.template left_bits<T2, T1>();
-    }
+    SweepCell<D, F> cell(a, id, x, y, z, kind & 1);
+    cell.loadw();
+    const unsigned left = cell.left_bits();
     if (kind >= 4) {
         // an even number (>= 2) of advected crossings met on an edge that keeps
         // no marker (Fig. 5)
         if (cell.count_crossings(left) >= 2) ev[C_ANNIHILATE]++;
-    } else if (kind == 0) {
-        cell.template unaligned<T1, T2>(left, ev, half);
-    } else if (kind == 1) {
-        cell.template unaligned<T2, T1>(left, ev, half);
+    } else if (kind < 2) {
+        cell.unaligned(left, ev, half);
     } else {
         int ncol0 = ld_in<F>(a.cbo + id) & 1;
-        int bit = (kind == 2) ? (cell.template face_phase<T1, T2>(ncol0) << (1 + T2))
-                              : (cell.template face_phase<T2, T1>(ncol0) << (1 + T1));
+        const int bit = cell.face_phase(ncol0) << (1 + (kind == 2 ? T2 : T1));
         if (bit) {
             uintptr_t addr = (uintptr_t)(a.cbo + id);
             unsigned *w = (unsigned *)(addr & ~(uintptr_t)3);
