@@ -9,12 +9,13 @@
 #include "../../include/ebit.h"
 #include "common.cuh"
 #include "devmem.h"
+#include "sweep_args.cuh"
 
 using ebit::Grid;
 
-// work lists of a context's sweep: unaligned edges and saddle faces of the two
-// face families, and the annihilation checks of the two families
-constexpr int NLISTS = 6;
+// arrays of a sweep's work lists (see SweepArgs::work)
+constexpr int NWORK = 4;
+constexpr int NLISTS = ebit::SWEEP_LISTS;
 
 struct ebit_mlp {
     ebit::DevMem mem;  // the allocator the network was created with
@@ -69,12 +70,13 @@ struct ebit_ctx {
     unsigned long long *amr_ctr;  // refined cells | brick count, ids out of range (two ints)
     double *adv[3];           // advected marker coordinates of the current sweep (scratch)
     int8_t *bin[3];           // floor(2 adv) (scratch)
-    unsigned *work[NLISTS];   // work lists of a sweep (scratch; a batch view has the first 4)
-    int *wcount;              // [NLISTS] list lengths ([4] in a batch view), then the band pass's tile counter
+    unsigned *work[NWORK];    // work lists of a sweep (scratch)
+    int *wcount;              // [NLISTS] list lengths, then (not in a batch view) the band pass's tile counter
     // A context's band sweeps alternate between two sets of lists: a sweep
     // reads set mk_par (the markers and band the previous sweep listed) and
     // writes set mk_par ^ 1.  Set 0 is work/wcount above, set 1 work2/wcount2.
-    unsigned *work2[NLISTS];
+    unsigned *work2[NWORK];
+    int *scan_count;          // [3] lengths of the marker lists of a whole-grid scan
     int *wcount2;
     unsigned *mk_al[2];       // aligned edges that carry a marker, per set
     int *mk_count;            // [2] their lengths
@@ -100,7 +102,7 @@ struct ebit_ctx {
     const double *last_C;
     const double *last_kh;
     const uint8_t *last_st;
-    int grid_sweep, grid_adv, grid_advl, grid_fp64, grid_f2v, grid_f2vl, grid_hf, grid_hfl;
+    int grid_sweep, grid_advl, grid_fp64, grid_f2v, grid_f2vl, grid_hf, grid_hfl;
     // per-kernel CUDA-event timing (ebit_profile)
     int prof_on;
     std::vector<cudaEvent_t> ev;
@@ -119,7 +121,7 @@ struct ebit_state_arrays {
     double *s[2][3];
     double *adv[3];
     int8_t *bin[3];
-    unsigned *work[4];
+    unsigned *work[NWORK];
     int *wcount;
     uint32_t *tile_marker;
     uint8_t *tile_dirty;

@@ -178,25 +178,21 @@ struct ProfScope {
 };
 
 template <int D>
-int sweep_launch(ebit_ctx *ctx, const SweepArgs &args, const MarkerLists *ml) {
+int sweep_launch(ebit_ctx *ctx, const SweepArgs &args, const MarkerLists &ml) {
     {
         ProfScope ps(ctx, EBIT_PROF_ADVECT);
-        int r = ml ? launched(ctx, launch_pdl(advect_list_kernel<D, NLISTS>, ctx->grid_advl, 256, 0, ctx->stream,
-                                              args, *ml),
-                              "advect_list_kernel")
-                   : launched(ctx, launch_pdl(advect_kernel<D, NLISTS>, ctx->grid_adv, 256, 0, ctx->stream, args),
-                              "advect_kernel");
+        int r = launched(ctx, launch_pdl(advect_list_kernel<D>, ctx->grid_advl, 256, 0, ctx->stream, args, ml),
+                         "advect_list_kernel");
         if (r) return r;
     }
     {
         ProfScope ps(ctx, EBIT_PROF_SWEEP);
-        int r = launched(ctx, launch_pdl(sweep_kernel<D, NLISTS>, ctx->grid_sweep, 256, 0, ctx->stream, args),
+        int r = launched(ctx, launch_pdl(sweep_kernel<D>, ctx->grid_sweep, BAND_THREADS, 0, ctx->stream, args),
                          "sweep_kernel");
         if (r) return r;
     }
     ProfScope ps(ctx, EBIT_PROF_FP64);
-    return launched(ctx, launch_pdl(fp64_kernel<D, NLISTS>, ctx->grid_fp64, 128, 0, ctx->stream, args),
-                    "fp64_kernel");
+    return launched(ctx, launch_pdl(fp64_kernel<D>, ctx->grid_fp64, 128, 0, ctx->stream, args), "fp64_kernel");
 }
 
 }  // namespace
@@ -232,8 +228,8 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
         ctx->adv[a] = nullptr;
         ctx->bin[a] = nullptr;
     }
-    for (int k = 0; k < NLISTS; k++) ctx->work[k] = ctx->work2[k] = nullptr;
-    ctx->wcount2 = ctx->mk_count = ctx->mt_count = ctx->band_list2 = nullptr;
+    for (int k = 0; k < NWORK; k++) ctx->work[k] = ctx->work2[k] = nullptr;
+    ctx->wcount2 = ctx->mk_count = ctx->mt_count = ctx->band_list2 = ctx->scan_count = nullptr;
     ctx->mk_al[0] = ctx->mk_al[1] = nullptr;
     ctx->mtiles[0] = ctx->mtiles[1] = nullptr;
     ctx->band_flag = nullptr;
@@ -297,7 +293,7 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
             ctx->adv[a] = st->adv[a];
             ctx->bin[a] = st->bin[a];
         }
-        for (int k = 0; k < 4; k++) ctx->work[k] = st->work[k];
+        for (int k = 0; k < NWORK; k++) ctx->work[k] = st->work[k];
         ctx->wcount = st->wcount;
         ctx->tile_marker = st->tile_marker;
         ctx->tile_dirty = st->tile_dirty;
@@ -309,14 +305,14 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
         }
         for (int a = 0; a < 3 && ok; a++)
             ok = ok && alloc((void **)&ctx->adv[a], ctx->N * sizeof(double)) && alloc((void **)&ctx->bin[a], ctx->N);
-        for (int k = 0; k < NLISTS && ok; k++) ok = ok && alloc((void **)&ctx->work[k], ctx->N * sizeof(unsigned));
+        for (int k = 0; k < NWORK && ok; k++) ok = ok && alloc((void **)&ctx->work[k], ctx->N * sizeof(unsigned));
         ok = ok && alloc((void **)&ctx->wcount, (NLISTS + 1) * sizeof(int)) && alloc((void **)&ctx->tile_marker, nt * sizeof(uint32_t)) &&
              alloc((void **)&ctx->tile_dirty, nt) && alloc((void **)&ctx->ctr, C_TOTAL * sizeof(unsigned long long));
-        for (int k = 0; k < NLISTS && ok; k++) ok = ok && alloc((void **)&ctx->work2[k], ctx->N * sizeof(unsigned));
+        for (int k = 0; k < NWORK && ok; k++) ok = ok && alloc((void **)&ctx->work2[k], ctx->N * sizeof(unsigned));
         for (int q = 0; q < 2 && ok; q++)
             ok = ok && alloc((void **)&ctx->mk_al[q], ctx->N * sizeof(unsigned)) &&
                  alloc((void **)&ctx->mtiles[q], nt * sizeof(int));
-        ok = ok && alloc((void **)&ctx->wcount2, (NLISTS + 1) * sizeof(int)) && alloc((void **)&ctx->mk_count, 2 * sizeof(int)) &&
+        ok = ok && alloc((void **)&ctx->wcount2, (NLISTS + 1) * sizeof(int)) && alloc((void **)&ctx->scan_count, 3 * sizeof(int)) && alloc((void **)&ctx->mk_count, 2 * sizeof(int)) &&
              alloc((void **)&ctx->mt_count, 2 * sizeof(int)) && alloc((void **)&ctx->band_list2, nt * sizeof(int)) &&
              alloc((void **)&ctx->band_flag, nt * sizeof(uint32_t)) && alloc((void **)&ctx->tile_dirty2, nt);
     }
@@ -335,13 +331,11 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
         return EBIT_ENOMEM;
     }
     int occ = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sweep_kernel<0, NLISTS>, 256, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sweep_kernel<0>, BAND_THREADS, 0);
     ctx->grid_sweep = std::max(1, std::min(nt, ctx->sms * std::max(occ, 1)));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, advect_kernel<0, NLISTS>, 256, 0);
-    ctx->grid_adv = std::max(1, std::min(nt, ctx->sms * std::max(occ, 1)));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, advect_list_kernel<0, NLISTS>, 256, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, advect_list_kernel<0>, 256, 0);
     ctx->grid_advl = ctx->sms * std::max(occ, 1);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fp64_kernel<0, NLISTS>, 128, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fp64_kernel<0>, 128, 0);
     ctx->grid_fp64 = ctx->sms * std::max(occ, 1);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f2v_band_kernel, 256, 0);
     ctx->grid_f2v = std::max(1, std::min(ntc, ctx->sms * std::max(occ, 1)));
@@ -351,10 +345,11 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
     ctx->grid_hf = std::max(1, std::min(ntc, ctx->sms * std::max(occ, 1)));
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, hf_list_kernel<true>, 128, 0);
     ctx->grid_hfl = ctx->sms * std::max(occ, 1);
-    cudaMemsetAsync(ctx->wcount, 0, (ctx->owns_state ? NLISTS + 1 : 4) * sizeof(int), ctx->stream);
+    cudaMemsetAsync(ctx->wcount, 0, (ctx->owns_state ? NLISTS + 1 : NLISTS) * sizeof(int), ctx->stream);
     if (ctx->owns_state) {
         cudaMemsetAsync(ctx->wcount2, 0, (NLISTS + 1) * sizeof(int), ctx->stream);
         cudaMemsetAsync(ctx->mk_count, 0, 2 * sizeof(int), ctx->stream);
+        cudaMemsetAsync(ctx->scan_count, 0, 3 * sizeof(int), ctx->stream);
         cudaMemsetAsync(ctx->mt_count, 0, 2 * sizeof(int), ctx->stream);
     }
     cudaMemsetAsync(ctx->ncut, 0, sizeof(int), ctx->stream);
@@ -426,12 +421,13 @@ void ebit_destroy(ebit_ctx *ctx) {
             dev_free(ctx->mem, ctx->adv[a]);
             dev_free(ctx->mem, ctx->bin[a]);
         }
-        for (int k = 0; k < NLISTS; k++) {
+        for (int k = 0; k < NWORK; k++) {
             dev_free(ctx->mem, ctx->work[k]);
             dev_free(ctx->mem, ctx->work2[k]);
         }
         dev_free(ctx->mem, ctx->wcount);
         dev_free(ctx->mem, ctx->wcount2);
+        dev_free(ctx->mem, ctx->scan_count);
         dev_free(ctx->mem, ctx->mk_al[0]);
         dev_free(ctx->mem, ctx->mk_al[1]);
         dev_free(ctx->mem, ctx->mk_count);
@@ -640,8 +636,8 @@ int ebit_advect_sweep(ebit_ctx *ctx, int dir, const double *u_face, double dt) {
     // sweep reads set rd (the markers to move and the tiles with markers
     // nearby, listed by the previous sweep), builds its band into band list
     // rd from the latter, and writes set wr for the next one.  After a state
-    // change, and in dense mode, every tile is processed and the markers are
-    // found from the colours of each tile instead.
+    // change, and in dense mode, every tile is processed and a scan of the
+    // colours lists the markers (into the arrays of set rd, free then).
     // an asynchronous Front2VOF may still read the buffer this sweep writes
     if (ctx->f2v_pending && (ctx->cur ^ 1) == ctx->f2v_buf) {
         CU(cudaStreamWaitEvent(ctx->stream, ctx->ev_f2v, 0));
@@ -663,7 +659,8 @@ int ebit_advect_sweep(ebit_ctx *ctx, int dir, const double *u_face, double dt) {
         a.bin[k] = ctx->bin[k];
     }
     unsigned *const *wk_wr = wr ? ctx->work2 : ctx->work;
-    for (int k = 0; k < NLISTS; k++) a.work[k] = wk_wr[k];
+    for (int k = 0; k < NWORK; k++) a.work[k] = wk_wr[k];
+    a.cb_whole = (ctx->N + 7) & ~7LL;
     a.wcount = wr ? ctx->wcount2 : ctx->wcount;
     a.tile_next = a.wcount + NLISTS;  // one int after the list lengths
     a.u = u_face;
@@ -682,30 +679,43 @@ int ebit_advect_sweep(ebit_ctx *ctx, int dir, const double *u_face, double dt) {
         a.band_next_count = ctx->band_count + wr;
     }
     MarkerLists ml;
+    unsigned *const *wk_rd = rd ? ctx->work2 : ctx->work;
+    const int *wc_rd = rd ? ctx->wcount2 : ctx->wcount;
+    ml.list[0] = ctx->mk_al[rd];
+    ml.list[1] = wk_rd[0];
+    ml.list[2] = wk_rd[1];
     if (lists) {
         // the previous sweep's aligned markers and its unaligned work lists
-        const int pd = ctx->mk_dir;
-        unsigned *const *wk_rd = rd ? ctx->work2 : ctx->work;
-        const int *wc_rd = rd ? ctx->wcount2 : ctx->wcount;
-        ml.list[0] = ctx->mk_al[rd];
         ml.count[0] = ctx->mk_count + rd;
-        ml.axis[0] = pd;
-        ml.list[1] = wk_rd[0];
         ml.count[1] = wc_rd + 0;
-        ml.axis[1] = (pd + 1) % 3;
-        ml.list[2] = wk_rd[1];
         ml.count[2] = wc_rd + 1;
-        ml.axis[2] = (pd + 2) % 3;
+        for (int k = 0; k < 3; k++) ml.axis[k] = (ctx->mk_dir + k) % 3;
         ml.mtiles = ctx->mtiles[rd];
         ml.mtiles_count = ctx->mt_count + rd;
         ml.band = rd ? ctx->band_list2 : ctx->band_list;
         ml.band_count = ctx->band_count + rd;
+    } else {
+        for (int k = 0; k < 3; k++) {
+            ml.count[k] = ctx->scan_count + k;
+            ml.axis[k] = k;
+        }
+        ml.mtiles = nullptr;
+        ml.mtiles_count = ctx->zero;
+        ml.band = nullptr;
+        ml.band_count = nullptr;
+        a.scan_count = ctx->scan_count;
+        ProfScope ps(ctx, EBIT_PROF_ADVECT);
+        const long long groups = (ctx->N / ctx->g.n[0]) * ((ctx->g.n[0] + 7) / 8);
+        int r = launched(ctx, launch_pdl(mark_scan_kernel, blocks_for(groups, 256, ctx->sms), 256, 0, ctx->stream, a,
+                                         ctx->mk_al[rd], wk_rd[0], wk_rd[1], ctx->scan_count),
+                         "mark_scan_kernel");
+        if (r) return r;
     }
     int r;
     switch (dir) {
-    case 0: r = sweep_launch<0>(ctx, a, lists ? &ml : nullptr); break;
-    case 1: r = sweep_launch<1>(ctx, a, lists ? &ml : nullptr); break;
-    default: r = sweep_launch<2>(ctx, a, lists ? &ml : nullptr); break;
+    case 0: r = sweep_launch<0>(ctx, a, ml); break;
+    case 1: r = sweep_launch<1>(ctx, a, ml); break;
+    default: r = sweep_launch<2>(ctx, a, ml); break;
     }
     if (r) return r;
     ctx->band_last = lists ? rd : -1;

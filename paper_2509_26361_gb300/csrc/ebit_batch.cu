@@ -35,6 +35,16 @@
 
 namespace ebit {
 
+// the largest colour block of advect_tile
+__host__ __device__ constexpr int adv_stage_max() {
+    int m = 0;
+    for (int sh = 0; sh < N_TILE_SHAPES; sh++) {
+        const int v = (tile_edge(sh, 0) + 1) * (tile_edge(sh, 1) + 1) * (tile_edge(sh, 2) + 1);
+        m = v > m ? v : m;
+    }
+    return m;
+}
+
 constexpr int BATCH_MAX = 1024;      // instances per batch (tile ids keep 20 bits)
 constexpr int BATCH_THREADS = 256;
 constexpr long long BAR_POLLS = 1LL << 24;  // polls of 64 ns sleep: about a second
@@ -52,7 +62,7 @@ struct BatchParams {
     const double *lam;        // [n] dt / h
     int *band;                // (instance << 20) | tile
     int *nband;
-    int *wcount;              // [4 n] FP64 list lengths (all instances)
+    int *wcount;              // [6 n] FP64 list lengths (all instances)
     unsigned *bar;            // [2] arrivals, generation
     int *err;
 };
@@ -104,18 +114,22 @@ template <int D, int SH>
 __global__ void __launch_bounds__(BATCH_THREADS, 4) batch_sweep_kernel(BatchParams p) {
     __shared__ uint16_t s_mk[3 * TILE_CELLS];
     __shared__ uint8_t s_c[adv_stage_max()];
-    __shared__ uint8_t s_b[stage_n(D, SH)];
-    __shared__ int8_t s_bn[stage_n(D, SH)];
+    // the band pass's staging and the FP64 phase's prefix sums, in turn
+    constexpr int GROUPS = BATCH_THREADS / BAND_THREADS;
+    constexpr size_t SHARED = sizeof(BandSmem<D, SH>) * GROUPS > sizeof(int) * (SWEEP_LISTS * BATCH_MAX + 1)
+                                  ? sizeof(BandSmem<D, SH>) * GROUPS
+                                  : sizeof(int) * (SWEEP_LISTS * BATCH_MAX + 1);
+    __shared__ __align__(16) unsigned char s_raw[SHARED];
+    BandSmem<D, SH> *s_band = reinterpret_cast<BandSmem<D, SH> *>(s_raw);
+    int *s_pre = reinterpret_cast<int *>(s_raw);
     __shared__ int s_n, s_ok;
-    __shared__ unsigned s_flag;
-    __shared__ int s_pre[4 * BATCH_MAX + 1];
     __shared__ int s_wsum[BATCH_THREADS / 32];
     if (*(volatile int *)p.err) return;
     const int stride = gridDim.x * blockDim.x;
     const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
 
     // ---- band: tiles near a marker, all instances
-    for (int k = gtid; k < 4 * p.n; k += stride) p.wcount[k] = 0;
+    for (int k = gtid; k < SWEEP_LISTS * p.n; k += stride) p.wcount[k] = 0;
     {
         const int iters = (p.total_tiles + stride - 1) / stride;
         for (int it = 0; it < iters; it++) {
@@ -145,21 +159,26 @@ __global__ void __launch_bounds__(BATCH_THREADS, 4) batch_sweep_kernel(BatchPara
     if (!grid_barrier(p, &s_ok)) return;
 
     // ---- integer band pass
-    for (int li = blockIdx.x; li < nb; li += gridDim.x) {
-        const int e = __ldcg(p.band + li);
-        const int i = e >> 20;
-        const SweepArgs &a = p.inst[i].a;
-        sweep_tile<D, true, 4, SH>(a, e & 0xFFFFF, s_b, s_bn, &s_flag);
-        if (threadIdx.x == 0) atomicAdd(a.ctr + C_TILES, 1ull);
+    {
+        const int grp = threadIdx.x / BAND_THREADS;
+        for (int li = grp * gridDim.x + blockIdx.x; li < nb; li += gridDim.x * GROUPS) {
+            const int e = __ldcg(p.band + li);
+            const SweepArgs &a = p.inst[e >> 20].a;
+            BandEvents ev;
+            band_tile<D, true, SH>(a, e & 0xFFFFF, s_band[grp], 1 + grp, ev);
+            flush_events(ev, a.ctr);
+            if ((threadIdx.x & (BAND_THREADS - 1)) == 0) atomicAdd(a.ctr + C_TILES, 1ull);
+            band_sync(1 + grp);
+        }
     }
     if (!grid_barrier(p, &s_ok)) return;
 
     // ---- FP64 lists of every instance as one index space: block-wide prefix
-    // sums of the 4 n list lengths
+    // sums of the list lengths
     {
-        const int m = 4 * p.n;
+        const int m = SWEEP_LISTS * p.n;
         const int per = (m + blockDim.x - 1) / blockDim.x;
-        int loc[4 * BATCH_MAX / BATCH_THREADS];
+        int loc[SWEEP_LISTS * BATCH_MAX / BATCH_THREADS];
         int sum = 0;
         for (int q = 0; q < per; q++) {
             const int j = threadIdx.x * per + q;
@@ -187,7 +206,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, 4) batch_sweep_kernel(BatchPara
         // marker counts of the unaligned lists (one per entry)
         if (blockIdx.x == 0)
             for (int i = threadIdx.x; i < p.n; i += blockDim.x) {
-                const int nm = (s_pre[4 * i + 2] - s_pre[4 * i]);
+                const int nm = (s_pre[SWEEP_LISTS * i + 2] - s_pre[SWEEP_LISTS * i]);
                 if (nm) atomicAdd(p.inst[i].a.ctr + C_MARKERS, (unsigned long long)nm);
             }
         const int total = s_pre[m];
@@ -198,7 +217,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, 4) batch_sweep_kernel(BatchPara
                 if (s_pre[mid] <= t) lo = mid;
                 else hi = mid;
             }
-            const int i = lo >> 2, kind = lo & 3;
+            const int i = lo / SWEEP_LISTS, kind = lo - i * SWEEP_LISTS;
             unsigned ev[C_N] = {0, 0, 0, 0, 0};
             fp64_item<D, true>(p.inst[i].a, kind, t - s_pre[lo], ev);
 #pragma unroll
@@ -549,7 +568,7 @@ int ebit_batch_create(int n, const ebit_desc *descs, ebit_batch **out) {
     for (int a = 0; a < 3 && ok; a++)
         ok = ok && alloc((void **)&b->adv[a], cells * sizeof(double)) && alloc((void **)&b->bin[a], cells);
     for (int k = 0; k < 4 && ok; k++) ok = ok && alloc((void **)&b->work[k], cells * sizeof(unsigned));
-    ok = ok && alloc((void **)&b->wcount, 4 * n * sizeof(int)) && alloc((void **)&b->tile_marker, tiles * sizeof(uint32_t)) &&
+    ok = ok && alloc((void **)&b->wcount, SWEEP_LISTS * n * sizeof(int)) && alloc((void **)&b->tile_marker, tiles * sizeof(uint32_t)) &&
          alloc((void **)&b->tile_dirty, tiles) && alloc((void **)&b->ctr, (size_t)n * C_TOTAL * 8) &&
          alloc((void **)&b->table[0], n * sizeof(BatchInst)) && alloc((void **)&b->table[1], n * sizeof(BatchInst)) &&
          alloc((void **)&b->d_toff, (n + 1) * sizeof(int)) && alloc((void **)&b->lam, n * sizeof(double)) &&
@@ -580,7 +599,7 @@ int ebit_batch_create(int n, const ebit_desc *descs, ebit_batch **out) {
             st.bin[a] = b->bin[a] + c0;
         }
         for (int k = 0; k < 4; k++) st.work[k] = b->work[k] + c0;
-        st.wcount = b->wcount + 4 * i;
+        st.wcount = b->wcount + SWEEP_LISTS * i;
         st.tile_marker = b->tile_marker + t0;
         st.tile_dirty = b->tile_dirty + t0;
         st.ctr = b->ctr + (size_t)i * C_TOTAL;
@@ -604,6 +623,7 @@ int ebit_batch_create(int n, const ebit_desc *descs, ebit_batch **out) {
             }
             for (int k = 0; k < 4; k++) a.work[k] = st.work[k];
             a.wcount = st.wcount;
+            a.cb_whole = (c->N + 7) & ~7LL;
             a.ctr = st.ctr;
             a.tile_marker = st.tile_marker;
             a.tile_dirty = st.tile_dirty;
@@ -617,7 +637,7 @@ int ebit_batch_create(int n, const ebit_desc *descs, ebit_batch **out) {
             cudaSuccess ||
         cudaMemsetAsync(b->bar, 0, 2 * sizeof(unsigned), b->stream) != cudaSuccess ||
         cudaMemsetAsync(b->err, 0, sizeof(int), b->stream) != cudaSuccess ||
-        cudaMemsetAsync(b->wcount, 0, 4 * n * sizeof(int), b->stream) != cudaSuccess ||
+        cudaMemsetAsync(b->wcount, 0, SWEEP_LISTS * n * sizeof(int), b->stream) != cudaSuccess ||
         cudaStreamSynchronize(b->stream) != cudaSuccess) {
         cudaGetLastError();
         ebit_batch_destroy(b);

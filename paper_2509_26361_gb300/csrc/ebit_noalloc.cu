@@ -46,8 +46,9 @@ constexpr long long OFF_ADV = 0;
 constexpr long long OFF_BIN = align256(OFF_ADV + 3 * NA_MAX_CELLS * 8);
 constexpr long long OFF_WORK = align256(OFF_BIN + 3 * NA_MAX_CELLS);
 constexpr long long OFF_LIST = align256(OFF_WORK + 4 * NA_MAX_CELLS * 4);
-constexpr long long OFF_INTS = align256(OFF_LIST + NA_MAX_TILES * 4);  // all_count, wcount[4]
-constexpr long long OFF_CTR = align256(OFF_INTS + 8 * 4);
+constexpr long long OFF_INTS = align256(OFF_LIST + NA_MAX_TILES * 4);  // all_count, wcount[6], scan_count[3], a zero
+constexpr int NA_INTS = 11;
+constexpr long long OFF_CTR = align256(OFF_INTS + NA_INTS * 4);
 constexpr long long OFF_TILES = align256(OFF_CTR + C_TOTAL * 8);       // tile_marker (u32), tile_dirty
 constexpr long long NA_BYTES = align256(OFF_TILES + 5 * NA_MAX_TILES);
 
@@ -91,9 +92,12 @@ __global__ void na_zero_empty_kernel(Grid g, const uint8_t *__restrict__ cb, dou
 }
 
 template <int D>
-void launch_all(const SweepArgs &a, cudaStream_t st, int grid_tiles, int grid_fp64) {
-    advect_kernel<D><<<grid_tiles, 256, 0, st>>>(a);
-    sweep_kernel<D><<<grid_tiles, 256, 0, st>>>(a);
+void launch_all(const SweepArgs &a, const MarkerLists &m, cudaStream_t st, int grid_scan, int grid_tiles, int grid_fp64) {
+    // the marker lists use the work lists' arrays: they are read before the
+    // band pass writes those
+    mark_scan_kernel<<<grid_scan, 256, 0, st>>>(a, a.work[0], a.work[1], a.work[2], a.scan_count);
+    advect_list_kernel<D><<<grid_fp64, 256, 0, st>>>(a, m);
+    sweep_kernel<D><<<grid_tiles, BAND_THREADS, 0, st>>>(a);
     fp64_kernel<D><<<grid_fp64, 128, 0, st>>>(a);
 }
 
@@ -124,7 +128,7 @@ extern "C" int ebit_advect_sweep_noalloc(int nx, int ny, int nz, double h, int d
     unsigned long long *ctr = (unsigned long long *)(base + OFF_CTR);
 
     // zero what must start at zero: list lengths and counters
-    if (cudaMemsetAsync(ints, 0, 8 * sizeof(int), st) != cudaSuccess) return EBIT_ECUDA;
+    if (cudaMemsetAsync(ints, 0, NA_INTS * sizeof(int), st) != cudaSuccess) return EBIT_ECUDA;
     if (cudaMemsetAsync(ctr, 0, C_TOTAL * sizeof(unsigned long long), st) != cudaSuccess) return EBIT_ECUDA;
     // every tile is processed: the list is 0 .. ntiles-1
     na_tiles_kernel<<<(g.ntiles + 255) / 256, 256, 0, st>>>(list, g.ntiles, ints);
@@ -145,6 +149,8 @@ extern "C" int ebit_advect_sweep_noalloc(int nx, int ny, int nz, double h, int d
     a.list = list;
     a.count = ints;
     a.wcount = ints + 1;
+    a.scan_count = ints + 7;
+    a.cb_whole = ((uintptr_t)cb_in & 7) == 0 ? N & ~7LL : 0;
     a.ctr = ctr;
     a.tile_marker = reinterpret_cast<uint32_t *>(base + OFF_TILES);
     a.tile_dirty = base + OFF_TILES + 4 * NA_MAX_TILES;
@@ -153,10 +159,21 @@ extern "C" int ebit_advect_sweep_noalloc(int nx, int ny, int nz, double h, int d
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int grid_tiles = g.ntiles < sms * 4 ? g.ntiles : sms * 4;
+    const int grid_scan = (int)(((long long)((nx + 7) / 8) * ny * nz + 255) / 256);
+    MarkerLists m;
+    for (int k = 0; k < 3; k++) {
+        m.list[k] = a.work[k];
+        m.count[k] = a.scan_count + k;
+        m.axis[k] = k;
+    }
+    m.mtiles = nullptr;
+    m.mtiles_count = ints + 10;
+    m.band = nullptr;
+    m.band_count = nullptr;
     switch (dir) {
-    case 0: launch_all<0>(a, st, grid_tiles, sms * 4); break;
-    case 1: launch_all<1>(a, st, grid_tiles, sms * 4); break;
-    default: launch_all<2>(a, st, grid_tiles, sms * 4); break;
+    case 0: launch_all<0>(a, m, st, grid_scan, grid_tiles, sms * 4); break;
+    case 1: launch_all<1>(a, m, st, grid_scan, grid_tiles, sms * 4); break;
+    default: launch_all<2>(a, m, st, grid_scan, grid_tiles, sms * 4); break;
     }
     // offsets of edges without a marker set to 0
     na_zero_empty_kernel<<<(int)((N + 255) / 256), 256, 0, st>>>(g, cb_out, s_out);

@@ -16,16 +16,17 @@
 // instruction costs its issue slots whatever the number of active lanes, so all
 // FP64 arithmetic runs from compacted lists with full warps, and the band pass
 // over the cells is integer work:
-//   advect_kernel -- per band tile, the markers owned by the tile are listed in
-//                    shared memory and each is moved once (trilinear velocity):
+//   mark_scan_kernel -- after a state change, the markers of the whole grid
+//                    listed from the colours.
+//   advect_list_kernel -- every listed marker moved once (trilinear velocity):
 //                    adv = its advected coordinate along D relative to its node
 //                    (s + u dt/h for an aligned marker, u dt/h for an unaligned
 //                    one) and bin = floor(2 adv), both in scratch arrays.
-//   sweep_kernel  -- per band tile, one thread per cell, integer only: new node
-//                    colours, aligned edges, canonical face colours; unaligned
-//                    edges that carry a marker and saddle faces are appended to
-//                    global work lists (with six lists, also the unaligned
-//                    edges whose annihilation count needs their crossings).
+//   sweep_kernel  -- (band.cuh) per band tile, integers only: new node colours,
+//                    aligned edges, canonical face colours; unaligned edges that
+//                    carry a marker, saddle faces and unaligned edges whose
+//                    annihilation count needs their crossings go to global
+//                    work lists.
 //   fp64_kernel   -- one thread per list entry (two per unaligned edge when
 //                    the lists are short, the circle fits split between them):
 //                    crossings, circle fits, face phases, crossing counts.
@@ -37,73 +38,15 @@
 // saddle faces are OR-ed into the byte written by the band pass), and old and
 // new state live in separate buffers.
 #pragma once
+#include "band.cuh"
 #include "common.cuh"
+#include "sweep_args.cuh"
 
 namespace ebit {
-
-struct SweepArgs {
-    Grid g;
-    const uint8_t *__restrict__ cb;  // old colour bytes
-    uint8_t *__restrict__ cbo;       // new colour bytes
-    const double *__restrict__ s[3]; // old offsets per edge axis
-    double *__restrict__ so[3];      // new offsets (written only where a marker is)
-    const double *__restrict__ u;    // u_D on D-faces
-    double lam;                      // dt / h
-    double *__restrict__ adv[3];     // advected coordinate of each marker (scratch)
-    int8_t *__restrict__ bin[3];     // floor(2 adv) (scratch)
-    const int *__restrict__ list;    // band tile ids
-    const int *__restrict__ count;   // number of band tiles (device)
-    unsigned *__restrict__ work[6];  // work lists: unaligned fam.1, fam.2, saddle fam.1, fam.2
-                                     // (and, with six lists, annihilation checks fam.1, fam.2)
-    int *__restrict__ wcount;        // [4] or [6] list lengths (device)
-    unsigned long long *ctr;         // event counters
-    uint32_t *tile_marker;           // per tile: proximity mask of its markers in the input or the output
-    uint8_t *tile_dirty;             // per tile: processed since the last Front2VOF
-    // Lists for the next sweep (a context's band sweeps; null elsewhere).  The
-    // band pass appends every aligned edge that carries a marker after the
-    // sweep to mk_out (the unaligned ones are its work lists 0 and 1) and every
-    // tile whose new proximity mask is not empty to mt_out; it clears the band
-    // flag of each tile it processes.  The next sweep's advection builds that
-    // sweep's band from mt_out and the masks.
-    unsigned *mk_out = nullptr;
-    int *mk_out_count = nullptr;
-    int *mt_out = nullptr;
-    int *mt_out_count = nullptr;
-    uint32_t *band_flag = nullptr;
-    // the count of the band list the following sweep builds (cleared here)
-    int *band_next_count = nullptr;
-    // next band tile to take (blocks of the band pass take tiles in turn from
-    // this counter; null: a fixed stride over the list)
-    int *tile_next = nullptr;
-};
-
-// The markers of the state before a sweep, as node ids of their edges, one
-// list per edge axis, and the tiles whose proximity mask is not empty (the
-// previous sweep's band pass wrote them); the band this sweep processes is
-// built from the latter into band / band_count, with band_flag against
-// duplicates.
-struct MarkerLists {
-    const unsigned *list[3];
-    const int *count[3];
-    int axis[3];
-    const int *mtiles;
-    const int *mtiles_count;
-    int *band;
-    int *band_count;
-};
 
 struct P2 {
     double x, y;
 };
-
-// Loads of data produced earlier in the same launch (the persistent batched
-// sweep, F = true) bypass the non-coherent read-only path and L1; separate
-// launches (F = false) read them through the read-only cache.
-template <bool F, typename T>
-__device__ __forceinline__ T ld_in(const T *p) {
-    if (F) return __ldcg(p);
-    return __ldg(p);
-}
 
 // 2D cell edges in a plane spanned by (a, t): B a-edge at c00, R t-edge at c10,
 // T a-edge at c01, L t-edge at c00.
@@ -297,6 +240,59 @@ __device__ __forceinline__ int warp_append(int *counter, bool flag) {
 }
 
 // ---------------------------------------------------------------- advection
+// The markers of the whole grid, one list per edge axis, from the node colours
+// (after a state change, in dense mode and in the allocation-free sweep).  One
+// thread per 8 cells of an x-row: the row's colours and those of the next rows
+// along y and z are 8-bit masks, their exclusive-ors the marked edges; a warp
+// reserves its slots with one round of atomics.  count[3] starts at zero.  (6 us
+// at 128^3; the staged pass per tile that it and the marker lists replace, 24-30.)
+static __global__ void __launch_bounds__(256) mark_scan_kernel(SweepArgs a, unsigned *l0, unsigned *l1, unsigned *l2,
+                                                               int *count) {
+    pdl_wait();
+    const int nx = a.g.n[0], ny = a.g.n[1], nz = a.g.n[2];
+    const long long n = (long long)nx * ny * nz;
+    const int gx = (nx + 7) / 8;
+    const long long groups = (long long)gx * ny * nz;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long t0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); t0 < groups; t0 += stride) {
+        const long long t = t0 + lane;
+        unsigned m[3] = {0, 0, 0};
+        int id = 0;
+        if (t < groups) {
+            const int row = (int)(t / gx), x = 8 * (int)(t - (long long)row * gx);
+            const int z = row / ny, y = row - z * ny;
+            id = row * nx + x;
+            const unsigned ok = nx - x >= 8 ? 0xFFu : (1u << (nx - x)) - 1u;
+            const unsigned c = gather_bits(load_colours8(a.cb, id, a.cb_whole, n));
+            const unsigned cy = gather_bits(load_colours8(a.cb, (long long)(z * ny + wrapc(y + 1, ny)) * nx + x, a.cb_whole, n));
+            const unsigned cz = gather_bits(load_colours8(a.cb, (long long)(wrapc(z + 1, nz) * ny + y) * nx + x, a.cb_whole, n));
+            // the node after the group's last valid one
+            const int last = min(x + 8, nx) - x - 1;
+            const unsigned cn = __ldg(a.cb + row * nx + wrapc(x + last + 1, nx)) & 1u;
+            const unsigned up = (c >> 1 & ~(1u << last)) | cn << last;
+            m[0] = (c ^ up) & ok;
+            m[1] = (c ^ cy) & ok;
+            m[2] = (c ^ cz) & ok;
+        }
+        if (!__any_sync(full, m[0] | m[1] | m[2])) continue;
+        unsigned tot;
+        const unsigned pre = warp_prefix(__popc(m[0]) | __popc(m[1]) << 10 | __popc(m[2]) << 20, &tot);
+        int base = 0;
+        if (lane < 3) {
+            const unsigned c = (tot >> (10 * lane)) & 1023u;
+            if (c) base = atomicAdd(count + lane, (int)c);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            unsigned *l = k == 0 ? l0 : (k == 1 ? l1 : l2);
+            int pos = __shfl_sync(full, base, k) + (int)((pre >> (10 * k)) & 1023u);
+            for (unsigned w = m[k]; w; w &= w - 1) l[pos++] = (unsigned)(id + __ffs((int)w) - 1);
+        }
+    }
+}
+
 // Move every marker of one band tile once (Eq. 2).  CFL >= 1 is counted and
 // clamped; a displacement that is not finite (NaN or infinite velocity) is
 // counted apart and the marker stays where it is.  Called by all threads of the block; s_mk/s_c/s_n are its shared
@@ -361,34 +357,22 @@ __device__ __forceinline__ void advect_tile(const SweepArgs &a, const double *__
 }
 
 // the counters the band pass appends to start at zero (cleared by the launch before it)
-template <int NL>
 __device__ __forceinline__ void clear_sweep_counts(const SweepArgs &a) {
     if (blockIdx.x != 0) return;
-    if (threadIdx.x < NL) a.wcount[threadIdx.x] = 0;
+    if (threadIdx.x < SWEEP_LISTS) a.wcount[threadIdx.x] = 0;
     if (threadIdx.x == 32 && a.mk_out_count) *a.mk_out_count = 0;
     if (threadIdx.x == 33 && a.mt_out_count) *a.mt_out_count = 0;
     if (threadIdx.x == 34 && a.tile_next) *a.tile_next = 0;
     if (threadIdx.x == 35 && a.band_next_count) *a.band_next_count = 0;
 }
 
-template <int D, int NL = 4>
-__global__ void __launch_bounds__(256) advect_kernel(SweepArgs a) {
-    __shared__ uint16_t s_mk[3 * TILE_CELLS];
-    __shared__ uint8_t s_c[9 * 9 * 9];  // node colours of the tile and its +1 layer
-    __shared__ int s_n;
-    pdl_wait();
-    const int ntl = *a.count;
-    clear_sweep_counts<NL>(a);
-    for (int li = blockIdx.x; li < ntl; li += gridDim.x) advect_tile<D>(a, a.u, a.lam, a.list[li], s_mk, s_c, &s_n);
-}
-
 // Advection from the marker lists (Eq. 2): one thread per marker, no tile
 // staging.  Every marker of the state is on a list, so the same markers as in
 // advect_tile are moved, with the same arithmetic.
-template <int D, int NL = 4>
+template <int D>
 __global__ void __launch_bounds__(256) advect_list_kernel(SweepArgs a, MarkerLists m) {
     pdl_wait();
-    clear_sweep_counts<NL>(a);
+    clear_sweep_counts(a);
     // One index space: the markers, then this sweep's band items (tile of the
     // marker-tile list, direction); a thread takes one item per round, so the
     // two kinds of work run side by side rather than one after the other.
@@ -725,348 +709,14 @@ struct SweepCell {
     }
 };
 
-__device__ __forceinline__ bool saddle4(int c00, int c10, int c01, int c11) {
-    return c00 == c11 && c10 == c01 && c00 != c10;
-}
-
-// ------------------------------------------------------- band pass (integer)
-// staged colour region of a tile, in sweep-local axes: A in [-1, TA + 1], T1
-// in [0, T1], T2 in [0, T2] relative to the tile origin (TA, T1, T2: the
-// tile's edges along the sweep axis and the two others)
-__host__ __device__ constexpr int tile_edge(int sh, int a) { return 1 << tile_log2(sh, a); }
-__host__ __device__ constexpr int stage_n(int d, int sh) {
-    return (tile_edge(sh, d) + 3) * (tile_edge(sh, (d + 1) % 3) + 1) * (tile_edge(sh, (d + 2) % 3) + 1);
-}
-template <int D, int SH>
-struct Stage {
-    static constexpr int RA = tile_edge(SH, D) + 3, R1 = tile_edge(SH, (D + 1) % 3) + 1,
-                         R2 = tile_edge(SH, (D + 2) % 3) + 1;
-};
-// the largest staged region over directions and shapes, and the largest
-// colour block of advect_tile
-__host__ __device__ constexpr int stage_max() {
-    int m = 0;
-    for (int sh = 0; sh < N_TILE_SHAPES; sh++)
-        for (int d = 0; d < 3; d++) m = stage_n(d, sh) > m ? stage_n(d, sh) : m;
-    return m;
-}
-__host__ __device__ constexpr int adv_stage_max() {
-    int m = 0;
-    for (int sh = 0; sh < N_TILE_SHAPES; sh++) {
-        const int v = (tile_edge(sh, 0) + 1) * (tile_edge(sh, 1) + 1) * (tile_edge(sh, 2) + 1);
-        m = v > m ? v : m;
-    }
-    return m;
-}
-constexpr int RA = 11, R1 = 9, R2 = 9;  // 8^3 tiles (every direction)
-static_assert(stage_n(0, 0) == RA * R1 * R2, "8^3 staging");
-
-// One band tile, all threads of the block; s_b/s_n/s_flag are its shared
-// staging (colour bytes and the A-axis bins of the same window; a bin is read
-// only where its node owns a marker).
-// NL = 6: an unaligned edge without a marker whose window shows a colour change
-// goes to work list 4 or 5 (the crossing count of the annihilation counter is
-// taken by the FP64-list kernel, with full warps); NL = 4: counted here.
-template <int D, bool F, int NL = 4, int SH = 0>
-__device__ __forceinline__ int sweep_tile(const SweepArgs &a, int tile, uint8_t *s_b, int8_t *s_n, unsigned *s_flag) {
-    constexpr int A = D, T1 = (D + 1) % 3, T2 = (D + 2) % 3;
-    using S = TileShape<SH>;
-    constexpr int RA = Stage<D, SH>::RA, R1 = Stage<D, SH>::R1, R2 = Stage<D, SH>::R2;
-    {
-        int o[3];
-        tile_origin(a.g, tile, o);
-        if (threadIdx.x == 0) *s_flag = 0;
-        // walk the region in global order (x fastest), so that a warp's loads
-        // fall on a few rows of the grid whatever the sweep axis; the staged
-        // copy is indexed in sweep-local order (A fastest)
-        constexpr int E0 = A == 0 ? RA : (T1 == 0 ? R1 : R2);
-        constexpr int E1 = A == 1 ? RA : (T1 == 1 ? R1 : R2);
-        int seen = 0;  // bit 0: a staged node of colour 1, bit 1: one of colour 0
-        for (int r = threadIdx.x; r < RA * R1 * R2; r += blockDim.x) {
-            const int gl[3] = {r % E0, (r / E0) % E1, r / (E0 * E1)};
-            const int ka = gl[A], k1 = gl[T1], k2 = gl[T2];
-            int q[3];
-            q[A] = o[A] + ka - 1;
-            q[T1] = o[T1] + k1;
-            q[T2] = o[T2] + k2;
-            const int id = lin3(a.g, q);
-            const int sr = ka + RA * (k1 + R1 * k2);
-            const uint8_t b = __ldg(a.cb + id);
-            seen |= (b & 1) ? 1 : 2;
-            s_b[sr] = b;
-            s_n[sr] = ld_in<F>(a.bin[A] + id);
-        }
-        // (__syncthreads_or returns whether any thread's value is non-zero)
-        const int has1 = __syncthreads_or(seen & 1), has0 = __syncthreads_or(seen & 2);
-        if (!(has1 && has0)) {
-            // Every staged node has one colour: no marker lies on an edge whose
-            // crossing could change a node, face or edge of this tile's cells,
-            // so the sweep leaves them as they are (the band pass's uniform
-            // window, for the whole tile): canonical colour bytes, no markers,
-            // no work, and nothing for Front2VOF to redo.
-            const uint8_t byte = has1 ? 0x0F : 0x00;
-            for (int c = threadIdx.x; c < TILE_CELLS; c += blockDim.x) {
-                int l[3];
-                S::cell(c, l);
-                const int x = o[0] + l[0], y = o[1] + l[1], z = o[2] + l[2];
-                if (x < a.g.n[0] && y < a.g.n[1] && z < a.g.n[2]) a.cbo[lin(a.g, x, y, z)] = byte;
-            }
-            if (threadIdx.x == 0) {
-                a.tile_marker[tile] = 0u;
-                if (a.band_flag) a.band_flag[tile] = 0u;
-            }
-            return -1;
-        }
-        unsigned ev[C_N] = {0, 0, 0, 0, 0};
-        unsigned mk = 0;  // proximity mask of the markers of this thread's cells
-        for (int c = threadIdx.x; c < TILE_CELLS; c += blockDim.x) {
-            int l[3];
-            S::cell(c, l);
-            int x = o[0] + l[0], y = o[1] + l[1], z = o[2] + l[2];
-            bool valid = x < a.g.n[0] && y < a.g.n[1] && z < a.g.n[2];
-            bool push[6] = {false, false, false, false, false, false};
-            bool push_al = false;
-            int myid = 0;
-            if (valid) {
-                myid = lin(a.g, x, y, z);
-                // staged index of node (da, d1, d2) relative to the cell
-                const int r0 = (l[A] + 1) + RA * (l[T1] + R1 * l[T2]);
-                auto sidx = [&](int da, int d1, int d2) { return r0 + da + RA * (d1 + R1 * d2); };
-                int col[4][2][2];
-                const int myb = s_b[r0];
-                const int c0 = myb & 1;
-                int any = 0;
-#pragma unroll
-                for (int da = 0; da < 4; da++)
-#pragma unroll
-                    for (int d1 = 0; d1 < 2; d1++)
-#pragma unroll
-                        for (int d2 = 0; d2 < 2; d2++) {
-                            int v = s_b[sidx(da - 1, d1, d2)] & 1;
-                            col[da][d1][d2] = v;
-                            any |= v ^ c0;
-                        }
-                if (!any) {
-                    a.cbo[myid] = (uint8_t)(c0 | (c0 << 1) | (c0 << 2) | (c0 << 3));
-                } else {
-                    bool in_marker = (c0 != col[2][0][0]) || (c0 != col[1][1][0]) || (c0 != col[1][0][1]);
-                    // bins of the aligned markers on the A-edges (da in {-1,0,1}) of 4 lines
-                    int bn[3][2][2];
-                    bool has[3][2][2];
-#pragma unroll
-                    for (int da = 0; da < 3; da++)
-#pragma unroll
-                        for (int d1 = 0; d1 < 2; d1++)
-#pragma unroll
-                            for (int d2 = 0; d2 < 2; d2++) {
-                                has[da][d1][d2] = col[da][d1][d2] != col[da + 1][d1][d2];
-                                bn[da][d1][d2] = has[da][d1][d2] ? (int)s_n[sidx(da - 1, d1, d2)] : 0;
-                            }
-                    // new colours: X >= 1 <=> bin >= 2 (crossed the right node),
-                    // X < 0 <=> bin < 0 (crossed the left node)  (Fig. 4)
-                    int nc[2][2][2];
-#pragma unroll
-                    for (int dA = 0; dA < 2; dA++)
-#pragma unroll
-                        for (int d1 = 0; d1 < 2; d1++)
-#pragma unroll
-                            for (int d2 = 0; d2 < 2; d2++) {
-                                int v = col[dA + 1][d1][d2];
-                                if (has[dA][d1][d2] && bn[dA][d1][d2] >= 2) v ^= 1;
-                                if (has[dA + 1][d1][d2] && bn[dA + 1][d1][d2] < 0) v ^= 1;
-                                nc[dA][d1][d2] = v;
-                            }
-                    const int n0 = nc[0][0][0];
-                    bool out_marker = false;
-                    // aligned edge (Fig. 5): presence from the new colours, landing markers
-                    {
-                        bool present = n0 != nc[1][0][0];
-                        int land[3], nl = 0;
-#pragma unroll
-                        for (int e = -1; e <= 1; e++) {
-                            if (!has[e + 1][0][0]) continue;
-                            int b = bn[e + 1][0][0];
-                            int dest = (b < 0) ? -1 : (b >= 2 ? 1 : 0);
-                            if (e + dest != 0) continue;
-                            land[nl++] = e;
-                        }
-                        if (present) {
-                            double v;
-                            if (nl == 1 || nl == 3) {
-                                double sv[3];
-                                for (int k = 0; k < nl; k++) {
-                                    double xv = ld_in<F>(a.adv[A] + lin(a.g, x + (A == 0 ? land[k] : 0), y + (A == 1 ? land[k] : 0),
-                                                                      z + (A == 2 ? land[k] : 0)));
-                                    double sn = xv - (double)(-land[k]);
-                                    if (sn > ONE_MINUS) sn = ONE_MINUS;
-                                    sv[k] = sn;
-                                }
-                                if (nl == 1) {
-                                    v = sv[0];
-                                } else {
-                                    double a0 = sv[0], a1 = sv[1], a2 = sv[2], tmp;
-                                    if (a0 > a1) { tmp = a0; a0 = a1; a1 = tmp; }
-                                    if (a1 > a2) { tmp = a1; a1 = a2; a2 = tmp; }
-                                    if (a0 > a1) { tmp = a0; a0 = a1; a1 = tmp; }
-                                    v = a1;
-                                    ev[C_MULTI]++;
-                                }
-                            } else {
-                                v = 0.5;
-                                ev[C_INCONSISTENT]++;
-                            }
-                            a.so[A][myid] = v;
-                            ev[C_MARKERS]++;
-                            out_marker = true;
-                            push_al = true;
-                        } else if (nl >= 2) {
-                            ev[C_ANNIHILATE]++;
-                        }
-                    }
-                    // unaligned edges: a marker -> FP64 list; none -> count the
-                    // crossings that met there (topology change, Fig. 5)
-                    const int m = col[0][0][0];
-                    const bool pres1 = n0 != nc[0][1][0];
-                    const bool pres2 = n0 != nc[0][0][1];
-                    push[0] = pres1;
-                    push[1] = pres2;
-                    const bool chk1 = !pres1 && ((col[1][0][0] ^ m) | (col[2][0][0] ^ m) | (col[0][1][0] ^ m) |
-                                                 (col[1][1][0] ^ m) | (col[2][1][0] ^ m));
-                    const bool chk2 = !pres2 && ((col[1][0][0] ^ m) | (col[2][0][0] ^ m) | (col[0][0][1] ^ m) |
-                                                 (col[1][0][1] ^ m) | (col[2][0][1] ^ m));
-                    if (NL == 6) {
-                        push[4] = chk1;
-                        push[5] = chk2;
-                    } else {
-                        for (int fam = 0; fam < 2; fam++) {
-                            if (!(fam ? chk2 : chk1)) continue;
-                            SweepCell<D, F> cell(a, myid, x, y, z, fam);
-                            cell.loadw();
-                            if (cell.count_crossings(cell.left_bits()) >= 2) ev[C_ANNIHILATE]++;
-                        }
-                    }
-                    out_marker |= pres1 || pres2;
-                    // face colours: family 1 faces are normal to T2, family 2 to T1
-                    int byte = n0;
-                    push[2] = saddle4(n0, nc[1][0][0], nc[0][1][0], nc[1][1][0]);
-                    if (!push[2]) byte |= n0 << (1 + T2);
-                    push[3] = saddle4(n0, nc[1][0][0], nc[0][0][1], nc[1][0][1]);
-                    if (!push[3]) byte |= n0 << (1 + T1);
-                    int fa = saddle4(n0, nc[0][1][0], nc[0][0][1], nc[0][1][1]) ? ((myb >> (1 + A)) & 1) : n0;
-                    byte |= fa << (1 + A);
-                    a.cbo[myid] = (uint8_t)byte;
-                    if (in_marker || out_marker) mk |= near_bits(l[0], l[1], l[2], S::TX, S::TY, S::TZ);
-                }
-            }
-            // the warp's appends to the NL work lists and the marker list: all
-            // ballots first, then lane 0 reserves every list's slots with
-            // independent atomics (one round trip to L2 for all of them); a
-            // warp with nothing to append (cells away from the interface)
-            // skips it after one vote
-            bool any_push = push_al;
-#pragma unroll
-            for (int k = 0; k < NL; k++) any_push |= push[k];
-            if (__any_sync(0xffffffffu, any_push)) {
-                const unsigned full = 0xffffffffu;
-                const int lane = threadIdx.x & 31;
-                unsigned m[NL + 1];
-                int base[NL + 1];
-#pragma unroll
-                for (int k = 0; k < NL; k++) m[k] = __ballot_sync(full, push[k]);
-                m[NL] = a.mk_out ? __ballot_sync(full, push_al) : 0u;
-#pragma unroll
-                for (int k = 0; k <= NL; k++) base[k] = 0;
-                if (lane == 0) {
-#pragma unroll
-                    for (int k = 0; k < NL; k++)
-                        if (m[k]) base[k] = atomicAdd(a.wcount + k, __popc(m[k]));
-                    if (m[NL]) base[NL] = atomicAdd(a.mk_out_count, __popc(m[NL]));
-                }
-                const unsigned below = (1u << lane) - 1u;
-#pragma unroll
-                for (int k = 0; k < NL; k++) {
-                    const int b = __shfl_sync(full, base[k], 0);
-                    if (push[k]) a.work[k][b + __popc(m[k] & below)] = (unsigned)myid;
-                }
-                const int b = __shfl_sync(full, base[NL], 0);
-                if (push_al && a.mk_out) a.mk_out[b + __popc(m[NL] & below)] = (unsigned)myid;
-            }
-        }
-        {
-            const unsigned v = __reduce_or_sync(0xffffffffu, mk);
-            if ((threadIdx.x & 31) == 0 && v) atomicOr(s_flag, v);
-        }
-        if (__any_sync(0xffffffffu, (ev[0] | ev[1] | ev[2] | ev[3] | ev[4]) != 0u)) {
-#pragma unroll
-            for (int k = 0; k < C_N; k++) {
-                unsigned v = __reduce_add_sync(0xffffffffu, ev[k]);
-                if ((threadIdx.x & 31) == 0 && v) atomicAdd(a.ctr + k, (unsigned long long)v);
-            }
-        }
-        __syncthreads();
-        int pending = -1;
-        if (threadIdx.x == 0) {
-            const unsigned fl = *s_flag;
-            a.tile_marker[tile] = fl;
-            a.tile_dirty[tile] = 1;
-            if (a.band_flag) a.band_flag[tile] = 0u;
-            // a slot on the list of tiles with markers nearby; the caller
-            // stores the tile id there later, so that nothing waits for it
-            if (a.mt_out && fl) pending = atomicAdd(a.mt_out_count, 1);
-        }
-        __syncthreads();
-        return pending;
-    }
-}
-
-template <int D, int NL = 4>
-__global__ void __launch_bounds__(256, 4) sweep_kernel(SweepArgs a) {
-    __shared__ unsigned s_flag;
-    __shared__ uint8_t s_b[RA * R1 * R2];
-    __shared__ int8_t s_n[RA * R1 * R2];
-    __shared__ int s_li;
-    pdl_wait();
-    const int ntl = *a.count;
-    // the previous tile's slot on the marker-tile list (thread 0), stored one
-    // tile later so that the atomic that reserved it is not waited for
-    int pending = -1, pending_tile = 0;
-    if (a.tile_next) {
-        // tiles differ in cost (interface tiles against halo tiles): each block
-        // takes the next one when it is done, the counter read one tile ahead.
-        // Every thread reads s_li before the first barrier inside sweep_tile,
-        // and thread 0 rewrites it only after the last one.
-        int next = threadIdx.x == 0 ? atomicAdd(a.tile_next, 1) : 0;
-        for (;;) {
-            if (threadIdx.x == 0) s_li = next;
-            __syncthreads();
-            const int li = s_li;
-            if (li >= ntl) break;
-            if (threadIdx.x == 0) {
-                next = atomicAdd(a.tile_next, 1);
-                if (pending >= 0) a.mt_out[pending] = pending_tile;
-            }
-            pending_tile = a.list[li];
-            pending = sweep_tile<D, false, NL>(a, pending_tile, s_b, s_n, &s_flag);
-        }
-    } else {
-        for (int li = blockIdx.x; li < ntl; li += gridDim.x) {
-            if (threadIdx.x == 0 && pending >= 0) a.mt_out[pending] = pending_tile;
-            pending_tile = a.list[li];
-            pending = sweep_tile<D, false, NL>(a, pending_tile, s_b, s_n, &s_flag);
-        }
-    }
-    if (threadIdx.x == 0 && pending >= 0) a.mt_out[pending] = pending_tile;
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(a.ctr + C_TILES, (unsigned long long)ntl);
-}
-
-
 // ------------------------------------------------- FP64 work lists
 // Entry k of list `kind` (0, 1: unaligned edges of families 1, 2; 2, 3: saddle
-// faces of families 1, 2).
+// faces; 4, 5: annihilation checks, from the ends of lists 0, 1).
 template <int D, bool F>
 __device__ __forceinline__ void fp64_item(const SweepArgs &a, int kind, int k, unsigned ev[C_N], int half = -1) {
     constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
-    const int id = (int)ld_in<F>(a.work[kind] + k);
+    const int id = (int)ld_in<F>(kind < 4 ? a.work[kind] + k
+                                          : a.work[kind - 4] + (a.g.n[0] * a.g.n[1] * a.g.n[2] - 1 - k));
     const int x = id % a.g.n[0], y = (id / a.g.n[0]) % a.g.n[1], z = id / (a.g.n[0] * a.g.n[1]);
     SweepCell<D, F> cell(a, id, x, y, z, kind & 1);
     cell.loadw();
@@ -1088,11 +738,11 @@ __device__ __forceinline__ void fp64_item(const SweepArgs &a, int kind, int k, u
     }
 }
 
-template <int D, int NL = 4>
+template <int D>
 __global__ void __launch_bounds__(128, 8) fp64_kernel(SweepArgs a) {
     pdl_wait();
     const int n0 = a.wcount[0], n1 = a.wcount[1], n2 = a.wcount[2], n3 = a.wcount[3];
-    const int n4 = NL == 6 ? a.wcount[4] : 0, n5 = NL == 6 ? a.wcount[5] : 0;
+    const int n4 = a.wcount[4], n5 = a.wcount[5];
     const int total = n0 + n1 + n2 + n3 + n4 + n5;
     unsigned ev[C_N] = {0, 0, 0, 0, 0};
     const int stride = gridDim.x * blockDim.x;
