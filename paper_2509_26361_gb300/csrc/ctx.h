@@ -60,8 +60,7 @@ struct ebit_ctx {
     int f2v_buf;
     int *band_list, *band_count;  // band_count[2]: the lengths of band_list and band_list2
     int band_last;                // slot of the last sweep's band list (-1: every tile)
-    int *work_list, *work_count;  // work_count[2]: one slot per incremental Front2VOF parity
-    int f2v_par;
+    int f2v_par;              // slot of ncut that the last Front2VOF wrote
     int *all_list, *all_count;
     unsigned long long *ctr;  // C_N event counters + Front2VOF inconsistencies
     double *scratch;          // 3N doubles, allocated on first ebit_get_state
@@ -88,7 +87,7 @@ struct ebit_ctx {
     int mk_dir;               // sweep axis of the last sweep
     int mk_valid;             // the lists of set mk_par describe the current state
     unsigned *cut;            // cells cut by the interface at the last Front2VOF
-    int *ncut;
+    int *ncut;                // [2] its length, one slot per Front2VOF call modulo 2
     unsigned *iface[2];       // interface cells of the last two curvature calls
     int *niface;              // [3] list lengths, one slot per curvature call modulo 3
     int cur_if;               // list buffer of the last curvature call

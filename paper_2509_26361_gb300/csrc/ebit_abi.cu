@@ -253,7 +253,7 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
     ctx->own_mlp = nullptr;
     ctx->tile_marker = nullptr;
     ctx->tile_dirty = ctx->tile_cchg = nullptr;
-    ctx->band_list = ctx->band_count = ctx->work_list = ctx->work_count = ctx->all_list = ctx->all_count = nullptr;
+    ctx->band_list = ctx->band_count = ctx->all_list = ctx->all_count = nullptr;
     ctx->ctr = nullptr;
     ctx->g.n[0] = desc->nx;
     ctx->g.n[1] = desc->ny;
@@ -319,11 +319,11 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
     ok = ok && alloc((void **)&ctx->cut, ctx->N * sizeof(unsigned)) && alloc((void **)&ctx->scan, ctx->N * sizeof(unsigned)) &&
          alloc((void **)&ctx->iface[0], ctx->N * sizeof(unsigned)) &&
          alloc((void **)&ctx->iface[1], ctx->N * sizeof(unsigned)) &&
-         alloc((void **)&ctx->ncut, sizeof(int)) && alloc((void **)&ctx->niface, 3 * sizeof(int)) &&
+         alloc((void **)&ctx->ncut, 2 * sizeof(int)) && alloc((void **)&ctx->niface, 3 * sizeof(int)) &&
          alloc((void **)&ctx->nscan, sizeof(int)) && alloc((void **)&ctx->zero, sizeof(int));
     ok = ok && alloc((void **)&ctx->tile_cchg, ntc) && alloc((void **)&ctx->band_list, ntc * sizeof(int)) &&
-         alloc((void **)&ctx->band_count, 2 * sizeof(int)) && alloc((void **)&ctx->work_list, ntc * sizeof(int)) &&
-         alloc((void **)&ctx->work_count, 2 * sizeof(int)) && alloc((void **)&ctx->all_list, ntc * sizeof(int)) &&
+         alloc((void **)&ctx->band_count, 2 * sizeof(int)) &&
+         alloc((void **)&ctx->all_list, ntc * sizeof(int)) &&
          alloc((void **)&ctx->all_count, sizeof(int));
     if (!ok) {
         cudaGetLastError();
@@ -337,7 +337,7 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
     ctx->grid_advl = ctx->sms * std::max(occ, 1);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fp64_kernel<0>, 128, 0);
     ctx->grid_fp64 = ctx->sms * std::max(occ, 1);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f2v_band_kernel, 256, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f2v_band_kernel<0>, 64, 0);
     ctx->grid_f2v = std::max(1, std::min(ntc, ctx->sms * std::max(occ, 1)));
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f2v_list_kernel, 128, 0);
     ctx->grid_f2vl = ctx->sms * std::max(occ, 1);
@@ -352,10 +352,9 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
         cudaMemsetAsync(ctx->scan_count, 0, 3 * sizeof(int), ctx->stream);
         cudaMemsetAsync(ctx->mt_count, 0, 2 * sizeof(int), ctx->stream);
     }
-    cudaMemsetAsync(ctx->ncut, 0, sizeof(int), ctx->stream);
+    cudaMemsetAsync(ctx->ncut, 0, 2 * sizeof(int), ctx->stream);
     cudaMemsetAsync(ctx->niface, 0, 3 * sizeof(int), ctx->stream);
     cudaMemsetAsync(ctx->band_count, 0, 2 * sizeof(int), ctx->stream);
-    cudaMemsetAsync(ctx->work_count, 0, 2 * sizeof(int), ctx->stream);
     cudaMemsetAsync(ctx->nscan, 0, sizeof(int), ctx->stream);
     cudaMemsetAsync(ctx->zero, 0, sizeof(int), ctx->stream);
     iota_kernel<<<blocks_for(nt, 256, ctx->sms), 256, 0, ctx->stream>>>(ctx->all_list, nt, ctx->all_count);
@@ -441,8 +440,6 @@ void ebit_destroy(ebit_ctx *ctx) {
     dev_free(ctx->mem, ctx->tile_cchg);
     dev_free(ctx->mem, ctx->band_list);
     dev_free(ctx->mem, ctx->band_count);
-    dev_free(ctx->mem, ctx->work_list);
-    dev_free(ctx->mem, ctx->work_count);
     dev_free(ctx->mem, ctx->all_list);
     dev_free(ctx->mem, ctx->all_count);
     dev_free(ctx->mem, ctx->scratch);
@@ -732,52 +729,39 @@ int ebit_advect_sweep(ebit_ctx *ctx, int dir, const double *u_face, double dt) {
 
 int ebit_front2vof(ebit_ctx *ctx, double *C, int flags) {
     if (!ctx || !C) return fail(ctx, EBIT_EINVAL, "ebit_front2vof: null argument");
-    const int *list, *count;
     bool full = (flags & EBIT_FULL) || ctx->dense || C != ctx->last_C;
     // nothing was swept since the last call on this buffer: C is current
     if (!full && ctx->sweeps_since_f2v == 0) return EBIT_OK;
     cudaStream_t st;
     if (int r = call_stream(ctx, flags, &st)) return r;
-    // this call consumes the dirty set the sweeps since the last call marked;
-    // the next sweeps mark the other one (a batch view has one set)
-    uint8_t *dirty = ctx->dirty_set ? ctx->tile_dirty2 : ctx->tile_dirty;
-    if (ctx->tile_dirty2) ctx->dirty_set ^= 1;
-    if (full) {
-        CU(cudaMemsetAsync(ctx->ncut, 0, sizeof(int), st));
-        CU(cudaMemsetAsync(dirty, 0, ctx->g.ntiles, st));
-        list = ctx->all_list;
-        count = ctx->all_count;
-    } else {
-        // work_count[fp] is 0; the tile-list kernel clears the other slot for
-        // the next incremental call, and the cut-cell count (its readers, the
-        // previous Front2VOF and curvature, are complete)
-        ProfScope ps(ctx, EBIT_PROF_F2V, st);
-        const int fp = ctx->f2v_par;
-        int r = launched(ctx,
-                         launch_pdl(take_flagged_kernel, blocks_for(ctx->g.ntiles, 256, ctx->sms), 256, 0, st,
-                                    ctx->g, dirty, ctx->work_list, ctx->work_count + fp,
-                                    ctx->work_count + (fp ^ 1), ctx->ncut),
-                         "take_flagged_kernel");
-        if (r) return r;
-        list = ctx->work_list;
-        count = ctx->work_count + fp;
-        ctx->f2v_par = fp ^ 1;
-    }
     F2VArgs a;
     a.g = ctx->g;
     int c = ctx->cur;
     a.cb = ctx->cb[c];
+    a.cb_whole = (ctx->N + 7) & ~7LL;
     for (int k = 0; k < 3; k++) a.s[k] = ctx->s[c][k];
     a.C = C;
-    a.list = list;
-    a.count = count;
+    // this call consumes the dirty set the sweeps since the last call marked;
+    // the next sweeps mark the other one (a batch view has one set)
+    a.dirty = ctx->dirty_set ? ctx->tile_dirty2 : ctx->tile_dirty;
+    if (ctx->tile_dirty2) ctx->dirty_set ^= 1;
+    a.full = full ? 1 : 0;
     a.cut = ctx->cut;
-    a.ncut = ctx->ncut;
+    // ncut[fp] is 0: the previous call cleared it (the readers of that slot, the
+    // Front2VOF before and its curvature, were complete then)
+    const int fp = ctx->f2v_par ^ 1;
+    a.ncut = ctx->ncut + fp;
+    a.zero = ctx->ncut + (fp ^ 1);
     a.bad = ctx->ctr + C_F2V_BAD;
+    ctx->f2v_par = fp;
     int r;
     {
         ProfScope ps(ctx, EBIT_PROF_F2V, st);
-        r = launched(ctx, launch_pdl(f2v_band_kernel, ctx->grid_f2v, 256, 0, st, a), "f2v_band_kernel");
+        // one instantiation per tile shape (a batch instance may be re-tiled)
+        const cudaError_t e = ctx->g.tl[0] == 3   ? launch_pdl(f2v_band_kernel<0>, ctx->grid_f2v, 64, 0, st, a)
+                              : ctx->g.tl[0] == 4 ? launch_pdl(f2v_band_kernel<1>, ctx->grid_f2v, 64, 0, st, a)
+                                                  : launch_pdl(f2v_band_kernel<2>, ctx->grid_f2v, 64, 0, st, a);
+        r = launched(ctx, e, "f2v_band_kernel");
     }
     if (r) return r;
     {
@@ -838,7 +822,7 @@ int ebit_curvature(ebit_ctx *ctx, const double *C, double *kappa_h, uint8_t *sta
         a.prev = ctx->iface[ctx->cur_if];
         a.nprev = ctx->niface + cprev;
         a.cand = ctx->cut;
-        a.ncand = ctx->ncut;
+        a.ncand = ctx->ncut + ctx->f2v_par;
         // the fallback list of the learned pass below starts empty
         if (mode != EBIT_CURV_HF) a.zero[1] = ctx->nscan;
     }

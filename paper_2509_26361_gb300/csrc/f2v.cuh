@@ -11,6 +11,7 @@
 // where A_a1 is the reference-phase area on the cube face a = 1 (the faces
 // through the origin contribute nothing).  C = V clamped to [0, 1].
 #pragma once
+#include "band.cuh"
 #include "common.cuh"
 
 namespace ebit {
@@ -29,192 +30,112 @@ struct F2VArgs {
     const uint8_t *__restrict__ cb;
     const double *__restrict__ s[3];
     double *__restrict__ C;
-    const int *__restrict__ list;    // tiles to recompute
-    const int *__restrict__ count;
+    long long cb_whole;              // see load_colours8
+    uint8_t *__restrict__ dirty;     // per tile: swept since the last call (cleared here)
+    int full;                        // take every tile
     unsigned *__restrict__ cut;      // cells cut by the interface (output list)
-    int *__restrict__ ncut;
+    int *__restrict__ ncut;          // its length (0 on entry)
+    int *__restrict__ zero;          // the length of the next call's list, cleared here
     unsigned long long *bad;
 };
-
-struct V3 {
-    double x[3];
-};
-
-__device__ __forceinline__ V3 corner3(int c) {
-    V3 r;
-    r.x[0] = (double)(c & 1);
-    r.x[1] = (double)((c >> 1) & 1);
-    r.x[2] = (double)((c >> 2) & 1);
-    return r;
-}
-
-__device__ __forceinline__ double det3(const V3 &c, const V3 &p, const V3 &q) {
-    return c.x[0] * (p.x[1] * q.x[2] - p.x[2] * q.x[1]) + c.x[1] * (p.x[2] * q.x[0] - p.x[0] * q.x[2]) +
-           c.x[2] * (p.x[0] * q.x[1] - p.x[1] * q.x[0]);
-}
-
-// |area| of a polygon on a face, projected on the face axes (u, v)
-__device__ __forceinline__ double area_uv(const V3 *pts, int np, int u, int v) {
-    double acc = 0.0;
-    for (int i = 0; i < np; i++) {
-        const V3 &a = pts[i];
-        const V3 &b = pts[i + 1 == np ? 0 : i + 1];
-        acc += a.x[u] * b.x[v] - b.x[u] * a.x[v];
-    }
-    return 0.5 * fabs(acc);
-}
-
-// volume fraction of one cell; *bad set on an inconsistent configuration
-__device__ __noinline__ double cell_fraction(int K, const int F[6], const double E[12], int *bad) {
-    V3 mk[12];
-    for (int e = 0; e < 12; e++) {
-        int ax = e >> 2, r = e & 3;
-        V3 p;
-        if (ax == 0) { p.x[0] = E[e]; p.x[1] = (double)(r & 1); p.x[2] = (double)(r >> 1); }
-        else if (ax == 1) { p.x[0] = (double)(r & 1); p.x[1] = E[e]; p.x[2] = (double)(r >> 1); }
-        else { p.x[0] = (double)(r & 1); p.x[1] = (double)(r >> 1); p.x[2] = E[e]; }
-        mk[e] = p;
-    }
-    int8_t out[12];
-    for (int e = 0; e < 12; e++) out[e] = -1;
-    unsigned hasmask = 0;
-    double A1[3] = {0.0, 0.0, 0.0};
-    for (int f = 0; f < 6; f++) {
-        int kc[4], col[4], ed[4], mm[4], nm = 0;
-        for (int k = 0; k < 4; k++) {
-            kc[k] = kFaceCorner[f][k];
-            col[k] = (K >> kc[k]) & 1;
-            ed[k] = kFaceEdge[f][k];
-        }
-        for (int k = 0; k < 4; k++) {
-            mm[k] = col[k] != col[(k + 1) & 3];
-            nm += mm[k];
-            if (mm[k]) hasmask |= 1u << ed[k];
-        }
-        const int upper = f & 1, fa = f >> 1;
-        const int u = fa == 2 ? 0 : fa + 1, v = fa == 0 ? 2 : (fa == 1 ? 0 : 1);
-        double area1 = 0.0;
-        if (nm == 0) {
-            area1 = (double)col[0];
-        } else if (nm == 2) {
-            int ea = -1, eb = -1;
-            for (int k = 0; k < 4; k++)
-                if (mm[k]) {
-                    if (ea < 0) ea = k;
-                    else eb = k;
-                }
-            int arc = col[(ea + 1) & 3];
-            if (arc) out[ed[eb]] = (int8_t)ed[ea];
-            else out[ed[ea]] = (int8_t)ed[eb];
-            if (upper) {
-                V3 poly[6];
-                int np = 0;
-                poly[np++] = mk[ed[ea]];
-                for (int k = ea + 1; k <= eb; k++) poly[np++] = corner3(kc[k]);
-                poly[np++] = mk[ed[eb]];
-                double R = area_uv(poly, np, u, v);
-                area1 = arc ? R : 1.0 - R;
-            }
-        } else if (nm == 4) {
-            int phif = F[f];
-            double T = 0.0;
-            for (int m = 0; m < 4; m++) {
-                if (col[m] == phif) continue;
-                int ep = ed[(m + 3) & 3], en = ed[m];
-                if (col[m]) out[en] = (int8_t)ep;
-                else out[ep] = (int8_t)en;
-                if (upper) {
-                    V3 tri[3] = {mk[ep], corner3(kc[m]), mk[en]};
-                    T += area_uv(tri, 3, u, v);
-                }
-            }
-            area1 = (1 - phif) ? T : 1.0 - T;
-        } else {
-            *bad = 1;
-        }
-        if (upper) A1[fa] = area1;
-    }
-    if (!hasmask) return (double)(K & 1);
-    unsigned vis = 0;
-    double acc = 0.0;
-    for (int e0 = 0; e0 < 12; e0++) {
-        if (!((hasmask >> e0) & 1) || ((vis >> e0) & 1)) continue;
-        int idx[12];
-        int len = 0, e = e0;
-        while (len < 12) {
-            if (e < 0 || !((hasmask >> e) & 1) || ((vis >> e) & 1)) break;
-            vis |= 1u << e;
-            idx[len++] = e;
-            e = out[e];
-            if (e == e0) break;
-        }
-        if (e != e0) {
-            *bad = 1;
-            continue;
-        }
-        V3 cen;
-        for (int a = 0; a < 3; a++) {
-            double sm = 0.0;
-            for (int i = 0; i < len; i++) sm += mk[idx[i]].x[a];
-            cen.x[a] = sm / (double)len;
-        }
-        for (int i = 0; i < len; i++) acc += det3(cen, mk[idx[i]], mk[idx[i + 1 == len ? 0 : i + 1]]);
-    }
-    double V = ((A1[0] + A1[1]) + A1[2]) / 3.0 - acc / 6.0;
-    if (V < 0.0) V = 0.0;
-    if (V > 1.0) V = 1.0;
-    return V;
-}
 
 __device__ __forceinline__ void cell_ids(const Grid &g, int x, int y, int z, int ids[8]) {
 #pragma unroll
     for (int cid = 0; cid < 8; cid++) ids[cid] = lin(g, x + (cid & 1), y + ((cid >> 1) & 1), z + ((cid >> 2) & 1));
 }
 
-// Band pass (integer only): a cell with eight equal corner colours holds no
-// marker and its fraction is that colour (written as a bit pattern); the other
-// cells go to the global cut list.
-__global__ void __launch_bounds__(256) f2v_band_kernel(F2VArgs a) {
+// Band pass (integers only) over the tiles swept since the last call: a cell
+// with eight equal corner colours holds no marker and its fraction is that
+// colour (written as a bit pattern); the others go to the global cut list (their
+// fraction is written by the list kernel).
+//
+// 64 threads per tile, one x-row of cells each, bit-parallel as in band.cuh.
+// A block finds its tiles among every gridDim-th flag, so that neighbouring
+// tiles, which are swept together, fall to different blocks; that takes the
+// place of a launch that listed the flagged tiles (with it and one byte load per
+// cell corner a step's Front2VOF took 40 us at 128^3 with its list pass, 95 at
+// 512^3; 27 and 64 now.)
+template <int SH>
+__global__ void __launch_bounds__(64, 16) f2v_band_kernel(F2VArgs a) {
+    constexpr int TX = tile_edge(SH, 0), TY = tile_edge(SH, 1), TZ = tile_edge(SH, 2);
+    constexpr int RY = TY + 1, ROWS = RY * (TZ + 1);
+    constexpr uint32_t MT = TX == 32 ? 0xFFFFFFFFu : (1u << (TX & 31)) - 1u;
+    using M = typename RowMask<(TX + 1 > 32)>::type;
+    __shared__ M s_row[ROWS];
+    __shared__ int s_tile[64], s_n;
     pdl_wait();
-    const int ntl = *a.count;
-    for (int li = blockIdx.x; li < ntl; li += gridDim.x) {
-        const int tile = a.list[li];
-        int o[3];
-        tile_origin(a.g, tile, o);
-        for (int c = threadIdx.x; c < TILE_CELLS; c += blockDim.x) {
-            int l[3];
-            tile_cell(a.g, c, l);
-            int x = o[0] + l[0], y = o[1] + l[1], z = o[2] + l[2];
-            bool cutc = false;
-            int id0 = 0;
-            if (x < a.g.n[0] && y < a.g.n[1] && z < a.g.n[2]) {
-                int ids[8];
-                cell_ids(a.g, x, y, z, ids);
-                int K = 0;
+    if (a.zero && blockIdx.x == 0 && threadIdx.x == 0) *a.zero = 0;
+    const unsigned full = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int nx = a.g.n[0], ny = a.g.n[1], nz = a.g.n[2];
+    const long long n = (long long)nx * ny * nz;
+    const bool even = nx % 2 == 0 && ((uintptr_t)a.C & 15) == 0;  // rows of C start on 16 bytes
+    for (long long t0 = blockIdx.x; t0 < a.g.ntiles; t0 += 64ll * gridDim.x) {
+        if (tid == 0) s_n = 0;
+        __syncthreads();
+        const long long t = t0 + (long long)tid * gridDim.x;
+        bool on = false;
+        if (t < a.g.ntiles) {
+            const uint8_t d = a.dirty[t];
+            if (d) a.dirty[t] = 0;
+            on = d || a.full;
+        }
+        if (on) s_tile[atomicAdd(&s_n, 1)] = (int)t;
+        __syncthreads();
+        const int nt = s_n;
+        for (int k = 0; k < nt; k++) {
+            int o[3];
+            tile_origin(a.g, s_tile[k], o);
 #pragma unroll
-                for (int cid = 0; cid < 8; cid++) K |= (__ldg(a.cb + ids[cid]) & 1) << cid;
-                id0 = ids[0];
-                if (K == 0 || K == 255)
-                    reinterpret_cast<unsigned long long *>(a.C)[id0] = (K & 1) ? 0x3FF0000000000000ull : 0ull;
-                else
-                    cutc = true;
+            for (int q = 0; q < (ROWS + 63) / 64; q++) {
+                const int r = tid + 64 * q;
+                if (r >= ROWS) continue;
+                uint32_t f;
+                s_row[r] = load_row<M, TX, 0, TX + 1>(
+                    a.cb, (wrapc(o[2] + r / RY, nz) * ny + wrapc(o[1] + r % RY, ny)) * nx, o[0], nx, a.cb_whole, n, 1, &f);
             }
-            const unsigned full = 0xffffffffu;
-            unsigned m = __ballot_sync(full, cutc);
-            if (m) {
-                const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
+            __syncthreads();
+            const int ly = tid % TY, lz = tid / TY, y = o[1] + ly, z = o[2] + lz;
+            const bool row_ok = tid < TY * TZ && y < ny && z < nz;
+            uint32_t ones = 0, cut = 0, vx = 0;
+            const int id = (z * ny + y) * nx + o[0];
+            if (row_ok) {
+                vx = nx - o[0] >= TX ? MT : (1u << (nx - o[0])) - 1u;
+                const M *r = s_row + ly + RY * lz;
+                const M all = r[0] & r[1] & r[RY] & r[RY + 1], any = r[0] | r[1] | r[RY] | r[RY + 1];
+                ones = (uint32_t)(all & all >> 1) & MT;
+                cut = (uint32_t)(any | any >> 1) & ~ones & vx;
+            }
+            unsigned total;
+            int pos = (int)warp_prefix((unsigned)__popc(cut), &total);
+            if (total) {
                 int base = 0;
-                if (lane == leader) base = atomicAdd(a.ncut, __popc(m));
-                base = __shfl_sync(full, base, leader);
-                if (cutc) a.cut[base + __popc(m & ((1u << lane) - 1u))] = (unsigned)id0;
+                if (lane == 0) base = atomicAdd(a.ncut, (int)total);
+                pos += __shfl_sync(full, base, 0);
+                for (uint32_t m = cut; m; m &= m - 1) a.cut[pos++] = (unsigned)(id + __ffs((int)m) - 1);
             }
+            // the fractions, 16 bytes per lane along the rows
+            constexpr int LPR = TX / 2;  // lanes per row
+#pragma unroll
+            for (int j = 0; j < LPR; j++) {
+                const int from = j * (32 / LPR) + lane / LPR, b = 2 * (lane % LPR);
+                const uint32_t w = __shfl_sync(full, ones, from) >> b, ok = __shfl_sync(full, vx, from) >> b;
+                unsigned long long *p = reinterpret_cast<unsigned long long *>(a.C) + __shfl_sync(full, id, from) + b;
+                const unsigned long long v0 = (w & 1u) ? 0x3FF0000000000000ull : 0ull,
+                                         v1 = (w & 2u) ? 0x3FF0000000000000ull : 0ull;
+                if (even && (ok & 3u) == 3u) {
+                    *reinterpret_cast<ulonglong2 *>(p) = make_ulonglong2(v0, v1);
+                } else {
+                    if (ok & 1u) p[0] = v0;
+                    if (ok & 2u) p[1] = v1;
+                }
+            }
+            __syncthreads();
         }
     }
 }
 
-// Per-cell reconstruction used by the list kernel.  Same geometry as
-// cell_fraction (the reference form above, kept for the exhaustive checks), in
-// a register-only formulation:
+// Per-cell reconstruction, registers only:
 //   * face areas from closed forms -- a corner cut is the triangle l1*l2/2, a
 //     cut across the face the trapezoid (l1 + l2)/2, three corners the
 //     complement of a corner cut (l = distances from the cut corner or side);
@@ -222,13 +143,18 @@ __global__ void __launch_bounds__(256) f2v_band_kernel(F2VArgs a) {
 //   * sum_i det(c, p_i, p_i+1) = c . sum_i (p_i x p_i+1) with c the mean of
 //     the loop's markers (Eq. 7) -- the same sum reassociated, so C agrees
 //     with the fan-by-fan evaluation to rounding (about 1e-16).
-// face corner k -> k+1 runs along +axis when the edge goes from its lower to its
-// upper node: kFaceFwd[f][k] = 1 (then the marker sits at distance s from
-// corner k).
-__constant__ int8_t kFaceFwd[6][4] = {
-    {1, 1, 0, 0}, {1, 1, 0, 0}, {1, 1, 0, 0}, {1, 1, 0, 0}, {1, 1, 0, 0}, {1, 1, 0, 0}};
-
+// Bound by the FP64 pipe on long lists and by the chain of one cell on short
+// ones.  A marker's coordinates but one are 0 or 1, so of the six products of a
+// cross product five are selections; the faces' cases differ by selected
+// operands, not by branches, so lanes with different cuts share one instruction
+// stream (72 registers, where the branching form took 160).
 __device__ __forceinline__ double sel01(int b) { return __longlong_as_double(b ? 0x3FF0000000000000ll : 0ll); }
+
+// a loop's number of markers (up to 12) as a double, by its bit pattern
+__device__ __forceinline__ double small_count(int k) {
+    const int e = 31 - __clz(k);
+    return __hiloint2double((1023 + e) << 20 | (k << (20 - e) & 0xFFFFF), 0);
+}
 
 __device__ __forceinline__ void marker_xyz(int e, double s, double &x, double &y, double &z) {
     const int ax = e >> 2, r = e & 3;
@@ -238,62 +164,62 @@ __device__ __forceinline__ void marker_xyz(int e, double s, double &x, double &y
     z = ax == 2 ? s : v;
 }
 
-// distance from face corner k to the marker on face edge k (corner k -> k+1)
-// and from corner k+1 to it
-__device__ __forceinline__ double dist_from_k(int fwd, double s) { return fwd ? s : 1.0 - s; }
-__device__ __forceinline__ double dist_from_k1(int fwd, double s) { return fwd ? 1.0 - s : s; }
-
+// Links the segments of face F into the successor codes (a segment runs from one
+// cube edge to the next with the reference phase on its left) and, for an upper
+// face (odd F), returns its reference-phase area.  Of the face's edges 0 and 1
+// run from corner k to k + 1, 2 and 3 back, on every face, which fixes
+// whether a distance is s or 1 - s.
 template <int F>
 __device__ __forceinline__ double face_area_and_links(int K, int phif, const double *sE, int stride,
                                                       unsigned long long &nxt) {
-    int col[4], ed[4], fw[4];
+    // the face's edges as nibbles
+    unsigned eds = 0;
+    int cols = 0;
 #pragma unroll
     for (int k = 0; k < 4; k++) {
-        col[k] = (K >> kFaceCorner[F][k]) & 1;
-        ed[k] = kFaceEdge[F][k];
-        fw[k] = kFaceFwd[F][k];
+        cols |= ((K >> kFaceCorner[F][k]) & 1) << k;
+        eds |= (unsigned)kFaceEdge[F][k] << (4 * k);
     }
-    int mm = 0;
-#pragma unroll
-    for (int k = 0; k < 4; k++) mm |= (col[k] != col[(k + 1) & 3]) << k;
-    const int nm = __popc(mm);
-    double area = 0.0;
-    auto link = [&](int from, int to) {
-        nxt = (nxt & ~(0xFull << (4 * from))) | ((unsigned long long)to << (4 * from));
+    auto edge = [&](int k) -> int { return (int)((eds >> (4 * k)) & 15u); };
+    auto link = [&](int from, int to, bool on) {
+        const unsigned long long m = on ? 0xFull << (4 * from) : 0ull;
+        nxt = (nxt & ~m) | (((unsigned long long)to << (4 * from)) & m);
     };
-    if (nm == 0) {
-        area = sel01(col[0]);
-    } else if (nm == 2) {
-        const int ea = __ffs(mm) - 1, eb = 31 - __clz(mm);
-        const int arc = col[(ea + 1) & 3];
-        if (arc) link(ed[eb], ed[ea]);
-        else link(ed[ea], ed[eb]);
-        if (F & 1) {
-            const double sa = sE[ed[ea] * stride], sb = sE[ed[eb] * stride];
-            double R;
-            if (eb == ea + 1) {
-                // triangle at corner ea+1: legs along E_ea (to corner ea+1) and E_eb (from it)
-                R = 0.5 * (dist_from_k1(fw[ea], sa) * dist_from_k(fw[eb], sb));
-            } else if (eb == ea + 2) {
-                // corners ea+1, ea+2 on the opposite parallel edges E_ea, E_eb
-                R = 0.5 * (dist_from_k1(fw[ea], sa) + dist_from_k(fw[eb], sb));
-            } else {
-                // three corners: complement of the triangle at corner ea (= eb + 1)
-                R = 1.0 - 0.5 * (dist_from_k(fw[ea], sa) * dist_from_k1(fw[eb], sb));
-            }
-            area = arc ? R : 1.0 - R;
-        }
-    } else if (nm == 4) {
+    const int mm = cols ^ ((cols >> 1) | (cols & 1) << 3);  // edge k marked: corners k, k + 1 differ
+    const bool saddle = mm == 15, one = mm != 0 && !saddle;
+    // one segment between the marked edges ea < eb, or on a saddle the cuts of
+    // the two corners m0, m0 + 2 whose colour differs from the face's
+    const int m0 = (cols & 1) == phif ? 1 : 0, ea = one ? __ffs(mm) - 1 : (m0 + 3) & 3, eb = one ? 31 - __clz(mm) : m0;
+    const int arc = one ? (cols >> ((ea + 1) & 3)) & 1 : !phif;
+    const int ce_a = edge(ea), ce_b = edge(eb);
+    link(arc ? ce_b : ce_a, arc ? ce_a : ce_b, one || saddle);
+    const int ce_c = edge((ea + 2) & 3), ce_d = edge((eb + 2) & 3);  // the saddle's other cut
+    link(arc ? ce_d : ce_c, arc ? ce_c : ce_d, saddle);
+    if (!(F & 1)) return 0.0;
+    double area = sel01(cols & 1);
+    if (one) {
+        // corner ea + 1 cut off (eb = ea + 1), corners ea + 1 and ea + 2 (eb =
+        // ea + 2), or all but corner 0 (ea = 0, eb = 3: its complement)
+        const bool rest = eb == ea + 3, side = eb == ea + 2;
+        double l1 = sE[ce_a * stride], l2 = sE[ce_b * stride];
+        if (ea < 2 && !rest) l1 = 1.0 - l1;
+        if (eb >= 2 && !rest) l2 = 1.0 - l2;
+        double R = 0.5 * (side ? l1 + l2 : l1 * l2);
+        if (rest) R = 1.0 - R;
+        area = arc ? R : 1.0 - R;
+    } else if (saddle) {
         double T = 0.0;
 #pragma unroll
         for (int m = 0; m < 4; m++) {
-            if (col[m] == phif) continue;
-            const int ep = ed[(m + 3) & 3], en = ed[m];
-            if (col[m]) link(en, ep);
-            else link(ep, en);
-            if (F & 1) T += 0.5 * (dist_from_k1(fw[(m + 3) & 3], sE[ep * stride]) * dist_from_k(fw[m], sE[en * stride]));
+            if (((cols >> m) & 1) == phif) continue;
+            // legs from corner m back along edge m - 1 and on along edge m
+            const int p = (m + 3) & 3;
+            double lp = sE[kFaceEdge[F][p] * stride], ln = sE[kFaceEdge[F][m] * stride];
+            if (p < 2) lp = 1.0 - lp;
+            if (m >= 2) ln = 1.0 - ln;
+            T += 0.5 * (lp * ln);
         }
-        area = (1 - phif) ? T : 1.0 - T;
+        area = phif ? 1.0 - T : T;
     }
     return area;
 }
@@ -321,42 +247,48 @@ __device__ double cell_fraction_fast(int K, const int Fc[6], const double *sE, i
     double acc = 0.0;
     while (todo) {
         const int e0 = __ffs(todo) - 1;
-        double x0, y0, z0;
-        marker_xyz(e0, sE[e0 * stride], x0, y0, z0);
-        double sx = x0, sy = y0, sz = z0;
-        double px = x0, py = y0, pz = z0;
+        double sp = sE[e0 * stride];
+        const double s0 = sp;
+        double sx, sy, sz;
+        marker_xyz(e0, sp, sx, sy, sz);
+        double px = sx, py = sy, pz = sz;
         double cxs = 0.0, cys = 0.0, czs = 0.0;
         int len = 1, e = e0;
         todo &= ~(1u << e0);
         bool closed = false;
         for (int guard = 0; guard < 12; guard++) {
-            int nx_ = (int)((nxt >> (4 * e)) & 0xF);
-            if (nx_ == 0xF) break;
+            const int to = (int)((nxt >> (4 * e)) & 0xF);
+            closed = to == e0;
+            if (!closed && (to == 0xF || !((todo >> to) & 1))) break;
+            const double sq = closed ? s0 : sE[to * stride];
             double qx, qy, qz;
-            if (nx_ == e0) {
-                qx = x0; qy = y0; qz = z0;
-            } else {
-                if (!((todo >> nx_) & 1)) break;
-                marker_xyz(nx_, sE[nx_ * stride], qx, qy, qz);
-            }
-            cxs += py * qz - pz * qy;
-            cys += pz * qx - px * qz;
-            czs += px * qy - py * qx;
-            if (nx_ == e0) {
-                closed = true;
-                break;
-            }
+            marker_xyz(to, sq, qx, qy, qz);
+            // p x q: the one product of two offsets, the others selected
+            const double pq = sp * sq;
+            const int ap = e >> 2, aq = to >> 2;
+            auto mul = [&](double u, double v, int au, int av) -> double {
+                // u = p's coordinate au, v = q's coordinate av
+                const bool us = ap == au, vs = aq == av;
+                const double w = us ? u : v;             // the factor that is an offset (or 0, 1)
+                const double z = us ? v : u;             // the other one
+                return (us && vs) ? pq : (__double2hiint(z) ? w : 0.0);
+            };
+            cxs += mul(py, qz, 1, 2) - mul(pz, qy, 2, 1);
+            cys += mul(pz, qx, 2, 0) - mul(px, qz, 0, 2);
+            czs += mul(px, qy, 0, 1) - mul(py, qx, 1, 0);
+            if (closed) break;
             sx += qx; sy += qy; sz += qz;
             px = qx; py = qy; pz = qz;
-            todo &= ~(1u << nx_);
-            e = nx_;
+            sp = sq;
+            todo &= ~(1u << to);
+            e = to;
             len++;
         }
         if (!closed) {
             *bad = 1;
             continue;
         }
-        acc += (sx * cxs + sy * cys + sz * czs) / (double)len;
+        acc += (sx * cxs + sy * cys + sz * czs) / small_count(len);
     }
     double V = (2.0 * ((A1 + A2) + A3) - acc) / 6.0;
     if (V < 0.0) V = 0.0;

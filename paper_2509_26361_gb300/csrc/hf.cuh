@@ -40,65 +40,28 @@ __device__ __forceinline__ bool is_interface(double c) {
     return b > 0 && b < 0x3FF0000000000000ll;
 }
 
-// C at offset (dx, dy, dz) from the cell; WRAP = false uses direct strides (the
-// cell is at least HFH+1 cells from every periodic seam)
-template <bool WRAP>
-struct CAccess {
+// The cell's neighbourhood: offsets along one axis are wrapped by two selects, so
+// cells at a periodic seam run the same code as the others.
+struct HFCell {
     const double *__restrict__ C;
-    Grid g;
-    int x, y, z, id, sy, sz;
-    __device__ __forceinline__ double operator()(int dx, int dy, int dz) const {
-        if (WRAP) return __ldg(C + lin(g, x + dx, y + dy, z + dz));
-        return __ldg(C + id + dx + dy * sy + dz * sz);
-    }
-};
+    int p[3], n[3], s[3];  // coordinates, extents, strides
+    int id;
 
-// heights along axis d on the 3x3 stencil of 9-cell columns; returns false when
-// a column's ends are not pure with the reference phase on the expected side.
-// The axis is a run-time value so that lanes of a warp with different
-// dominant axes share one instruction stream.
-template <bool WRAP>
-__device__ __forceinline__ bool hf_axis(const CAccess<WRAP> &c, int d, bool below, double *out) {
-    const int t1 = (d == 0) ? 1 : 0, t2 = (d == 2) ? 1 : 2;
-    int ed[3] = {0, 0, 0}, e1[3] = {0, 0, 0}, e2[3] = {0, 0, 0};
-    ed[d] = 1;
-    e1[t1] = 1;
-    e2[t2] = 1;
-    double eta[3][3];
-    bool ok = true;
-#pragma unroll 1
-    for (int b2 = -1; b2 <= 1; b2++)
-#pragma unroll
-        for (int b1 = -1; b1 <= 1; b1++) {
-            const int ox = b1 * e1[0] + b2 * e2[0], oy = b1 * e1[1] + b2 * e2[1], oz = b1 * e1[2] + b2 * e2[2];
-            double H = 0.0;
-            unsigned long long lo = 0ull, hi = 0ull;
-#pragma unroll
-            for (int m = -HFH; m <= HFH; m++) {
-                double cv = c(ox + m * ed[0], oy + m * ed[1], oz + m * ed[2]);
-                H += cv;
-                if (m == -HFH) lo = (unsigned long long)__double_as_longlong(cv);
-                if (m == HFH) hi = (unsigned long long)__double_as_longlong(cv);
-            }
-            // pure ends on the bit patterns: == 1.0 is one pattern, == 0.0 two (+0, -0)
-            const bool lo1 = lo == 0x3FF0000000000000ull, lo0 = (lo << 1) == 0ull;
-            const bool hi1 = hi == 0x3FF0000000000000ull, hi0 = (hi << 1) == 0ull;
-            ok = ok && (below ? (lo1 && hi0) : (lo0 && hi1));
-            eta[b1 + 1][b2 + 1] = below ? H - (HFH + 0.5) : (HFH + 0.5) - H;
-        }
-    if (!ok) return false;
-    double hx = (eta[2][1] - eta[0][1]) * 0.5;
-    double hy = (eta[1][2] - eta[1][0]) * 0.5;
-    double hxx = (eta[2][1] + eta[0][1]) - 2.0 * eta[1][1];
-    double hyy = (eta[1][2] + eta[1][0]) - 2.0 * eta[1][1];
-    double hxy = ((eta[2][2] - eta[2][0]) - (eta[0][2] - eta[0][0])) * 0.25;
-    double num = (1.0 + hy * hy) * hxx + (1.0 + hx * hx) * hyy - 2.0 * hx * hy * hxy;
-    double q2 = 1.0 + hx * hx + hy * hy;
-    double den = q2 * sqrt(q2);
-    double kap = num / den;
-    *out = below ? -kap : kap;
-    return true;
-}
+    __device__ HFCell(const double *C_, const Grid &g, int id_) : C(C_), id(id_) {
+        n[0] = g.n[0];
+        n[1] = g.n[1];
+        n[2] = g.n[2];
+        s[0] = 1;
+        s[1] = n[0];
+        s[2] = n[0] * n[1];
+        p[2] = id / s[2];
+        const int r = id - p[2] * s[2];
+        p[1] = r / n[0];
+        p[0] = r - p[1] * n[0];
+    }
+    // id offset of m cells along an axis (coordinate q, extent nn, stride st)
+    __device__ __forceinline__ static int off(int q, int nn, int st, int m) { return (wrapc(q + m, nn) - q) * st; }
+};
 
 // The float at or below c for c in [+0, 1], from the bit pattern (values
 // under 2^-126 give 0): an error below one float ulp, at most 2^-24.
@@ -109,21 +72,67 @@ __device__ __forceinline__ float trunc_unit_float(double c) {
     return e < 1023 - 126 ? 0.0f : __uint_as_float(f);
 }
 
-template <bool WRAP>
-__device__ int hf_cell_impl(const CAccess<WRAP> &c, double *out) {
-    // the 3x3x3 block once; Youngs sums in the order (b2 outer, b1 inner)
-    double blk[3][3][3];
+// axes in the order they are tried (bits 0-5, two each) and, in bits 6-8, the
+// axes with n > 0 (reference phase below)
+template <typename T>
+__device__ __forceinline__ int hf_order(T n0, T n1, T n2) {
+    const T a0 = n0 < T(0) ? -n0 : n0, a1 = n1 < T(0) ? -n1 : n1, a2 = n2 < T(0) ? -n2 : n2;
+    int o0 = 0, o1 = 1, o2 = 2, tmp;
+    T f0 = a0, f1 = a1, f2 = a2, t;
+    if (f1 > f0) { tmp = o0; o0 = o1; o1 = tmp; t = f0; f0 = f1; f1 = t; }
+    if (f2 > f1) {
+        tmp = o1; o1 = o2; o2 = tmp; t = f1; f1 = f2; f2 = t;
+        if (f1 > f0) { tmp = o0; o0 = o1; o1 = tmp; }
+    }
+    return o0 | o1 << 2 | o2 << 4 | (n0 > T(0) ? 64 : 0) | (n1 > T(0) ? 128 : 0) | (n2 > T(0) ? 256 : 0);
+}
+
+// The order by the FP64 normal, Youngs sums in the order (b2 outer, b1 inner):
+// the rare cells whose float normal does not decide.
+static __device__ __noinline__ int hf_order_exact(const double *__restrict__ C, int id, const int *ox, const int *oy,
+                                                  const int *oz) {
+    double n[3];
+    const double w[3] = {1.0, 2.0, 1.0};
+    for (int d = 0; d < 3; d++) {
+        double gsum = 0.0;
+        for (int b2 = 0; b2 < 3; b2++)
+            for (int b1 = 0; b1 < 3; b1++) {
+                // the block's cells at +1 and -1 along d, b1 and b2 along the other two axes
+                const int up = d == 0 ? ox[2] + oy[b1] + oz[b2] : (d == 1 ? ox[b1] + oy[2] + oz[b2] : ox[b1] + oy[b2] + oz[2]);
+                const int dn = d == 0 ? ox[0] + oy[b1] + oz[b2] : (d == 1 ? ox[b1] + oy[0] + oz[b2] : ox[b1] + oy[b2] + oz[0]);
+                gsum += (w[b1] * w[b2]) * (__ldg(C + id + up) - __ldg(C + id + dn));
+            }
+        n[d] = -gsum;
+    }
+    return hf_order<double>(n[0], n[1], n[2]);
+}
+
+// Height-function curvature of an interface cell: its status, and kappa h in
+// *out.
+//
+// The axis is chosen first, by integer tests of the columns' ends alone: the
+// ends of the 3x3 columns along the axis must be pure with the reference phase
+// on the expected side.  The heights are then summed once, for the one axis that
+// has them.  Every lane of a warp follows one instruction stream (wrapped
+// offsets, the axis a run-time value, one path for both ways of ordering the
+// axes): with separate code for cells at the seams, for each way of ordering and
+// a whole sum per axis tried, a warp ran up to twelve sums one after another.
+// The FP64 pipe (2 lanes per clock and SM) bounds long lists: 81 additions and
+// about 50 operations for the formula per cell with heights.  4.2e5 cells at
+// 256^3 took 286 us and take 88, the 500 of a sphere at 32^3 45 us and 12.
+__device__ __forceinline__ int hf_cell(const HFCell &c, double *out) {
+    int ox[3], oy[3], oz[3];
 #pragma unroll
-    for (int dz = -1; dz <= 1; dz++)
-#pragma unroll
-        for (int dy = -1; dy <= 1; dy++)
-#pragma unroll
-            for (int dx = -1; dx <= 1; dx++) blk[dz + 1][dy + 1][dx + 1] = c(dx, dy, dz);
+    for (int i = 0; i < 3; i++) {
+        ox[i] = HFCell::off(c.p[0], c.n[0], c.s[0], i - 1);
+        oy[i] = HFCell::off(c.p[1], c.n[1], c.s[1], i - 1);
+        oz[i] = HFCell::off(c.p[2], c.n[2], c.s[2], i - 1);
+    }
     // The normal decides only the axis order and the side of the reference
     // phase.  A float normal decides them when every |n_d| and every gap
     // between two |n_d| clears the float rounding bound CANON_EPS with margin
     // (then the FP64 sums, within 2e-14 of the exact ones, order and sign them
-    // the same); otherwise the FP64 sums below, in the oracle's order.
+    // the same); otherwise the FP64 sums, in the oracle's order.
     // (the bound holds for values in [+0, 1], checked on the bit patterns).
     // The floats are the doubles truncated by integer operations, not rounded
     // by conversion instructions: an input error below 2^-24 instead of 2^-25,
@@ -131,82 +140,77 @@ __device__ int hf_cell_impl(const CAccess<WRAP> &c, double *out) {
     float fv[27];
     bool unit = true;
 #pragma unroll
-    for (int dz = 0; dz < 3; dz++)
-#pragma unroll
-        for (int dy = 0; dy < 3; dy++)
-#pragma unroll
-            for (int dx = 0; dx < 3; dx++) {
-                unit = unit && (unsigned long long)__double_as_longlong(blk[dz][dy][dx]) <= 0x3FF0000000000000ull;
-                fv[dz * 9 + dy * 3 + dx] = trunc_unit_float(blk[dz][dy][dx]);
-            }
+    for (int i = 0; i < 27; i++) {
+        const double v = __ldg(c.C + c.id + ox[i % 3] + oy[(i / 3) % 3] + oz[i / 9]);
+        unit = unit && (unsigned long long)__double_as_longlong(v) <= 0x3FF0000000000000ull;
+        fv[i] = trunc_unit_float(v);
+    }
     float nf[3];
     youngs<float>(fv, nf);
     const float f0 = fabsf(nf[0]), f1 = fabsf(nf[1]), f2 = fabsf(nf[2]);
+    int ord;
     if (unit && f0 > CANON_EPS && f1 > CANON_EPS && f2 > CANON_EPS && fabsf(f0 - f1) > 2.0f * CANON_EPS &&
-        fabsf(f0 - f2) > 2.0f * CANON_EPS && fabsf(f1 - f2) > 2.0f * CANON_EPS) {
-        int o0 = 0, o1 = 1, o2 = 2, tmp;
-        const float fa[3] = {f0, f1, f2};
-        if (fa[o1] > fa[o0]) { tmp = o0; o0 = o1; o1 = tmp; }
-        if (fa[o2] > fa[o1]) {
-            tmp = o1; o1 = o2; o2 = tmp;
-            if (fa[o1] > fa[o0]) { tmp = o0; o0 = o1; o1 = tmp; }
+        fabsf(f0 - f2) > 2.0f * CANON_EPS && fabsf(f1 - f2) > 2.0f * CANON_EPS)
+        ord = hf_order<float>(nf[0], nf[1], nf[2]);
+    else
+        ord = hf_order_exact(c.C, c.id, ox, oy, oz);
+    // the first axis whose columns end pure, the reference phase below (above)
+    int axis = -1, q = 0, nn = 0, st = 0, t1[3], t2[3];
+    for (int k = 0; k < 3 && axis < 0; k++) {
+        const int d = (ord >> (2 * k)) & 3;
+        q = d == 0 ? c.p[0] : (d == 1 ? c.p[1] : c.p[2]);
+        nn = d == 0 ? c.n[0] : (d == 1 ? c.n[1] : c.n[2]);
+        st = d == 0 ? c.s[0] : (d == 1 ? c.s[1] : c.s[2]);
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            t1[i] = d == 0 ? oy[i] : ox[i];
+            t2[i] = d == 2 ? oy[i] : oz[i];
         }
-        const int ord[3] = {o0, o1, o2};
-        for (int oi = 0; oi < 3; oi++) {
-            const int d = ord[oi];
-            if (hf_axis<WRAP>(c, d, nf[d] > 0.0f, out)) return 1 + d;
-        }
+        const int lo = c.id + HFCell::off(q, nn, st, -HFH), hi = c.id + HFCell::off(q, nn, st, HFH);
+        const bool below = (ord >> (6 + d)) & 1;
+        bool ok = true;
+#pragma unroll
+        for (int b2 = 0; b2 < 3; b2++)
+#pragma unroll
+            for (int b1 = 0; b1 < 3; b1++) {
+                // == 1.0 is one pattern, == 0.0 two (+0, -0)
+                const unsigned long long l = (unsigned long long)__double_as_longlong(__ldg(c.C + lo + t1[b1] + t2[b2]));
+                const unsigned long long h = (unsigned long long)__double_as_longlong(__ldg(c.C + hi + t1[b1] + t2[b2]));
+                const unsigned long long f = below ? l : h, e = below ? h : l;
+                ok = ok && f == 0x3FF0000000000000ull && (e << 1) == 0ull;
+            }
+        if (ok) axis = d;
+    }
+    if (axis < 0) {
         *out = 0.0;
         return 4;
     }
-    const double w[3] = {1.0, 2.0, 1.0};
-    double n[3];
+    // heights: each column summed from its lower end
+    const bool below = (ord >> (6 + axis)) & 1;
+    int om[9];
 #pragma unroll
-    for (int d = 0; d < 3; d++) {
-        const int t1 = (d == 0) ? 1 : 0, t2 = (d == 2) ? 1 : 2;
-        double gsum = 0.0;
+    for (int m = 0; m < 9; m++) om[m] = HFCell::off(q, nn, st, m - HFH);
+    double eta[3][3];
 #pragma unroll
-        for (int b2 = -1; b2 <= 1; b2++)
+    for (int b2 = 0; b2 < 3; b2++)
 #pragma unroll
-            for (int b1 = -1; b1 <= 1; b1++) {
-                int op[3] = {0, 0, 0}, om[3] = {0, 0, 0};
-                op[d] = 1;
-                om[d] = -1;
-                op[t1] += b1;
-                om[t1] += b1;
-                op[t2] += b2;
-                om[t2] += b2;
-                gsum += (w[b1 + 1] * w[b2 + 1]) *
-                        (blk[op[2] + 1][op[1] + 1][op[0] + 1] - blk[om[2] + 1][om[1] + 1][om[0] + 1]);
-            }
-        n[d] = -gsum;
-    }
-    int o0 = 0, o1 = 1, o2 = 2, tmp;
-    if (fabs(n[o1]) > fabs(n[o0])) { tmp = o0; o0 = o1; o1 = tmp; }
-    if (fabs(n[o2]) > fabs(n[o1])) {
-        tmp = o1; o1 = o2; o2 = tmp;
-        if (fabs(n[o1]) > fabs(n[o0])) { tmp = o0; o0 = o1; o1 = tmp; }
-    }
-    const int ord[3] = {o0, o1, o2};
-    for (int oi = 0; oi < 3; oi++) {
-        const int d = ord[oi];
-        const bool below = n[d] > 0.0;
-        if (hf_axis<WRAP>(c, d, below, out)) return 1 + d;
-    }
-    *out = 0.0;
-    return 4;
-}
-
-__device__ __noinline__ int hf_cell(const HFArgs &a, int x, int y, int z, double *out) {
-    const int R = HFH + 1;
-    const int id = lin(a.g, x, y, z);
-    const int sy = a.g.n[0], sz = a.g.n[0] * a.g.n[1];
-    if (x >= R && x < a.g.n[0] - R && y >= R && y < a.g.n[1] - R && z >= R && z < a.g.n[2] - R) {
-        CAccess<false> c{a.C, a.g, x, y, z, id, sy, sz};
-        return hf_cell_impl<false>(c, out);
-    }
-    CAccess<true> c{a.C, a.g, x, y, z, id, sy, sz};
-    return hf_cell_impl<true>(c, out);
+        for (int b1 = 0; b1 < 3; b1++) {
+            const double *col = c.C + c.id + t1[b1] + t2[b2];
+            double H = __ldg(col + om[0]);
+#pragma unroll
+            for (int m = 1; m < 9; m++) H += __ldg(col + om[m]);
+            eta[b1][b2] = (below ? H : HFH + 0.5) - (below ? HFH + 0.5 : H);
+        }
+    const double hx = (eta[2][1] - eta[0][1]) * 0.5;
+    const double hy = (eta[1][2] - eta[1][0]) * 0.5;
+    const double hxx = (eta[2][1] + eta[0][1]) - 2.0 * eta[1][1];
+    const double hyy = (eta[1][2] + eta[1][0]) - 2.0 * eta[1][1];
+    const double hxy = ((eta[2][2] - eta[2][0]) - (eta[0][2] - eta[0][0])) * 0.25;
+    const double num = (1.0 + hy * hy) * hxx + (1.0 + hx * hx) * hyy - 2.0 * hx * hy * hxy;
+    const double q2 = 1.0 + hx * hx + hy * hy;
+    const double kap = num / (q2 * sqrt(q2));
+    *out = below ? -kap : kap;
+    return 1 + axis;
 }
 
 // Interface-cell pass: entries [0, nprev) reset the previous interface cells
@@ -216,9 +220,7 @@ __device__ __noinline__ int hf_cell(const HFArgs &a, int x, int y, int z, double
 // complete; one thread per entry, full warps for the FP64 work.  Without
 // COMPUTE the interface cells are only listed (the learned curvature writes
 // them next).
-// 4 blocks of 128 per SM: with the outer column loop kept rolled the kernel
-// fits 127 registers without spilling, where the fully unrolled one took 226
-// (2 blocks per SM) to keep all 81 column loads in flight
+// 4 blocks of 128 per SM (128 registers without spilling)
 template <bool COMPUTE>
 __global__ void __launch_bounds__(128, 4) hf_list_kernel(HFArgs a) {
     pdl_wait();
@@ -244,9 +246,8 @@ __global__ void __launch_bounds__(128, 4) hf_list_kernel(HFArgs a) {
                 }
             } else if (iface) {
                 if (COMPUTE) {
-                    const int x = id % a.g.n[0], y = (id / a.g.n[0]) % a.g.n[1], z = id / (a.g.n[0] * a.g.n[1]);
                     double kv = 0.0;
-                    int st = hf_cell(a, x, y, z, &kv);
+                    const int st = hf_cell(HFCell(a.C, a.g, id), &kv);
                     a.kh[id] = kv;
                     a.st[id] = (uint8_t)st;
                 }

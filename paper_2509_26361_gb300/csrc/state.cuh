@@ -75,25 +75,6 @@ __global__ void canonical_s_kernel(Grid g, const uint8_t *__restrict__ cb, const
     }
 }
 
-// List of the flagged tiles (no dilation), clearing the flags; zero0 and
-// zero1 (may be null) are counters of later launches, cleared as in
-// band_kernel.
-__global__ void take_flagged_kernel(Grid g, uint8_t *__restrict__ flag, int *__restrict__ list, int *__restrict__ count,
-                                    int *zero0, int *zero1) {
-    pdl_wait();
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        if (zero0) *zero0 = 0;
-        if (zero1) *zero1 = 0;
-    }
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.ntiles; t += gridDim.x * blockDim.x) {
-        if (flag[t]) {
-            flag[t] = 0;
-            int slot = atomicAdd(count, 1);
-            list[slot] = t;
-        }
-    }
-}
-
 __global__ void iota_kernel(int *list, int n, int *count) {
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) list[t] = t;
     if (blockIdx.x == 0 && threadIdx.x == 0) *count = n;
