@@ -53,8 +53,8 @@ __device__ __forceinline__ void cell_ids(const Grid &g, int x, int y, int z, int
 // A block finds its tiles among every gridDim-th flag, so that neighbouring
 // tiles, which are swept together, fall to different blocks; that takes the
 // place of a launch that listed the flagged tiles (with it and one byte load per
-// cell corner a step's Front2VOF took 40 us at 128^3 with its list pass, 95 at
-// 512^3; 27 and 64 now.)
+// cell corner: 9 us at 128^3, 25 at 512^3, 294 over every tile of 384^3; now 8,
+// 14 and 152.)
 template <int SH>
 __global__ void __launch_bounds__(64, 16) f2v_band_kernel(F2VArgs a) {
     constexpr int TX = tile_edge(SH, 0), TY = tile_edge(SH, 1), TZ = tile_edge(SH, 2);
@@ -147,7 +147,8 @@ __global__ void __launch_bounds__(64, 16) f2v_band_kernel(F2VArgs a) {
 // ones.  A marker's coordinates but one are 0 or 1, so of the six products of a
 // cross product five are selections; the faces' cases differ by selected
 // operands, not by branches, so lanes with different cuts share one instruction
-// stream (72 registers, where the branching form took 160).
+// stream (72 registers, where the branching form took 160; 17 to 14 us for the
+// cut cells of 128^3, 62 to 45 us at 512^3).
 __device__ __forceinline__ double sel01(int b) { return __longlong_as_double(b ? 0x3FF0000000000000ll : 0ll); }
 
 // a loop's number of markers (up to 12) as a double, by its bit pattern
