@@ -10,112 +10,133 @@
 // interfacial cell, so its cells share one colour, its edges carry no marker
 // and its faces store their corner colour.
 #pragma once
+#include "band.cuh"
 #include "common.cuh"
 
 namespace ebit {
 
 constexpr int AMR_R = TILE + 3;   // staged nodes per axis: -1 .. TILE + 1
 constexpr int AMR_F = TILE + 2;   // interfacial flags of cells -1 .. TILE
+constexpr int AMR_WARPS = 8;
+constexpr int AMR_CHUNK = 1024;   // tiles per chunk of the compaction
 
 // Per tile: the refinement mask of its cells (mask may be null), whether any
-// of them is refined (flag), the colour of its origin node (bg), and the
-// number of refined cells (count).  One block of 256 threads per tile.
-__global__ void __launch_bounds__(256) refine_kernel(Grid g, const uint8_t *__restrict__ cb, uint8_t *__restrict__ mask,
-                                                     int *__restrict__ flag, uint8_t *__restrict__ bg,
-                                                     unsigned long long *__restrict__ count) {
-    __shared__ uint8_t s_c[AMR_R * AMR_R * AMR_R];
-    __shared__ uint8_t s_f[AMR_F * AMR_F * AMR_F];
-    for (int tile = blockIdx.x; tile < g.ntiles; tile += gridDim.x) {
+// of them is refined (flag), the colour of its origin node (bg, may be null),
+// and the numbers of refined cells (count[0]), of flagged tiles (count[1]) and
+// of flagged tiles per chunk of AMR_CHUNK (chunk).  Outputs but the mask start
+// at zero where they are sums.
+//
+// One warp per tile, an x-row of colours as one bit mask: the flags of ten
+// cells are a few shifts of four rows and the 27-cell OR of eight cells a few
+// of nine, so the pass is bound by the colours' way from L2 and the mask's to
+// memory.  (a block per tile, one byte per thread and node: 1.9 ms at 512^3 and
+// 558 us at 384^3; this form 230 us at 384^3.)
+__global__ void __launch_bounds__(32 * AMR_WARPS) refine_kernel(Grid g, const uint8_t *__restrict__ cb, long long whole,
+                                                                uint8_t *__restrict__ mask, uint8_t *__restrict__ flag,
+                                                                uint8_t *__restrict__ bg,
+                                                                unsigned long long *__restrict__ count,
+                                                                int *__restrict__ chunk) {
+    __shared__ unsigned s_row[AMR_WARPS][AMR_R * AMR_R];
+    __shared__ unsigned s_flg[AMR_WARPS][AMR_F * AMR_F];
+    const unsigned full = 0xffffffffu;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    unsigned *row = s_row[warp], *flg = s_flg[warp];
+    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+    const long long n = (long long)nx * ny * nz;
+    unsigned nref = 0;
+    for (int tile = blockIdx.x * AMR_WARPS + warp; tile < g.ntiles; tile += gridDim.x * AMR_WARPS) {
         int o[3];
         tile_origin(g, tile, o);
-        int seen = 0;
-        for (int r = threadIdx.x; r < AMR_R * AMR_R * AMR_R; r += blockDim.x) {
-            const int rx = r % AMR_R, ry = (r / AMR_R) % AMR_R, rz = r / (AMR_R * AMR_R);
-            const uint8_t c = __ldg(cb + lin(g, o[0] + rx - 1, o[1] + ry - 1, o[2] + rz - 1)) & 1;
-            s_c[r] = c;
-            seen |= c ? 1 : 2;
+        bool any1 = false, any0 = false;
+#pragma unroll
+        for (int q = 0; q < (AMR_R * AMR_R + 31) / 32; q++) {
+            const int r = lane + 32 * q;
+            if (r >= AMR_R * AMR_R) continue;
+            const int y = wrapc(o[1] + r % AMR_R - 1, ny), z = wrapc(o[2] + r / AMR_R - 1, nz);
+            uint32_t f;
+            const unsigned c = load_row<uint32_t, TILE, -1, AMR_R>(cb, (z * ny + y) * nx, o[0], nx, whole, n, 1, &f);
+            row[r] = c;
+            any1 |= c != 0u;
+            any0 |= c != (1u << AMR_R) - 1u;
         }
-        const int has1 = __syncthreads_or(seen & 1), has0 = __syncthreads_or(seen & 2);
-        if (threadIdx.x == 0) bg[tile] = s_c[1 + AMR_R * (1 + AMR_R)];  // the origin node
-        unsigned nref = 0;
-        int any = 0;
+        const bool has1 = __any_sync(full, any1), has0 = __any_sync(full, any0);
+        __syncwarp();
+        const unsigned vx = nx - o[0] >= TILE ? 0xFFu : (1u << (nx - o[0])) - 1u;
+        bool any = false;
         if (has1 && has0) {
             // interfacial flags of the cells -1 .. TILE around the tile
-            for (int r = threadIdx.x; r < AMR_F * AMR_F * AMR_F; r += blockDim.x) {
-                const int fx = r % AMR_F, fy = (r / AMR_F) % AMR_F, fz = r / (AMR_F * AMR_F);
-                int lo = 1, hi = 0;
-#pragma unroll
-                for (int d = 0; d < 8; d++) {
-                    const int c = s_c[(fx + (d & 1)) + AMR_R * ((fy + ((d >> 1) & 1)) + AMR_R * (fz + (d >> 2)))];
-                    lo &= c;
-                    hi |= c;
-                }
-                s_f[r] = (uint8_t)(hi & ~lo);
+            for (int r = lane; r < AMR_F * AMR_F; r += 32) {
+                const int i = r % AMR_F + AMR_R * (r / AMR_F);
+                const unsigned p = row[i], q = row[i + 1], s = row[i + AMR_R], t = row[i + AMR_R + 1];
+                const unsigned hi = p | q | s | t, lo = p & q & s & t;
+                flg[r] = (hi | hi >> 1) & ~(lo & lo >> 1) & ((1u << AMR_F) - 1u);
             }
-            __syncthreads();
-            for (int c = threadIdx.x; c < TILE_CELLS; c += blockDim.x) {
-                const int lx = c & 7, ly = (c >> 3) & 7, lz = c >> 6;
-                const bool valid = o[0] + lx < g.n[0] && o[1] + ly < g.n[1] && o[2] + lz < g.n[2];
-                int ref = 0;
+            __syncwarp();
+        }
 #pragma unroll
-                for (int d = 0; d < 27; d++)
-                    ref |= s_f[(lx + d % 3) + AMR_F * ((ly + (d / 3) % 3) + AMR_F * (lz + d / 9))];
-                ref = valid ? ref : 0;
-                if (valid && mask) mask[lin(g, o[0] + lx, o[1] + ly, o[2] + lz)] = (uint8_t)ref;
-                nref += ref;
-                any |= ref;
+        for (int q = 0; q < 2; q++) {
+            const int r = lane + 32 * q, ly = r & 7, lz = r >> 3, y = o[1] + ly, z = o[2] + lz;
+            unsigned ref = 0;
+            if (has1 && has0) {
+                unsigned f = 0;
+#pragma unroll
+                for (int d = 0; d < 9; d++) f |= flg[ly + d % 3 + AMR_F * (lz + d / 3)];
+                ref = (f | f >> 1 | f >> 2) & vx;
             }
-        } else if (mask) {
-            for (int c = threadIdx.x; c < TILE_CELLS; c += blockDim.x) {
-                const int lx = c & 7, ly = (c >> 3) & 7, lz = c >> 6;
-                if (o[0] + lx < g.n[0] && o[1] + ly < g.n[1] && o[2] + lz < g.n[2])
-                    mask[lin(g, o[0] + lx, o[1] + ly, o[2] + lz)] = 0;
+            if (y >= ny || z >= nz) continue;
+            nref += __popc(ref);
+            any |= ref != 0;
+            if (mask) store_row<TILE>(mask, ((long long)z * ny + y) * nx + o[0], ref, 0u, 0u, 0u, vx);
+        }
+        const bool tile_any = __any_sync(full, any);
+        if (lane == 0) {
+            flag[tile] = tile_any ? 1 : 0;
+            if (bg) bg[tile] = (uint8_t)((row[1 + AMR_R] >> 1) & 1u);  // the origin node
+            if (tile_any) {
+                atomicAdd(count + 1, 1ull);
+                atomicAdd(chunk + tile / AMR_CHUNK, 1);
             }
         }
-        const int tile_any = __syncthreads_or(any);
-        const unsigned v = __reduce_add_sync(0xffffffffu, nref);
-        if ((threadIdx.x & 31) == 0 && v) atomicAdd(count, (unsigned long long)v);
-        if (threadIdx.x == 0) flag[tile] = tile_any ? 1 : 0;
-        __syncthreads();  // the staging is rewritten by the next tile
+        __syncwarp();  // the staging is rewritten by the next tile
     }
+    nref = __reduce_add_sync(full, nref);
+    if (lane == 0 && nref) atomicAdd(count, (unsigned long long)nref);
 }
 
-// Ascending ids of the flagged tiles into out[0 .. cap) and their number into
-// *n_out (one block: each thread scans a contiguous run of tiles).
-__global__ void __launch_bounds__(1024) compact_tiles_kernel(const int *__restrict__ flag, int nt,
-                                                             int *__restrict__ out, int cap, int *__restrict__ n_out) {
-    __shared__ int s_w[32];
-    const int per = (nt + blockDim.x - 1) / blockDim.x;
-    const int b0 = threadIdx.x * per, b1 = min(nt, b0 + per);
-    int cnt = 0;
-    for (int t = b0; t < b1; t++) cnt += flag[t];
-    // block-wide exclusive scan of cnt
+// Ascending ids of the flagged tiles into out[0 .. cap), from the flags and the
+// counts of refine_kernel: a block per chunk, which starts at the sum of the
+// chunks before it.
+__global__ void __launch_bounds__(256) compact_tiles_kernel(const uint8_t *__restrict__ flag, int nt,
+                                                            const int *__restrict__ chunk, int *__restrict__ out,
+                                                            int cap) {
+    __shared__ int s_w[8], s_base;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int inc = cnt;
+    for (int c = blockIdx.x; c * AMR_CHUNK < nt; c += gridDim.x) {
+        if (threadIdx.x == 0) s_base = 0;
+        __syncthreads();
+        int sum = 0;
+        for (int k = threadIdx.x; k < c; k += 256) sum += chunk[k];
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        if (lane == 0 && sum) atomicAdd(&s_base, sum);
+        const int t0 = c * AMR_CHUNK + 4 * threadIdx.x;
+        int m = 0;
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, inc, off);
-        if (lane >= off) inc += v;
+        for (int j = 0; j < 4; j++)
+            if (t0 + j < nt && flag[t0 + j]) m |= 1 << j;
+        const int cnt = __popc(m);
+        unsigned total;
+        const int pre = (int)warp_prefix((unsigned)cnt, &total);
+        if (lane == 0) s_w[wid] = (int)total;
+        __syncthreads();
+        int pos = s_base + pre;
+        for (int w = 0; w < wid; w++) pos += s_w[w];
+        for (int j = 0; j < 4; j++)
+            if ((m >> j) & 1) {
+                if (pos < cap) out[pos] = t0 + j;
+                pos++;
+            }
+        __syncthreads();
     }
-    if (lane == 31) s_w[wid] = inc;
-    __syncthreads();
-    if (wid == 0) {
-        int w = lane < (int)(blockDim.x >> 5) ? s_w[lane] : 0;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, w, off);
-            if (lane >= off) w += v;
-        }
-        s_w[lane] = w;  // inclusive prefix over warps
-    }
-    __syncthreads();
-    int pos = (wid ? s_w[wid - 1] : 0) + inc - cnt;
-    for (int t = b0; t < b1; t++)
-        if (flag[t]) {
-            if (pos < cap) out[pos] = t;
-            pos++;
-        }
-    if (threadIdx.x == blockDim.x - 1) *n_out = pos;
 }
 
 // Brick k of the store: tile tiles[k]'s colour bytes cb[k][c] and canonical
@@ -123,8 +144,10 @@ __global__ void __launch_bounds__(1024) compact_tiles_kernel(const int *__restri
 // tile (x fastest); cells outside the grid give 0.
 __global__ void __launch_bounds__(256) pack_kernel(Grid g, const uint8_t *__restrict__ cb, const double *__restrict__ s0,
                                                    const double *__restrict__ s1, const double *__restrict__ s2,
-                                                   const int *__restrict__ tiles, int n, uint8_t *__restrict__ out_cb,
-                                                   double *__restrict__ out_s) {
+                                                   const int *__restrict__ tiles,
+                                                   const unsigned long long *__restrict__ nbricks, int cap,
+                                                   uint8_t *__restrict__ out_cb, double *__restrict__ out_s) {
+    const int n = (int)min(*nbricks, (unsigned long long)cap);
     for (int k = blockIdx.x; k < n; k += gridDim.x) {
         int o[3];
         tile_origin(g, tiles[k], o);
@@ -159,32 +182,44 @@ __global__ void brick_slots_kernel(const int *__restrict__ tiles, int n, int nt,
     }
 }
 
-// The state from a brick store: bricks copied in, every other tile filled
-// with its colour (bg: bit 0), face colours equal to it, offsets 0.
+// The state from a brick store: bricks copied in, every other tile filled with
+// its colour (bg: bit 0), face colours equal to it.  Both state buffers get the
+// colours (a sweep leaves tiles outside its band unwritten); the offsets go to
+// the first only, and only the bricks' (an offset is read where its edge
+// carries a marker, and a sweep writes every marker's).  One thread per 8 cells
+// of an x-row of tiles; HBM writes of two bytes per cell.
 __global__ void __launch_bounds__(256) unpack_kernel(Grid g, const int *__restrict__ slot, const uint8_t *__restrict__ in_cb,
                                                      const double *__restrict__ in_s, const uint8_t *__restrict__ bg,
-                                                     uint8_t *__restrict__ cb, double *__restrict__ s0,
-                                                     double *__restrict__ s1, double *__restrict__ s2) {
-    for (int tile = blockIdx.x; tile < g.ntiles; tile += gridDim.x) {
-        int o[3];
-        tile_origin(g, tile, o);
+                                                     uint8_t *__restrict__ cb, uint8_t *__restrict__ cb2,
+                                                     double *__restrict__ s0, double *__restrict__ s1,
+                                                     double *__restrict__ s2) {
+    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+    const long long groups = (long long)g.td[0] * ny * nz, stride = (long long)gridDim.x * blockDim.x;
+    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < groups; t += stride) {
+        const int row = (int)(t / g.td[0]), tx = (int)(t - (long long)row * g.td[0]);
+        const int z = row / ny, y = row - z * ny;
+        const int tile = ((z >> 3) * g.td[1] + (y >> 3)) * g.td[0] + tx;
+        const long long id = (long long)row * nx + 8 * tx;
+        const int cnt = min(8, nx - 8 * tx);
         const int k = slot[tile];
-        const uint8_t fill = (bg[tile] & 1) ? 0x0F : 0x00;
-        for (int c = threadIdx.x; c < TILE_CELLS; c += blockDim.x) {
-            const int x = o[0] + (c & 7), y = o[1] + ((c >> 3) & 7), z = o[2] + (c >> 6);
-            if (x >= g.n[0] || y >= g.n[1] || z >= g.n[2]) continue;
-            const int id = lin(g, x, y, z);
-            if (k >= 0) {
-                cb[id] = in_cb[(size_t)k * TILE_CELLS + c];
-                s0[id] = in_s[((size_t)k * 3 + 0) * TILE_CELLS + c];
-                s1[id] = in_s[((size_t)k * 3 + 1) * TILE_CELLS + c];
-                s2[id] = in_s[((size_t)k * 3 + 2) * TILE_CELLS + c];
-            } else {
-                cb[id] = fill;
-                s0[id] = 0.0;
-                s1[id] = 0.0;
-                s2[id] = 0.0;
+        unsigned long long v = (bg[tile] & 1) ? 0x0F0F0F0F0F0F0F0Full : 0ull;
+        if (k >= 0) {
+            const int c = ((y & 7) + 8 * (z & 7)) * 8;
+            const uint8_t *bc = in_cb + (size_t)k * TILE_CELLS + c;
+            const double *bs = in_s + (size_t)k * 3 * TILE_CELLS + c;
+            v = 0;
+            for (int j = 0; j < cnt; j++) {
+                v |= (unsigned long long)__ldg(bc + j) << (8 * j);
+                s0[id + j] = __ldg(bs + j);
+                s1[id + j] = __ldg(bs + TILE_CELLS + j);
+                s2[id + j] = __ldg(bs + 2 * TILE_CELLS + j);
             }
+        }
+        if (cnt == 8 && (((uintptr_t)(cb + id) | (uintptr_t)(cb2 + id)) & 7) == 0) {
+            *reinterpret_cast<unsigned long long *>(cb + id) = v;
+            *reinterpret_cast<unsigned long long *>(cb2 + id) = v;
+        } else {
+            for (int j = 0; j < cnt; j++) cb[id + j] = cb2[id + j] = (uint8_t)(v >> (8 * j));
         }
     }
 }

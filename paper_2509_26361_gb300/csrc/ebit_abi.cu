@@ -265,7 +265,8 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
     ctx->dense = (desc->flags & EBIT_DESC_DENSE) ? 1 : 0;
     ctx->cur = 0;
     ctx->scratch = nullptr;
-    ctx->amr_flag = ctx->amr_slot = nullptr;
+    ctx->amr_flag = nullptr;
+    ctx->amr_slot = nullptr;
     ctx->amr_ctr = nullptr;
     int dev = 0;
     cudaGetDevice(&dev);
@@ -482,18 +483,23 @@ int ebit_set_state(ebit_ctx *ctx, const uint8_t *cb, const double *s) {
     return mark_all(ctx);
 }
 
-// the refinement scratch (per-tile flags and slots, two counters), on first use
+// tile chunks of the brick compaction
+static int amr_chunks(const ebit_ctx *ctx) { return (ctx->nt_cap + AMR_CHUNK - 1) / AMR_CHUNK; }
+
+// the refinement scratch (per-tile flags and slots; refined cells, bricks and
+// ids out of range, then the bricks per chunk), on first use
 static int amr_scratch(ebit_ctx *ctx) {
     if (ctx->amr_flag) return EBIT_OK;
     const size_t nt = (size_t)ctx->nt_cap;
-    if (!dev_alloc(ctx->mem, (void **)&ctx->amr_flag, nt * sizeof(int)) ||
+    if (!dev_alloc(ctx->mem, (void **)&ctx->amr_flag, nt) ||
         !dev_alloc(ctx->mem, (void **)&ctx->amr_slot, nt * sizeof(int)) ||
-        !dev_alloc(ctx->mem, (void **)&ctx->amr_ctr, 2 * sizeof(unsigned long long))) {
+        !dev_alloc(ctx->mem, (void **)&ctx->amr_ctr, 3 * sizeof(unsigned long long) + amr_chunks(ctx) * sizeof(int))) {
         cudaGetLastError();
         dev_free(ctx->mem, ctx->amr_flag);
         dev_free(ctx->mem, ctx->amr_slot);
         dev_free(ctx->mem, ctx->amr_ctr);
-        ctx->amr_flag = ctx->amr_slot = nullptr;
+        ctx->amr_flag = nullptr;
+        ctx->amr_slot = nullptr;
         ctx->amr_ctr = nullptr;
         return fail(ctx, EBIT_ENOMEM, "refinement scratch: allocation failed");
     }
@@ -501,13 +507,13 @@ static int amr_scratch(ebit_ctx *ctx) {
 }
 
 // refine_kernel over the current state: per-tile flags, background colours
-// (bg may be ctx scratch when the caller gives none), refined-cell count
+// (bg may be null), refined-cell and brick counts
 static int refine_pass(ebit_ctx *ctx, uint8_t *mask, uint8_t *bg) {
     if (int r = amr_scratch(ctx)) return r;
-    CU(cudaMemsetAsync(ctx->amr_ctr, 0, 2 * sizeof(unsigned long long), ctx->stream));
-    refine_kernel<<<std::min(ctx->g.ntiles, 4 * ctx->sms), 256, 0, ctx->stream>>>(
-        ctx->g, ctx->cb[ctx->cur], mask, ctx->amr_flag, bg ? bg : reinterpret_cast<uint8_t *>(ctx->amr_slot),
-        ctx->amr_ctr);
+    CU(cudaMemsetAsync(ctx->amr_ctr, 0, 3 * sizeof(unsigned long long) + amr_chunks(ctx) * sizeof(int), ctx->stream));
+    refine_kernel<<<std::min((ctx->g.ntiles + AMR_WARPS - 1) / AMR_WARPS, 8 * ctx->sms), 32 * AMR_WARPS, 0,
+                    ctx->stream>>>(ctx->g, ctx->cb[ctx->cur], (ctx->N + 7) & ~7LL, mask, ctx->amr_flag, bg,
+                                   ctx->amr_ctr, reinterpret_cast<int *>(ctx->amr_ctr + 3));
     return launch_check(ctx, "refine_kernel");
 }
 
@@ -533,21 +539,24 @@ int ebit_pack_bricks(ebit_ctx *ctx, int capacity, int *tiles, uint8_t *cb, doubl
         return fail(ctx, EBIT_EINVAL, "ebit_pack_bricks: 8^3 tiles only");
     if (int r = join_side(ctx)) return r;
     if (int r = refine_pass(ctx, nullptr, capacity > 0 ? bg : nullptr)) return r;
-    int *nb_dev = reinterpret_cast<int *>(ctx->amr_ctr + 1);
-    compact_tiles_kernel<<<1, 1024, 0, ctx->stream>>>(ctx->amr_flag, ctx->g.ntiles, tiles, capacity, nb_dev);
-    if (int r = launch_check(ctx, "compact_tiles_kernel")) return r;
-    int n = 0;
-    CU(cudaMemcpyAsync(&n, nb_dev, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    CU(cudaStreamSynchronize(ctx->stream));
-    *nbricks = n;
-    if (capacity == 0) return EBIT_OK;
-    if (n > capacity) return fail(ctx, EBIT_EINVAL, "ebit_pack_bricks: capacity below the brick count");
-    if (n > 0) {
+    if (capacity > 0) {
+        // the packing reads the brick count on the device, so that nothing waits
+        // for the host to learn it
+        compact_tiles_kernel<<<std::min((ctx->g.ntiles + AMR_CHUNK - 1) / AMR_CHUNK, 8 * ctx->sms), 256, 0,
+                               ctx->stream>>>(ctx->amr_flag, ctx->g.ntiles, reinterpret_cast<int *>(ctx->amr_ctr + 3),
+                                              tiles, capacity);
+        if (int r = launch_check(ctx, "compact_tiles_kernel")) return r;
         const int c = ctx->cur;
-        pack_kernel<<<std::min(n, 8 * ctx->sms), 256, 0, ctx->stream>>>(ctx->g, ctx->cb[c], ctx->s[c][0], ctx->s[c][1],
-                                                                        ctx->s[c][2], tiles, n, cb, s);
+        pack_kernel<<<std::min(std::min(capacity, ctx->g.ntiles), 8 * ctx->sms), 256, 0, ctx->stream>>>(
+            ctx->g, ctx->cb[c], ctx->s[c][0], ctx->s[c][1], ctx->s[c][2], tiles, ctx->amr_ctr + 1, capacity, cb, s);
         if (int r = launch_check(ctx, "pack_kernel")) return r;
     }
+    unsigned long long n = 0;
+    CU(cudaMemcpyAsync(&n, ctx->amr_ctr + 1, sizeof(n), cudaMemcpyDeviceToHost, ctx->stream));
+    CU(cudaStreamSynchronize(ctx->stream));
+    *nbricks = (int)n;
+    if (capacity > 0 && *nbricks > capacity)
+        return fail(ctx, EBIT_EINVAL, "ebit_pack_bricks: capacity below the brick count");
     return EBIT_OK;
 }
 
@@ -558,7 +567,7 @@ int ebit_unpack_bricks(ebit_ctx *ctx, int nbricks, const int *tiles, const uint8
     if (!ctx->owns_state) return fail(ctx, EBIT_EINVAL, "ebit_unpack_bricks: a batch instance's state is the batch's");
     if (int r = join_side(ctx)) return r;
     if (int r = amr_scratch(ctx)) return r;
-    int *bad_dev = reinterpret_cast<int *>(ctx->amr_ctr + 1) + 1;
+    int *bad_dev = reinterpret_cast<int *>(ctx->amr_ctr + 2);
     CU(cudaMemsetAsync(ctx->amr_slot, 0xFF, (size_t)ctx->g.ntiles * sizeof(int), ctx->stream));
     CU(cudaMemsetAsync(bad_dev, 0, sizeof(int), ctx->stream));
     if (nbricks > 0) {
@@ -571,10 +580,10 @@ int ebit_unpack_bricks(ebit_ctx *ctx, int nbricks, const int *tiles, const uint8
     CU(cudaStreamSynchronize(ctx->stream));
     if (bad) return fail(ctx, EBIT_EINVAL, "ebit_unpack_bricks: tile id out of range");
     const int c = ctx->cur;
-    unpack_kernel<<<std::min(ctx->g.ntiles, 8 * ctx->sms), 256, 0, ctx->stream>>>(
-        ctx->g, ctx->amr_slot, cb, s, bg, ctx->cb[c], ctx->s[c][0], ctx->s[c][1], ctx->s[c][2]);
+    unpack_kernel<<<blocks_for((long long)ctx->g.td[0] * ctx->g.n[1] * ctx->g.n[2], 256, ctx->sms), 256, 0,
+                    ctx->stream>>>(ctx->g, ctx->amr_slot, cb, s, bg, ctx->cb[c], ctx->cb[c ^ 1], ctx->s[c][0],
+                                   ctx->s[c][1], ctx->s[c][2]);
     if (int r = launch_check(ctx, "unpack_kernel")) return r;
-    if (int r = copy_other(ctx)) return r;
     return mark_all(ctx);
 }
 
