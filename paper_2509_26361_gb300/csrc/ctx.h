@@ -76,6 +76,7 @@ struct ebit_ctx {
     // writes set mk_par ^ 1.  Set 0 is work/wcount above, set 1 work2/wcount2.
     unsigned *work2[NWORK];
     int *scan_count;          // [3] lengths of the marker lists of a whole-grid scan
+    int scan_done;            // those lists describe the current state
     int *wcount2;
     unsigned *mk_al[2];       // aligned edges that carry a marker, per set
     int *mk_count;            // [2] their lengths

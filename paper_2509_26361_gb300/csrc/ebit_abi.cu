@@ -75,18 +75,29 @@ int launched(ebit_ctx *ctx, cudaError_t e, const char *what) {
     return launch_check(ctx, what);
 }
 
+int blocks_for(long long n, int threads, int sms) {
+    long long b = (n + threads - 1) / threads;
+    long long cap = (long long)sms * 16;
+    if (b > cap) b = cap;
+    if (b < 1) b = 1;
+    return (int)b;
+}
+
 int mark_all(ebit_ctx *ctx) {
     ctx->sweeps_since_f2v = 1;
-    CU(cudaMemsetAsync(ctx->tile_marker, 0xFF, ctx->g.ntiles * sizeof(uint32_t), ctx->stream));
-    CU(cudaMemsetAsync(ctx->dirty_set ? ctx->tile_dirty2 : ctx->tile_dirty, 1, ctx->g.ntiles, ctx->stream));
-    if (ctx->tile_dirty2)
-        CU(cudaMemsetAsync(ctx->dirty_set ? ctx->tile_dirty : ctx->tile_dirty2, 0, ctx->g.ntiles, ctx->stream));
+    MarkAllArgs m;
+    m.ntiles = ctx->g.ntiles;
+    m.tile_marker = ctx->tile_marker;
+    m.dirty = ctx->dirty_set ? ctx->tile_dirty2 : ctx->tile_dirty;
+    m.clean = ctx->tile_dirty2 ? (ctx->dirty_set ? ctx->tile_dirty : ctx->tile_dirty2) : nullptr;
+    m.band_flag = ctx->band_flag;
+    m.band_count = ctx->owns_state ? ctx->band_count : nullptr;
+    m.scan_count = ctx->scan_count;
+    mark_all_kernel<<<blocks_for(ctx->g.ntiles, 256, ctx->sms), 256, 0, ctx->stream>>>(m);
+    if (int r = launch_check(ctx, "mark_all_kernel")) return r;
     // the next sweep processes every tile and lists the markers and band anew
     ctx->mk_valid = 0;
-    if (ctx->owns_state) {
-        CU(cudaMemsetAsync(ctx->band_flag, 0, ctx->g.ntiles * sizeof(uint32_t), ctx->stream));
-        CU(cudaMemsetAsync(ctx->band_count, 0, 2 * sizeof(int), ctx->stream));
-    }
+    ctx->scan_done = 0;
     ctx->last_C = nullptr;
     ctx->last_kh = nullptr;
     ctx->last_st = nullptr;
@@ -125,21 +136,41 @@ int call_stream(ebit_ctx *ctx, int flags, cudaStream_t *st) {
     return EBIT_OK;
 }
 
+// The colours into the other buffer: a sweep leaves the tiles outside its band
+// unwritten.  (Offsets need no copy: they are read only on edges with a marker,
+// and a sweep writes every marker's.)
 int copy_other(ebit_ctx *ctx) {
-    int o = ctx->cur ^ 1;
-    CU(cudaMemcpyAsync(ctx->cb[o], ctx->cb[ctx->cur], ctx->N, cudaMemcpyDeviceToDevice, ctx->stream));
-    for (int a = 0; a < 3; a++)
-        CU(cudaMemcpyAsync(ctx->s[o][a], ctx->s[ctx->cur][a], ctx->N * sizeof(double), cudaMemcpyDeviceToDevice,
-                           ctx->stream));
+    CU(cudaMemcpyAsync(ctx->cb[ctx->cur ^ 1], ctx->cb[ctx->cur], ctx->N, cudaMemcpyDeviceToDevice, ctx->stream));
     return EBIT_OK;
 }
 
-int blocks_for(long long n, int threads, int sms) {
-    long long b = (n + threads - 1) / threads;
-    long long cap = (long long)sms * 16;
-    if (b > cap) b = cap;
-    if (b < 1) b = 1;
-    return (int)b;
+// Is p memory that this device's kernels may access as T?
+template <typename T>
+bool on_device(const T *p) {
+    cudaPointerAttributes a;
+    const cudaError_t e = cudaPointerGetAttributes(&a, p);
+    cudaGetLastError();
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return e == cudaSuccess && ((a.type == cudaMemoryTypeDevice && a.device == dev) || a.type == cudaMemoryTypeManaged) &&
+           (uintptr_t)p % sizeof(T) == 0;
+}
+
+// lists and grid of a whole-grid marker scan (set mk_par's arrays, free then)
+ScanArgs scan_args(ebit_ctx *ctx) {
+    ScanArgs a;
+    unsigned *const *wk = ctx->mk_par ? ctx->work2 : ctx->work;
+    a.g = ctx->g;
+    a.cb = ctx->cb[ctx->cur];
+    a.whole = (ctx->N + 7) & ~7LL;
+    a.list[0] = ctx->mk_al[ctx->mk_par];
+    a.list[1] = wk[0];
+    a.list[2] = wk[1];
+    a.list_count = ctx->scan_count;
+    return a;
+}
+int scan_grid(const ebit_ctx *ctx) {
+    return blocks_for((ctx->N / ctx->g.n[0]) * ((ctx->g.n[0] + 7) / 8), 256, ctx->sms);
 }
 
 // Event pairs around the timed launches; drained into per-kind sums.
@@ -241,6 +272,7 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
     ctx->mk_par = 0;
     ctx->mk_dir = 0;
     ctx->mk_valid = 0;
+    ctx->scan_done = 0;
     ctx->iface[0] = ctx->iface[1] = nullptr;
     ctx->wcount = ctx->ncut = ctx->niface = ctx->nscan = ctx->zero = nullptr;
     ctx->cut = ctx->scan = nullptr;
@@ -474,7 +506,23 @@ int ebit_init(ebit_ctx *ctx, const double *phi_nodes, const double *phi_faces, c
 int ebit_set_state(ebit_ctx *ctx, const uint8_t *cb, const double *s) {
     if (!ctx || !cb || !s) return fail(ctx, EBIT_EINVAL, "ebit_set_state: null argument");
     if (int r = join_side(ctx)) return r;
-    int c = ctx->cur;
+    const int c = ctx->cur;
+    if (ctx->owns_state && on_device(cb) && on_device(s)) {
+        // one pass: colours into both buffers, the markers' offsets, and the
+        // marker lists of the next sweep
+        if (int r = mark_all(ctx)) return r;
+        ScanArgs a = scan_args(ctx);
+        a.cb = cb;
+        a.whole = ((uintptr_t)cb & 7) == 0 ? ctx->N & ~7LL : 0;
+        a.cb1 = ctx->cb[c];
+        a.cb2 = ctx->cb[c ^ 1];
+        a.src = s;
+        for (int k = 0; k < 3; k++) a.s[k] = ctx->s[c][k];
+        mark_scan_kernel<<<scan_grid(ctx), 256, 0, ctx->stream>>>(a);
+        if (int r = launch_check(ctx, "mark_scan_kernel")) return r;
+        ctx->scan_done = 1;
+        return EBIT_OK;
+    }
     CU(cudaMemcpyAsync(ctx->cb[c], cb, ctx->N, cudaMemcpyDefault, ctx->stream));
     for (int a = 0; a < 3; a++)
         CU(cudaMemcpyAsync(ctx->s[c][a], s + a * ctx->N, ctx->N * sizeof(double), cudaMemcpyDefault, ctx->stream));
@@ -617,17 +665,24 @@ int ebit_one_fluid(ebit_ctx *ctx, const double *C, const double *kappa_h, const 
 int ebit_get_state(ebit_ctx *ctx, uint8_t *cb, double *s) {
     if (!ctx || !cb || !s) return fail(ctx, EBIT_EINVAL, "ebit_get_state: null argument");
     if (int r = join_side(ctx)) return r;
+    const int c = ctx->cur;
+    // straight into device arrays; host arrays through a scratch copy of the
+    // offsets, which the first call reserves whatever its arrays are, so that no
+    // later read-back fails for want of room
+    const bool direct = on_device(cb) && on_device(s);
     if (!ctx->scratch && !dev_alloc(ctx->mem, (void **)&ctx->scratch, 3 * ctx->N * sizeof(double))) {
         cudaGetLastError();
         return fail(ctx, EBIT_ENOMEM, "ebit_get_state: no room for the scratch copy");
     }
-    int c = ctx->cur;
-    canonical_s_kernel<<<blocks_for(ctx->N, 256, ctx->sms), 256, 0, ctx->stream>>>(
-        ctx->g, ctx->cb[c], ctx->s[c][0], ctx->s[c][1], ctx->s[c][2], ctx->scratch);
-    int r = launch_check(ctx, "canonical_s_kernel");
+    state_out_kernel<<<scan_grid(ctx), 256, 0, ctx->stream>>>(ctx->g, ctx->cb[c], (ctx->N + 7) & ~7LL, ctx->s[c][0],
+                                                              ctx->s[c][1], ctx->s[c][2], direct ? cb : nullptr,
+                                                              direct ? s : ctx->scratch);
+    int r = launch_check(ctx, "state_out_kernel");
     if (r) return r;
-    CU(cudaMemcpyAsync(cb, ctx->cb[c], ctx->N, cudaMemcpyDefault, ctx->stream));
-    CU(cudaMemcpyAsync(s, ctx->scratch, 3 * ctx->N * sizeof(double), cudaMemcpyDefault, ctx->stream));
+    if (!direct) {
+        CU(cudaMemcpyAsync(cb, ctx->cb[c], ctx->N, cudaMemcpyDefault, ctx->stream));
+        CU(cudaMemcpyAsync(s, ctx->scratch, 3 * ctx->N * sizeof(double), cudaMemcpyDefault, ctx->stream));
+    }
     return ebit_sync(ctx);
 }
 
@@ -710,12 +765,13 @@ int ebit_advect_sweep(ebit_ctx *ctx, int dir, const double *u_face, double dt) {
         ml.band = nullptr;
         ml.band_count = nullptr;
         a.scan_count = ctx->scan_count;
-        ProfScope ps(ctx, EBIT_PROF_ADVECT);
-        const long long groups = (ctx->N / ctx->g.n[0]) * ((ctx->g.n[0] + 7) / 8);
-        int r = launched(ctx, launch_pdl(mark_scan_kernel, blocks_for(groups, 256, ctx->sms), 256, 0, ctx->stream, a,
-                                         ctx->mk_al[rd], wk_rd[0], wk_rd[1], ctx->scan_count),
-                         "mark_scan_kernel");
-        if (r) return r;
+        if (!ctx->scan_done) {
+            ProfScope ps(ctx, EBIT_PROF_ADVECT);
+            int r = launched(ctx, launch_pdl(mark_scan_kernel, scan_grid(ctx), 256, 0, ctx->stream, scan_args(ctx)),
+                             "mark_scan_kernel");
+            if (r) return r;
+        }
+        ctx->scan_done = 0;
     }
     int r;
     switch (dir) {

@@ -27,6 +27,7 @@
 
 #include "../../include/ebit.h"
 #include "common.cuh"
+#include "state.cuh"
 #include "sweep.cuh"
 
 using namespace ebit;
@@ -95,7 +96,13 @@ template <int D>
 void launch_all(const SweepArgs &a, const MarkerLists &m, cudaStream_t st, int grid_scan, int grid_tiles, int grid_fp64) {
     // the marker lists use the work lists' arrays: they are read before the
     // band pass writes those
-    mark_scan_kernel<<<grid_scan, 256, 0, st>>>(a, a.work[0], a.work[1], a.work[2], a.scan_count);
+    ScanArgs sc;
+    sc.g = a.g;
+    sc.cb = a.cb;
+    sc.whole = a.cb_whole;
+    for (int k = 0; k < 3; k++) sc.list[k] = a.work[k];
+    sc.list_count = a.scan_count;
+    mark_scan_kernel<<<grid_scan, 256, 0, st>>>(sc);
     advect_list_kernel<D><<<grid_fp64, 256, 0, st>>>(a, m);
     sweep_kernel<D><<<grid_tiles, BAND_THREADS, 0, st>>>(a);
     fp64_kernel<D><<<grid_fp64, 128, 0, st>>>(a);

@@ -16,8 +16,8 @@
 // instruction costs its issue slots whatever the number of active lanes, so all
 // FP64 arithmetic runs from compacted lists with full warps, and the band pass
 // over the cells is integer work:
-//   mark_scan_kernel -- after a state change, the markers of the whole grid
-//                    listed from the colours.
+//   mark_scan_kernel -- (state.cuh) after a state change, the markers of the
+//                    whole grid listed from the colours.
 //   advect_list_kernel -- every listed marker moved once (trilinear velocity):
 //                    adv = its advected coordinate along D relative to its node
 //                    (s + u dt/h for an aligned marker, u dt/h for an unaligned
@@ -240,59 +240,6 @@ __device__ __forceinline__ int warp_append(int *counter, bool flag) {
 }
 
 // ---------------------------------------------------------------- advection
-// The markers of the whole grid, one list per edge axis, from the node colours
-// (after a state change, in dense mode and in the allocation-free sweep).  One
-// thread per 8 cells of an x-row: the row's colours and those of the next rows
-// along y and z are 8-bit masks, their exclusive-ors the marked edges; a warp
-// reserves its slots with one round of atomics.  count[3] starts at zero.  (6 us
-// at 128^3; the staged pass per tile that it and the marker lists replace, 24-30.)
-static __global__ void __launch_bounds__(256) mark_scan_kernel(SweepArgs a, unsigned *l0, unsigned *l1, unsigned *l2,
-                                                               int *count) {
-    pdl_wait();
-    const int nx = a.g.n[0], ny = a.g.n[1], nz = a.g.n[2];
-    const long long n = (long long)nx * ny * nz;
-    const int gx = (nx + 7) / 8;
-    const long long groups = (long long)gx * ny * nz;
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long t0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); t0 < groups; t0 += stride) {
-        const long long t = t0 + lane;
-        unsigned m[3] = {0, 0, 0};
-        int id = 0;
-        if (t < groups) {
-            const int row = (int)(t / gx), x = 8 * (int)(t - (long long)row * gx);
-            const int z = row / ny, y = row - z * ny;
-            id = row * nx + x;
-            const unsigned ok = nx - x >= 8 ? 0xFFu : (1u << (nx - x)) - 1u;
-            const unsigned c = gather_bits(load_colours8(a.cb, id, a.cb_whole, n));
-            const unsigned cy = gather_bits(load_colours8(a.cb, (long long)(z * ny + wrapc(y + 1, ny)) * nx + x, a.cb_whole, n));
-            const unsigned cz = gather_bits(load_colours8(a.cb, (long long)(wrapc(z + 1, nz) * ny + y) * nx + x, a.cb_whole, n));
-            // the node after the group's last valid one
-            const int last = min(x + 8, nx) - x - 1;
-            const unsigned cn = __ldg(a.cb + row * nx + wrapc(x + last + 1, nx)) & 1u;
-            const unsigned up = (c >> 1 & ~(1u << last)) | cn << last;
-            m[0] = (c ^ up) & ok;
-            m[1] = (c ^ cy) & ok;
-            m[2] = (c ^ cz) & ok;
-        }
-        if (!__any_sync(full, m[0] | m[1] | m[2])) continue;
-        unsigned tot;
-        const unsigned pre = warp_prefix(__popc(m[0]) | __popc(m[1]) << 10 | __popc(m[2]) << 20, &tot);
-        int base = 0;
-        if (lane < 3) {
-            const unsigned c = (tot >> (10 * lane)) & 1023u;
-            if (c) base = atomicAdd(count + lane, (int)c);
-        }
-#pragma unroll
-        for (int k = 0; k < 3; k++) {
-            unsigned *l = k == 0 ? l0 : (k == 1 ? l1 : l2);
-            int pos = __shfl_sync(full, base, k) + (int)((pre >> (10 * k)) & 1023u);
-            for (unsigned w = m[k]; w; w &= w - 1) l[pos++] = (unsigned)(id + __ffs((int)w) - 1);
-        }
-    }
-}
-
 // Move every marker of one band tile once (Eq. 2).  CFL >= 1 is counted and
 // clamped; a displacement that is not finite (NaN or infinite velocity) is
 // counted apart and the marker stays where it is.  Called by all threads of the block; s_mk/s_c/s_n are its shared
