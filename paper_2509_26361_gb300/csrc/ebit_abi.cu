@@ -375,7 +375,8 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f2v_list_kernel, 128, 0);
     ctx->grid_f2vl = ctx->sms * std::max(occ, 1);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, hf_scan_kernel, 256, 0);
-    ctx->grid_hf = std::max(1, std::min(ntc, ctx->sms * std::max(occ, 1)));
+    ctx->grid_hf = std::max(1, std::min(((ctx->g.n[0] + SCAN_X - 1) / SCAN_X) * ((ctx->g.n[1] + 7) / 8) * ((ctx->g.n[2] + 7) / 8),
+                                        ctx->sms * std::max(occ, 1)));
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, hf_list_kernel<true>, 128, 0);
     ctx->grid_hfl = ctx->sms * std::max(occ, 1);
     cudaMemsetAsync(ctx->wcount, 0, (ctx->owns_state ? NLISTS + 1 : NLISTS) * sizeof(int), ctx->stream);
@@ -867,21 +868,33 @@ int ebit_curvature(ebit_ctx *ctx, const double *C, double *kappa_h, uint8_t *sta
     a.st = status;
     a.iface = ctx->iface[nw];
     a.niface = ctx->niface + cs;
-    a.list = ctx->all_list;
-    a.count = ctx->all_count;
     a.zero[0] = ctx->niface + cnext;
     a.zero[1] = nullptr;
+    // Interface cells: listed in a.iface (slot cs), others reset to 0 / NONE.
     if (full) {
-        // any C: scan every tile, reset non-interface cells, list the interface cells
-        ProfScope ps(ctx, EBIT_PROF_SCAN, st);
-        CU(cudaMemsetAsync(ctx->nscan, 0, sizeof(int), st));
-        int r = launched(ctx, launch_pdl(hf_scan_kernel, ctx->grid_hf, 256, 0, st, a, ctx->scan, ctx->nscan),
-                         "hf_scan_kernel");
-        if (r) return r;
+        // any C: a scan of every cell lists them; height functions (mode HF) then
+        // run on that list
+        {
+            ProfScope ps(ctx, EBIT_PROF_SCAN, st);
+            int r = launched(ctx,
+                             launch_pdl(hf_scan_kernel, ctx->grid_hf, 256, 0, st, ctx->g, C, kappa_h, status, a.iface,
+                                        a.niface, ctx->niface + cnext, ctx->nscan),
+                             "hf_scan_kernel");
+            if (r) return r;
+        }
         a.prev = ctx->iface[ctx->cur_if];
         a.nprev = ctx->zero;
-        a.cand = ctx->scan;
-        a.ncand = ctx->nscan;
+        a.cand = a.iface;
+        a.ncand = a.niface;
+        if (mode == EBIT_CURV_HF) {
+            HFArgs f = a;
+            f.iface = nullptr;
+            f.niface = nullptr;
+            f.zero[0] = nullptr;
+            ProfScope ps(ctx, EBIT_PROF_HF, st);
+            int r = launched(ctx, launch_pdl(hf_list_kernel<true>, ctx->grid_hfl, 128, 0, st, f), "hf_list_kernel");
+            if (r) return r;
+        }
     } else {
         // C is this context's Front2VOF output: its cut cells hold every interface cell
         a.prev = ctx->iface[ctx->cur_if];
@@ -890,8 +903,6 @@ int ebit_curvature(ebit_ctx *ctx, const double *C, double *kappa_h, uint8_t *sta
         a.ncand = ctx->ncut + ctx->f2v_par;
         // the fallback list of the learned pass below starts empty
         if (mode != EBIT_CURV_HF) a.zero[1] = ctx->nscan;
-    }
-    {
         // height functions on every interface cell (mode HF), or only the list
         ProfScope ps(ctx, EBIT_PROF_HF, st);
         cudaError_t e = (mode == EBIT_CURV_HF)
@@ -914,9 +925,8 @@ int ebit_curvature(ebit_ctx *ctx, const double *C, double *kappa_h, uint8_t *sta
         m.kh = kappa_h;
         m.st = status;
         m.mode = mode;
-        m.fb = ctx->scan;  // free again: the listing pass above has consumed it
+        m.fb = ctx->scan;
         m.nfb = ctx->nscan;
-        if (full) CU(cudaMemsetAsync(ctx->nscan, 0, sizeof(int), st));
         int r;
         {
             ProfScope pm(ctx, EBIT_PROF_MLP, st);
