@@ -1235,8 +1235,7 @@ static int mlp_grad_launch(ebit_mlp *mlp, const uint16_t *X, const float *t, con
     a.grad = mlp->g;
     a.loss = mlp->loss;
     const int ntile = (batch + 127) / 128;
-    mlp_train_kernel<<<std::min(ntile, mlp->sms), TRAIN_THREADS, TRAIN_SMEM, mlp->stream>>>(a);
-    MCU(cudaGetLastError());
+    MCU(launch_pdl(mlp_train_kernel, std::min(ntile, mlp->sms), TRAIN_THREADS, TRAIN_SMEM, mlp->stream, a));
     return EBIT_OK;
 }
 
@@ -1268,9 +1267,8 @@ int ebit_mlp_train_step(ebit_mlp *mlp, const uint16_t *X, const float *t, const 
         cudaGetLastError();
     }
     float *dst = loss_out ? (dev_out ? loss_out : mlp->loss + 1) : nullptr;
-    mlp_adam_kernel<<<(MLP_NP + 255) / 256, 256, 0, mlp->stream>>>(mlp->p, mlp->g, mlp->m, mlp->v, mlp->w1b, mlp->w2b,
-                                                                  lr, bc1, bc2, mlp->loss, dst);
-    MCU(cudaGetLastError());
+    MCU(launch_pdl(mlp_adam_kernel, (MLP_NP + 255) / 256, 256, 0, mlp->stream, mlp->p, mlp->g, mlp->m, mlp->v, mlp->w1b,
+                   mlp->w2b, lr, bc1, bc2, mlp->loss, dst));
     if (loss_out && !dev_out) MCU(cudaMemcpyAsync(loss_out, mlp->loss + 1, 4, cudaMemcpyDefault, mlp->stream));
     return EBIT_OK;
 }

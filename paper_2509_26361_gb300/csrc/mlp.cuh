@@ -315,6 +315,20 @@ __device__ __forceinline__ void ldsm4(const __nv_bfloat16 *p, uint32_t r[4]) {
                  : "r"((uint32_t)__cvta_generic_to_shared(p)));
 }
 
+// the same with each 8x8 matrix transposed: lanes give the rows of a matrix
+// stored with K as the row index, the registers get the operand layout
+__device__ __forceinline__ void ldsm4t(const __nv_bfloat16 *p, uint32_t r[4]) {
+#ifdef EBIT_MLP_CHECK
+    if (!__all_sync(0xffffffffu, MLP_S(p, 16, 1))) {
+        r[0] = r[1] = r[2] = r[3] = 0u;
+        return;
+    }
+#endif
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)));
+}
+
 __device__ __forceinline__ void mma16816(float c[4], const uint32_t a[4], uint32_t b0, uint32_t b1) {
     asm volatile(
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
@@ -324,11 +338,12 @@ __device__ __forceinline__ void mma16816(float c[4], const uint32_t a[4], uint32
 }
 
 // acc = A[m0 .. m0+31][0..K) * B[n0 .. n0+31][0..K)^T for the calling warp:
-// A rows are the M index, B rows the N index, both K contiguous.  Element
-// acc[mt][nt][e] is row m0 + 16 mt + g + 8 (e >> 1), column n0 + 8 nt + 2 t + (e & 1)
+// A rows are the M index, B rows the N index, both K contiguous; with TA (TB)
+// the operand is stored the other way, [K][M] ([K][N]), and read transposed.
+// Element acc[mt][nt][e] is row m0 + 16 mt + g + 8 (e >> 1), column n0 + 8 nt + 2 t + (e & 1)
 // with g = lane / 4, t = lane % 4.  A and B are 16-byte aligned shared
 // memory and LDA, LDB multiples of 8 elements (ldmatrix rows).
-template <int K, int LDA, int LDB>
+template <int K, int LDA, int LDB, bool TA = false, bool TB = false>
 __device__ __forceinline__ void warp_gemm32(const __nv_bfloat16 *A, const __nv_bfloat16 *B, int m0, int n0,
                                             float acc[2][4][4]) {
     const int lane = threadIdx.x & 31;
@@ -342,15 +357,23 @@ __device__ __forceinline__ void warp_gemm32(const __nv_bfloat16 *A, const __nv_b
     // (rows +0, k +0), (rows +8, k +0), (rows +0, k +8), (rows +8, k +8); for B
     // (n +0, k +0), (n +0, k +8), (n +8, k +0), (n +8, k +8), two n-tiles at once
     const int li = lane & 7, lm = lane >> 3;
-    const __nv_bfloat16 *pa = A + (m0 + li + 8 * (lm & 1)) * LDA + 8 * (lm >> 1);
-    const __nv_bfloat16 *pb = B + (n0 + li + 8 * (lm >> 1)) * LDB + 8 * (lm & 1);
+    const __nv_bfloat16 *pa = TA ? A + (li + 8 * (lm >> 1)) * LDA + m0 + 8 * (lm & 1)
+                                 : A + (m0 + li + 8 * (lm & 1)) * LDA + 8 * (lm >> 1);
+    const __nv_bfloat16 *pb = TB ? B + (li + 8 * (lm & 1)) * LDB + n0 + 8 * (lm >> 1)
+                                 : B + (n0 + li + 8 * (lm >> 1)) * LDB + 8 * (lm & 1);
 #pragma unroll
     for (int k0 = 0; k0 < K; k0 += 16) {
         uint32_t a[2][4], b[2][4];
 #pragma unroll
-        for (int mt = 0; mt < 2; mt++) ldsm4(pa + mt * 16 * LDA + k0, a[mt]);
+        for (int mt = 0; mt < 2; mt++) {
+            if (TA) ldsm4t(pa + mt * 16 + k0 * LDA, a[mt]);
+            else ldsm4(pa + mt * 16 * LDA + k0, a[mt]);
+        }
 #pragma unroll
-        for (int np = 0; np < 2; np++) ldsm4(pb + np * 16 * LDB + k0, b[np]);
+        for (int np = 0; np < 2; np++) {
+            if (TB) ldsm4t(pb + np * 16 + k0 * LDB, b[np]);
+            else ldsm4(pb + np * 16 * LDB + k0, b[np]);
+        }
 #pragma unroll
         for (int nt = 0; nt < 4; nt++)
 #pragma unroll
@@ -766,54 +789,61 @@ __device__ __forceinline__ void add_block4(float *G, int ld, int m0, int n0, con
 }
 
 // ------------------------------------------------------------ training
-// smem (bf16 tiles, row-major, padded):
-//   W1 [128][72] | W2 [128][136] (dH1^T after the dH1 product) | W2T [128][136] |
-//   X [128][72] | XT [64][136] | B1 [128][136] (H1, then dH2) | H1T [128][136] |
-//   dH2T [128][136] | reductions 512 floats
+// smem (bf16 tiles, row-major, padded): W1 [128][72] | W2 [128][136] |
+//   X [128][72] | H1 | dH2 | dH1 [128][136] each | reductions and parameters
+//
+// Every operand has one copy: the products that contract over rows (dW2 = dH2^T
+// H1, dW1 = dH1^T X) or take W2 the other way (dH1 = dH2 W2) read it through
+// ldmatrix.trans, and epilogues store two columns at a time.  With second,
+// transposed copies a thread made 208 two-byte shared stores per tile where it
+// now makes 48 four-byte ones, and the loss was added by 256 shared atomics to
+// two addresses where a warp now adds once.  What bounds the kernel is the chain
+// of one tile's phases (a batch of 16 384 is 128 tiles, one per SM): 31 us, now 21.
 constexpr int TR_W1 = 0;
 constexpr int TR_W2 = TR_W1 + 128 * LD64 * 2;
-constexpr int TR_W2T = TR_W2 + 128 * LD128 * 2;
-constexpr int TR_X = TR_W2T + 128 * LD128 * 2;
-constexpr int TR_XT = TR_X + 128 * LD64 * 2;
-constexpr int TR_B1 = TR_XT + 64 * LD128 * 2;
-constexpr int TR_H1T = TR_B1 + 128 * LD128 * 2;
-constexpr int TR_DH2T = TR_H1T + 128 * LD128 * 2;
-constexpr int TR_RED = TR_DH2T + 128 * LD128 * 2;
-// after the bf16 tiles: reductions (388 floats), b1 | b2 | w3 (384), the tile's targets (128)
-constexpr int TRAIN_SMEM = TR_RED + 900 * 4;
+constexpr int TR_X = TR_W2 + 128 * LD128 * 2;
+constexpr int TR_H1 = TR_X + 128 * LD64 * 2;
+constexpr int TR_DH2 = TR_H1 + 128 * LD128 * 2;
+constexpr int TR_DH1 = TR_DH2 + 128 * LD128 * 2;
+constexpr int TR_RED = TR_DH1 + 128 * LD128 * 2;
+// after the bf16 tiles: reductions (388 floats), b1 | b2 | w3 (384), the tile's
+// targets (128), shares of y (512)
+constexpr int TRAIN_SMEM = TR_RED + (388 + 384 + 128 + 512) * 4;
 constexpr int TRAIN_THREADS = 512;            // 16 warps: 4 row blocks x 4 column blocks of 32
 static_assert(MLP_IN == 64 && MLP_H == 128, "the training kernel's warp split assumes 64 inputs, 128 hidden units");
 static_assert(TRAIN_SMEM <= 227 * 1024, "training tile exceeds the shared memory of one block");
 
+// two neighbouring columns of a bf16 tile (p: 4-byte aligned)
+__device__ __forceinline__ void store_pair(__nv_bfloat16 *p, float lo, float hi) {
+    *reinterpret_cast<uint32_t *>(p) = pack_bf16x2(lo, hi);
+}
+
 __global__ void __launch_bounds__(TRAIN_THREADS) mlp_train_kernel(MlpArgs a) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __nv_bfloat16 *sW1 = reinterpret_cast<__nv_bfloat16 *>(smem_raw + TR_W1);
     __nv_bfloat16 *sW2 = reinterpret_cast<__nv_bfloat16 *>(smem_raw + TR_W2);
-    __nv_bfloat16 *sW2T = reinterpret_cast<__nv_bfloat16 *>(smem_raw + TR_W2T);
     __nv_bfloat16 *sX = reinterpret_cast<__nv_bfloat16 *>(smem_raw + TR_X);
-    __nv_bfloat16 *sXT = reinterpret_cast<__nv_bfloat16 *>(smem_raw + TR_XT);
-    __nv_bfloat16 *sB1 = reinterpret_cast<__nv_bfloat16 *>(smem_raw + TR_B1);
-    __nv_bfloat16 *sH1T = reinterpret_cast<__nv_bfloat16 *>(smem_raw + TR_H1T);
-    __nv_bfloat16 *sdH2T = reinterpret_cast<__nv_bfloat16 *>(smem_raw + TR_DH2T);
+    __nv_bfloat16 *sH1 = reinterpret_cast<__nv_bfloat16 *>(smem_raw + TR_H1);
+    __nv_bfloat16 *sdH2 = reinterpret_cast<__nv_bfloat16 *>(smem_raw + TR_DH2);
+    __nv_bfloat16 *sdH1 = reinterpret_cast<__nv_bfloat16 *>(smem_raw + TR_DH1);
     float *red = reinterpret_cast<float *>(smem_raw + TR_RED);  // dw3 | db1 | db2 | db3, loss
     float *prm = red + 388;  // b1 | b2 | w3, staged once
     float *st = red + 772;   // targets of the tile's rows
-    // [column block][row]: partial sums of y over 32 hidden units of layer 2,
-    // over the X tile, which layer 1 has finished reading
-    float *sy = reinterpret_cast<float *>(sX);
+    float *sy = red + 900;   // [column block][row]: partial sums of y over 32 hidden units of layer 2
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t4 = lane & 3;
     // warp (row block, column block) of every 128 x 128 product
     const int m0 = (warp & 3) * 32, cb = warp >> 2, n0 = cb * 32;
     const int row_t = tid & 127, part = tid >> 7;  // the tile row and quarter a thread stages
-    if (tid < 128) load_row(sW1, LD64, tid, a.w1b, tid, MLP_IN, MLP_H);
-    {
-        // W2^T: a quarter of row row_t by 16-byte loads, written down column row_t
-        __align__(16) __nv_bfloat16 wv[32];
-        const uint4 *s4 = reinterpret_cast<const uint4 *>(a.w2b + row_t * MLP_H) + 4 * part;
 #pragma unroll
-        for (int q = 0; q < 4; q++) reinterpret_cast<uint4 *>(wv)[q] = s4[q];
+    for (int q = 0; q < 2; q++) {  // 8 threads per row of W1, 16 bytes each
+        const int c = q * TRAIN_THREADS + tid, r = c >> 3;
+        reinterpret_cast<uint4 *>(sW1 + r * LD64)[c & 7] = reinterpret_cast<const uint4 *>(a.w1b + r * MLP_IN)[c & 7];
+    }
 #pragma unroll
-        for (int j = 0; j < 32; j++) sW2T[(part * 32 + j) * LD128 + row_t] = wv[j];
+    for (int q = 0; q < 4; q++) {  // 16 threads per row of W2
+        const int c = q * TRAIN_THREADS + tid, r = c >> 4;
+        reinterpret_cast<uint4 *>(sW2 + r * LD128)[c & 15] = reinterpret_cast<const uint4 *>(a.w2b + r * MLP_H)[c & 15];
     }
     for (int k = tid; k < 388; k += TRAIN_THREADS) red[k] = 0.0f;
     if (tid < 384) prm[tid] = ldp(a.params, tid < 256 ? (tid < 128 ? P_B1 + tid : P_B2 + tid - 128) : P_W3 + tid - 256);
@@ -822,36 +852,23 @@ __global__ void __launch_bounds__(TRAIN_THREADS) mlp_train_kernel(MlpArgs a) {
     const int ntile = (B + 127) / 128;
     const float invB = 1.0f / (float)B;
     for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
-        // W2 (its buffer holds dH1^T by the end of a tile), this tile's rows
-        // of X and their transpose; each thread stages a quarter of one row
-#pragma unroll
-        for (int q = 0; q < 4; q++) {  // 16 threads per row of W2, 16 bytes each
-            const int c = q * TRAIN_THREADS + tid, r = c >> 4;
-            reinterpret_cast<uint4 *>(sW2 + r * LD128)[c & 15] =
-                reinterpret_cast<const uint4 *>(a.w2b + r * MLP_H)[c & 15];
-        }
+        // this tile's rows of X; each thread stages a quarter of one row
         {
             const int row = tile * 128 + row_t;
-            __align__(16) __nv_bfloat16 xv[16];
-            uint4 *x4 = reinterpret_cast<uint4 *>(xv);
+            uint4 x0 = make_uint4(0u, 0u, 0u, 0u), x1 = x0;
             if (row < B) {
                 const long long src = a.idx ? a.idx[row] : row;
                 const uint4 *s4 = reinterpret_cast<const uint4 *>(a.X + src * MLP_IN) + 2 * part;
-                x4[0] = s4[0];
-                x4[1] = s4[1];
+                x0 = s4[0];
+                x1 = s4[1];
                 if (part == 0) st[row_t] = a.t[src];
-            } else {
-                x4[0] = make_uint4(0u, 0u, 0u, 0u);
-                x4[1] = x4[0];
             }
             uint4 *d4 = reinterpret_cast<uint4 *>(sX + row_t * LD64) + 2 * part;
-            d4[0] = x4[0];
-            d4[1] = x4[1];
-#pragma unroll
-            for (int i = 0; i < 16; i++) sXT[(part * 16 + i) * LD128 + row_t] = xv[i];
+            d4[0] = x0;
+            d4[1] = x1;
         }
         __syncthreads();
-        // ---- layer 1: the warp's block of H1 (rows) and H1T; ReLU mask kept
+        // ---- layer 1: the warp's block of H1; ReLU mask kept
         uint32_t mask1 = 0;
         {
             float acc[2][4][4];
@@ -859,22 +876,23 @@ __global__ void __launch_bounds__(TRAIN_THREADS) mlp_train_kernel(MlpArgs a) {
 #pragma unroll
             for (int mt = 0; mt < 2; mt++)
 #pragma unroll
-                for (int nt = 0; nt < 4; nt++)
+                for (int nt = 0; nt < 4; nt++) {
+                    const int col = n0 + nt * 8 + 2 * t4;
+                    const float2 b1 = *reinterpret_cast<const float2 *>(prm + col);
 #pragma unroll
-                    for (int e = 0; e < 4; e++) {
-                        const int r = m0 + mt * 16 + g + 8 * (e >> 1), col = n0 + nt * 8 + 2 * t4 + (e & 1);
-                        const float z = acc[mt][nt][e] + prm[col];
-                        if (z > 0.0f) mask1 |= 1u << (mt * 16 + nt * 4 + e);
-                        const __nv_bfloat16 hb = __float2bfloat16_rn(fmaxf(z, 0.0f));
-                        sB1[r * LD128 + col] = hb;
-                        sH1T[col * LD128 + r] = hb;
+                    for (int hh = 0; hh < 2; hh++) {
+                        const float z0 = acc[mt][nt][2 * hh] + b1.x, z1 = acc[mt][nt][2 * hh + 1] + b1.y;
+                        if (z0 > 0.0f) mask1 |= 1u << (mt * 16 + nt * 4 + 2 * hh);
+                        if (z1 > 0.0f) mask1 |= 1u << (mt * 16 + nt * 4 + 2 * hh + 1);
+                        store_pair(sH1 + (m0 + mt * 16 + g + 8 * hh) * LD128 + col, fmaxf(z0, 0.0f), fmaxf(z1, 0.0f));
                     }
+                }
         }
         __syncthreads();
         // ---- layer 2, pass A: Z2 of the warp's block stays in registers for
         // pass B; its 32 hidden units' share of y per row goes to shared memory
         float acc2[2][4][4];
-        warp_gemm32<MLP_H, LD128, LD128>(sB1, sW2, m0, n0, acc2);
+        warp_gemm32<MLP_H, LD128, LD128>(sH1, sW2, m0, n0, acc2);
         {
             float yp[2][2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
 #pragma unroll
@@ -899,7 +917,7 @@ __global__ void __launch_bounds__(TRAIN_THREADS) mlp_train_kernel(MlpArgs a) {
         __syncthreads();
         // y per row from the four column blocks' shares, in a fixed order;
         // dy = dL/dy of the weighted squared error (replicated over the quad)
-        float dyv[2][2];
+        float dyv[2][2], sl = 0.0f, sd = 0.0f;
 #pragma unroll
         for (int mt = 0; mt < 2; mt++)
 #pragma unroll
@@ -914,17 +932,26 @@ __global__ void __launch_bounds__(TRAIN_THREADS) mlp_train_kernel(MlpArgs a) {
                     const float wgt = 1.0f / (den * den);
                     const float r = yv - tv;
                     d = 2.0f * wgt * r * invB;
-                    if (cb == 0 && t4 == 0) {  // once per row
-                        atomicAdd(&red[385], wgt * r * r);
-                        atomicAdd(&red[384], d);
-                    }
+                    sl += wgt * r * r;
+                    sd += d;
                 }
                 dyv[mt][hh] = d;
             }
-        // ---- layer 2, pass B: dH2 = dy w3 (Z2 > 0) as rows (over H1, which
-        // pass A has finished reading) and transposed; dw3, db2
+        if (cb == 0) {  // once per row: the lanes of a quad hold the same rows
 #pragma unroll
-        for (int nt = 0; nt < 4; nt++)
+            for (int o = 4; o < 32; o <<= 1) {
+                sl += __shfl_xor_sync(0xffffffffu, sl, o);
+                sd += __shfl_xor_sync(0xffffffffu, sd, o);
+            }
+            if (lane == 0) {
+                atomicAdd(&red[385], sl);
+                atomicAdd(&red[384], sd);
+            }
+        }
+        // ---- layer 2, pass B: dH2 = dy w3 (Z2 > 0); dw3, db2
+#pragma unroll
+        for (int nt = 0; nt < 4; nt++) {
+            float dh[2][2][2];  // [mt][hh][q]
 #pragma unroll
             for (int q = 0; q < 2; q++) {
                 const int col = n0 + nt * 8 + 2 * t4 + q;
@@ -935,13 +962,9 @@ __global__ void __launch_bounds__(TRAIN_THREADS) mlp_train_kernel(MlpArgs a) {
 #pragma unroll
                     for (int hh = 0; hh < 2; hh++) {
                         const float z = acc2[mt][nt][2 * hh + q] + b2v;
-                        const float dh = z > 0.0f ? dyv[mt][hh] * w3v : 0.0f;
+                        dh[mt][hh][q] = z > 0.0f ? dyv[mt][hh] * w3v : 0.0f;
                         sdw3 += dyv[mt][hh] * fmaxf(z, 0.0f);
-                        sdb2 += dh;
-                        const int r = m0 + mt * 16 + g + 8 * hh;
-                        const __nv_bfloat16 hb = __float2bfloat16_rn(dh);
-                        sB1[r * LD128 + col] = hb;
-                        sdH2T[col * LD128 + r] = hb;
+                        sdb2 += dh[mt][hh][q];
                     }
 #pragma unroll
                 for (int o = 4; o < 32; o <<= 1) {  // over the 8 row groups of the warp
@@ -953,46 +976,56 @@ __global__ void __launch_bounds__(TRAIN_THREADS) mlp_train_kernel(MlpArgs a) {
                     atomicAdd(&red[256 + col], sdb2);
                 }
             }
+#pragma unroll
+            for (int mt = 0; mt < 2; mt++)
+#pragma unroll
+                for (int hh = 0; hh < 2; hh++)
+                    store_pair(sdH2 + (m0 + mt * 16 + g + 8 * hh) * LD128 + n0 + nt * 8 + 2 * t4, dh[mt][hh][0], dh[mt][hh][1]);
+        }
         __syncthreads();
-        // ---- dH1 = (dH2 W2) (Z1 > 0), transposed over W2; db1
+        // ---- dH1 = (dH2 W2) (Z1 > 0); db1
         {
             float acc[2][4][4];
-            warp_gemm32<MLP_H, LD128, LD128>(sB1, sW2T, m0, n0, acc);
+            warp_gemm32<MLP_H, LD128, LD128, false, true>(sdH2, sW2, m0, n0, acc);
 #pragma unroll
-            for (int nt = 0; nt < 4; nt++)
+            for (int nt = 0; nt < 4; nt++) {
+#pragma unroll
+                for (int mt = 0; mt < 2; mt++)
+#pragma unroll
+                    for (int e = 0; e < 4; e++)
+                        if (!((mask1 >> (mt * 16 + nt * 4 + e)) & 1)) acc[mt][nt][e] = 0.0f;
+                const int col = n0 + nt * 8 + 2 * t4;
 #pragma unroll
                 for (int q = 0; q < 2; q++) {
-                    const int col = n0 + nt * 8 + 2 * t4 + q;
                     float sdb1 = 0.0f;
 #pragma unroll
                     for (int mt = 0; mt < 2; mt++)
 #pragma unroll
-                        for (int hh = 0; hh < 2; hh++) {
-                            const int e = 2 * hh + q;
-                            const bool on = (mask1 >> (mt * 16 + nt * 4 + e)) & 1;
-                            const float d1 = on ? acc[mt][nt][e] : 0.0f;
-                            sdb1 += d1;
-                            const int r = m0 + mt * 16 + g + 8 * hh;
-                            sW2[col * LD128 + r] = __float2bfloat16_rn(d1);
-                        }
+                        for (int hh = 0; hh < 2; hh++) sdb1 += acc[mt][nt][2 * hh + q];
 #pragma unroll
                     for (int o = 4; o < 32; o <<= 1) sdb1 += __shfl_xor_sync(0xffffffffu, sdb1, o);
-                    if (g == 0) atomicAdd(&red[128 + col], sdb1);
+                    if (g == 0) atomicAdd(&red[128 + col + q], sdb1);
                 }
+#pragma unroll
+                for (int mt = 0; mt < 2; mt++)
+#pragma unroll
+                    for (int hh = 0; hh < 2; hh++)
+                        store_pair(sdH1 + (m0 + mt * 16 + g + 8 * hh) * LD128 + col, acc[mt][nt][2 * hh], acc[mt][nt][2 * hh + 1]);
+            }
         }
-        __syncthreads();
-        // ---- dW2 = dH2^T H1 (A = dH2T, B = H1T): the warp's 32 x 32 block
+        // ---- dW2 = dH2^T H1: the warp's 32 x 32 block (needs nothing of dH1)
         {
             float acc[2][4][4];
-            warp_gemm32<128, LD128, LD128>(sdH2T, sH1T, m0, n0, acc);
+            warp_gemm32<128, LD128, LD128, true, true>(sdH2, sH1, m0, n0, acc);
             add_block4(a.grad + P_W2, MLP_H, m0, n0, acc);
         }
-        // ---- dW1 = dH1^T X (A = dH1T, B = XT): 8 blocks of 32 x 32, each
-        // split over the tile's two halves of 64 rows
+        __syncthreads();
+        // ---- dW1 = dH1^T X: 8 blocks of 32 x 32, each split over the tile's
+        // two halves of 64 rows
         {
             const int n1 = ((warp >> 2) & 1) * 32, k1 = (warp >> 3) * 64;
             float acc[2][4][4];
-            warp_gemm32<64, LD128, LD128>(sW2 + k1, sXT + k1, m0, n1, acc);
+            warp_gemm32<64, LD128, LD64, true, true>(sdH1 + k1 * LD128, sX + k1 * LD64, m0, n1, acc);
             add_block4(a.grad + P_W1, MLP_IN, m0, n1, acc);
         }
         __syncthreads();
@@ -1014,6 +1047,7 @@ __global__ void __launch_bounds__(TRAIN_THREADS) mlp_train_kernel(MlpArgs a) {
 __global__ void mlp_adam_kernel(float *__restrict__ p, float *__restrict__ g, float *__restrict__ m,
                                 float *__restrict__ v, __nv_bfloat16 *__restrict__ w1b, __nv_bfloat16 *__restrict__ w2b,
                                 float lr, float bc1, float bc2, float *__restrict__ loss, float *__restrict__ loss_dst) {
+    pdl_wait();
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (loss_dst) *loss_dst = *loss;
