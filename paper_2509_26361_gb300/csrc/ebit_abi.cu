@@ -659,7 +659,12 @@ int ebit_one_fluid(ebit_ctx *ctx, const double *C, const double *kappa_h, const 
     for (int d = 0; d < 3; d++) a.f[d] = force ? force + d * ctx->N : nullptr;
     if (!rho && !mu && !force) return EBIT_OK;
     ProfScope ps(ctx, EBIT_PROF_COUPLING, ctx->stream);
-    coupling_kernel<<<std::min(ctx->g.n[1] * ctx->g.n[2], 8 * ctx->sms), 256, 0, ctx->stream>>>(a);
+    // two cells per thread where every row of every array starts on a 16-byte boundary
+    auto even = [](const void *p) { return ((uintptr_t)p & 15) == 0; };
+    if (ctx->g.n[0] % 2 == 0 && even(C) && even(rho) && even(mu) && even(force))
+        coupling_kernel<2><<<(unsigned)((ctx->N / 2 + 255) / 256), 256, 0, ctx->stream>>>(a);
+    else
+        coupling_kernel<1><<<(unsigned)((ctx->N + 255) / 256), 256, 0, ctx->stream>>>(a);
     return launch_check(ctx, "coupling_kernel");
 }
 
