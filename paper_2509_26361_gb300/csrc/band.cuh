@@ -213,11 +213,16 @@ __device__ __forceinline__ unsigned warp_prefix(unsigned v, unsigned *total) {
     return inc - v;
 }
 
-// One band tile, 64 threads (`bar`: a named barrier of theirs); the caller
-// synchronises them before `sm` is used again.  With F, data written earlier in the same launch
+// One band tile of grid g, 64 threads (`bar`: a named barrier of theirs); the
+// caller synchronises them before `sm` is used again.  The grid's cells start
+// at `base` and its tiles at `tbase` of the arrays (0, 0 for a single context, its
+// slice of the arena for an instance of a batch); `whole`: see load_colours8,
+// for the colours from base on.  Ids on the lists count from the arrays' start.
+// With F, data written earlier in the same launch
 // (bins, advected coordinates) is read through L2.
 template <int D, bool F, int SH = 0>
-__device__ __forceinline__ void band_tile(const SweepArgs &a, int tile, BandSmem<D, SH> &sm, int bar, BandEvents &ev) {
+__device__ __forceinline__ void band_tile(const SweepArgs &a, const Grid &g, int base0, int tbase, long long whole, int tile,
+                                          BandSmem<D, SH> &sm, int bar, BandEvents &ev) {
     using R = BandRegion<D, SH>;
     using M = typename BandSmem<D, SH>::M;
     constexpr int A = D, T1 = (D + 1) % 3, T2 = (D + 2) % 3;
@@ -227,11 +232,12 @@ __device__ __forceinline__ void band_tile(const SweepArgs &a, int tile, BandSmem
     constexpr M MR = ((M)1 << R::RX) - 1;
     const unsigned full = 0xffffffffu;
     const int tid = threadIdx.x & (BAND_THREADS - 1), lane = tid & 31, warp = tid >> 5;
-    const int nx = a.g.n[0], ny = a.g.n[1], nz = a.g.n[2];
+    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
     const long long n = (long long)nx * ny * nz;
+    const uint8_t *cb = a.cb + base0;
     uint16_t *list = sm.list + (warp ? BandSmem<D, SH>::LIST1 : 0);
     int o[3];
-    tile_origin(a.g, tile, o);
+    tile_origin(g, tile, o);
 
     // ---- the region's colours
     M mine[RPL];
@@ -243,8 +249,8 @@ __device__ __forceinline__ void band_tile(const SweepArgs &a, int tile, BandSmem
         if (r >= R::ROWS) continue;
         const int ry = r % RY + Y0, rz = r / RY + Z0;
         uint32_t f;
-        const M c = load_row<M, TX, X0, R::RX>(a.cb, (wrapc(o[2] + rz, nz) * ny + wrapc(o[1] + ry, ny)) * nx, o[0], nx,
-                                              a.cb_whole, n, 1 + A, &f);
+        const M c = load_row<M, TX, X0, R::RX>(cb, (wrapc(o[2] + rz, nz) * ny + wrapc(o[1] + ry, ny)) * nx, o[0], nx,
+                                              whole, n, 1 + A, &f);
         mine[q] = c;
         sm.C[r] = c;
         sm.up[r] = 0;
@@ -262,7 +268,7 @@ __device__ __forceinline__ void band_tile(const SweepArgs &a, int tile, BandSmem
     // the lane's row of cells
     const int ly = tid % TY, lz = tid / TY, y = o[1] + ly, z = o[2] + lz;
     const bool row_ok = tid < R::CELL_ROWS && y < ny && z < nz;
-    const int rowid = (z * ny + y) * nx + o[0];
+    const int rowid = base0 + (z * ny + y) * nx + o[0];
     if (colours != 3u) {
         // Every staged node has one colour: no marker lies on an edge whose
         // crossing could change a node, face or edge of this tile's cells, so
@@ -271,8 +277,8 @@ __device__ __forceinline__ void band_tile(const SweepArgs &a, int tile, BandSmem
         const uint32_t c = colours == 1u ? MT : 0u;
         if (row_ok) store_row<TX>(a.cbo, rowid, c, c, c, c, vx);
         if (tid == 0) {
-            a.tile_marker[tile] = 0u;
-            if (a.band_flag) a.band_flag[tile] = 0u;
+            a.tile_marker[tbase + tile] = 0u;
+            if (a.band_flag) a.band_flag[tbase + tile] = 0u;
         }
         return;
     }
@@ -307,7 +313,7 @@ __device__ __forceinline__ void band_tile(const SweepArgs &a, int tile, BandSmem
             b[j] = 0;
             if (code[j] >= 0) {
                 const int r = code[j] >> 6;
-                b[j] = ld_in<F>(a.bin[A] + lin(a.g, o[0] + (code[j] & 63) + X0, o[1] + r % RY + Y0, o[2] + r / RY + Z0));
+                b[j] = ld_in<F>(a.bin[A] + base0 + lin(g, o[0] + (code[j] & 63) + X0, o[1] + r % RY + Y0, o[2] + r / RY + Z0));
             }
         }
 #pragma unroll
@@ -367,7 +373,6 @@ __device__ __forceinline__ void band_tile(const SweepArgs &a, int tile, BandSmem
         lost = pres & ~odd;
         below = la;
         above = lc;
-        ev.markers += __popc(pres);
         ev.multi += __popc(many);
         ev.inconsistent += __popc(lost);
         ev.annihilate += __popc(~pres & two & vx);
@@ -377,6 +382,7 @@ __device__ __forceinline__ void band_tile(const SweepArgs &a, int tile, BandSmem
         const uint32_t along = (v000 ^ vm00) | (v100 ^ vm00);
         wk[0] = p1;
         wk[1] = p2;
+        ev.markers += __popc(pres) + __popc(p1) + __popc(p2);
         wk[4] = (along | (V(-1, 1, 0) ^ vm00) | (v010 ^ vm00) | (V(1, 1, 0) ^ vm00)) & ~p1 & vx;
         wk[5] = (along | (V(-1, 0, 1) ^ vm00) | (v001 ^ vm00) | (V(1, 0, 1) ^ vm00)) & ~p2 & vx;
         // face colours: family 1 faces are normal to T2, family 2 to T1
@@ -425,7 +431,7 @@ __device__ __forceinline__ void band_tile(const SweepArgs &a, int tile, BandSmem
         int pos = __shfl_sync(full, base, k) + (int)(((k < 3 ? w0 : w1) >> (10 * (k % 3))) & 1023u);
         // an unaligned edge is on list k or, checked for annihilation, on list
         // k + 4, never on both: the two share an array, from its two ends
-        unsigned *w = k < 4 ? a.work[k] : a.work[k - 4] + (n - 1);
+        unsigned *w = k < 4 ? a.work[k] : a.work[k - 4] + (a.cells - 1);
         for (uint32_t m = wk[k]; m; m &= m - 1, pos++) w[k < 4 ? pos : -pos] = (unsigned)(rowid + __ffs((int)m) - 1);
     }
     const int bal = __shfl_sync(full, base, 6);
@@ -433,10 +439,10 @@ __device__ __forceinline__ void band_tile(const SweepArgs &a, int tile, BandSmem
     for (int k = lane; k < (int)t2; k += 32) {
         const int c = list[k], src = c >> 11, r = (c >> 5) & 63;
         const int cx = o[0] + (c & 31), cy = o[1] + r % TY, cz = o[2] + r / TY;
-        const int id = (cz * ny + cy) * nx + cx;
+        const int id = base0 + (cz * ny + cy) * nx + cx;
         auto landed = [&](int e) -> double {
             const double xv =
-                ld_in<F>(a.adv[A] + lin(a.g, cx + (A == 0 ? e : 0), cy + (A == 1 ? e : 0), cz + (A == 2 ? e : 0)));
+                ld_in<F>(a.adv[A] + base0 + lin(g, cx + (A == 0 ? e : 0), cy + (A == 1 ? e : 0), cz + (A == 2 ? e : 0)));
             const double s = e == 0 ? xv : xv + (e < 0 ? -1.0 : 1.0);
             return __double_as_longlong(s) > __double_as_longlong(ONE_MINUS) ? ONE_MINUS : s;
         };
@@ -458,10 +464,10 @@ __device__ __forceinline__ void band_tile(const SweepArgs &a, int tile, BandSmem
     band_sync(bar);
     if (tid == 0) {
         const unsigned nm = sm.near[0] | sm.near[1];
-        a.tile_marker[tile] = nm;
-        a.tile_dirty[tile] = 1;
-        if (a.band_flag) a.band_flag[tile] = 0u;
-        if (a.mt_out && nm) a.mt_out[atomicAdd(a.mt_out_count, 1)] = tile;
+        a.tile_marker[tbase + tile] = nm;
+        a.tile_dirty[tbase + tile] = 1;
+        if (a.band_flag) a.band_flag[tbase + tile] = 0u;
+        if (a.mt_out && nm) a.mt_out[atomicAdd(a.mt_out_count, 1)] = tbase + tile;
     }
 }
 
@@ -476,7 +482,7 @@ __global__ void __launch_bounds__(BAND_THREADS, 16) sweep_kernel(SweepArgs a) {
     // cost), read one tile ahead
     for (int li = blockIdx.x; li < ntl;) {
         if (threadIdx.x == 0) s_next = a.tile_next ? (int)gridDim.x + atomicAdd(a.tile_next, 1) : li + (int)gridDim.x;
-        band_tile<D, false>(a, a.list[li], sm, 0, ev);
+        band_tile<D, false>(a, a.g, 0, 0, a.cb_whole, a.list[li], sm, 0, ev);
         __syncthreads();
         li = s_next;
         __syncthreads();

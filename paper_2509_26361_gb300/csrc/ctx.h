@@ -70,7 +70,7 @@ struct ebit_ctx {
     double *adv[3];           // advected marker coordinates of the current sweep (scratch)
     int8_t *bin[3];           // floor(2 adv) (scratch)
     unsigned *work[NWORK];    // work lists of a sweep (scratch)
-    int *wcount;              // [NLISTS] list lengths, then (not in a batch view) the band pass's tile counter
+    int *wcount;              // [NLISTS] list lengths, then the band pass's tile counter
     // A context's band sweeps alternate between two sets of lists: a sweep
     // reads set mk_par (the markers and band the previous sweep listed) and
     // writes set mk_par ^ 1.  Set 0 is work/wcount above, set 1 work2/wcount2.
@@ -86,7 +86,7 @@ struct ebit_ctx {
     uint32_t *band_flag;      // per tile: in the band list being built or processed
     int mk_par;               // set written by the last sweep
     int mk_dir;               // sweep axis of the last sweep
-    int mk_valid;             // the lists of set mk_par describe the current state
+    int mk_valid;             // the lists of set mk_par (a batch instance: of its batch) describe the current state
     unsigned *cut;            // cells cut by the interface at the last Front2VOF
     int *ncut;                // [2] its length, one slot per Front2VOF call modulo 2
     unsigned *iface[2];       // interface cells of the last two curvature calls
@@ -119,10 +119,6 @@ struct ebit_ctx {
 struct ebit_state_arrays {
     uint8_t *cb[2];
     double *s[2][3];
-    double *adv[3];
-    int8_t *bin[3];
-    unsigned *work[NWORK];
-    int *wcount;
     uint32_t *tile_marker;
     uint8_t *tile_dirty;
     unsigned long long *ctr;

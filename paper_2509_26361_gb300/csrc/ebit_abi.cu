@@ -322,12 +322,6 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
             ctx->cb[b] = st->cb[b];
             for (int a = 0; a < 3; a++) ctx->s[b][a] = st->s[b][a];
         }
-        for (int a = 0; a < 3; a++) {
-            ctx->adv[a] = st->adv[a];
-            ctx->bin[a] = st->bin[a];
-        }
-        for (int k = 0; k < NWORK; k++) ctx->work[k] = st->work[k];
-        ctx->wcount = st->wcount;
         ctx->tile_marker = st->tile_marker;
         ctx->tile_dirty = st->tile_dirty;
         ctx->ctr = st->ctr;
@@ -379,8 +373,8 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
                                         ctx->sms * std::max(occ, 1)));
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, hf_list_kernel<true>, 128, 0);
     ctx->grid_hfl = ctx->sms * std::max(occ, 1);
-    cudaMemsetAsync(ctx->wcount, 0, (ctx->owns_state ? NLISTS + 1 : NLISTS) * sizeof(int), ctx->stream);
     if (ctx->owns_state) {
+        cudaMemsetAsync(ctx->wcount, 0, (NLISTS + 1) * sizeof(int), ctx->stream);
         cudaMemsetAsync(ctx->wcount2, 0, (NLISTS + 1) * sizeof(int), ctx->stream);
         cudaMemsetAsync(ctx->mk_count, 0, 2 * sizeof(int), ctx->stream);
         cudaMemsetAsync(ctx->scan_count, 0, 3 * sizeof(int), ctx->stream);
@@ -727,6 +721,7 @@ int ebit_advect_sweep(ebit_ctx *ctx, int dir, const double *u_face, double dt) {
     }
     unsigned *const *wk_wr = wr ? ctx->work2 : ctx->work;
     for (int k = 0; k < NWORK; k++) a.work[k] = wk_wr[k];
+    a.cells = ctx->N;
     a.cb_whole = (ctx->N + 7) & ~7LL;
     a.wcount = wr ? ctx->wcount2 : ctx->wcount;
     a.tile_next = a.wcount + NLISTS;  // one int after the list lengths

@@ -10,17 +10,27 @@
 // arena, so Front2VOF, curvature, state access and counters work per instance
 // through the ordinary entry points' code.
 //
-// A sweep is one cooperative launch that runs four phases over all instances,
+// A sweep is one cooperative launch that runs three phases over all instances,
 // separated by a grid barrier:
-//   band    -- every (instance, tile) whose 3x3x3 tile neighbourhood held a
-//              marker is listed; the FP64 list lengths are cleared;
-//   advect  -- per listed tile: each marker moved once (velocity interpolated);
-//   sweep   -- per listed tile: integer colour/aligned-edge pass, FP64 lists;
-//   fp64    -- the FP64 lists of all instances as one index space.
+//   advect  -- each listed marker moved once (velocity interpolated); the band
+//              built from the previous sweep's list of tiles with markers nearby;
+//   sweep   -- per band tile: integer colour/aligned-edge pass (band.cuh), FP64
+//              lists, the marker and tile lists of the next sweep;
+//   fp64    -- the FP64 lists.
+// The lists are the batch's, not the instances': their entries count cells and
+// tiles of the arena, and an entry's instance is found by bisection of the
+// instances' first cells (or tiles).  Two sets of lists alternate with the state
+// buffers, as in a context.  After a state change of any instance (or the
+// autotuner's) batch_scan_kernel lists the markers and the band anew before the
+// next sweep.
 // Data written in one phase and read in a later one is loaded through L2 (not
 // the read-only path).  The barrier waits a bounded number of polls; on
 // timeout it sets an error flag, every block leaves, and ebit_batch_sync
 // reports EBIT_ETIMEOUT.
+//
+// Four steps and the fractions of 64 instances (32^3 to 128^3) take 2.4 ms; with
+// the band listed by testing every tile, the markers found by staging each band
+// tile and a third barrier they took 3.4.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -30,39 +40,33 @@
 #include "../../include/ebit.h"
 #include "common.cuh"
 #include "ctx.h"
+#include "state.cuh"
 #include "sweep.cuh"
 #include "tc.cuh"
 
 namespace ebit {
 
-// the largest colour block of advect_tile
-__host__ __device__ constexpr int adv_stage_max() {
-    int m = 0;
-    for (int sh = 0; sh < N_TILE_SHAPES; sh++) {
-        const int v = (tile_edge(sh, 0) + 1) * (tile_edge(sh, 1) + 1) * (tile_edge(sh, 2) + 1);
-        m = v > m ? v : m;
-    }
-    return m;
-}
-
-constexpr int BATCH_MAX = 1024;      // instances per batch (tile ids keep 20 bits)
+constexpr int BATCH_MAX = 1024;      // instances per batch
 constexpr int BATCH_THREADS = 256;
 constexpr long long BAR_POLLS = 1LL << 24;  // polls of 64 ns sleep: about a second
 
-struct BatchInst {
-    SweepArgs a;  // u, lam, list and count are unused (per-sweep arrays below)
-};
+// counters of one set of lists
+enum { B_WORK = 0, B_AL = SWEEP_LISTS, B_MT, B_BAND, B_DIR, B_N = 16 };
 
 struct BatchParams {
-    const BatchInst *inst;    // [n], for the current buffer parity
+    SweepArgs a;              // over the arena: its g, u, lam, list, count and ctr are unused
+    const Grid *grid;         // [n]
+    const int *coff;          // [n + 1] first cell of each instance
+    const int *toff;          // [n + 1] first tile of each instance
     int n;
-    int total_tiles;
-    const int *toff;          // [n + 1] first global tile of each instance
     const double *const *u;   // [n] velocity component of the sweep direction
     const double *lam;        // [n] dt / h
-    int *band;                // (instance << 20) | tile
-    int *nband;
-    int *wcount;              // [6 n] FP64 list lengths (all instances)
+    unsigned long long *ctr;  // [n][C_TOTAL]
+    // the previous sweep's lists (set rd) and counters, this sweep's counters
+    const unsigned *al, *un0, *un1;
+    const int *mtiles;
+    int *band;
+    int *rd, *wr;
     unsigned *bar;            // [2] arrivals, generation
     int *err;
 };
@@ -100,11 +104,11 @@ __device__ bool grid_barrier(const BatchParams &p, int *s_ok, long long max_poll
     return *s_ok != 0;
 }
 
-__device__ __forceinline__ int find_inst(const int *toff, int n, int gt) {
-    int lo = 0, hi = n;  // toff[lo] <= gt < toff[hi]
+__device__ __forceinline__ int find_inst(const int *off, int n, int i) {
+    int lo = 0, hi = n;  // off[lo] <= i < off[hi]
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
-        if (__ldg(toff + mid) <= gt) lo = mid;
+        if (off[mid] <= i) lo = mid;
         else hi = mid;
     }
     return lo;
@@ -112,118 +116,141 @@ __device__ __forceinline__ int find_inst(const int *toff, int n, int gt) {
 
 template <int D, int SH>
 __global__ void __launch_bounds__(BATCH_THREADS, 4) batch_sweep_kernel(BatchParams p) {
-    __shared__ uint16_t s_mk[3 * TILE_CELLS];
-    __shared__ uint8_t s_c[adv_stage_max()];
-    // the band pass's staging and the FP64 phase's prefix sums, in turn
     constexpr int GROUPS = BATCH_THREADS / BAND_THREADS;
-    constexpr size_t SHARED = sizeof(BandSmem<D, SH>) * GROUPS > sizeof(int) * (SWEEP_LISTS * BATCH_MAX + 1)
-                                  ? sizeof(BandSmem<D, SH>) * GROUPS
-                                  : sizeof(int) * (SWEEP_LISTS * BATCH_MAX + 1);
-    __shared__ __align__(16) unsigned char s_raw[SHARED];
-    BandSmem<D, SH> *s_band = reinterpret_cast<BandSmem<D, SH> *>(s_raw);
-    int *s_pre = reinterpret_cast<int *>(s_raw);
-    __shared__ int s_n, s_ok;
-    __shared__ int s_wsum[BATCH_THREADS / 32];
+    __shared__ BandSmem<D, SH> s_band[GROUPS];
+    __shared__ int s_ok;
+    __shared__ int s_coff[BATCH_MAX + 1], s_toff[BATCH_MAX + 1];
     if (*(volatile int *)p.err) return;
     const int stride = gridDim.x * blockDim.x;
-    const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
-
-    // ---- band: tiles near a marker, all instances
-    for (int k = gtid; k < SWEEP_LISTS * p.n; k += stride) p.wcount[k] = 0;
-    {
-        const int iters = (p.total_tiles + stride - 1) / stride;
-        for (int it = 0; it < iters; it++) {
-            const int gt = it * stride + gtid;
-            bool on = false;
-            int i = 0, t = 0;
-            if (gt < p.total_tiles) {
-                i = find_inst(p.toff, p.n, gt);
-                t = gt - __ldg(p.toff + i);
-                const Grid g = p.inst[i].a.g;
-                const int tx = t % g.td[0], ty = (t / g.td[0]) % g.td[1], tz = t / (g.td[0] * g.td[1]);
-                on = in_band(g, p.inst[i].a.tile_marker, tx, ty, tz);
-            }
-            const int slot = warp_append(p.nband, on);
-            if (slot >= 0) p.band[slot] = (i << 20) | t;
-        }
+    for (int k = threadIdx.x; k <= p.n; k += blockDim.x) {
+        s_coff[k] = __ldg(p.coff + k);
+        s_toff[k] = __ldg(p.toff + k);
     }
-    if (!grid_barrier(p, &s_ok)) return;
-    const int nb = __ldcg(p.nband);
+    // this sweep's counters (last read by the sweep before the previous one)
+    if (blockIdx.x == 0 && threadIdx.x < B_DIR) p.wr[threadIdx.x] = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 32) p.wr[B_DIR] = D;
+    __syncthreads();
 
-    // ---- advect
-    for (int li = blockIdx.x; li < nb; li += gridDim.x) {
-        const int e = __ldcg(p.band + li);
-        const int i = e >> 20;
-        advect_tile<D, SH>(p.inst[i].a, p.u[i], p.lam[i], e & 0xFFFFF, s_mk, s_c, &s_n);
+    // ---- advect, and the band
+    {
+        const int n0 = p.rd[B_AL], n1 = p.rd[B_WORK], n2 = p.rd[B_WORK + 1], pd = p.rd[B_DIR];
+        const int total = n0 + n1 + n2;
+        const long long all = total + 27ll * p.rd[B_MT];
+        for (int it = 0; (long long)it * stride < all; it++) {
+            const int t = list_item(it);
+            if (t >= all) continue;
+            if (t >= total) {
+                const int tb = t - total, gt = __ldg(p.mtiles + tb / 27);
+                const int i = find_inst(s_toff, p.n, gt);
+                band_item(p.grid[i], s_toff[i], gt - s_toff[i], tb % 27, p.a.tile_marker, p.a.band_flag, p.band,
+                          p.rd + B_BAND);
+                continue;
+            }
+            const int k = t < n0 ? 0 : (t < n0 + n1 ? 1 : 2);
+            const int j = t - (k == 0 ? 0 : (k == 1 ? n0 : n0 + n1));
+            const int gid = (int)__ldg((k == 0 ? p.al : (k == 1 ? p.un0 : p.un1)) + j);
+            const int i = find_inst(s_coff, p.n, gid);
+            unsigned hits = 0, bad = 0;
+            move_marker<D>(p.a, p.grid[i], s_coff[i], p.u[i], p.lam[i], pd + k < 3 ? pd + k : pd + k - 3, gid, hits, bad);
+            if (hits) atomicAdd(p.ctr + (size_t)i * C_TOTAL + C_CFL, 1ull);
+            if (bad) atomicAdd(p.ctr + (size_t)i * C_TOTAL + C_NONFINITE, 1ull);
+        }
     }
     if (!grid_barrier(p, &s_ok)) return;
 
     // ---- integer band pass
     {
+        const int nb = __ldcg(p.rd + B_BAND);
         const int grp = threadIdx.x / BAND_THREADS;
         for (int li = grp * gridDim.x + blockIdx.x; li < nb; li += gridDim.x * GROUPS) {
-            const int e = __ldcg(p.band + li);
-            const SweepArgs &a = p.inst[e >> 20].a;
+            const int gt = __ldcg(p.band + li);
+            const int i = find_inst(s_toff, p.n, gt);
+            const Grid g = p.grid[i];
+            const long long n = (long long)g.n[0] * g.n[1] * g.n[2];
+            unsigned long long *ctr = p.ctr + (size_t)i * C_TOTAL;
             BandEvents ev;
-            band_tile<D, true, SH>(a, e & 0xFFFFF, s_band[grp], 1 + grp, ev);
-            flush_events(ev, a.ctr);
-            if ((threadIdx.x & (BAND_THREADS - 1)) == 0) atomicAdd(a.ctr + C_TILES, 1ull);
+            band_tile<D, true, SH>(p.a, g, s_coff[i], s_toff[i], (n + 7) & ~7LL, gt - s_toff[i], s_band[grp], 1 + grp, ev);
+            flush_events(ev, ctr);
+            if ((threadIdx.x & (BAND_THREADS - 1)) == 0) atomicAdd(ctr + C_TILES, 1ull);
             band_sync(1 + grp);
         }
     }
     if (!grid_barrier(p, &s_ok)) return;
 
-    // ---- FP64 lists of every instance as one index space: block-wide prefix
-    // sums of the list lengths
+    // ---- FP64 lists
     {
-        const int m = SWEEP_LISTS * p.n;
-        const int per = (m + blockDim.x - 1) / blockDim.x;
-        int loc[SWEEP_LISTS * BATCH_MAX / BATCH_THREADS];
-        int sum = 0;
-        for (int q = 0; q < per; q++) {
-            const int j = threadIdx.x * per + q;
-            loc[q] = j < m ? __ldcg(p.wcount + j) : 0;
-            sum += loc[q];
-        }
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-        int inc = sum;
-        for (int off = 1; off < 32; off <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, inc, off);
-            if (lane >= off) inc += v;
-        }
-        if (lane == 31) s_wsum[wid] = inc;
-        __syncthreads();
-        int base = 0;
-        for (int w = 0; w < wid; w++) base += s_wsum[w];
-        int run = base + inc - sum;
-        for (int q = 0; q < per; q++) {
-            const int j = threadIdx.x * per + q;
-            if (j < m) s_pre[j] = run;
-            run += loc[q];
-        }
-        if (threadIdx.x == blockDim.x - 1) s_pre[m] = run;
-        __syncthreads();
-        // marker counts of the unaligned lists (one per entry)
-        if (blockIdx.x == 0)
-            for (int i = threadIdx.x; i < p.n; i += blockDim.x) {
-                const int nm = (s_pre[SWEEP_LISTS * i + 2] - s_pre[SWEEP_LISTS * i]);
-                if (nm) atomicAdd(p.inst[i].a.ctr + C_MARKERS, (unsigned long long)nm);
-            }
-        const int total = s_pre[m];
-        for (int t = gtid; t < total; t += stride) {
-            int lo = 0, hi = m;  // s_pre[lo] <= t < s_pre[hi]
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (s_pre[mid] <= t) lo = mid;
-                else hi = mid;
-            }
-            const int i = lo / SWEEP_LISTS, kind = lo - i * SWEEP_LISTS;
+        const WorkLanes<true> w(p.a, stride);
+        for (int it = 0; (long long)it * stride < w.lanes; it++) {
+            const int t = list_item(it);
+            if (t >= w.lanes) continue;
+            int kind, half;
+            const int gid = w.item(p.a, t, &kind, &half);
+            const int i = find_inst(s_coff, p.n, gid);
             unsigned ev[C_N] = {0, 0, 0, 0, 0};
-            fp64_item<D, true>(p.inst[i].a, kind, t - s_pre[lo], ev);
+            fp64_item<D, true>(p.a, p.grid[i], s_coff[i], kind, gid, ev, half);
 #pragma unroll
             for (int k = 0; k < C_N; k++)
-                if (k != C_MARKERS && ev[k]) atomicAdd(p.inst[i].a.ctr + k, (unsigned long long)ev[k]);
+                if (ev[k]) atomicAdd(p.ctr + (size_t)i * C_TOTAL + k, (unsigned long long)ev[k]);
         }
+    }
+}
+
+// The lists of set rd from the state: the markers of every instance (as
+// mark_scan_kernel lists a context's) and the band by the tiles' masks.  The
+// set's counters start at zero (direction 0).
+struct BatchScanArgs {
+    const uint8_t *cb;
+    const Grid *grid;
+    const int *coff, *toff, *goff;  // first cell, tile, group of 8 cells
+    int n;
+    const uint32_t *mask;
+    unsigned *list[3];  // edge axes 0, 1, 2
+    int *band;
+    int *counts;
+};
+__global__ void __launch_bounds__(256) batch_scan_kernel(BatchScanArgs a) {
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu;
+    const int stride = gridDim.x * blockDim.x;
+    const int first = blockIdx.x * blockDim.x + (threadIdx.x & ~31);
+    for (int t0 = first; t0 < a.goff[a.n]; t0 += stride) {
+        RowGroup r{{0u, 0u, 0u}, 0, 0, 0ull};
+        int base = 0;
+        if (t0 + lane < a.goff[a.n]) {
+            const int i = find_inst(a.goff, a.n, t0 + lane);
+            const Grid g = a.grid[i];
+            base = a.coff[i];
+            const long long n = (long long)g.n[0] * g.n[1] * g.n[2];
+            r = row_group(g, a.cb + base, (n + 7) & ~7LL, (g.n[0] + 7) / 8, t0 + lane - a.goff[i]);
+        }
+        if (!__any_sync(full, r.m[0] | r.m[1] | r.m[2])) continue;
+        unsigned tot;
+        const unsigned pre = warp_prefix(__popc(r.m[0]) | __popc(r.m[1]) << 10 | __popc(r.m[2]) << 20, &tot);
+        int slot = 0;
+        if (lane < 3) {
+            const unsigned c = (tot >> (10 * lane)) & 1023u;
+            if (c) slot = atomicAdd(a.counts + (lane == 0 ? B_AL : B_WORK + lane - 1), (int)c);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            int pos = __shfl_sync(full, slot, k) + (int)((pre >> (10 * k)) & 1023u);
+            for (unsigned w = r.m[k]; w; w &= w - 1) a.list[k][pos++] = (unsigned)(base + r.id + __ffs((int)w) - 1);
+        }
+    }
+    const int tiles = a.toff[a.n];
+    for (int t0 = first; t0 < tiles; t0 += stride) {
+        const int gt = t0 + lane;
+        bool on = false;
+        if (gt < tiles) {
+            const int i = find_inst(a.toff, a.n, gt), t = gt - a.toff[i];
+            const Grid g = a.grid[i];
+            on = in_band(g, a.mask + a.toff[i], t % g.td[0], (t / g.td[0]) % g.td[1], t / (g.td[0] * g.td[1]));
+        }
+        const unsigned m = __ballot_sync(full, on);
+        int base = 0;
+        if (lane == 0 && m) base = atomicAdd(a.counts + B_BAND, __popc(m));
+        base = __shfl_sync(full, base, 0);
+        if (on) a.band[base + __popc(m & ((1u << lane) - 1u))] = gt;
     }
 }
 
@@ -269,7 +296,6 @@ struct ebit_batch {
     std::vector<long long> coff;   // first cell of each instance in the arena
     std::vector<int> toff;         // first tile (current tile shape)
     std::vector<int> dims;         // nx, ny, nz of each instance
-    std::vector<BatchInst> htab[2];  // host copy of the launch tables
     long long cells = 0;
     int tiles = 0;
     int parity = 0;                // buffer holding the current state
@@ -278,17 +304,23 @@ struct ebit_batch {
     double *s[2][3] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}};
     double *adv[3] = {nullptr, nullptr, nullptr};
     int8_t *bin[3] = {nullptr, nullptr, nullptr};
-    unsigned *work[4] = {nullptr, nullptr, nullptr, nullptr};
-    int *wcount = nullptr;
+    // the sweeps' lists; sets alternate with the state buffers: set q's unaligned
+    // edges (two families, with the checks) and aligned markers, its tiles with
+    // markers nearby, and its counters (B_*)
+    unsigned *un[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}}, *saddle[2] = {nullptr, nullptr};
+    unsigned *al[2] = {nullptr, nullptr};
+    int *mtiles[2] = {nullptr, nullptr};
+    int *counts = nullptr;         // [2][B_N]
+    int *band = nullptr;
+    uint32_t *band_flag = nullptr;
     uint32_t *tile_marker = nullptr;
     uint8_t *tile_dirty = nullptr;
     unsigned long long *ctr = nullptr;
     // launch data
-    BatchInst *table[2] = {nullptr, nullptr};
-    int *d_toff = nullptr;
+    Grid *d_grid = nullptr;
+    int *d_off = nullptr;          // coff, toff, goff: [n + 1] each
     double **u[3] = {nullptr, nullptr, nullptr};
     double *lam = nullptr;
-    int *band = nullptr, *nband = nullptr;
     unsigned *bar = nullptr;
     int *err = nullptr;
     int have_u[3] = {0, 0, 0};
@@ -336,20 +368,98 @@ const void *sweep_fn(int d, int sh) {
 // co-resident blocks per SM that every direction's kernel of shape sh allows
 int max_ctas(const ebit_batch *b, int sh) { return std::min({b->occ[sh][0], b->occ[sh][1], b->occ[sh][2]}); }
 
+const int *off_cells(const ebit_batch *b) { return b->d_off; }
+const int *off_tiles(const ebit_batch *b) { return b->d_off + (b->n + 1); }
+const int *off_groups(const ebit_batch *b) { return b->d_off + 2 * (b->n + 1); }
+
 BatchParams sweep_params(const ebit_batch *b, int d, int parity) {
-    BatchParams p;
-    p.inst = b->table[parity];
+    BatchParams p{};
+    const int rd = parity, wr = parity ^ 1;
+    p.a.cb = b->cb[rd];
+    p.a.cbo = b->cb[wr];
+    for (int k = 0; k < 3; k++) {
+        p.a.s[k] = b->s[rd][k];
+        p.a.so[k] = b->s[wr][k];
+        p.a.adv[k] = b->adv[k];
+        p.a.bin[k] = b->bin[k];
+    }
+    for (int k = 0; k < 2; k++) {
+        p.a.work[k] = b->un[wr][k];
+        p.a.work[2 + k] = b->saddle[k];
+    }
+    p.a.cells = b->cells;
+    p.rd = b->counts + rd * B_N;
+    p.wr = b->counts + wr * B_N;
+    p.a.wcount = p.wr + B_WORK;
+    p.a.tile_marker = b->tile_marker;
+    p.a.tile_dirty = b->tile_dirty;
+    p.a.mk_out = b->al[wr];
+    p.a.mk_out_count = p.wr + B_AL;
+    p.a.mt_out = b->mtiles[wr];
+    p.a.mt_out_count = p.wr + B_MT;
+    p.a.band_flag = b->band_flag;
+    p.grid = b->d_grid;
+    p.coff = off_cells(b);
+    p.toff = off_tiles(b);
     p.n = b->n;
-    p.total_tiles = b->tiles;
-    p.toff = b->d_toff;
     p.u = b->u[d];
     p.lam = b->lam;
+    p.ctr = b->ctr;
+    p.al = b->al[rd];
+    p.un0 = b->un[rd][0];
+    p.un1 = b->un[rd][1];
+    p.mtiles = b->mtiles[rd];
     p.band = b->band;
-    p.nband = b->nband;
-    p.wcount = b->wcount;
     p.bar = b->bar;
     p.err = b->err;
     return p;
+}
+
+// The instances' grids and offsets on the device (the current tile shape).
+int upload_layout(ebit_batch *b) {
+    std::vector<int> off(3 * (b->n + 1));
+    std::vector<Grid> grid(b->n);
+    long long groups = 0;
+    for (int i = 0; i <= b->n; i++) {
+        off[i] = (int)b->coff[i];
+        off[b->n + 1 + i] = b->toff[i];
+        off[2 * (b->n + 1) + i] = (int)groups;
+        if (i == b->n) break;
+        grid[i] = b->inst[i]->g;
+        groups += (long long)((grid[i].n[0] + 7) / 8) * grid[i].n[1] * grid[i].n[2];
+    }
+    BCU(cudaMemcpyAsync(b->d_off, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice, b->stream));
+    BCU(cudaMemcpyAsync(b->d_grid, grid.data(), grid.size() * sizeof(Grid), cudaMemcpyHostToDevice, b->stream));
+    BCU(cudaStreamSynchronize(b->stream));  // the host copies go out of scope
+    return EBIT_OK;
+}
+
+// Before a sweep (or a graph of them): if any instance's state was changed
+// since the last one, the lists of the current set from the state.
+int ensure_lists(ebit_batch *b) {
+    bool valid = true;
+    for (const ebit_ctx *c : b->inst) valid = valid && c->mk_valid;
+    if (valid) return EBIT_OK;
+    const int rd = b->parity;
+    BCU(cudaMemsetAsync(b->counts, 0, 2 * B_N * sizeof(int), b->stream));
+    BCU(cudaMemsetAsync(b->band_flag, 0, b->tiles_cap * sizeof(uint32_t), b->stream));
+    BatchScanArgs a;
+    a.cb = b->cb[rd];
+    a.grid = b->d_grid;
+    a.coff = off_cells(b);
+    a.toff = off_tiles(b);
+    a.goff = off_groups(b);
+    a.n = b->n;
+    a.mask = b->tile_marker;
+    a.list[0] = b->al[rd];
+    a.list[1] = b->un[rd][0];
+    a.list[2] = b->un[rd][1];
+    a.band = b->band;
+    a.counts = b->counts + rd * B_N;
+    batch_scan_kernel<<<8 * b->sms, 256, 0, b->stream>>>(a);
+    BCU(cudaGetLastError());
+    for (ebit_ctx *c : b->inst) c->mk_valid = 1;
+    return EBIT_OK;
 }
 
 int sweep_grid(const ebit_batch *b, int d, int ctas_per_sm) {
@@ -359,7 +469,6 @@ int sweep_grid(const ebit_batch *b, int d, int ctas_per_sm) {
 // cooperative launch (all blocks co-resident: the grid barrier needs it)
 int launch_dir(ebit_batch *b, int d, int ctas_per_sm) {
     BatchParams p = sweep_params(b, d, b->parity);
-    BCU(cudaMemsetAsync(b->nband, 0, sizeof(int), b->stream));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(sweep_grid(b, d, ctas_per_sm));
     cfg.blockDim = dim3(BATCH_THREADS);
@@ -375,8 +484,8 @@ int launch_dir(ebit_batch *b, int d, int ctas_per_sm) {
     return EBIT_OK;
 }
 
-// Two steps (x y z, then z y x) as an explicitly built graph: a memset of the
-// band count and a cooperative kernel node per sweep.
+// Two steps (x y z, then z y x) as an explicitly built graph: a cooperative
+// kernel node per sweep.
 cudaError_t build_graph(ebit_batch *b, cudaGraph_t *out) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaGraphCreate(&g, 0);
@@ -386,16 +495,7 @@ cudaError_t build_graph(ebit_batch *b, cudaGraph_t *out) {
     cudaGraphNode_t prev = nullptr;
     for (int q = 0; q < 6 && e == cudaSuccess; q++) {
         const int d = ord[q];
-        cudaMemsetParams mp = {};
-        mp.dst = b->nband;
-        mp.value = 0;
-        mp.elementSize = sizeof(int);
-        mp.width = 1;
-        mp.height = 1;
-        mp.pitch = 0;
-        cudaGraphNode_t mn = nullptr, kn = nullptr;
-        e = cudaGraphAddMemsetNode(&mn, g, prev ? &prev : nullptr, prev ? 1 : 0, &mp);
-        if (e != cudaSuccess) break;
+        cudaGraphNode_t kn = nullptr;
         BatchParams p = sweep_params(b, d, par);
         void *args[] = {&p};
         cudaKernelNodeParams kp = {};
@@ -405,7 +505,7 @@ cudaError_t build_graph(ebit_batch *b, cudaGraph_t *out) {
         kp.sharedMemBytes = 0;
         kp.kernelParams = args;
         kp.extra = nullptr;
-        e = cudaGraphAddKernelNode(&kn, g, &mn, 1, &kp);
+        e = cudaGraphAddKernelNode(&kn, g, prev ? &prev : nullptr, prev ? 1 : 0, &kp);
         if (e != cudaSuccess) break;
         cudaLaunchAttributeValue v = {};
         v.cooperative = 1;
@@ -422,7 +522,8 @@ cudaError_t build_graph(ebit_batch *b, cudaGraph_t *out) {
 }
 
 int sweep_once(ebit_batch *b, int dir, int ctas_per_sm) {
-    int r = launch_dir(b, dir, ctas_per_sm);
+    int r = ensure_lists(b);
+    if (r == EBIT_OK) r = launch_dir(b, dir, ctas_per_sm);
     if (r) return r;
     b->parity ^= 1;
     for (ebit_ctx *c : b->inst) {
@@ -469,30 +570,21 @@ void tile_offsets(const ebit_batch *b, int sh, std::vector<int> &toff) {
 
 // Switch the batch to tile shape sh: tile offsets, every instance context
 // re-tiled over its new slice of the tile tables (every tile marked for the
-// next sweep and Front2VOF), the launch tables rewritten, the graph dropped.
+// next sweep and Front2VOF), the layout uploaded, the graph dropped.
 int retile(ebit_batch *b, int sh) {
     if (!shape_fits(b, sh)) return bfail(b, EBIT_EINVAL, "tile shape too large for an instance");
     std::vector<int> toff;
     tile_offsets(b, sh, toff);
     if (toff[b->n] > b->tiles_cap) return bfail(b, EBIT_EINVAL, "retile: tile tables too small");
-    std::vector<BatchInst> *tab = b->htab;
     for (int i = 0; i < b->n; i++) {
         ebit_ctx *c = b->inst[i];
         int r = ctx_retile(c, sh, b->tile_marker + toff[i], b->tile_dirty + toff[i]);
         if (r) return bfail(b, r, "retile: " + c->err);
-        for (int q = 0; q < 2; q++) {
-            tab[q][i].a.g = c->g;
-            tab[q][i].a.tile_marker = c->tile_marker;
-            tab[q][i].a.tile_dirty = c->tile_dirty;
-        }
     }
-    for (int q = 0; q < 2; q++)
-        BCU(cudaMemcpyAsync(b->table[q], tab[q].data(), b->n * sizeof(BatchInst), cudaMemcpyHostToDevice, b->stream));
-    BCU(cudaMemcpyAsync(b->d_toff, toff.data(), (b->n + 1) * sizeof(int), cudaMemcpyHostToDevice, b->stream));
-    BCU(cudaStreamSynchronize(b->stream));  // toff goes out of scope
     b->toff = toff;
     b->tiles = toff[b->n];
     b->shape = sh;
+    if (int r = upload_layout(b)) return r;
     b->ctas_per_sm = std::min(b->ctas_per_sm, max_ctas(b, sh));
     drop_graph(b);
     return EBIT_OK;
@@ -567,13 +659,15 @@ int ebit_batch_create(int n, const ebit_desc *descs, ebit_batch **out) {
     }
     for (int a = 0; a < 3 && ok; a++)
         ok = ok && alloc((void **)&b->adv[a], cells * sizeof(double)) && alloc((void **)&b->bin[a], cells);
-    for (int k = 0; k < 4 && ok; k++) ok = ok && alloc((void **)&b->work[k], cells * sizeof(unsigned));
-    ok = ok && alloc((void **)&b->wcount, SWEEP_LISTS * n * sizeof(int)) && alloc((void **)&b->tile_marker, tiles * sizeof(uint32_t)) &&
+    for (int q = 0; q < 2 && ok; q++)
+        ok = ok && alloc((void **)&b->un[q][0], cells * sizeof(unsigned)) &&
+             alloc((void **)&b->un[q][1], cells * sizeof(unsigned)) && alloc((void **)&b->al[q], cells * sizeof(unsigned)) &&
+             alloc((void **)&b->saddle[q], cells * sizeof(unsigned)) && alloc((void **)&b->mtiles[q], tiles * sizeof(int));
+    ok = ok && alloc((void **)&b->counts, 2 * B_N * sizeof(int)) && alloc((void **)&b->tile_marker, tiles * sizeof(uint32_t)) &&
          alloc((void **)&b->tile_dirty, tiles) && alloc((void **)&b->ctr, (size_t)n * C_TOTAL * 8) &&
-         alloc((void **)&b->table[0], n * sizeof(BatchInst)) && alloc((void **)&b->table[1], n * sizeof(BatchInst)) &&
-         alloc((void **)&b->d_toff, (n + 1) * sizeof(int)) && alloc((void **)&b->lam, n * sizeof(double)) &&
-         alloc((void **)&b->band, std::max<long long>(tiles, 1) * sizeof(int)) &&
-         alloc((void **)&b->nband, sizeof(int)) && alloc((void **)&b->bar, 2 * sizeof(unsigned)) &&
+         alloc((void **)&b->band_flag, tiles * sizeof(uint32_t)) && alloc((void **)&b->d_grid, n * sizeof(Grid)) &&
+         alloc((void **)&b->d_off, 3 * (n + 1) * sizeof(int)) && alloc((void **)&b->lam, n * sizeof(double)) &&
+         alloc((void **)&b->band, tiles * sizeof(int)) && alloc((void **)&b->bar, 2 * sizeof(unsigned)) &&
          alloc((void **)&b->err, sizeof(int));
     for (int d = 0; d < 3 && ok; d++) ok = ok && alloc((void **)&b->u[d], n * sizeof(double *));
     if (!ok) {
@@ -583,9 +677,6 @@ int ebit_batch_create(int n, const ebit_desc *descs, ebit_batch **out) {
     }
     // instance contexts over the arena slices
     b->inst.assign(n, nullptr);
-    std::vector<BatchInst> tab[2];
-    tab[0].resize(n);
-    tab[1].resize(n);
     for (int i = 0; i < n; i++) {
         const long long c0 = b->coff[i];
         const int t0 = b->toff[i];
@@ -594,12 +685,6 @@ int ebit_batch_create(int n, const ebit_desc *descs, ebit_batch **out) {
             st.cb[q] = b->cb[q] + c0;
             for (int a = 0; a < 3; a++) st.s[q][a] = b->s[q][a] + c0;
         }
-        for (int a = 0; a < 3; a++) {
-            st.adv[a] = b->adv[a] + c0;
-            st.bin[a] = b->bin[a] + c0;
-        }
-        for (int k = 0; k < 4; k++) st.work[k] = b->work[k] + c0;
-        st.wcount = b->wcount + SWEEP_LISTS * i;
         st.tile_marker = b->tile_marker + t0;
         st.tile_dirty = b->tile_dirty + t0;
         st.ctr = b->ctr + (size_t)i * C_TOTAL;
@@ -608,37 +693,9 @@ int ebit_batch_create(int n, const ebit_desc *descs, ebit_batch **out) {
             ebit_batch_destroy(b);
             return r;
         }
-        const ebit_ctx *c = b->inst[i];
-        for (int q = 0; q < 2; q++) {
-            SweepArgs &a = tab[q][i].a;
-            std::memset(&a, 0, sizeof(a));
-            a.g = c->g;
-            a.cb = st.cb[q];
-            a.cbo = st.cb[q ^ 1];
-            for (int k = 0; k < 3; k++) {
-                a.s[k] = st.s[q][k];
-                a.so[k] = st.s[q ^ 1][k];
-                a.adv[k] = st.adv[k];
-                a.bin[k] = st.bin[k];
-            }
-            for (int k = 0; k < 4; k++) a.work[k] = st.work[k];
-            a.wcount = st.wcount;
-            a.cb_whole = (c->N + 7) & ~7LL;
-            a.ctr = st.ctr;
-            a.tile_marker = st.tile_marker;
-            a.tile_dirty = st.tile_dirty;
-        }
     }
-    if (cudaMemcpyAsync(b->table[0], tab[0].data(), n * sizeof(BatchInst), cudaMemcpyHostToDevice, b->stream) !=
-            cudaSuccess ||
-        cudaMemcpyAsync(b->table[1], tab[1].data(), n * sizeof(BatchInst), cudaMemcpyHostToDevice, b->stream) !=
-            cudaSuccess ||
-        cudaMemcpyAsync(b->d_toff, b->toff.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice, b->stream) !=
-            cudaSuccess ||
-        cudaMemsetAsync(b->bar, 0, 2 * sizeof(unsigned), b->stream) != cudaSuccess ||
-        cudaMemsetAsync(b->err, 0, sizeof(int), b->stream) != cudaSuccess ||
-        cudaMemsetAsync(b->wcount, 0, SWEEP_LISTS * n * sizeof(int), b->stream) != cudaSuccess ||
-        cudaStreamSynchronize(b->stream) != cudaSuccess) {
+    if (cudaMemsetAsync(b->bar, 0, 2 * sizeof(unsigned), b->stream) != cudaSuccess ||
+        cudaMemsetAsync(b->err, 0, sizeof(int), b->stream) != cudaSuccess || upload_layout(b) != EBIT_OK) {
         cudaGetLastError();
         ebit_batch_destroy(b);
         return EBIT_ECUDA;
@@ -648,8 +705,6 @@ int ebit_batch_create(int n, const ebit_desc *descs, ebit_batch **out) {
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b->occ[sh][d], sweep_fn(d, sh), BATCH_THREADS, 0);
             b->occ[sh][d] = std::max(1, b->occ[sh][d]);
         }
-    b->htab[0] = tab[0];
-    b->htab[1] = tab[1];
     b->shape = 0;
     b->ctas_per_sm = max_ctas(b, 0);
     *out = b;
@@ -670,17 +725,22 @@ void ebit_batch_destroy(ebit_batch *b) {
         dev_free(b->mem, b->bin[a]);
         dev_free(b->mem, b->u[a]);
     }
-    for (int k = 0; k < 4; k++) dev_free(b->mem, b->work[k]);
-    dev_free(b->mem, b->wcount);
+    for (int q = 0; q < 2; q++) {
+        dev_free(b->mem, b->un[q][0]);
+        dev_free(b->mem, b->un[q][1]);
+        dev_free(b->mem, b->al[q]);
+        dev_free(b->mem, b->saddle[q]);
+        dev_free(b->mem, b->mtiles[q]);
+    }
+    dev_free(b->mem, b->counts);
+    dev_free(b->mem, b->band_flag);
     dev_free(b->mem, b->tile_marker);
     dev_free(b->mem, b->tile_dirty);
     dev_free(b->mem, b->ctr);
-    dev_free(b->mem, b->table[0]);
-    dev_free(b->mem, b->table[1]);
-    dev_free(b->mem, b->d_toff);
+    dev_free(b->mem, b->d_grid);
+    dev_free(b->mem, b->d_off);
     dev_free(b->mem, b->lam);
     dev_free(b->mem, b->band);
-    dev_free(b->mem, b->nband);
     dev_free(b->mem, b->bar);
     dev_free(b->mem, b->err);
     delete b;
@@ -760,6 +820,7 @@ int ebit_batch_run(ebit_batch *b, int first_step, int steps, int use_graph) {
         left--;
     }
     if (use_graph && left >= 2) {
+        if (int r = ensure_lists(b)) return r;
         if (b->graph_ok && b->graph_parity != b->parity) drop_graph(b);
         if (!b->graph_ok) {
             // two steps from the current parity (a replay restores it): stream

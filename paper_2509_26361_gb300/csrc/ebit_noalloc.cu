@@ -155,6 +155,7 @@ extern "C" int ebit_advect_sweep_noalloc(int nx, int ny, int nz, double h, int d
     a.lam = dt / h;
     a.list = list;
     a.count = ints;
+    a.cells = N;
     a.wcount = ints + 1;
     a.scan_count = ints + 7;
     a.cb_whole = ((uintptr_t)cb_in & 7) == 0 ? N & ~7LL : 0;

@@ -240,69 +240,6 @@ __device__ __forceinline__ int warp_append(int *counter, bool flag) {
 }
 
 // ---------------------------------------------------------------- advection
-// Move every marker of one band tile once (Eq. 2).  CFL >= 1 is counted and
-// clamped; a displacement that is not finite (NaN or infinite velocity) is
-// counted apart and the marker stays where it is.  Called by all threads of the block; s_mk/s_c/s_n are its shared
-// staging; u is u_D on the D-faces and lam = dt / h.
-// Tile shape SH (TileShape<SH>); s_c holds (TX + 1) (TY + 1) (TZ + 1) colours.
-template <int D, int SH = 0>
-__device__ __forceinline__ void advect_tile(const SweepArgs &a, const double *__restrict__ u, double lam, int tile,
-                                            uint16_t *s_mk, uint8_t *s_c, int *s_n) {
-    using S = TileShape<SH>;
-    constexpr int CX = S::TX + 1, CY = S::TY + 1, CZ = S::TZ + 1;
-    int o[3];
-    tile_origin(a.g, tile, o);
-    if (threadIdx.x == 0) *s_n = 0;
-    for (int r = threadIdx.x; r < CX * CY * CZ; r += blockDim.x) {
-        int rx = r % CX, ry = (r / CX) % CY, rz = r / (CX * CY);
-        s_c[r] = __ldg(a.cb + lin(a.g, o[0] + rx, o[1] + ry, o[2] + rz)) & 1;
-    }
-    __syncthreads();
-    for (int c = threadIdx.x; c < TILE_CELLS; c += blockDim.x) {
-        int l[3];
-        S::cell(c, l);
-        int q[3] = {o[0] + l[0], o[1] + l[1], o[2] + l[2]};
-        bool valid = q[0] < a.g.n[0] && q[1] < a.g.n[1] && q[2] < a.g.n[2];
-        int mask = 0;
-        if (valid) {
-            const int r = l[0] + CX * (l[1] + CY * l[2]);
-            const int c0 = s_c[r];
-            mask = (s_c[r + 1] != c0) | ((s_c[r + CX] != c0) << 1) | ((s_c[r + CX * CY] != c0) << 2);
-        }
-        for (int e = 0; e < 3; e++) {
-            int slot = warp_append(s_n, (mask >> e) & 1);
-            if (slot >= 0) s_mk[slot] = (uint16_t)(c | (e << 9));
-        }
-    }
-    __syncthreads();
-    const int n = *s_n;
-    unsigned hits = 0, bad = 0;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        int it = s_mk[k], c = it & 511, e = it >> 9;
-        int l[3];
-        S::cell(c, l);
-        int q[3] = {o[0] + l[0], o[1] + l[1], o[2] + l[2]};
-        const int id = lin3(a.g, q);
-        double sv = __ldg(a.s[e] + id);
-        double cf = interp_u<D>(a.g, u, q, e, sv) * lam;
-        if (!isfinite(cf)) {
-            bad++;
-            cf = 0.0;
-        } else if (!(fabs(cf) < 1.0)) {
-            hits++;
-            cf = cf > 0.0 ? ONE_MINUS : -ONE_MINUS;
-        }
-        double x = (e == D) ? sv + cf : cf;
-        a.adv[e][id] = x;
-        a.bin[e][id] = (int8_t)(int)floor(2.0 * x);
-    }
-    unsigned v = __reduce_add_sync(0xffffffffu, hits);
-    if ((threadIdx.x & 31) == 0 && v) atomicAdd(a.ctr + C_CFL, (unsigned long long)v);
-    v = __reduce_add_sync(0xffffffffu, bad);
-    if ((threadIdx.x & 31) == 0 && v) atomicAdd(a.ctr + C_NONFINITE, (unsigned long long)v);
-    __syncthreads();
-}
-
 // the counters the band pass appends to start at zero (cleared by the launch before it)
 __device__ __forceinline__ void clear_sweep_counts(const SweepArgs &a) {
     if (blockIdx.x != 0) return;
@@ -313,9 +250,51 @@ __device__ __forceinline__ void clear_sweep_counts(const SweepArgs &a) {
     if (threadIdx.x == 35 && a.band_next_count) *a.band_next_count = 0;
 }
 
+// Move the marker on the e-edge of node gid once (Eq. 2); the grid's cells start
+// at base, u is u_D on its D-faces and lam = dt / h.  CFL >= 1 is counted and
+// clamped; a displacement that is not finite (NaN or infinite velocity) is
+// counted apart and the marker stays where it is.
+template <int D>
+__device__ __forceinline__ void move_marker(const SweepArgs &a, const Grid &g, int base, const double *__restrict__ u,
+                                            double lam, int e, int gid, unsigned &hits, unsigned &bad) {
+    const int nx = g.n[0], nxy = nx * g.n[1], id = gid - base;
+    const int z = id / nxy, r = id - z * nxy;
+    const int y = r / nx;
+    const int q[3] = {r - y * nx, y, z};
+    // selects rather than indexing, which would copy the parameter arrays to
+    // local memory
+    const double *se = e == 0 ? a.s[0] : (e == 1 ? a.s[1] : a.s[2]);
+    double *adv = e == 0 ? a.adv[0] : (e == 1 ? a.adv[1] : a.adv[2]);
+    int8_t *bin = e == 0 ? a.bin[0] : (e == 1 ? a.bin[1] : a.bin[2]);
+    const double sv = __ldg(se + gid);
+    double cf = interp_u<D>(g, u, q, e, sv) * lam;
+    if (!isfinite(cf)) {
+        bad++;
+        cf = 0.0;
+    } else if (!(fabs(cf) < 1.0)) {
+        hits++;
+        cf = cf > 0.0 ? ONE_MINUS : -ONE_MINUS;
+    }
+    const double x = (e == D) ? sv + cf : cf;
+    adv[gid] = x;
+    bin[gid] = (int8_t)(int)floor(2.0 * x);
+}
+
+// Band item b (a direction) of a listed tile of grid g (its tiles start at
+// tbase): the neighbour the tile's mask points to that way (bit
+// near_bit(dx, dy, dz)), listed once.
+__device__ __forceinline__ void band_item(const Grid &g, int tbase, int tile, int b, const uint32_t *__restrict__ mask,
+                                          uint32_t *band_flag, int *band, int *band_count) {
+    if (!((__ldg(mask + tbase + tile) >> b) & 1u)) return;
+    const int tx = tile % g.td[0], ty = (tile / g.td[0]) % g.td[1], tz = tile / (g.td[0] * g.td[1]);
+    const int bx = wrapc(tx + b % 3 - 1, g.td[0]), by = wrapc(ty + (b / 3) % 3 - 1, g.td[1]),
+              bz = wrapc(tz + b / 9 - 1, g.td[2]);
+    const int nt = tbase + (bz * g.td[1] + by) * g.td[0] + bx;
+    if (atomicExch(band_flag + nt, 1u) == 0u) band[atomicAdd(band_count, 1)] = nt;
+}
+
 // Advection from the marker lists (Eq. 2): one thread per marker, no tile
-// staging.  Every marker of the state is on a list, so the same markers as in
-// advect_tile are moved, with the same arithmetic.
+// staging.
 template <int D>
 __global__ void __launch_bounds__(256) advect_list_kernel(SweepArgs a, MarkerLists m) {
     pdl_wait();
@@ -329,50 +308,20 @@ __global__ void __launch_bounds__(256) advect_list_kernel(SweepArgs a, MarkerLis
     const int all = total + 27 * nmt;
     const int stride = gridDim.x * blockDim.x;
     const int iters = (all + stride - 1) / stride;
-    const int nx = a.g.n[0], nxy = a.g.n[0] * a.g.n[1];
     unsigned hits = 0, bad = 0;
     for (int it = 0; it < iters; it++) {
         const int t = list_item(it);
         if (t >= all) continue;
         if (t >= total) {
-            // the band: every tile a listed tile's mask points to (bit
-            // near_bit(dx, dy, dz) names the neighbour in that direction),
-            // listed once
             const int tb = t - total;
-            const int tile = __ldg(m.mtiles + tb / 27), b = tb % 27;
-            if (!((__ldg(a.tile_marker + tile) >> b) & 1u)) continue;
-            const int tx = tile % a.g.td[0], ty = (tile / a.g.td[0]) % a.g.td[1], tz = tile / (a.g.td[0] * a.g.td[1]);
-            const int bx = wrapc(tx + b % 3 - 1, a.g.td[0]), by = wrapc(ty + (b / 3) % 3 - 1, a.g.td[1]),
-                      bz = wrapc(tz + b / 9 - 1, a.g.td[2]);
-            const int nt = (bz * a.g.td[1] + by) * a.g.td[0] + bx;
-            if (atomicExch(a.band_flag + nt, 1u) == 0u) m.band[atomicAdd(m.band_count, 1)] = nt;
+            band_item(a.g, 0, __ldg(m.mtiles + tb / 27), tb % 27, a.tile_marker, a.band_flag, m.band, m.band_count);
             continue;
         }
-        // selects rather than indexing, which would copy the parameter arrays
-        // to local memory
         const int k = t < n0 ? 0 : (t < n0 + n1 ? 1 : 2);
         const int j = t - (k == 0 ? 0 : (k == 1 ? n0 : n0 + n1));
         const unsigned *lst = k == 0 ? m.list[0] : (k == 1 ? m.list[1] : m.list[2]);
         const int e = k == 0 ? m.axis[0] : (k == 1 ? m.axis[1] : m.axis[2]);
-        const int id = (int)__ldg(lst + j);
-        const int z = id / nxy, r = id - z * nxy;
-        const int y = r / nx;
-        const int q[3] = {r - y * nx, y, z};
-        const double *se = e == 0 ? a.s[0] : (e == 1 ? a.s[1] : a.s[2]);
-        double *adv = e == 0 ? a.adv[0] : (e == 1 ? a.adv[1] : a.adv[2]);
-        int8_t *bin = e == 0 ? a.bin[0] : (e == 1 ? a.bin[1] : a.bin[2]);
-        const double sv = __ldg(se + id);
-        double cf = interp_u<D>(a.g, a.u, q, e, sv) * a.lam;
-        if (!isfinite(cf)) {
-            bad++;
-            cf = 0.0;
-        } else if (!(fabs(cf) < 1.0)) {
-            hits++;
-            cf = cf > 0.0 ? ONE_MINUS : -ONE_MINUS;
-        }
-        const double x = (e == D) ? sv + cf : cf;
-        adv[id] = x;
-        bin[id] = (int8_t)(int)floor(2.0 * x);
+        move_marker<D>(a, a.g, 0, a.u, a.lam, e, (int)__ldg(lst + j), hits, bad);
     }
     unsigned v = __reduce_add_sync(0xffffffffu, hits);
     if ((threadIdx.x & 31) == 0 && v) atomicAdd(a.ctr + C_CFL, (unsigned long long)v);
@@ -425,13 +374,16 @@ struct SweepCell {
     // bit (da + 2) + 5 (dt + 1): node colour, and the colour of the node's face
     unsigned col, face;
 
-    __device__ SweepCell(const SweepArgs &args, int id_, int x, int y, int z, int fam_) : a(args), id(id_), fam(fam_) {
-        const int p[3] = {x, y, z}, s[3] = {1, a.g.n[0], a.g.n[0] * a.g.n[1]};
+    // node id_ of grid g, whose cells start at base
+    __device__ SweepCell(const SweepArgs &args, const Grid &g, int base, int id_, int fam_)
+        : a(args), id(id_), fam(fam_) {
+        const int nx = g.n[0], nxy = nx * g.n[1], l = id_ - base, z = l / nxy, r = l - z * nxy, y = r / nx;
+        const int p[3] = {r - y * nx, y, z}, s[3] = {1, nx, nxy};
         pa = p[A];
-        na = a.g.n[A];
+        na = g.n[A];
         sa = s[A];
         pt = fam ? p[T2] : p[T1];
-        nt = fam ? a.g.n[T2] : a.g.n[T1];
+        nt = fam ? g.n[T2] : g.n[T1];
         st = fam ? s[T2] : s[T1];
     }
     // per-family arrays by selects (indexing would copy the arguments to local memory)
@@ -579,7 +531,6 @@ struct SweepCell {
     __device__ __forceinline__ void unaligned(unsigned left, unsigned ev[C_N], int half = -1) const {
         const Crossings c = crossings(left);
         const bool lead = half <= 0;
-        if (lead) ev[C_MARKERS]++;
         if ((c.n & 1) == 0) {
             if (lead) {
                 ev[C_INCONSISTENT]++;
@@ -657,15 +608,13 @@ struct SweepCell {
 };
 
 // ------------------------------------------------- FP64 work lists
-// Entry k of list `kind` (0, 1: unaligned edges of families 1, 2; 2, 3: saddle
-// faces; 4, 5: annihilation checks, from the ends of lists 0, 1).
+// Entry of list `kind` (0, 1: unaligned edges of families 1, 2; 2, 3: saddle
+// faces; 4, 5: annihilation checks): node id of grid g, whose cells start at base.
 template <int D, bool F>
-__device__ __forceinline__ void fp64_item(const SweepArgs &a, int kind, int k, unsigned ev[C_N], int half = -1) {
+__device__ __forceinline__ void fp64_item(const SweepArgs &a, const Grid &g, int base, int kind, int id, unsigned ev[C_N],
+                                          int half = -1) {
     constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
-    const int id = (int)ld_in<F>(kind < 4 ? a.work[kind] + k
-                                          : a.work[kind - 4] + (a.g.n[0] * a.g.n[1] * a.g.n[2] - 1 - k));
-    const int x = id % a.g.n[0], y = (id / a.g.n[0]) % a.g.n[1], z = id / (a.g.n[0] * a.g.n[1]);
-    SweepCell<D, F> cell(a, id, x, y, z, kind & 1);
+    SweepCell<D, F> cell(a, g, base, id, kind & 1);
     cell.loadw();
     const unsigned left = cell.left_bits();
     if (kind >= 4) {
@@ -685,47 +634,67 @@ __device__ __forceinline__ void fp64_item(const SweepArgs &a, int kind, int k, u
     }
 }
 
+// The work lists of a sweep as one index space of lanes.  Unaligned edges come
+// first, then saddle faces and annihilation checks, one lane each.  When the
+// lists fit one round of `stride` lanes with two per unaligned edge, each edge
+// gets two adjacent lanes and the circle fits are split between them: a shorter
+// chain per warp where few warps run.  Long lists keep one lane per edge, since
+// the pairs repeat the work before the fits.
+template <bool F>
+struct WorkLanes {
+    int n[SWEEP_LISTS], lanes_u, lanes;
+    bool pairs;
+    __device__ WorkLanes(const SweepArgs &a, int stride) {
+#pragma unroll
+        for (int k = 0; k < SWEEP_LISTS; k++) n[k] = ld_in<F>(a.wcount + k);
+        const int nu = n[0] + n[1], rest = n[2] + n[3] + n[4] + n[5];
+        pairs = 2 * nu + rest <= stride;
+        lanes_u = pairs ? 2 * nu : nu;
+        lanes = lanes_u + rest;
+    }
+    // lane t's list and node, and its half of the edge (-1: all of it)
+    __device__ __forceinline__ int item(const SweepArgs &a, int t, int *kind, int *half) const {
+        *half = -1;
+        if (t < lanes_u) {
+            if (pairs) {
+                *half = t & 1;
+                t >>= 1;
+            }
+        } else {
+            t += n[0] + n[1] - lanes_u;
+        }
+        int k = 0;
+#pragma unroll
+        for (int q = 0; q < SWEEP_LISTS - 1; q++)
+            if (k == q && t >= n[q]) {
+                t -= n[q];
+                k = q + 1;
+            }
+        *kind = k;
+        // the checks fill the unaligned lists' arrays from the end
+        const unsigned *w = (k & 1) ? ((k & 2) ? a.work[3] : a.work[1]) : ((k & 2) ? a.work[2] : a.work[0]);
+        return (int)ld_in<F>(k < 4 ? w + t : w + (a.cells - 1 - t));
+    }
+};
+
 template <int D>
 __global__ void __launch_bounds__(128, 8) fp64_kernel(SweepArgs a) {
     pdl_wait();
-    const int n0 = a.wcount[0], n1 = a.wcount[1], n2 = a.wcount[2], n3 = a.wcount[3];
-    const int n4 = a.wcount[4], n5 = a.wcount[5];
-    const int total = n0 + n1 + n2 + n3 + n4 + n5;
     unsigned ev[C_N] = {0, 0, 0, 0, 0};
     const int stride = gridDim.x * blockDim.x;
-    // Unaligned edges first, then saddle faces and annihilation checks, one lane
-    // each.  When the lists fit one round of the grid with two lanes per
-    // unaligned edge, each edge gets two adjacent lanes and the circle fits are
-    // split between them: a shorter chain per warp where few warps run.  Long
-    // lists keep one lane per edge, since the pairs repeat the work before the
-    // fits.  The trip count is uniform so that every lane reaches the warp
-    // reductions.
-    const int nu = n0 + n1, rest = total - nu;
-    const bool pairs = 2 * nu + rest <= stride;
-    const int lanes_u = pairs ? 2 * nu : nu;
-    const int iters = (lanes_u + rest + stride - 1) / stride;
+    const WorkLanes<false> w(a, stride);
+    // (the trip count is uniform so that every lane reaches the warp reductions)
+    const int iters = (w.lanes + stride - 1) / stride;
     for (int it = 0; it < iters; it++) {
-        const int t2 = list_item(it);
-        int t, half;
-        if (t2 < lanes_u) {
-            t = pairs ? t2 >> 1 : t2;
-            half = pairs ? (t2 & 1) : -1;
-        } else {
-            t = nu + (t2 - lanes_u);
-            half = -1;
-        }
-        if (t >= total) continue;
-        int k, kind;
-        if (t < n0) { kind = 0; k = t; }
-        else if (t < n0 + n1) { kind = 1; k = t - n0; }
-        else if (t < n0 + n1 + n2) { kind = 2; k = t - n0 - n1; }
-        else if (t < n0 + n1 + n2 + n3) { kind = 3; k = t - n0 - n1 - n2; }
-        else if (t < n0 + n1 + n2 + n3 + n4) { kind = 4; k = t - n0 - n1 - n2 - n3; }
-        else { kind = 5; k = t - n0 - n1 - n2 - n3 - n4; }
-        fp64_item<D, false>(a, kind, k, ev, half);
+        const int t = list_item(it);
+        if (t >= w.lanes) continue;
+        int kind, half;
+        const int id = w.item(a, t, &kind, &half);
+        fp64_item<D, false>(a, a.g, 0, kind, id, ev, half);
     }
 #pragma unroll
     for (int k = 0; k < C_N; k++) {
+        if (k == C_MARKERS || k == C_CFL) continue;  // counted by the band pass and the advection
         unsigned v = __reduce_add_sync(0xffffffffu, ev[k]);
         if ((threadIdx.x & 31) == 0 && v) atomicAdd(a.ctr + k, (unsigned long long)v);
     }

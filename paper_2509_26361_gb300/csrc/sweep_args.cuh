@@ -24,6 +24,7 @@ struct SweepArgs {
                                      // fam.2; the annihilation checks of a family fill its unaligned list from
                                      // the end (an edge is on one of the two at most)
     int *__restrict__ wcount;        // [6] list lengths (device): unaligned, saddle, annihilation checks
+    long long cells = 0;             // entries of each work list (a batch: the cells of its arena)
     long long cb_whole = 0;          // bytes from cb that may be read as aligned 8-byte words (see load_colours8)
     unsigned long long *ctr;         // event counters
     uint32_t *tile_marker;           // per tile: proximity mask of its markers in the input or the output
