@@ -111,6 +111,15 @@ __host__ __device__ inline void grid_tiles(Grid &g, int sh) {
     }
 }
 
+// Does a tile reach past the grid on some axis?  The proximity masks measure from
+// the tile's edges, so across the seam behind such a clipped tile they can miss
+// the neighbour of a marker: that tile stays out of the band and keeps its old
+// colours, and an edge it owns may then carry a marker that no list names and
+// whose offset was written by no sweep.
+__host__ __device__ inline bool has_clipped_tiles(const Grid &g) {
+    return ((g.n[0] & ((1 << g.tl[0]) - 1)) | (g.n[1] & ((1 << g.tl[1]) - 1)) | (g.n[2] & ((1 << g.tl[2]) - 1))) != 0;
+}
+
 __host__ __device__ inline int wrapc(int v, int n) {
     // v is within a few cells of [0, n)
     return v < 0 ? v + n : (v >= n ? v - n : v);
