@@ -476,13 +476,13 @@ __global__ void __launch_bounds__(BAND_THREADS, 16) sweep_kernel(SweepArgs a) {
     __shared__ BandSmem<D, 0> sm;
     __shared__ int s_next;
     pdl_wait();
-    const int ntl = *a.count;
+    const int ntl = a.list ? *a.count : a.g.ntiles;
     BandEvents ev;
     // after the first, each block takes tiles from a counter (tiles differ in
     // cost), read one tile ahead
     for (int li = blockIdx.x; li < ntl;) {
         if (threadIdx.x == 0) s_next = a.tile_next ? (int)gridDim.x + atomicAdd(a.tile_next, 1) : li + (int)gridDim.x;
-        band_tile<D, false>(a, a.g, 0, 0, a.cb_whole, a.list[li], sm, 0, ev);
+        band_tile<D, false>(a, a.g, 0, 0, a.cb_whole, a.list ? a.list[li] : li, sm, 0, ev);
         __syncthreads();
         li = s_next;
         __syncthreads();

@@ -18,6 +18,7 @@
 #include "../../include/ebit.h"
 #include "common.cuh"
 #include "ctx.h"
+#include "launch.h"
 #include "f2v.cuh"
 #include "hf.cuh"
 #include "mlp.cuh"
@@ -45,26 +46,6 @@ int launch_check(ebit_ctx *ctx, const char *what) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(ctx, EBIT_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
     return EBIT_OK;
-}
-
-// Launch with programmatic stream serialization: the kernel is launched as
-// the previous kernel's blocks exit, and waits (pdl_wait) for that kernel's
-// completion before it touches global memory.  Counters that a
-// launch appends to are cleared by an earlier kernel of the chain (in its
-// zero arguments) instead of by memsets, which would break the overlap.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 int launched(ebit_ctx *ctx, cudaError_t e, const char *what) {

@@ -116,6 +116,8 @@ struct ScanArgs {
     uint8_t *cb1 = nullptr, *cb2 = nullptr;
     const double *src = nullptr;  // [3][n]
     double *s[3] = {nullptr, nullptr, nullptr};
+    // zeros into the offsets of an output state, before a sweep writes its markers'
+    double *clear = nullptr;      // [3][n]
 };
 static __global__ void __launch_bounds__(256) mark_scan_kernel(ScanArgs a) {
     pdl_wait();
@@ -125,6 +127,16 @@ static __global__ void __launch_bounds__(256) mark_scan_kernel(ScanArgs a) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const long long stride = (long long)gridDim.x * blockDim.x;
+    if (a.clear) {
+        const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+        if (((uintptr_t)a.clear & 15) == 0) {
+            double2 *p = reinterpret_cast<double2 *>(a.clear);
+            for (long long k = t; k < 3 * n / 2; k += stride) p[k] = make_double2(0.0, 0.0);
+            if (t == 0 && (n & 1)) a.clear[3 * n - 1] = 0.0;
+        } else {
+            for (long long k = t; k < 3 * n; k += stride) a.clear[k] = 0.0;
+        }
+    }
     for (long long t0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); t0 < groups; t0 += stride) {
         const RowGroup r = row_group(a.g, a.cb, a.whole, gx, t0 + lane);
         if (a.cb2) {

@@ -18,7 +18,7 @@ struct SweepArgs {
     double lam;                      // dt / h
     double *__restrict__ adv[3];     // advected coordinate of each marker (scratch)
     int8_t *__restrict__ bin[3];     // floor(2 adv) (scratch)
-    const int *__restrict__ list;    // band tile ids
+    const int *__restrict__ list;    // band tile ids (null: every tile of g)
     const int *__restrict__ count;   // number of band tiles (device)
     unsigned *__restrict__ work[4];  // work lists, one entry per node each: unaligned fam.1, fam.2, saddle fam.1,
                                      // fam.2; the annihilation checks of a family fill its unaligned list from
