@@ -26,78 +26,104 @@ constexpr int AMR_CHUNK = 1024;   // tiles per chunk of the compaction
 // of flagged tiles per chunk of AMR_CHUNK (chunk).  Outputs but the mask start
 // at zero where they are sums.
 //
-// One warp per tile, an x-row of colours as one bit mask: the flags of ten
-// cells are a few shifts of four rows and the 27-cell OR of eight cells a few
-// of nine, so the pass is bound by the colours' way from L2 and the mask's to
-// memory.  (a block per tile, one byte per thread and node: 1.9 ms at 512^3 and
-// 558 us at 384^3; this form 230 us at 384^3.)
+// A block takes a strip of eight tiles along x.  Its colours come as groups of 8
+// cells, consecutive lanes along the rows, and are kept as one byte of bits per
+// group; each warp then works on one tile, whose rows of 11 nodes it reads off
+// three bytes: the flags of ten cells are a few shifts of four rows and the
+// 27-cell OR of eight cells a few of nine.  The mask is written the way the
+// colours are read.  Bound by the colours' way from L2 and the mask's to memory.
+// (a block per tile, one byte per thread and node: 558 us at 384^3; a warp per
+// tile, a lane per row: 230 us, bound by the cache lines its loads touch, one per
+// lane; this form 89.)
+constexpr int AMR_G = 10;  // groups of 8 nodes per row: x0 - 8 .. x0 + 71
+
 __global__ void __launch_bounds__(32 * AMR_WARPS) refine_kernel(Grid g, const uint8_t *__restrict__ cb, long long whole,
                                                                 uint8_t *__restrict__ mask, uint8_t *__restrict__ flag,
                                                                 uint8_t *__restrict__ bg,
                                                                 unsigned long long *__restrict__ count,
                                                                 int *__restrict__ chunk) {
-    __shared__ unsigned s_row[AMR_WARPS][AMR_R * AMR_R];
+    __shared__ uint8_t s_col[AMR_R * AMR_R][AMR_G + 2];  // (a row of 12 bytes)
     __shared__ unsigned s_flg[AMR_WARPS][AMR_F * AMR_F];
+    __shared__ uint8_t s_ref[TILE * TILE][AMR_WARPS];
     const unsigned full = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    unsigned *row = s_row[warp], *flg = s_flg[warp];
+    unsigned *flg = s_flg[warp];
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
     const long long n = (long long)nx * ny * nz;
+    const int sx = (g.td[0] + AMR_WARPS - 1) / AMR_WARPS;
+    const long long strips = (long long)sx * g.td[1] * g.td[2];
     unsigned nref = 0;
-    for (int tile = blockIdx.x * AMR_WARPS + warp; tile < g.ntiles; tile += gridDim.x * AMR_WARPS) {
-        int o[3];
-        tile_origin(g, tile, o);
-        bool any1 = false, any0 = false;
+    for (long long st = blockIdx.x; st < strips; st += gridDim.x) {
+        const int ix = (int)(st % sx), iyz = (int)(st / sx), ty = iyz % g.td[1], tz = iyz / g.td[1];
+        const int x0 = ix * AMR_WARPS * TILE, y0 = ty * TILE, z0 = tz * TILE;
+        int seen = 0;
 #pragma unroll
-        for (int q = 0; q < (AMR_R * AMR_R + 31) / 32; q++) {
-            const int r = lane + 32 * q;
-            if (r >= AMR_R * AMR_R) continue;
-            const int y = wrapc(o[1] + r % AMR_R - 1, ny), z = wrapc(o[2] + r / AMR_R - 1, nz);
-            uint32_t f;
-            const unsigned c = load_row<uint32_t, TILE, -1, AMR_R>(cb, (z * ny + y) * nx, o[0], nx, whole, n, 1, &f);
-            row[r] = c;
-            any1 |= c != 0u;
-            any0 |= c != (1u << AMR_R) - 1u;
+        for (int q = 0; q < (AMR_R * AMR_R * AMR_G + 255) / 256; q++) {
+            const int k = threadIdx.x + 256 * q;
+            if (k >= AMR_R * AMR_R * AMR_G) continue;
+            const int r = k / AMR_G, gr = k - r * AMR_G;
+            const int y = wrapc(y0 + r % AMR_R - 1, ny), z = wrapc(z0 + r / AMR_R - 1, nz);
+            const unsigned c = group_colours(cb, (z * ny + y) * nx, x0 + 8 * (gr - 1), nx, whole, n);
+            s_col[r][gr] = (uint8_t)c;
+            // uniform strips (of the nodes that are read) need no flags
+            const unsigned used = gr == 0 ? 0x80u : (gr == AMR_G - 1 ? 0x03u : 0xFFu);
+            seen |= ((c & used) ? 1 : 0) | ((~c & used) ? 2 : 0);
         }
-        const bool has1 = __any_sync(full, any1), has0 = __any_sync(full, any0);
-        __syncwarp();
-        const unsigned vx = nx - o[0] >= TILE ? 0xFFu : (1u << (nx - o[0])) - 1u;
+        const int has1 = __syncthreads_or(seen & 1), has0 = __syncthreads_or(seen & 2);
+        const int tx = ix * AMR_WARPS + warp, o0 = x0 + TILE * warp;
+        const bool tile_ok = tx < g.td[0];
+        const int tile = (tz * g.td[1] + ty) * g.td[0] + tx;
+        const unsigned vx = !tile_ok ? 0u : (nx - o0 >= TILE ? 0xFFu : (1u << (nx - o0)) - 1u);
         bool any = false;
         if (has1 && has0) {
+            // node row r of the warp's tile, nodes -1 .. TILE + 1
+            auto row = [&](int r) -> unsigned {
+                const uint8_t *c = s_col[r] + warp;
+                return (unsigned)c[0] >> 7 | (unsigned)c[1] << 1 | ((unsigned)c[2] & 3u) << 9;
+            };
             // interfacial flags of the cells -1 .. TILE around the tile
             for (int r = lane; r < AMR_F * AMR_F; r += 32) {
                 const int i = r % AMR_F + AMR_R * (r / AMR_F);
-                const unsigned p = row[i], q = row[i + 1], s = row[i + AMR_R], t = row[i + AMR_R + 1];
+                const unsigned p = row(i), q = row(i + 1), s = row(i + AMR_R), t = row(i + AMR_R + 1);
                 const unsigned hi = p | q | s | t, lo = p & q & s & t;
                 flg[r] = (hi | hi >> 1) & ~(lo & lo >> 1) & ((1u << AMR_F) - 1u);
             }
             __syncwarp();
-        }
 #pragma unroll
-        for (int q = 0; q < 2; q++) {
-            const int r = lane + 32 * q, ly = r & 7, lz = r >> 3, y = o[1] + ly, z = o[2] + lz;
-            unsigned ref = 0;
-            if (has1 && has0) {
+            for (int q = 0; q < 2; q++) {
+                const int r = lane + 32 * q, ly = r & 7, lz = r >> 3;
                 unsigned f = 0;
 #pragma unroll
                 for (int d = 0; d < 9; d++) f |= flg[ly + d % 3 + AMR_F * (lz + d / 3)];
-                ref = (f | f >> 1 | f >> 2) & vx;
+                const unsigned ref = y0 + ly < ny && z0 + lz < nz ? (f | f >> 1 | f >> 2) & vx : 0u;
+                nref += __popc(ref);
+                any |= ref != 0u;
+                s_ref[r][warp] = (uint8_t)ref;
             }
-            if (y >= ny || z >= nz) continue;
-            nref += __popc(ref);
-            any |= ref != 0;
-            if (mask) store_row<TILE>(mask, ((long long)z * ny + y) * nx + o[0], ref, 0u, 0u, 0u, vx);
+        } else {
+            s_ref[lane][warp] = s_ref[lane + 32][warp] = 0;
         }
         const bool tile_any = __any_sync(full, any);
-        if (lane == 0) {
+        if (lane == 0 && tile_ok) {
             flag[tile] = tile_any ? 1 : 0;
-            if (bg) bg[tile] = (uint8_t)((row[1 + AMR_R] >> 1) & 1u);  // the origin node
+            if (bg) bg[tile] = s_col[1 + AMR_R][warp + 1] & 1u;  // the origin node
             if (tile_any) {
                 atomicAdd(count + 1, 1ull);
                 atomicAdd(chunk + tile / AMR_CHUNK, 1);
             }
         }
-        __syncwarp();  // the staging is rewritten by the next tile
+        __syncthreads();
+        if (mask) {
+#pragma unroll
+            for (int q = 0; q < TILE * TILE * AMR_WARPS / 256; q++) {
+                const int k = threadIdx.x + 256 * q, r = k / AMR_WARPS, gr = k % AMR_WARPS;
+                const int y = y0 + (r & 7), z = z0 + (r >> 3), x = x0 + TILE * gr;
+                if (y >= ny || z >= nz || x >= nx) continue;
+                store_row<TILE>(mask, ((long long)z * ny + y) * nx + x, s_ref[r][gr], 0u, 0u, 0u,
+                                nx - x >= TILE ? 0xFFu : (1u << (nx - x)) - 1u);
+            }
+        }
+        __syncthreads();  // the staging is rewritten by the next strip
     }
     nref = __reduce_add_sync(full, nref);
     if (lane == 0 && nref) atomicAdd(count, (unsigned long long)nref);

@@ -113,6 +113,20 @@ __device__ __forceinline__ unsigned long long load_colours8(const uint8_t *__res
     return v;
 }
 
+// Colours of nodes x .. x + 7 (periodic) of the row that starts at node `row`, as
+// bits, for passes over whole strips of tiles; x from -8 (only node -1 is read)
+// to past the end of the row.
+__device__ __forceinline__ unsigned group_colours(const uint8_t *__restrict__ cb, int row, int x, int nx, long long whole,
+                                                  long long n) {
+    if (x < 0) return (unsigned)(__ldg(cb + row + nx - 1) & 1) << 7;
+    if (x >= nx) x -= nx;
+    if (x >= nx) return 0u;
+    const unsigned c = gather_bits(load_colours8(cb, (long long)row + x, whole, n));
+    if (x + 8 <= nx) return c;
+    const int v = nx - x;
+    return (c & ((1u << v) - 1u)) | ((gather_bits(load_colours8(cb, row, whole, n)) << v) & 0xFFu);
+}
+
 // The colours of nodes x0 + X0 .. x0 + X0 + RX - 1 (periodic) of the x-row that
 // starts at node `row`, bit x - x0 - X0, and bit `fbit` of the bytes of the TX
 // cells (bit x - x0) in *fa.

@@ -543,8 +543,8 @@ static int amr_scratch(ebit_ctx *ctx) {
 static int refine_pass(ebit_ctx *ctx, uint8_t *mask, uint8_t *bg) {
     if (int r = amr_scratch(ctx)) return r;
     CU(cudaMemsetAsync(ctx->amr_ctr, 0, 3 * sizeof(unsigned long long) + amr_chunks(ctx) * sizeof(int), ctx->stream));
-    refine_kernel<<<std::min((ctx->g.ntiles + AMR_WARPS - 1) / AMR_WARPS, 8 * ctx->sms), 32 * AMR_WARPS, 0,
-                    ctx->stream>>>(ctx->g, ctx->cb[ctx->cur], (ctx->N + 7) & ~7LL, mask, ctx->amr_flag, bg,
+    const long long strips = (long long)((ctx->g.td[0] + AMR_WARPS - 1) / AMR_WARPS) * ctx->g.td[1] * ctx->g.td[2];
+    refine_kernel<<<(int)std::min<long long>(strips, 8 * ctx->sms), 32 * AMR_WARPS, 0, ctx->stream>>>(ctx->g, ctx->cb[ctx->cur], (ctx->N + 7) & ~7LL, mask, ctx->amr_flag, bg,
                                    ctx->amr_ctr, reinterpret_cast<int *>(ctx->amr_ctr + 3));
     return launch_check(ctx, "refine_kernel");
 }

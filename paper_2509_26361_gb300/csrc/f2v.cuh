@@ -135,6 +135,88 @@ __global__ void __launch_bounds__(64, 16) f2v_band_kernel(F2VArgs a) {
     }
 }
 
+// The band pass over every tile (8^3 tiles): a block takes a strip of eight tiles
+// along x, so that consecutive lanes read colours and write fractions along the
+// rows; HBM bound by the fractions (a tile at a time, a lane per row, 152 us at
+// 384^3; this form 112).
+constexpr int F2V_STRIP = 8;
+__global__ void __launch_bounds__(256) f2v_full_kernel(F2VArgs a) {
+    constexpr int R = TILE + 1, G = F2V_STRIP + 1;
+    __shared__ uint8_t s_col[R * R][G + 3];
+    __shared__ uint8_t s_one[TILE * TILE][F2V_STRIP];
+    pdl_wait();
+    if (a.zero && blockIdx.x == 0 && threadIdx.x == 0) *a.zero = 0;
+    const unsigned full = 0xffffffffu;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nx = a.g.n[0], ny = a.g.n[1], nz = a.g.n[2];
+    const long long n = (long long)nx * ny * nz;
+    const bool even = nx % 2 == 0 && ((uintptr_t)a.C & 15) == 0;  // rows of C start on 16 bytes
+    const int sx = (a.g.td[0] + F2V_STRIP - 1) / F2V_STRIP;
+    const long long strips = (long long)sx * a.g.td[1] * a.g.td[2];
+    for (long long st = blockIdx.x; st < strips; st += gridDim.x) {
+        const int ix = (int)(st % sx), iyz = (int)(st / sx), ty = iyz % a.g.td[1], tz = iyz / a.g.td[1];
+        const int x0 = ix * F2V_STRIP * TILE, y0 = ty * TILE, z0 = tz * TILE;
+#pragma unroll
+        for (int q = 0; q < (R * R * G + 255) / 256; q++) {
+            const int k = threadIdx.x + 256 * q;
+            if (k >= R * R * G) continue;
+            const int r = k / G, gr = k - r * G;
+            s_col[r][gr] = (uint8_t)group_colours(a.cb, (wrapc(z0 + r / R, nz) * ny + wrapc(y0 + r % R, ny)) * nx,
+                                                  x0 + 8 * gr, nx, a.cb_whole, n);
+        }
+        __syncthreads();
+        // warp w takes tile w of the strip, two rows of cells per lane
+        const int o0 = x0 + TILE * warp;
+        const unsigned vx = o0 >= nx ? 0u : (nx - o0 >= TILE ? 0xFFu : (1u << (nx - o0)) - 1u);
+        if (lane == 0 && o0 < nx) a.dirty[(tz * a.g.td[1] + ty) * a.g.td[0] + ix * F2V_STRIP + warp] = 0;
+        unsigned cut[2];
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+            const int r = lane + 32 * q, i = (r & 7) + R * (r >> 3);
+            auto row = [&](int k) -> unsigned {
+                const uint8_t *c = s_col[i + k] + warp;
+                return (unsigned)c[0] | ((unsigned)c[1] & 1u) << 8;
+            };
+            const unsigned c0 = row(0), c1 = row(1), c2 = row(R), c3 = row(R + 1);
+            const unsigned all = c0 & c1 & c2 & c3, any = c0 | c1 | c2 | c3;
+            const unsigned one = all & all >> 1 & 0xFFu;
+            s_one[r][warp] = (uint8_t)one;
+            cut[q] = y0 + (r & 7) < ny && z0 + (r >> 3) < nz ? (any | any >> 1) & ~one & vx : 0u;
+        }
+        unsigned total;
+        int pos = (int)warp_prefix(__popc(cut[0]) + __popc(cut[1]), &total);
+        if (total) {
+            int base = 0;
+            if (lane == 0) base = atomicAdd(a.ncut, (int)total);
+            pos += __shfl_sync(full, base, 0);
+#pragma unroll
+            for (int q = 0; q < 2; q++) {
+                const int r = lane + 32 * q;
+                const int id = ((z0 + (r >> 3)) * ny + y0 + (r & 7)) * nx + o0;
+                for (unsigned m = cut[q]; m; m &= m - 1) a.cut[pos++] = (unsigned)(id + __ffs((int)m) - 1);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < TILE * TILE * F2V_STRIP * TILE / 512; q++) {
+            const int k = threadIdx.x + 256 * q, r = k >> 5, xl = 2 * (k & 31);
+            const int y = y0 + (r & 7), z = z0 + (r >> 3), x = x0 + xl;
+            if (y >= ny || z >= nz || x >= nx) continue;
+            const unsigned w = s_one[r][xl >> 3] >> (xl & 7);
+            unsigned long long *p = reinterpret_cast<unsigned long long *>(a.C) + ((long long)z * ny + y) * nx + x;
+            const unsigned long long v0 = (w & 1u) ? 0x3FF0000000000000ull : 0ull,
+                                     v1 = (w & 2u) ? 0x3FF0000000000000ull : 0ull;
+            if (even) {
+                *reinterpret_cast<ulonglong2 *>(p) = make_ulonglong2(v0, v1);
+            } else {
+                p[0] = v0;
+                if (x + 1 < nx) p[1] = v1;
+            }
+        }
+        __syncthreads();
+    }
+}
+
 // Per-cell reconstruction, registers only:
 //   * face areas from closed forms -- a corner cut is the triangle l1*l2/2, a
 //     cut across the face the trapezoid (l1 + l2)/2, three corners the
