@@ -543,9 +543,9 @@ static int amr_scratch(ebit_ctx *ctx) {
 static int refine_pass(ebit_ctx *ctx, uint8_t *mask, uint8_t *bg) {
     if (int r = amr_scratch(ctx)) return r;
     CU(cudaMemsetAsync(ctx->amr_ctr, 0, 3 * sizeof(unsigned long long) + amr_chunks(ctx) * sizeof(int), ctx->stream));
-    const long long strips = (long long)((ctx->g.td[0] + AMR_WARPS - 1) / AMR_WARPS) * ctx->g.td[1] * ctx->g.td[2];
-    refine_kernel<<<(int)std::min<long long>(strips, 8 * ctx->sms), 32 * AMR_WARPS, 0, ctx->stream>>>(ctx->g, ctx->cb[ctx->cur], (ctx->N + 7) & ~7LL, mask, ctx->amr_flag, bg,
-                                   ctx->amr_ctr, reinterpret_cast<int *>(ctx->amr_ctr + 3));
+    refine_kernel<<<(int)std::min<long long>(refine_blocks(ctx->g), 1 << 20), AMR_THREADS, 0, ctx->stream>>>(
+        ctx->g, ctx->cb[ctx->cur], (ctx->N + 7) & ~7LL, mask, ctx->amr_flag, bg, ctx->amr_ctr,
+        reinterpret_cast<int *>(ctx->amr_ctr + 3));
     return launch_check(ctx, "refine_kernel");
 }
 
@@ -833,7 +833,7 @@ int ebit_front2vof(ebit_ctx *ctx, double *C, int flags) {
         const long long strips =
             (long long)((ctx->g.td[0] + F2V_STRIP - 1) / F2V_STRIP) * ctx->g.td[1] * ctx->g.td[2];
         const cudaError_t e =
-            full && sh == 0 ? launch_pdl(f2v_full_kernel, (int)std::min<long long>(strips, 8 * ctx->sms), 256, 0, st, a)
+            full && sh == 0 ? launch_pdl(f2v_full_kernel, (int)std::min<long long>(strips, 1 << 20), 256, 0, st, a)
             : sh == 0       ? launch_pdl(f2v_band_kernel<0>, ctx->grid_f2v, 64, 0, st, a)
             : sh == 1       ? launch_pdl(f2v_band_kernel<1>, ctx->grid_f2v, 64, 0, st, a)
                             : launch_pdl(f2v_band_kernel<2>, ctx->grid_f2v, 64, 0, st, a);

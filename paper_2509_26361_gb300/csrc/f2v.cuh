@@ -138,11 +138,12 @@ __global__ void __launch_bounds__(64, 16) f2v_band_kernel(F2VArgs a) {
 // The band pass over every tile (8^3 tiles): a block takes a strip of eight tiles
 // along x, so that consecutive lanes read colours and write fractions along the
 // rows; HBM bound by the fractions (a tile at a time, a lane per row, 152 us at
-// 384^3; this form 112).
+// 384^3; this form 105, of which the fractions take 68).
 constexpr int F2V_STRIP = 8;
 __global__ void __launch_bounds__(256) f2v_full_kernel(F2VArgs a) {
     constexpr int R = TILE + 1, G = F2V_STRIP + 1;
     __shared__ uint8_t s_col[R * R][G + 3];
+    __shared__ int s_off[R * R];
     __shared__ uint8_t s_one[TILE * TILE][F2V_STRIP];
     pdl_wait();
     if (a.zero && blockIdx.x == 0 && threadIdx.x == 0) *a.zero = 0;
@@ -154,15 +155,23 @@ __global__ void __launch_bounds__(256) f2v_full_kernel(F2VArgs a) {
     const int sx = (a.g.td[0] + F2V_STRIP - 1) / F2V_STRIP;
     const long long strips = (long long)sx * a.g.td[1] * a.g.td[2];
     for (long long st = blockIdx.x; st < strips; st += gridDim.x) {
-        const int ix = (int)(st % sx), iyz = (int)(st / sx), ty = iyz % a.g.td[1], tz = iyz / a.g.td[1];
+        const int iyz = (int)((unsigned)st / (unsigned)sx), ix = (int)st - iyz * sx;
+        const int tz = iyz / a.g.td[1], ty = iyz - tz * a.g.td[1];
         const int x0 = ix * F2V_STRIP * TILE, y0 = ty * TILE, z0 = tz * TILE;
+        if (threadIdx.x < R * R) {  // the rows' first nodes, once per row
+            const int r = threadIdx.x;
+            s_off[r] = (wrapc(z0 + r / R, nz) * ny + wrapc(y0 + r % R, ny)) * nx;
+        }
+        __syncthreads();
+        // no group of the strip at the seam, and its rows start on 8 bytes
+        const bool inner = x0 + 8 * G <= nx && nx % 8 == 0 && a.cb_whole > 0;
 #pragma unroll
         for (int q = 0; q < (R * R * G + 255) / 256; q++) {
             const int k = threadIdx.x + 256 * q;
             if (k >= R * R * G) continue;
-            const int r = k / G, gr = k - r * G;
-            s_col[r][gr] = (uint8_t)group_colours(a.cb, (wrapc(z0 + r / R, nz) * ny + wrapc(y0 + r % R, ny)) * nx,
-                                                  x0 + 8 * gr, nx, a.cb_whole, n);
+            const int r = k / G, gr = k - r * G, x = x0 + 8 * gr;
+            s_col[r][gr] = (uint8_t)(inner ? gather_bits(__ldg(reinterpret_cast<const unsigned long long *>(a.cb + (s_off[r] + x))))
+                                           : group_colours(a.cb, s_off[r], x, nx, a.cb_whole, n));
         }
         __syncthreads();
         // warp w takes tile w of the strip, two rows of cells per lane

@@ -74,7 +74,8 @@ __device__ __forceinline__ RowGroup row_group(const Grid &g, const uint8_t *__re
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
     if (t >= (long long)gx * ny * nz) return r;
     const long long n = (long long)nx * ny * nz;
-    const int row = (int)(t / gx), x = 8 * (int)(t - (long long)row * gx);
+    // (fewer groups than cells: 32-bit divisions)
+    const int row = (int)((unsigned)t / (unsigned)gx), x = 8 * ((int)t - row * gx);
     const int z = row / ny, y = row - z * ny;
     r.id = row * nx + x;
     r.cnt = min(8, nx - x);
