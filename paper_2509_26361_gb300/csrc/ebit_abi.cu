@@ -1223,7 +1223,7 @@ int ebit_mlp_forward(ebit_mlp *mlp, const uint16_t *X, int m, float *y) {
     const int ntile = (m + 127) / 128;
     a.err = mlp->err;
     if (mlp->path == EBIT_MLP_PATH_TCGEN05)
-        mlp_fwd_tc_kernel<false, false><<<std::min((ntile + TC_GROUPS - 1) / TC_GROUPS, mlp->sms), TC_THREADS,
+        mlp_fwd_tc_kernel<false, false><<<std::min(ntile, mlp->sms), TC_THREADS,
                                           FWD_TC_SMEM, mlp->stream>>>(a);
     else
         mlp_fwd_kernel<false, false><<<std::min(ntile, mlp->fwd_blocks * mlp->sms), 128, FWD_SMEM, mlp->stream>>>(a);

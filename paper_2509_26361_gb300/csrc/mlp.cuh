@@ -600,12 +600,6 @@ constexpr int FWD_TC_SMEM = TCF_PRM + 388 * 4 + 1024;
 constexpr int TC_THREADS = 128 * TC_GROUPS;
 constexpr long long MLP_WAIT = 1LL << 20;  // mbarrier polls before a wait gives up
 
-__device__ __forceinline__ void load_row_kmaj(unsigned char *tile, const __nv_bfloat16 *__restrict__ src, int tr,
-                                              long long r, int cols) {
-    const uint4 *s = reinterpret_cast<const uint4 *>(src + r * cols);
-    for (int q = 0; q < cols / 8; q++) *reinterpret_cast<uint4 *>(tile + tc::kmaj_off(tr, q * 8, cols)) = s[q];
-}
-
 // barrier of one 128-thread group (named barrier 1 + group)
 __device__ __forceinline__ void group_sync(int grp) {
     asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
@@ -633,32 +627,31 @@ __global__ void __launch_bounds__(TC_THREADS) mlp_fwd_tc_kernel(MlpArgs a) {
         *sBad = 0;
     }
     if (tid < 32) tc::tmem_alloc(tc::smem_u32(tbase), 512);
-    if (tid < 128) {
-        load_row_kmaj(sW1, a.w1b, tid, tid, MLP_IN);
-        load_row_kmaj(sW2, a.w2b, tid, tid, MLP_H);
-    }
+    // the weights, 16 bytes per thread and round, every thread
+#pragma unroll
+    for (int c = tid; c < MLP_H * MLP_IN / 8; c += TC_THREADS)
+        *reinterpret_cast<uint4 *>(sW1 + tc::kmaj_off(c / (MLP_IN / 8), c % (MLP_IN / 8) * 8, MLP_IN)) =
+            reinterpret_cast<const uint4 *>(a.w1b)[c];
+#pragma unroll
+    for (int c = tid; c < MLP_H * MLP_H / 8; c += TC_THREADS)
+        *reinterpret_cast<uint4 *>(sW2 + tc::kmaj_off(c / (MLP_H / 8), c % (MLP_H / 8) * 8, MLP_H)) =
+            reinterpret_cast<const uint4 *>(a.w2b)[c];
     stage_params(prm, a.params);
-    tc::fence_proxy_async();
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    const uint32_t tm0 = *tbase;
-    const uint32_t tm = tm0 + (uint32_t)(grp * 128);          // this group's columns
-    const uint32_t lane_base = tm + ((uint32_t)(wq * 32) << 16);
     const int m = a.ncells ? *a.ncells : a.m;
-    // the allocation must be the whole of tensor memory, from lane 0, column 0
-    const bool tm_ok = tm0 == 0;
-    const int ntile = tm_ok ? (m + 127) / 128 : 0;
-    if (!tm_ok && tid == 0) atomicExch(a.err, 2);
+    const int ntile = (m + 127) / 128;
+    uint32_t tm = 0, lane_base = 0;
+    bool tm_ok = true, staged = false;
     const uint32_t idesc = tc::idesc_bf16(128, 128);
     uint32_t phase = 0;
     bool ok = true;
-    for (int tile = blockIdx.x * TC_GROUPS + grp; tile < ntile; tile += gridDim.x * TC_GROUPS) {
+    // tiles go to the blocks in turn (group 0 of every block, then group 1, ...),
+    // so that a short list spreads over all SMs
+    for (int tile = grp * gridDim.x + blockIdx.x;; tile += gridDim.x * TC_GROUPS) {
         const int row = tile * 128 + t;
-        const bool live = row < m;
+        const bool live = tile < ntile && row < m;
         int cell = 0;
         // ---- inputs: row t of the group's tile
-        {
+        if (tile < ntile) {
             __nv_bfloat16 v[MLP_IN];
             if (GATHER && live) {
                 cell = a.cells[row];
@@ -675,7 +668,20 @@ __global__ void __launch_bounds__(TC_THREADS) mlp_fwd_tc_kernel(MlpArgs a) {
         }
         tc::fence_proxy_async();
         tc::fence_before_sync();
-        group_sync(grp);
+        if (staged) {
+            group_sync(grp);
+        } else {
+            // the first tile's inputs are gathered while the weights arrive; the
+            // tensor-memory allocation must be all of it, from lane 0, column 0
+            __syncthreads();
+            tc::fence_after_sync();
+            staged = true;
+            tm_ok = *tbase == 0;
+            if (!tm_ok && tid == 0) atomicExch(a.err, 2);
+            tm = *tbase + (uint32_t)(grp * 128);  // this group's columns
+            lane_base = tm + ((uint32_t)(wq * 32) << 16);
+        }
+        if (tile >= ntile || !tm_ok) break;
         // ---- layer 1: D = X W1^T
         if (t == 0) {
             tc::fence_after_sync();
@@ -764,7 +770,7 @@ __global__ void __launch_bounds__(TC_THREADS) mlp_fwd_tc_kernel(MlpArgs a) {
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (tid < 32 && tm_ok) tc::tmem_dealloc(tm0, 512);
+    if (tid < 32 && tm_ok) tc::tmem_dealloc(*tbase, 512);
 }
 
 // Adds a warp's 32 x 32 accumulator block (warp_gemm32 layout) to the FP32
