@@ -84,8 +84,8 @@ __device__ __noinline__ unsigned f64_bits_to_f32_rare(unsigned long long u) {
     return sign | f;  // f = 2^23 reads as the smallest normal
 }
 
-// Values of float exponent 1 .. 254, zeros and double subnormals, without a
-// branch; *rare is set for any other.
+// Values of float exponent 1 .. 254 and zeros, without a branch; *rare is set for
+// any other.
 __device__ __forceinline__ float f64_bits_to_f32_common(long long bits, bool *rare) {
     const unsigned long long u = (unsigned long long)bits;
     const unsigned long long x = u & 0x7FFFFFFFFFFFFFFFull;
@@ -95,7 +95,7 @@ __device__ __forceinline__ float f64_bits_to_f32_common(long long bits, bool *ra
     // bit); a carry out of the fraction raises the exponent, to infinity from the
     // largest binade
     const unsigned long long t = x + 0x0FFFFFFFull + ((x >> 29) & 1ull);
-    *rare |= !normal && e != 0;
+    *rare |= !normal && x != 0;
     return __uint_as_float(sign | (normal ? (unsigned)(t >> 29) - (896u << 23) : 0u));
 }
 
@@ -158,19 +158,17 @@ __device__ __forceinline__ void transpose27(float (&f)[27], bool on) {
             }
 }
 
-// 3x3x3 block around cell (x, y, z); reflect the axes with n < 0; order the
-// axes by increasing |n| (stable); write the 27 values in z-major order of the
-// canonical axes, split into bf16 head and tail.  The normal is taken in float
-// and its decisions (signs, order) kept when every sign and comparison clears
-// twice the bound above, so they equal those of the double-precision normal;
-// otherwise the double-precision normal decides.  The symmetry is applied in
-// registers: the reflections, then the axis transpositions of the three-step
-// sorting network that orders |n| (output axis j takes input axis o_j; each
-// exchange of two entries of o exchanges those two output axes).  Returns the
-// fragment flag.
-__device__ __forceinline__ bool canon_encode(const double *__restrict__ C, const Grid &g, int x, int y, int z,
-                                             __nv_bfloat16 out[MLP_IN]) {
+__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
+    __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<uint32_t *>(&v);
+}
+
+// The 3x3x3 block of C around a cell, as bit patterns in z-major order.
+__device__ __forceinline__ void stencil_load(const double *__restrict__ C, const Grid &g, int cell,
+                                             long long (&bits)[27]) {
     const long long *Cb = reinterpret_cast<const long long *>(C);
+    const int row = (int)((unsigned)cell / (unsigned)g.n[0]), x = cell - row * g.n[0];
+    const int z = (int)((unsigned)row / (unsigned)g.n[1]), y = row - z * g.n[1];
     int xo[3], yo[3], zo[3];
 #pragma unroll
     for (int i = 0; i < 3; i++) {
@@ -178,21 +176,44 @@ __device__ __forceinline__ bool canon_encode(const double *__restrict__ C, const
         yo[i] = wrapc(y + i - 1, g.n[1]) * g.n[0];
         zo[i] = wrapc(z + i - 1, g.n[2]) * (g.n[0] * g.n[1]);
     }
+#pragma unroll
+    for (int b = 0; b < 27; b++) bits[b] = __ldg(Cb + (zo[b / 9] + yo[(b / 3) % 3] + xo[b % 3]));
+}
+
+// The 64 inputs (bf16, as eight 16-byte pieces) of the block `bits` around `cell`:
+// reflect the axes with n < 0; order the
+// axes by increasing |n| (stable); write the 27 values in z-major order of the
+// canonical axes, split into bf16 head and tail.  The normal is taken in float
+// and its decisions (signs, order) kept when every sign and comparison clears
+// twice the bound above, so they equal those of the double-precision normal;
+// otherwise the double-precision normal decides (from the block, read again: a
+// rare case, and its bits need not be kept).  The symmetry is applied in
+// registers: the reflections, then the axis transpositions of the three-step
+// sorting network that orders |n| (output axis j takes input axis o_j; each
+// exchange of two entries of o exchanges those two output axes).  Returns the
+// fragment flag.
+__device__ __forceinline__ bool canon_encode(const double *__restrict__ C, const Grid &g, int cell,
+                                             const long long (&bits)[27], uint4 (&out)[MLP_IN / 8]) {
     float f[27];
     unsigned pos = 0;
     bool rare = false;
 #pragma unroll
     for (int b = 0; b < 27; b++) {
-        const long long bits = __ldg(Cb + zo[b / 9] + yo[(b / 3) % 3] + xo[b % 3]);
-        if (f64_bits_positive(bits)) pos |= 1u << b;
-        f[b] = f64_bits_to_f32_common(bits, &rare);
+        f[b] = f64_bits_to_f32_common(bits[b], &rare);
+        if (f[b] > 0.0f) pos |= 1u << b;
     }
     // one branch for all 27 (with one for each, the empty cells of a stencil, +0,
-    // cost a call each: 16 000 cycles of a tile, now 7600)
-    if (rare)
+    // cost a call each: 16 000 cycles of a tile, 3900 with this one)
+    if (rare) {
+        long long again[27];
+        stencil_load(C, g, cell, again);
+        pos = 0;
 #pragma unroll
-        for (int b = 0; b < 27; b++)
-            f[b] = f64_bits_to_f32(__ldg(Cb + zo[b / 9] + yo[(b / 3) % 3] + xo[b % 3]));
+        for (int b = 0; b < 27; b++) {
+            f[b] = f64_bits_to_f32(again[b]);
+            if (f64_bits_positive(again[b])) pos |= 1u << b;
+        }
+    }
     float nf[3];
     youngs<float>(f, nf);
     const float a0 = fabsf(nf[0]), a1 = fabsf(nf[1]), a2 = fabsf(nf[2]);
@@ -210,9 +231,11 @@ __device__ __forceinline__ bool canon_encode(const double *__restrict__ C, const
         if (s2) { t = p1; p1 = p2; p2 = t; }
         s3 = s2 && p1 < p0;
     } else {
+        long long again[27];
+        stencil_load(C, g, cell, again);
         double v[27];
 #pragma unroll
-        for (int b = 0; b < 27; b++) v[b] = __ldg(C + zo[b / 9] + yo[(b / 3) % 3] + xo[b % 3]);
+        for (int b = 0; b < 27; b++) v[b] = __longlong_as_double(again[b]);
         double n[3];
         youngs<double>(v, n);
         neg0 = n[0] < 0.0;
@@ -231,17 +254,17 @@ __device__ __forceinline__ bool canon_encode(const double *__restrict__ C, const
     transpose27<0, 1>(f, s1);
     transpose27<1, 2>(f, s2);
     transpose27<0, 1>(f, s3);
+    uint32_t w[MLP_IN / 2];
 #pragma unroll
-    for (int k = 0; k < 27; k++) {
-        const __nv_bfloat16 hi = __float2bfloat16_rn(f[k]);
-        out[k] = hi;
-        out[32 + k] = __float2bfloat16_rn(f[k] - __bfloat162float(hi));
+    for (int k = 0; k < 16; k++) {
+        w[k] = w[16 + k] = 0u;
+        if (k >= 14) continue;
+        const float lo = f[2 * k], hi = 2 * k + 1 < 27 ? f[2 * k + 1 < 27 ? 2 * k + 1 : 0] : 0.0f;
+        w[k] = pack_bf16x2(lo, hi);  // heads, and what they leave
+        w[16 + k] = pack_bf16x2(lo - __uint_as_float(w[k] << 16), hi - __uint_as_float(w[k] & 0xFFFF0000u));
     }
 #pragma unroll
-    for (int q = 27; q < 32; q++) {
-        out[q] = __float2bfloat16_rn(0.0f);
-        out[32 + q] = __float2bfloat16_rn(0.0f);
-    }
+    for (int q = 0; q < MLP_IN / 8; q++) out[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
     return fragmented27(pos);
 }
 
@@ -259,14 +282,14 @@ __global__ void __launch_bounds__(GATHER_THREADS) mlp_gather_kernel(const double
                                                                     uint8_t *__restrict__ frag) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
         const int id = cells[i];
-        const int x = id % g.n[0], y = (id / g.n[0]) % g.n[1], z = id / (g.n[0] * g.n[1]);
-        __nv_bfloat16 v[MLP_IN];
-        const bool fr = canon_encode(C, g, x, y, z, v);
+        long long bits[27];
+        stencil_load(C, g, id, bits);
+        uint4 v[MLP_IN / 8];
+        const bool fr = canon_encode(C, g, id, bits, v);
         if (frag) frag[i] = fr ? 1 : 0;
         uint4 *dst = reinterpret_cast<uint4 *>(X + (long long)i * MLP_IN);
-        const uint4 *src = reinterpret_cast<const uint4 *>(v);
 #pragma unroll
-        for (int q = 0; q < MLP_IN / 8; q++) dst[q] = src[q];
+        for (int q = 0; q < MLP_IN / 8; q++) dst[q] = v[q];
     }
 }
 
@@ -453,11 +476,6 @@ __device__ __forceinline__ void stage_params(float *prm, const float *__restrict
         prm[k] = ldp(p, k < 256 ? (k < 128 ? P_B1 + k : P_B2 + k - 128) : (k < 384 ? P_W3 + k - 256 : P_B3));
 }
 
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-    __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<uint32_t *>(&v);
-}
-
 template <bool GATHER, bool CURV>
 __global__ void __launch_bounds__(128, 3) mlp_fwd_kernel(MlpArgs a) {
     pdl_wait();
@@ -479,16 +497,19 @@ __global__ void __launch_bounds__(128, 3) mlp_fwd_kernel(MlpArgs a) {
         const bool live = row < m;
         // ---- inputs: row tid of the tile
         if (GATHER) {
-            __nv_bfloat16 v[MLP_IN];
+            uint4 v[MLP_IN / 8];
             if (live) {
                 const int cell = a.cells[row];
-                const int x = cell % a.g.n[0], y = (cell / a.g.n[0]) % a.g.n[1], z = cell / (a.g.n[0] * a.g.n[1]);
-                sFrag[tid] = canon_encode(a.C, a.g, x, y, z, v) ? 1 : 0;
+                long long bits[27];
+                stencil_load(a.C, a.g, cell, bits);
+                sFrag[tid] = canon_encode(a.C, a.g, cell, bits, v) ? 1 : 0;
             } else {
-                for (int q = 0; q < MLP_IN; q++) v[q] = __float2bfloat16_rn(0.0f);
+#pragma unroll
+                for (int q = 0; q < MLP_IN / 8; q++) v[q] = make_uint4(0u, 0u, 0u, 0u);
             }
             uint4 *d = reinterpret_cast<uint4 *>(sX + tid * LD64);
-            for (int q = 0; q < MLP_IN / 8; q++) d[q] = reinterpret_cast<uint4 *>(v)[q];
+#pragma unroll
+            for (int q = 0; q < MLP_IN / 8; q++) d[q] = v[q];
         } else if (live) {
             load_row(sX, LD64, tid, a.X, row, MLP_IN, m);
         } else {
@@ -619,9 +640,13 @@ __device__ __forceinline__ void group_sync(int grp) {
     asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
 }
 
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 template <bool GATHER, bool CURV>
 __global__ void __launch_bounds__(TC_THREADS) mlp_fwd_tc_kernel(MlpArgs a) {
-    pdl_wait();
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int tid = threadIdx.x, grp = tid >> 7, t = tid & 127, wq = (tid >> 5) & 3;
@@ -635,58 +660,79 @@ __global__ void __launch_bounds__(TC_THREADS) mlp_fwd_tc_kernel(MlpArgs a) {
     volatile int *sBad = reinterpret_cast<volatile int *>(base + TCF_BAD) + grp;
     float *prm = reinterpret_cast<float *>(base + TCF_PRM);
     const uint32_t mb = tc::smem_u32(mbar);
+    // nothing here depends on the kernel before
     if (t == 0) {
         tc::mbar_init(mb, 1);
         tc::fence_mbar_init();
         *sBad = 0;
     }
     if (tid < 32) tc::tmem_alloc(tc::smem_u32(tbase), 512);
-    // the weights, 16 bytes per thread and round, every thread
-#pragma unroll
-    for (int c = tid; c < MLP_H * MLP_IN / 8; c += TC_THREADS)
-        *reinterpret_cast<uint4 *>(sW1 + tc::kmaj_off(c / (MLP_IN / 8), c % (MLP_IN / 8) * 8, MLP_IN)) =
-            reinterpret_cast<const uint4 *>(a.w1b)[c];
-#pragma unroll
-    for (int c = tid; c < MLP_H * MLP_H / 8; c += TC_THREADS)
-        *reinterpret_cast<uint4 *>(sW2 + tc::kmaj_off(c / (MLP_H / 8), c % (MLP_H / 8) * 8, MLP_H)) =
-            reinterpret_cast<const uint4 *>(a.w2b)[c];
-    stage_params(prm, a.params);
+    pdl_wait();
+    // tiles go to the blocks in turn (group 0 of every block, then group 1, ...),
+    // so that a short list spreads over all SMs
+    int tile = grp * gridDim.x + blockIdx.x;
+    const int step = gridDim.x * TC_GROUPS;
+    // a tile's stencils are loaded while the one before is in its second layer, its
+    // cells a layer earlier; those of the first at once, with the list's length
+    // (entries past it are read, within the list's capacity, and not used)
+    int cell = 0;
+    long long bits[27];
+    if (GATHER) {
+        const long long row = (long long)tile * 128 + t;
+        if (row < (long long)a.g.n[0] * a.g.n[1] * a.g.n[2]) cell = __ldg(a.cells + row);
+    }
     const int m = a.ncells ? *a.ncells : a.m;
     const int ntile = (m + 127) / 128;
+    // the weights on their way, 16 bytes per thread and round, while the first
+    // tile is gathered and encoded
+#pragma unroll
+    for (int c = tid; c < MLP_H * MLP_IN / 8; c += TC_THREADS)
+        cp_async16(sW1 + tc::kmaj_off(c / (MLP_IN / 8), c % (MLP_IN / 8) * 8, MLP_IN), a.w1b + 8 * c);
+#pragma unroll
+    for (int c = tid; c < MLP_H * MLP_H / 8; c += TC_THREADS)
+        cp_async16(sW2 + tc::kmaj_off(c / (MLP_H / 8), c % (MLP_H / 8) * 8, MLP_H), a.w2b + 8 * c);
+    if (tid < 385) {
+        const int k = tid, src = k < 256 ? (k < 128 ? P_B1 + k : P_B2 + k - 128) : (k < 384 ? P_W3 + k - 256 : P_B3);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(tc::smem_u32(prm + k)), "l"(a.params + src)
+                     : "memory");
+    }
+    if (GATHER && tile < ntile && tile * 128 + t < m) stencil_load(a.C, a.g, cell, bits);
     uint32_t tm = 0, lane_base = 0;
     bool tm_ok = true, staged = false;
     const uint32_t idesc = tc::idesc_bf16(128, 128);
     uint32_t phase = 0;
     bool ok = true;
-    // tiles go to the blocks in turn (group 0 of every block, then group 1, ...),
-    // so that a short list spreads over all SMs
-    for (int tile = grp * gridDim.x + blockIdx.x;; tile += gridDim.x * TC_GROUPS) {
+    for (;; tile += step) {
         const int row = tile * 128 + t;
         const bool live = tile < ntile && row < m;
-        int cell = 0;
         // ---- inputs: row t of the group's tile
         if (tile < ntile) {
-            __nv_bfloat16 v[MLP_IN];
+            uint4 v[MLP_IN / 8];
             if (GATHER && live) {
-                cell = a.cells[row];
-                const int x = cell % a.g.n[0], y = (cell / a.g.n[0]) % a.g.n[1], z = cell / (a.g.n[0] * a.g.n[1]);
-                sFrag[t] = canon_encode(a.C, a.g, x, y, z, v) ? 1 : 0;
+                sFrag[t] = canon_encode(a.C, a.g, cell, bits, v) ? 1 : 0;
             } else if (!GATHER && live) {
                 const uint4 *s4 = reinterpret_cast<const uint4 *>(a.X + (long long)row * MLP_IN);
-                for (int q = 0; q < MLP_IN / 8; q++) reinterpret_cast<uint4 *>(v)[q] = s4[q];
+#pragma unroll
+                for (int q = 0; q < MLP_IN / 8; q++) v[q] = s4[q];
             } else {
-                for (int q = 0; q < MLP_IN; q++) v[q] = __float2bfloat16_rn(0.0f);
+#pragma unroll
+                for (int q = 0; q < MLP_IN / 8; q++) v[q] = make_uint4(0u, 0u, 0u, 0u);
             }
+#pragma unroll
             for (int q = 0; q < MLP_IN / 8; q++)
-                *reinterpret_cast<uint4 *>(sX + tc::kmaj_off(t, q * 8, MLP_IN)) = reinterpret_cast<uint4 *>(v)[q];
+                *reinterpret_cast<uint4 *>(sX + tc::kmaj_off(t, q * 8, MLP_IN)) = v[q];
         }
+        const bool more = GATHER && tile + step < ntile && (tile + step) * 128 + t < m;
+        int next = 0;
+        if (more) next = __ldg(a.cells + (tile + step) * 128 + t);
+        if (!staged) cp_async_wait();
         tc::fence_proxy_async();
         tc::fence_before_sync();
         if (staged) {
             group_sync(grp);
         } else {
-            // the first tile's inputs are gathered while the weights arrive; the
-            // tensor-memory allocation must be all of it, from lane 0, column 0
+            // the weights are in; the tensor-memory allocation must be all of it,
+            // from lane 0, column 0
             __syncthreads();
             tc::fence_after_sync();
             staged = true;
@@ -741,6 +787,7 @@ __global__ void __launch_bounds__(TC_THREADS) mlp_fwd_tc_kernel(MlpArgs a) {
                              idesc, kk > 0);
             tc::mma_commit(mb);
         }
+        if (more) stencil_load(a.C, a.g, next, bits);
         if (!tc::mbar_wait(mb, phase, MLP_WAIT)) *sBad = 1;
         group_sync(grp);
         ok = *sBad == 0;
@@ -775,6 +822,7 @@ __global__ void __launch_bounds__(TC_THREADS) mlp_fwd_tc_kernel(MlpArgs a) {
                 a.y[row] = yv;
             }
         }
+        cell = next;
         tc::fence_before_sync();
         group_sync(grp);
     }
