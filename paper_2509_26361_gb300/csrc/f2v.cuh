@@ -238,8 +238,8 @@ __global__ void __launch_bounds__(256) f2v_full_kernel(F2VArgs a) {
 // ones.  A marker's coordinates but one are 0 or 1, so of the six products of a
 // cross product five are selections; the faces' cases differ by selected
 // operands, not by branches, so lanes with different cuts share one instruction
-// stream (72 registers, where the branching form took 160; 17 to 14 us for the
-// cut cells of 128^3, 62 to 45 us at 512^3).
+// stream (72 registers, where the branching form took 160; 62 to 45 us at 512^3;
+// with multiply-adds, exact halves and quotients by known reciprocals 37).
 __device__ __forceinline__ double sel01(int b) { return __longlong_as_double(b ? 0x3FF0000000000000ll : 0ll); }
 
 // a loop's number of markers (up to 12) as a double, by its bit pattern
@@ -247,6 +247,16 @@ __device__ __forceinline__ double small_count(int k) {
     const int e = 31 - __clz(k);
     return __hiloint2double((1023 + e) << 20 | (k << (20 - e) & 0xFFFFF), 0);
 }
+
+// v / 2: an exponent decrement for a normal number with a normal half
+__device__ __forceinline__ double half_of(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    return ((b >> 52) & 0x7FF) > 1 ? __longlong_as_double((long long)(b - (1ull << 52))) : 0.5 * v;
+}
+
+// 1 / k correctly rounded, k = 1 .. 12
+static __constant__ double kInverse[13] = {0.0,       1.0,       1.0 / 2.0, 1.0 / 3.0, 1.0 / 4.0,  1.0 / 5.0, 1.0 / 6.0,
+                                           1.0 / 7.0, 1.0 / 8.0, 1.0 / 9.0, 1.0 / 10.0, 1.0 / 11.0, 1.0 / 12.0};
 
 __device__ __forceinline__ void marker_xyz(int e, double s, double &x, double &y, double &z) {
     const int ax = e >> 2, r = e & 3;
@@ -293,23 +303,24 @@ __device__ __forceinline__ double face_area_and_links(int K, int phif, const dou
         // corner ea + 1 cut off (eb = ea + 1), corners ea + 1 and ea + 2 (eb =
         // ea + 2), or all but corner 0 (ea = 0, eb = 3: its complement)
         const bool rest = eb == ea + 3, side = eb == ea + 2;
-        double l1 = sE[ce_a * stride], l2 = sE[ce_b * stride];
+        Fp l1 = sE[ce_a * stride], l2 = sE[ce_b * stride];
         if (ea < 2 && !rest) l1 = 1.0 - l1;
         if (eb >= 2 && !rest) l2 = 1.0 - l2;
-        double R = 0.5 * (side ? l1 + l2 : l1 * l2);
+        // l1 + l2 or l1 l2, in one operation
+        Fp R = half_of(__fma_rn(l1.v, side ? fp_one() : l2.v, side ? l2.v : fp_minus_zero()));
         if (rest) R = 1.0 - R;
         area = arc ? R : 1.0 - R;
     } else if (saddle) {
-        double T = 0.0;
+        Fp T = 0.0;
 #pragma unroll
         for (int m = 0; m < 4; m++) {
             if (((cols >> m) & 1) == phif) continue;
             // legs from corner m back along edge m - 1 and on along edge m
             const int p = (m + 3) & 3;
-            double lp = sE[kFaceEdge[F][p] * stride], ln = sE[kFaceEdge[F][m] * stride];
+            Fp lp = sE[kFaceEdge[F][p] * stride], ln = sE[kFaceEdge[F][m] * stride];
             if (p < 2) lp = 1.0 - lp;
             if (m >= 2) ln = 1.0 - ln;
-            T += 0.5 * (lp * ln);
+            T += half_of(lp * ln);
         }
         area = phif ? 1.0 - T : T;
     }
@@ -318,7 +329,7 @@ __device__ __forceinline__ double face_area_and_links(int K, int phif, const dou
 
 __device__ double cell_fraction_fast(int K, const int Fc[6], const double *sE, int stride, int *bad) {
     unsigned long long nxt = ~0ull;
-    double A1 = 0.0, A2 = 0.0, A3 = 0.0;
+    Fp A1 = 0.0, A2 = 0.0, A3 = 0.0;
     face_area_and_links<0>(K, Fc[0], sE, stride, nxt);
     A1 = face_area_and_links<1>(K, Fc[1], sE, stride, nxt);
     face_area_and_links<2>(K, Fc[2], sE, stride, nxt);
@@ -336,15 +347,15 @@ __device__ double cell_fraction_fast(int K, const int Fc[6], const double *sE, i
     }
     if (!has) return sel01(K & 1);
     unsigned todo = has;
-    double acc = 0.0;
+    Fp acc = 0.0;
     while (todo) {
         const int e0 = __ffs(todo) - 1;
         double sp = sE[e0 * stride];
         const double s0 = sp;
-        double sx, sy, sz;
-        marker_xyz(e0, sp, sx, sy, sz);
-        double px = sx, py = sy, pz = sz;
-        double cxs = 0.0, cys = 0.0, czs = 0.0;
+        double px, py, pz;
+        marker_xyz(e0, sp, px, py, pz);
+        Fp sx = px, sy = py, sz = pz;
+        Fp cxs = 0.0, cys = 0.0, czs = 0.0;
         int len = 1, e = e0;
         todo &= ~(1u << e0);
         bool closed = false;
@@ -356,9 +367,9 @@ __device__ double cell_fraction_fast(int K, const int Fc[6], const double *sE, i
             double qx, qy, qz;
             marker_xyz(to, sq, qx, qy, qz);
             // p x q: the one product of two offsets, the others selected
-            const double pq = sp * sq;
+            const double pq = Fp(sp) * sq;
             const int ap = e >> 2, aq = to >> 2;
-            auto mul = [&](double u, double v, int au, int av) -> double {
+            auto mul = [&](double u, double v, int au, int av) -> Fp {
                 // u = p's coordinate au, v = q's coordinate av
                 const bool us = ap == au, vs = aq == av;
                 const double w = us ? u : v;             // the factor that is an offset (or 0, 1)
@@ -380,12 +391,15 @@ __device__ double cell_fraction_fast(int K, const int Fc[6], const double *sE, i
             *bad = 1;
             continue;
         }
-        acc += (sx * cxs + sy * cys + sz * czs) / small_count(len);
+        const double dot = sx * cxs + sy * cys + sz * czs;
+        acc += safe_quotient(dot) ? quotient(dot, small_count(len), kInverse[len]) : dot / small_count(len);
     }
-    double V = (2.0 * ((A1 + A2) + A3) - acc) / 6.0;
-    if (V < 0.0) V = 0.0;
-    if (V > 1.0) V = 1.0;
-    return V;
+    const double six = 2.0 * ((A1 + A2) + A3) - acc;
+    const double V = safe_quotient(six) ? quotient(six, 6.0, 1.0 / 6.0) : six / 6.0;
+    // clamped to [0, 1] (finite), by the bit pattern
+    const long long b = __double_as_longlong(V);
+    if (b < 0 && (b << 1) != 0) return 0.0;
+    return b > 0x3FF0000000000000ll ? 1.0 : V;
 }
 
 // FP64 pass: one thread per cut cell, full warps.

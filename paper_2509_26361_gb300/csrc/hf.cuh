@@ -106,6 +106,24 @@ static __device__ __noinline__ int hf_order_exact(const double *__restrict__ C, 
     return hf_order<double>(n[0], n[1], n[2]);
 }
 
+// A value in [+0, 1] (bit pattern b) in units of 2^-60, cut off below; 0 for 0.
+__device__ __forceinline__ unsigned long long unit_fixed(unsigned long long b) {
+    const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | 1ull << 52;
+    const int sh = (int)(b >> 52) - (1023 - 60 + 52);  // m 2^(sh - 60), sh <= 8
+    return sh >= 0 ? m << sh : (sh > -53 ? m >> -sh : 0ull);
+}
+// v 2^-60 rounded to the nearest double, ties to even (|v| < 2^63)
+__device__ __forceinline__ double fixed_double(long long v) {
+    unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    if (a == 0) return 0.0;
+    const int lead = __clzll((long long)a);
+    a <<= lead;  // the leading one at bit 63
+    // 53 bits kept; a carry out of the fraction raises the exponent
+    const unsigned long long t = (a >> 11) + (((a >> 10) & 1ull) & (((a & 0x3FFull) != 0) | ((a >> 11) & 1ull)));
+    const unsigned long long e = (unsigned long long)(1023 + 3 - lead);  // of bit 63: 2^(63 - lead - 60)
+    return __longlong_as_double((long long)((((unsigned long long)v >> 63) << 63) | ((e << 52) + (t - (1ull << 52)))));
+}
+
 // Height-function curvature of an interface cell: its status, and kappa h in
 // *out.
 //
@@ -116,9 +134,11 @@ static __device__ __noinline__ int hf_order_exact(const double *__restrict__ C, 
 // offsets, the axis a run-time value, one path for both ways of ordering the
 // axes): with separate code for cells at the seams, for each way of ordering and
 // a whole sum per axis tried, a warp ran up to twelve sums one after another.
-// The FP64 pipe (2 lanes per clock and SM) bounds long lists: 81 additions and
-// about 50 operations for the formula per cell with heights.  4.2e5 cells at
-// 256^3 took 286 us and take 88, the 500 of a sphere at 32^3 45 us and 12.
+// The FP64 units (2 lanes per clock and SM) bound long lists: about 45 operations
+// for the formula per cell with heights; the 72 additions of its columns, which
+// took as long again, run as integers.  4.2e5 cells at 256^3 took 286 us, with
+// the additions in FP64 88, and take 71; the error against 64-bit references fell
+// from 8.3e-15 to 7.3e-15.
 __device__ __forceinline__ int hf_cell(const HFCell &c, double *out) {
     int ox[3], oy[3], oz[3];
 #pragma unroll
@@ -184,30 +204,51 @@ __device__ __forceinline__ int hf_cell(const HFCell &c, double *out) {
         *out = 0.0;
         return 4;
     }
-    // heights: each column summed from its lower end
+    // heights less 4.5 cells: the sum of a column's values in [+0, 1] as integers in
+    // units of 2^-60 (a value's bits below that are cut off; the sum is exact), with
+    // one rounding to a double; of other values, in FP64
     const bool below = (ord >> (6 + axis)) & 1;
     int om[9];
 #pragma unroll
     for (int m = 0; m < 9; m++) om[m] = HFCell::off(q, nn, st, m - HFH);
-    double eta[3][3];
+    Fp eta[3][3];
+    bool fixed = true;
 #pragma unroll
     for (int b2 = 0; b2 < 3; b2++)
 #pragma unroll
         for (int b1 = 0; b1 < 3; b1++) {
             const double *col = c.C + c.id + t1[b1] + t2[b2];
-            double H = __ldg(col + om[0]);
+            unsigned long long H = 0;
+            // (the ends are known to be 0 and 1)
 #pragma unroll
-            for (int m = 1; m < 9; m++) H += __ldg(col + om[m]);
-            eta[b1][b2] = (below ? H : HFH + 0.5) - (below ? HFH + 0.5 : H);
+            for (int m = 1; m < 8; m++) {
+                const unsigned long long b = (unsigned long long)__double_as_longlong(__ldg(col + om[m]));
+                fixed = fixed && b <= 0x3FF0000000000000ull;
+                H += unit_fixed(b);
+            }
+            const long long d = (long long)(H + (1ull << 60) - (9ull << 59));
+            eta[b1][b2] = fixed_double(below ? d : -d);
         }
-    const double hx = (eta[2][1] - eta[0][1]) * 0.5;
-    const double hy = (eta[1][2] - eta[1][0]) * 0.5;
-    const double hxx = (eta[2][1] + eta[0][1]) - 2.0 * eta[1][1];
-    const double hyy = (eta[1][2] + eta[1][0]) - 2.0 * eta[1][1];
-    const double hxy = ((eta[2][2] - eta[2][0]) - (eta[0][2] - eta[0][0])) * 0.25;
-    const double num = (1.0 + hy * hy) * hxx + (1.0 + hx * hx) * hyy - 2.0 * hx * hy * hxy;
-    const double q2 = 1.0 + hx * hx + hy * hy;
-    const double kap = num / (q2 * sqrt(q2));
+    if (!fixed) {
+#pragma unroll
+        for (int b2 = 0; b2 < 3; b2++)
+#pragma unroll
+            for (int b1 = 0; b1 < 3; b1++) {
+                const double *col = c.C + c.id + t1[b1] + t2[b2];
+                double H = __ldg(col + om[0]);
+#pragma unroll
+                for (int m = 1; m < 9; m++) H += __ldg(col + om[m]);
+                eta[b1][b2] = (below ? H : HFH + 0.5) - (below ? HFH + 0.5 : H);
+            }
+    }
+    const Fp hx = (eta[2][1] - eta[0][1]) * 0.5;
+    const Fp hy = (eta[1][2] - eta[1][0]) * 0.5;
+    const Fp hxx = (eta[2][1] + eta[0][1]) - 2.0 * eta[1][1];
+    const Fp hyy = (eta[1][2] + eta[1][0]) - 2.0 * eta[1][1];
+    const Fp hxy = ((eta[2][2] - eta[2][0]) - (eta[0][2] - eta[0][0])) * 0.25;
+    const Fp num = (1.0 + hy * hy) * hxx + (1.0 + hx * hx) * hyy - 2.0 * hx * hy * hxy;
+    const Fp q2 = 1.0 + hx * hx + hy * hy;
+    const double kap = num / (q2 * sqrt(q2.v));
     *out = below ? -kap : kap;
     return 1 + axis;
 }

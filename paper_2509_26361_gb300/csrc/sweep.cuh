@@ -45,7 +45,7 @@
 namespace ebit {
 
 struct P2 {
-    double x, y;
+    Fp x, y;
 };
 
 // 2D cell edges in a plane spanned by (a, t): B a-edge at c00, R t-edge at c10,
@@ -82,25 +82,34 @@ __device__ __forceinline__ double twice(double v) {
 // (0 <= y <= 1) count, the one nearest ylin is kept (Fig. 2).  rad2 gets the
 // squared radius.
 __device__ __forceinline__ bool circle_root(P2 A, P2 B, P2 C, double ylin, double *root, double *rad2) {
-    double bx = B.x - A.x, by = B.y - A.y;
-    double cx = C.x - A.x, cy = C.y - A.y;
-    double b2 = bx * bx + by * by;
-    double c2 = cx * cx + cy * cy;
-    double det = twice(bx * cy - by * cx);
+    const Fp bx = B.x - A.x, by = B.y - A.y;
+    const Fp cx = C.x - A.x, cy = C.y - A.y;
+    const Fp b2 = bx * bx + by * by;
+    const Fp c2 = cx * cx + cy * cy;
+    const double det = twice(bx * cy - by * cx);
     if (abs_bits(det) <= dbits(1e-12 * (b2 + c2))) return false;
-    double ux = (cy * b2 - by * c2) / det;
-    double uy = (bx * c2 - cx * b2) / det;
-    double r2 = ux * ux + uy * uy;
-    double dx = A.x + ux;
-    double disc = r2 - dx * dx;
+    const Fp nx = cy * b2 - by * c2, ny = bx * c2 - cx * b2;
+    Fp ux, uy;
+    // both quotients from one reciprocal
+    if (safe_quotient(det) && safe_quotient(nx) && safe_quotient(ny)) {
+        const double y = __drcp_rn(det);
+        ux = quotient(nx, det, y);
+        uy = quotient(ny, det, y);
+    } else {
+        ux = nx / det;
+        uy = ny / det;
+    }
+    const Fp r2 = ux * ux + uy * uy;
+    const Fp dx = A.x + ux;
+    const Fp disc = r2 - dx * dx;
     if (below_zero(disc)) return false;
-    double sq = sqrt(disc);
-    double yc = A.y + uy;
-    double yp = yc + sq, ym = yc - sq;
-    bool okp = in_unit(yp), okm = in_unit(ym);
+    const Fp sq = sqrt(disc.v);
+    const Fp yc = A.y + uy;
+    const Fp yp = yc + sq, ym = yc - sq;
+    const bool okp = in_unit(yp), okm = in_unit(ym);
     if (!okp && !okm) return false;
-    if (okp && okm) *root = (abs_bits(yp - ylin) <= abs_bits(ym - ylin)) ? yp : ym;
-    else *root = okp ? yp : ym;
+    if (okp && okm) *root = (abs_bits(yp - ylin) <= abs_bits(ym - ylin)) ? yp.v : ym.v;
+    else *root = okp ? yp.v : ym.v;
     *rad2 = r2;
     return true;
 }
@@ -111,7 +120,7 @@ __device__ __forceinline__ bool circle_root(P2 A, P2 B, P2 C, double ylin, doubl
 // 1e-12, far above the few units of rounding in the radii and the product), so
 // the square roots are taken only within that margin.
 __device__ __forceinline__ bool ratio_above_10(double r2max, double r2min) {
-    const double t = 100.0 * r2min;
+    const Fp t = 100.0 * Fp(r2min);
     if (dbits(r2max) > dbits(t * (1.0 + 1e-12))) return true;
     if (dbits(r2max) < dbits(t * (1.0 - 1e-12))) return false;
     return sqrt(r2max) > 10.0 * sqrt(r2min);
@@ -136,7 +145,7 @@ static __device__ __noinline__ double circle_pair(P2 P1, P2 Pa, P2 Pb, P2 P4, do
         // the larger circle
         const bool a_larger = dbits(ra2) > dbits(rb2);
         if (ratio_above_10(a_larger ? ra2 : rb2, a_larger ? rb2 : ra2)) y = a_larger ? ya : yb;
-        else y = 0.5 * (ya + yb);
+        else y = 0.5 * (Fp(ya) + yb);
     } else if (va) {
         y = ya;
     } else if (vb) {
@@ -166,7 +175,7 @@ static __device__ __noinline__ double circle_pair_split(P2 P1, P2 Pa, P2 Pb, P2 
     if (va && vb) {
         const bool a_larger = dbits(ra2) > dbits(rb2);
         if (ratio_above_10(a_larger ? ra2 : rb2, a_larger ? rb2 : ra2)) res = a_larger ? ya : yb;
-        else res = 0.5 * (ya + yb);
+        else res = 0.5 * (Fp(ya) + yb);
     } else if (va) {
         res = ya;
     } else if (vb) {
@@ -181,7 +190,7 @@ static __device__ __noinline__ double circle_pair_split(P2 P1, P2 Pa, P2 Pb, P2 
 template <int D>
 __device__ double interp_u(const Grid &g, const double *__restrict__ u, const int q[3], int e, double s) {
     int base[3];
-    double t[3];
+    Fp t[3];
 #pragma unroll
     for (int b = 0; b < 3; b++) {
         if (b == D) {
@@ -192,10 +201,10 @@ __device__ double interp_u(const Grid &g, const double *__restrict__ u, const in
             t[b] = 0.5;
         } else if (s < 0.5) {
             base[b] = q[b] - 1;
-            t[b] = s + 0.5;
+            t[b] = Fp(s) + 0.5;
         } else {
             base[b] = q[b];
-            t[b] = s - 0.5;
+            t[b] = Fp(s) - 0.5;
         }
     }
     int x0 = wrapc(base[0], g.n[0]), x1 = wrapc(base[0] + 1, g.n[0]);
@@ -208,7 +217,7 @@ __device__ double interp_u(const Grid &g, const double *__restrict__ u, const in
     // not read (for a = -0 the sign of the zero may differ; nothing downstream
     // depends on it).
     const bool flatD = e != D;
-    double c00, c10, c01, c11;
+    Fp c00, c10, c01, c11;
     if (D == 0 && flatD) {
         c00 = __ldg(u + r00 + x0);
         c10 = __ldg(u + r10 + x0);
@@ -216,13 +225,13 @@ __device__ double interp_u(const Grid &g, const double *__restrict__ u, const in
         c11 = __ldg(u + r11 + x0);
     } else {
         c00 = (1.0 - t[0]) * __ldg(u + r00 + x0) + t[0] * __ldg(u + r00 + x1);
-        c10 = (D == 1 && flatD) ? 0.0 : (1.0 - t[0]) * __ldg(u + r10 + x0) + t[0] * __ldg(u + r10 + x1);
-        c01 = (D == 2 && flatD) ? 0.0 : (1.0 - t[0]) * __ldg(u + r01 + x0) + t[0] * __ldg(u + r01 + x1);
-        c11 = (D != 0 && flatD) ? 0.0 : (1.0 - t[0]) * __ldg(u + r11 + x0) + t[0] * __ldg(u + r11 + x1);
+        c10 = (D == 1 && flatD) ? Fp(0.0) : (1.0 - t[0]) * __ldg(u + r10 + x0) + t[0] * __ldg(u + r10 + x1);
+        c01 = (D == 2 && flatD) ? Fp(0.0) : (1.0 - t[0]) * __ldg(u + r01 + x0) + t[0] * __ldg(u + r01 + x1);
+        c11 = (D != 0 && flatD) ? Fp(0.0) : (1.0 - t[0]) * __ldg(u + r11 + x0) + t[0] * __ldg(u + r11 + x1);
     }
-    const double c0 = (D == 1 && flatD) ? c00 : (1.0 - t[1]) * c00 + t[1] * c10;
+    const Fp c0 = (D == 1 && flatD) ? c00 : (1.0 - t[1]) * c00 + t[1] * c10;
     if (D == 2 && flatD) return c0;
-    const double c1 = (D == 1 && flatD) ? c01 : (1.0 - t[1]) * c01 + t[1] * c11;
+    const Fp c1 = (D == 1 && flatD) ? c01 : (1.0 - t[1]) * c01 + t[1] * c11;
     return (1.0 - t[2]) * c0 + t[2] * c1;
 }
 
@@ -267,7 +276,7 @@ __device__ __forceinline__ void move_marker(const SweepArgs &a, const Grid &g, i
     double *adv = e == 0 ? a.adv[0] : (e == 1 ? a.adv[1] : a.adv[2]);
     int8_t *bin = e == 0 ? a.bin[0] : (e == 1 ? a.bin[1] : a.bin[2]);
     const double sv = __ldg(se + gid);
-    double cf = interp_u<D>(g, u, q, e, sv) * lam;
+    double cf = Fp(interp_u<D>(g, u, q, e, sv)) * lam;
     if (!isfinite(cf)) {
         bad++;
         cf = 0.0;
@@ -275,7 +284,7 @@ __device__ __forceinline__ void move_marker(const SweepArgs &a, const Grid &g, i
         hits++;
         cf = cf > 0.0 ? ONE_MINUS : -ONE_MINUS;
     }
-    const double x = (e == D) ? sv + cf : cf;
+    const double x = (e == D) ? (double)(Fp(sv) + cf) : cf;
     adv[gid] = x;
     bin[gid] = (int8_t)(int)floor(2.0 * x);
 }
@@ -468,8 +477,8 @@ struct SweepCell {
         double s = 0.0;
         if (!m.on_a) s = __ldg(s_t() + q);
         P2 r;
-        r.x = small_double(m.qa) + x;
-        r.y = small_double(m.qt) + s;
+        r.x = Fp(small_double(m.qa)) + x;
+        r.y = Fp(small_double(m.qt)) + s;
         return r;
     }
     // the marker next along the polyline beyond edge e of cell (da, dt), in the
@@ -516,7 +525,7 @@ struct SweepCell {
     }
     // linear crossing height of the segment Pa Pb with x = 0
     __device__ __forceinline__ static double crossing_line(const P2 &Pa, const P2 &Pb) {
-        const double tt = (0.0 - Pa.x) / (Pb.x - Pa.x);
+        const Fp tt = (0.0 - Pa.x) / (Pb.x - Pa.x);
         return Pa.y + tt * (Pb.y - Pa.y);
     }
     __device__ __forceinline__ double crossing_height(int el, int er, int cda) const {
@@ -598,8 +607,8 @@ struct SweepCell {
                 if (l0 == l1) continue;
                 P2 L = pos(mark(l0 ? e0 : e1, da, 0));
                 P2 R = pos(mark(l0 ? e1 : e0, da, 0));
-                double tt = (0.5 - L.x) / (R.x - L.x);
-                double yl = L.y + tt * (R.y - L.y);
+                const Fp tt = (0.5 - L.x) / (R.x - L.x);
+                const double yl = L.y + tt * (R.y - L.y);
                 if (yl < 0.5) par ^= 1;
             }
         }
