@@ -348,7 +348,7 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
     int occ = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sweep_kernel<0>, BAND_THREADS, 0);
     ctx->grid_sweep = std::max(1, std::min(nt, ctx->sms * std::max(occ, 1)));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, advect_list_kernel<0>, 256, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, advect_list_kernel<1>, 256, 0);
     ctx->grid_advl = ctx->sms * std::max(occ, 1);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fp64_kernel<0>, 128, 0);
     ctx->grid_fp64 = ctx->sms * std::max(occ, 1);

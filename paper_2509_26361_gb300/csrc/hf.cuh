@@ -106,21 +106,20 @@ static __device__ __noinline__ int hf_order_exact(const double *__restrict__ C, 
     return hf_order<double>(n[0], n[1], n[2]);
 }
 
-// A value in [+0, 1] (bit pattern b) in units of 2^-60, cut off below; 0 for 0.
-__device__ __forceinline__ unsigned long long unit_fixed(unsigned long long b) {
-    const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | 1ull << 52;
-    const int sh = (int)(b >> 52) - (1023 - 60 + 52);  // m 2^(sh - 60), sh <= 8
-    return sh >= 0 ? m << sh : (sh > -53 ? m >> -sh : 0ull);
+// A value in [+0, 1] (bit pattern b) in units of 2^-58, cut off below.
+__device__ __forceinline__ long long unit_fixed(unsigned long long b) {
+    const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) << 6 | 1ull << 58;  // of a value in [1, 2)
+    return (long long)(m >> min(1023 - (int)(b >> 52), 63));                   // (0 from exponent 0)
 }
-// v 2^-60 rounded to the nearest double, ties to even (|v| < 2^63)
-__device__ __forceinline__ double fixed_double(long long v) {
+// v 2^-s rounded to the nearest double, ties to even
+__device__ __forceinline__ double fixed_double(long long v, int s) {
     unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
     if (a == 0) return 0.0;
     const int lead = __clzll((long long)a);
     a <<= lead;  // the leading one at bit 63
     // 53 bits kept; a carry out of the fraction raises the exponent
     const unsigned long long t = (a >> 11) + (((a >> 10) & 1ull) & (((a & 0x3FFull) != 0) | ((a >> 11) & 1ull)));
-    const unsigned long long e = (unsigned long long)(1023 + 3 - lead);  // of bit 63: 2^(63 - lead - 60)
+    const unsigned long long e = (unsigned long long)(1023 + 63 - s - lead);
     return __longlong_as_double((long long)((((unsigned long long)v >> 63) << 63) | ((e << 52) + (t - (1ull << 52)))));
 }
 
@@ -134,11 +133,11 @@ __device__ __forceinline__ double fixed_double(long long v) {
 // offsets, the axis a run-time value, one path for both ways of ordering the
 // axes): with separate code for cells at the seams, for each way of ordering and
 // a whole sum per axis tried, a warp ran up to twelve sums one after another.
-// The FP64 units (2 lanes per clock and SM) bound long lists: about 45 operations
-// for the formula per cell with heights; the 72 additions of its columns, which
-// took as long again, run as integers.  4.2e5 cells at 256^3 took 286 us, with
-// the additions in FP64 88, and take 71; the error against 64-bit references fell
-// from 8.3e-15 to 7.3e-15.
+// The FP64 units (2 lanes per clock and SM) bound long lists: about 32 operations
+// for the formula per cell with heights; its columns' 72 additions and
+// their differences run as integers.  4.2e5 cells at 256^3 took 286 us, with
+// the additions in FP64 88, and take 62; the error against 64-bit references fell
+// from 8.3e-15 to 7e-15.
 __device__ __forceinline__ int hf_cell(const HFCell &c, double *out) {
     int ox[3], oy[3], oz[3];
 #pragma unroll
@@ -204,32 +203,39 @@ __device__ __forceinline__ int hf_cell(const HFCell &c, double *out) {
         *out = 0.0;
         return 4;
     }
-    // heights less 4.5 cells: the sum of a column's values in [+0, 1] as integers in
-    // units of 2^-60 (a value's bits below that are cut off; the sum is exact), with
+    // heights: the sum of a column's values in [+0, 1] as integers in units of 2^-58
+    // (a value's bits below that are cut off); the differences are exact, with
     // one rounding to a double; of other values, in FP64
     const bool below = (ord >> (6 + axis)) & 1;
     int om[9];
 #pragma unroll
     for (int m = 0; m < 9; m++) om[m] = HFCell::off(q, nn, st, m - HFH);
-    Fp eta[3][3];
+    long long e[3][3];
     bool fixed = true;
 #pragma unroll
     for (int b2 = 0; b2 < 3; b2++)
 #pragma unroll
         for (int b1 = 0; b1 < 3; b1++) {
             const double *col = c.C + c.id + t1[b1] + t2[b2];
-            unsigned long long H = 0;
-            // (the ends are known to be 0 and 1)
+            long long H = 0;
+            // (the ends are 0 and 1 in every column: left out of the differences)
 #pragma unroll
             for (int m = 1; m < 8; m++) {
                 const unsigned long long b = (unsigned long long)__double_as_longlong(__ldg(col + om[m]));
                 fixed = fixed && b <= 0x3FF0000000000000ull;
                 H += unit_fixed(b);
             }
-            const long long d = (long long)(H + (1ull << 60) - (9ull << 59));
-            eta[b1][b2] = fixed_double(below ? d : -d);
+            e[b1][b2] = below ? H : -H;
         }
-    if (!fixed) {
+    Fp hx, hy, hxx, hyy, hxy;
+    if (fixed) {
+        hx = fixed_double(e[2][1] - e[0][1], 59);
+        hy = fixed_double(e[1][2] - e[1][0], 59);
+        hxx = fixed_double(e[2][1] + e[0][1] - 2 * e[1][1], 58);
+        hyy = fixed_double(e[1][2] + e[1][0] - 2 * e[1][1], 58);
+        hxy = fixed_double((e[2][2] - e[2][0]) - (e[0][2] - e[0][0]), 60);
+    } else {
+        double eta[3][3];
 #pragma unroll
         for (int b2 = 0; b2 < 3; b2++)
 #pragma unroll
@@ -240,12 +246,12 @@ __device__ __forceinline__ int hf_cell(const HFCell &c, double *out) {
                 for (int m = 1; m < 9; m++) H += __ldg(col + om[m]);
                 eta[b1][b2] = (below ? H : HFH + 0.5) - (below ? HFH + 0.5 : H);
             }
+        hx = (eta[2][1] - eta[0][1]) * 0.5;
+        hy = (eta[1][2] - eta[1][0]) * 0.5;
+        hxx = (eta[2][1] + eta[0][1]) - 2.0 * eta[1][1];
+        hyy = (eta[1][2] + eta[1][0]) - 2.0 * eta[1][1];
+        hxy = ((eta[2][2] - eta[2][0]) - (eta[0][2] - eta[0][0])) * 0.25;
     }
-    const Fp hx = (eta[2][1] - eta[0][1]) * 0.5;
-    const Fp hy = (eta[1][2] - eta[1][0]) * 0.5;
-    const Fp hxx = (eta[2][1] + eta[0][1]) - 2.0 * eta[1][1];
-    const Fp hyy = (eta[1][2] + eta[1][0]) - 2.0 * eta[1][1];
-    const Fp hxy = ((eta[2][2] - eta[2][0]) - (eta[0][2] - eta[0][0])) * 0.25;
     const Fp num = (1.0 + hy * hy) * hxx + (1.0 + hx * hx) * hyy - 2.0 * hx * hy * hxy;
     const Fp q2 = 1.0 + hx * hx + hy * hy;
     const double kap = num / (q2 * sqrt(q2.v));

@@ -305,7 +305,7 @@ __device__ __forceinline__ void band_item(const Grid &g, int tbase, int tile, in
 // Advection from the marker lists (Eq. 2): one thread per marker, no tile
 // staging.
 template <int D>
-__global__ void __launch_bounds__(256) advect_list_kernel(SweepArgs a, MarkerLists m) {
+__global__ void __launch_bounds__(256, 5) advect_list_kernel(SweepArgs a, MarkerLists m) {
     pdl_wait();
     clear_sweep_counts(a);
     // One index space: the markers, then this sweep's band items (tile of the
