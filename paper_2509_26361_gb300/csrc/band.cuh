@@ -490,15 +490,22 @@ __global__ void __launch_bounds__(BAND_THREADS, 16) sweep_kernel(SweepArgs a) {
     __shared__ BandSmem<D, 0> sm;
     __shared__ int s_next;
     pdl_wait();
+    // the first tile's id with the list's length (the list has room for every
+    // tile, and the grid no more blocks than tiles)
+    int tile = a.list ? a.list[blockIdx.x] : (int)blockIdx.x;
     const int ntl = a.list ? *a.count : a.g.ntiles;
     BandEvents ev;
     // after the first, each block takes tiles from a counter (tiles differ in
-    // cost), read one tile ahead
+    // cost), read one tile ahead: the value is stored after the tile, since the
+    // store waits for it, and with it all that follows in the warp
     for (int li = blockIdx.x; li < ntl;) {
-        if (threadIdx.x == 0) s_next = a.tile_next ? (int)gridDim.x + atomicAdd(a.tile_next, 1) : li + (int)gridDim.x;
-        band_tile<D, false>(a, a.g, 0, 0, a.cb_whole, a.list ? a.list[li] : li, sm, 0, ev);
+        int next = li + (int)gridDim.x;
+        if (threadIdx.x == 0 && a.tile_next) next = (int)gridDim.x + atomicAdd(a.tile_next, 1);
+        band_tile<D, false>(a, a.g, 0, 0, a.cb_whole, tile, sm, 0, ev);
+        if (threadIdx.x == 0) s_next = next;
         __syncthreads();
         li = s_next;
+        if (li < ntl) tile = a.list ? a.list[li] : li;
         __syncthreads();
     }
     flush_events(ev, a.ctr);

@@ -437,12 +437,16 @@ struct SweepCell {
     // (-1, 0) and (0, 0), in bits 0-3 and 4-7: x = q + adv < 0 <=> bin < -2 q for
     // the edge's node offset q.  (bins of edges without a marker are read and
     // not used)
-    __device__ __forceinline__ unsigned left_bits() const {
+    struct Bins {
+        int B1, T1, B0, T0, L1, L0, R0;
+    };
+    __device__ __forceinline__ Bins load_bins() const {
         const int8_t *ba = a.bin[A], *bt = bin_t();
-        const int bB1 = ld_in<F>(ba + pid(-1, 0)), bT1 = ld_in<F>(ba + pid(-1, 1));
-        const int bB0 = ld_in<F>(ba + pid(0, 0)), bT0 = ld_in<F>(ba + pid(0, 1));
-        const int bL1 = ld_in<F>(bt + pid(-1, 0)), bL0 = ld_in<F>(bt + pid(0, 0)),
-                  bR0 = ld_in<F>(bt + pid(1, 0));
+        return Bins{ld_in<F>(ba + pid(-1, 0)), ld_in<F>(ba + pid(-1, 1)), ld_in<F>(ba + pid(0, 0)), ld_in<F>(ba + pid(0, 1)),
+                    ld_in<F>(bt + pid(-1, 0)), ld_in<F>(bt + pid(0, 0)),  ld_in<F>(bt + pid(1, 0))};
+    }
+    __device__ __forceinline__ static unsigned left_bits(const Bins &b) {
+        const int bB1 = b.B1, bT1 = b.T1, bB0 = b.B0, bT0 = b.T0, bL1 = b.L1, bL0 = b.L0, bR0 = b.R0;
         const unsigned mid = bL0 < 0;  // the edge between the two cells
         return (unsigned)(bB1 < 2) | mid << ER | (unsigned)(bT1 < 2) << ET | (unsigned)(bL1 < 2) << EL |
                ((unsigned)(bB0 < 0) | (unsigned)(bR0 < -2) << ER | (unsigned)(bT0 < 0) << ET | mid << EL) << 4;
@@ -624,8 +628,9 @@ __device__ __forceinline__ void fp64_item(const SweepArgs &a, const Grid &g, int
                                           int half = -1) {
     constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
     SweepCell<D, F> cell(a, g, base, id, kind & 1);
+    const auto bins = cell.load_bins();  // (with the colours: one wait for both)
     cell.loadw();
-    const unsigned left = cell.left_bits();
+    const unsigned left = cell.left_bits(bins);
     if (kind >= 4) {
         // an even number (>= 2) of advected crossings met on an edge that keeps
         // no marker (Fig. 5)
