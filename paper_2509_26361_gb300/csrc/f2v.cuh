@@ -18,12 +18,14 @@ namespace ebit {
 
 // corners of the six cube faces, counter-clockwise seen from outside
 // (corner id = dx | dy<<1 | dz<<2); faces x=0, x=1, y=0, y=1, z=0, z=1
-__constant__ int8_t kFaceCorner[6][4] = {
-    {0, 4, 6, 2}, {1, 3, 7, 5}, {0, 1, 5, 4}, {2, 6, 7, 3}, {0, 2, 3, 1}, {4, 5, 7, 6}};
+__host__ __device__ constexpr unsigned face_corners(int F) {
+    return F == 0 ? 0x2640u : F == 1 ? 0x5731u : F == 2 ? 0x4510u : F == 3 ? 0x3762u : F == 4 ? 0x1320u : 0x6754u;
+}
 // cube edge between consecutive face corners k and k+1 (x-edges 0-3 by dy+2dz,
-// y-edges 4-7 by dx+2dz, z-edges 8-11 by dx+2dy)
-__constant__ int8_t kFaceEdge[6][4] = {
-    {8, 6, 10, 4}, {5, 11, 7, 9}, {0, 9, 2, 8}, {10, 3, 11, 1}, {4, 1, 5, 0}, {2, 7, 3, 6}};
+// y-edges 4-7 by dx+2dz, z-edges 8-11 by dx+2dy), nibble k
+__host__ __device__ constexpr unsigned face_edges(int F) {
+    return F == 0 ? 0x4A68u : F == 1 ? 0x97B5u : F == 2 ? 0x8290u : F == 3 ? 0x1B3Au : F == 4 ? 0x0514u : 0x6372u;
+}
 
 struct F2VArgs {
     Grid g;
@@ -271,17 +273,12 @@ __device__ __forceinline__ void marker_xyz(int e, double s, double &x, double &y
 // face (odd F), returns its reference-phase area.  Of the face's edges 0 and 1
 // run from corner k to k + 1, 2 and 3 back, on every face, which fixes
 // whether a distance is s or 1 - s.
-template <int F>
-__device__ __forceinline__ double face_area_and_links(int K, int phif, const double *sE, int stride,
-                                                      unsigned long long &nxt) {
-    // the face's edges as nibbles
-    unsigned eds = 0;
+// eds, cors: the face's edges and corners as nibbles; upper: an odd F.
+__device__ __forceinline__ double face_area_and_links(unsigned eds, unsigned cors, bool upper, int K, int phif,
+                                                      const double *sE, int stride, unsigned long long &nxt) {
     int cols = 0;
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
-        cols |= ((K >> kFaceCorner[F][k]) & 1) << k;
-        eds |= (unsigned)kFaceEdge[F][k] << (4 * k);
-    }
+    for (int k = 0; k < 4; k++) cols |= ((K >> ((cors >> (4 * k)) & 7)) & 1) << k;
     auto edge = [&](int k) -> int { return (int)((eds >> (4 * k)) & 15u); };
     auto link = [&](int from, int to, bool on) {
         const unsigned long long m = on ? 0xFull << (4 * from) : 0ull;
@@ -297,7 +294,7 @@ __device__ __forceinline__ double face_area_and_links(int K, int phif, const dou
     link(arc ? ce_b : ce_a, arc ? ce_a : ce_b, one || saddle);
     const int ce_c = edge((ea + 2) & 3), ce_d = edge((eb + 2) & 3);  // the saddle's other cut
     link(arc ? ce_d : ce_c, arc ? ce_c : ce_d, saddle);
-    if (!(F & 1)) return 0.0;
+    if (!upper) return 0.0;
     double area = sel01(cols & 1);
     if (one) {
         // corner ea + 1 cut off (eb = ea + 1), corners ea + 1 and ea + 2 (eb =
@@ -317,7 +314,7 @@ __device__ __forceinline__ double face_area_and_links(int K, int phif, const dou
             if (((cols >> m) & 1) == phif) continue;
             // legs from corner m back along edge m - 1 and on along edge m
             const int p = (m + 3) & 3;
-            Fp lp = sE[kFaceEdge[F][p] * stride], ln = sE[kFaceEdge[F][m] * stride];
+            Fp lp = sE[edge(p) * stride], ln = sE[edge(m) * stride];
             if (p < 2) lp = 1.0 - lp;
             if (m >= 2) ln = 1.0 - ln;
             T += half_of(lp * ln);
@@ -327,16 +324,14 @@ __device__ __forceinline__ double face_area_and_links(int K, int phif, const dou
     return area;
 }
 
-__device__ double cell_fraction_fast(int K, const int Fc[6], const double *sE, int stride, int *bad) {
-    unsigned long long nxt = ~0ull;
-    Fp A1 = 0.0, A2 = 0.0, A3 = 0.0;
-    face_area_and_links<0>(K, Fc[0], sE, stride, nxt);
-    A1 = face_area_and_links<1>(K, Fc[1], sE, stride, nxt);
-    face_area_and_links<2>(K, Fc[2], sE, stride, nxt);
-    A2 = face_area_and_links<3>(K, Fc[3], sE, stride, nxt);
-    face_area_and_links<4>(K, Fc[4], sE, stride, nxt);
-    A3 = face_area_and_links<5>(K, Fc[5], sE, stride, nxt);
-    // markers: edges whose end colours differ
+template <int F>
+__device__ __forceinline__ double face_of(int K, int phif, const double *sE, int stride, unsigned long long &nxt) {
+    constexpr unsigned eds = face_edges(F), cors = face_corners(F);
+    return face_area_and_links(eds, cors, F & 1, K, phif, sE, stride, nxt);
+}
+
+// edges whose end colours differ
+__device__ __forceinline__ unsigned marked_edges(int K) {
     unsigned has = 0;
     const int cx[4] = {0, 2, 4, 6}, cy[4] = {0, 1, 4, 5}, cz[4] = {0, 1, 2, 3};
 #pragma unroll
@@ -345,6 +340,31 @@ __device__ double cell_fraction_fast(int K, const int Fc[6], const double *sE, i
         has |= (unsigned)(((K >> cy[r]) ^ (K >> (cy[r] + 2))) & 1) << (4 + r);
         has |= (unsigned)(((K >> cz[r]) ^ (K >> (cz[r] + 4))) & 1) << (8 + r);
     }
+    return has;
+}
+
+// the volume from the upper faces' areas and the sum over the loops, clamped to
+// [0, 1] by the bit pattern
+__device__ __forceinline__ double volume(Fp A1, Fp A2, Fp A3, Fp acc) {
+    const double six = 2.0 * ((A1 + A2) + A3) - acc;
+    const double V = safe_quotient(six) ? quotient(six, 6.0, 1.0 / 6.0) : six / 6.0;
+    const long long b = __double_as_longlong(V);
+    if (b < 0 && (b << 1) != 0) return 0.0;
+    return b > 0x3FF0000000000000ll ? 1.0 : V;
+}
+__device__ __forceinline__ double loop_mean(double dot, int len) {
+    return safe_quotient(dot) ? quotient(dot, small_count(len), kInverse[len]) : dot / small_count(len);
+}
+
+__device__ double cell_fraction_fast(int K, const int Fc[6], const double *sE, int stride, int *bad) {
+    unsigned long long nxt = ~0ull;
+    face_of<0>(K, Fc[0], sE, stride, nxt);
+    const Fp A1 = face_of<1>(K, Fc[1], sE, stride, nxt);
+    face_of<2>(K, Fc[2], sE, stride, nxt);
+    const Fp A2 = face_of<3>(K, Fc[3], sE, stride, nxt);
+    face_of<4>(K, Fc[4], sE, stride, nxt);
+    const Fp A3 = face_of<5>(K, Fc[5], sE, stride, nxt);
+    const unsigned has = marked_edges(K);
     if (!has) return sel01(K & 1);
     unsigned todo = has;
     Fp acc = 0.0;
@@ -391,15 +411,9 @@ __device__ double cell_fraction_fast(int K, const int Fc[6], const double *sE, i
             *bad = 1;
             continue;
         }
-        const double dot = sx * cxs + sy * cys + sz * czs;
-        acc += safe_quotient(dot) ? quotient(dot, small_count(len), kInverse[len]) : dot / small_count(len);
+        acc += loop_mean(sx * cxs + sy * cys + sz * czs, len);
     }
-    const double six = 2.0 * ((A1 + A2) + A3) - acc;
-    const double V = safe_quotient(six) ? quotient(six, 6.0, 1.0 / 6.0) : six / 6.0;
-    // clamped to [0, 1] (finite), by the bit pattern
-    const long long b = __double_as_longlong(V);
-    if (b < 0 && (b << 1) != 0) return 0.0;
-    return b > 0x3FF0000000000000ll ? 1.0 : V;
+    return volume(A1, A2, A3, acc);
 }
 
 // FP64 pass: one thread per cut cell, full warps.
@@ -415,7 +429,8 @@ __global__ void __launch_bounds__(128) f2v_list_kernel(F2VArgs a) {
         const int t = list_item(it);
         if (t >= n) continue;
         const int id = (int)a.cut[t];
-        const int x = id % a.g.n[0], y = (id / a.g.n[0]) % a.g.n[1], z = id / (a.g.n[0] * a.g.n[1]);
+        const int row = (int)((unsigned)id / (unsigned)a.g.n[0]), x = id - row * a.g.n[0];
+        const int z = (int)((unsigned)row / (unsigned)a.g.n[1]), y = row - z * a.g.n[1];
         int ids[8];
         cell_ids(a.g, x, y, z, ids);
         int K = 0;
