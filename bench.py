@@ -874,7 +874,7 @@ def main():
             "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": config_dict(args.workload, w, "not flushed: the steps run back to back (Front2VOF and curvature "
-                                  "overlapping the next sweeps); the state (149 B per node) and the velocity "
+                                  "overlapping the next sweeps); the state (133 B per node) and the velocity "
                                   "fields are far larger than L2"),
             "roofline": dict(roofline_block(res_sync, prof), overlapped=overlapped(res),
                              timing="CUDA events around the three split-sweep calls of each step of the ordered "

@@ -247,7 +247,7 @@ int ebit_band_tiles(ebit_ctx *ctx);
 enum {
     EBIT_PROF_SWEEP = 0, /* split-sweep reconstruction kernels */
     EBIT_PROF_BAND = 1,  /* (no kernel of its own: each sweep's band pass lists the next sweep's band) */
-    EBIT_PROF_F2V = 2,   /* Front2VOF: list of the swept tiles (incremental calls), band and cut-cell kernels */
+    EBIT_PROF_F2V = 2,   /* Front2VOF: band and cut-cell kernels */
     EBIT_PROF_HF = 3,    /* height-function kernel (interface-cell list pass) */
     EBIT_PROF_MLP = 4,   /* learned-curvature kernels (with the height-function fallback pass) */
     EBIT_PROF_ADVECT = 5, /* marker advection (velocity interpolation) kernels */
@@ -308,7 +308,7 @@ int ebit_mlp_train_step(ebit_mlp *mlp, const uint16_t *X, const float *t, const 
 int ebit_mlp_sync(ebit_mlp *mlp);
 /* Inference path of ebit_mlp_forward and ebit_curvature:
  * EBIT_MLP_PATH_TCGEN05 (default): 5th-generation tensor cores, a persistent
- * block per SM with three pipelines, each issuing tcgen05.mma from shared
+ * block per SM with four pipelines, each issuing tcgen05.mma from shared
  * memory into its tensor-memory columns; EBIT_MLP_PATH_MMA: warp-level BF16
  * MMA (mma.sync m16n8k16), the layer-1 activations in registers.  Both compute
  * the same network in bf16 with FP32 accumulation. */

@@ -89,14 +89,21 @@ def test_sweeps_fractions_and_masks(n3, density):
     g.close()
 
 
+@pytest.mark.parametrize("wild", [False, True])
 @pytest.mark.parametrize("n3", EXTENTS)
-def test_full_curvature_scan(n3):
+def test_full_curvature_scan(n3, wild):
     """Fractions of random full and empty columns with a few cut cells between
-    them, some of whose stencils hold height functions."""
+    them, some of whose stencils hold height functions; wild: any C is taken, so
+    cells beside the cut ones outside [0, 1], negative zeros and values far below
+    the smallest fraction, which the heights sum in FP64."""
     rng = np.random.default_rng(5 + sum(n3))
     nx, ny, nz = n3
     lev = rng.integers(1, 3, size=(nz, ny)) + 0.25 * nx + rng.uniform(size=(nz, ny))
     C = np.clip(lev[:, :, None] - np.arange(nx), 0.0, 1.0)
+    if wild:
+        near = np.abs(np.arange(nx) - lev[:, :, None]) < 2.5
+        odd = rng.choice([1.25, -0.5, -0.0, 1e-300, 0.0, 1.0], size=C.shape)
+        C = np.where(near & (rng.uniform(size=C.shape) < 0.1), odd, C)
     okh, ost = oracle.hf_curvature(C)
     g = ebit.Grid(*n3)
     for place in (lambda t: t, shifted):
