@@ -830,10 +830,8 @@ int ebit_front2vof(ebit_ctx *ctx, double *C, int flags) {
         // one instantiation per tile shape (a batch instance may be re-tiled);
         // every 8^3 tile at once by strips
         const int sh = ctx->g.tl[0] - 3;
-        const long long strips =
-            (long long)((ctx->g.td[0] + F2V_STRIP - 1) / F2V_STRIP) * ctx->g.td[1] * ctx->g.td[2];
         const cudaError_t e =
-            full && sh == 0 ? launch_pdl(f2v_full_kernel, (int)std::min<long long>(strips, 1 << 20), 256, 0, st, a)
+            full && sh == 0 ? launch_pdl(f2v_full_kernel, (int)std::min<long long>(f2v_blocks(ctx->g), 1 << 20), F2V_THREADS, 0, st, a)
             : sh == 0       ? launch_pdl(f2v_band_kernel<0>, ctx->grid_f2v, 64, 0, st, a)
             : sh == 1       ? launch_pdl(f2v_band_kernel<1>, ctx->grid_f2v, 64, 0, st, a)
                             : launch_pdl(f2v_band_kernel<2>, ctx->grid_f2v, 64, 0, st, a);

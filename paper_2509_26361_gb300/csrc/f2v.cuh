@@ -137,94 +137,106 @@ __global__ void __launch_bounds__(64, 16) f2v_band_kernel(F2VArgs a) {
     }
 }
 
-// The band pass over every tile (8^3 tiles): a block takes a strip of eight tiles
-// along x, so that consecutive lanes read colours and write fractions along the
-// rows; HBM bound by the fractions (a tile at a time, a lane per row, 152 us at
-// 384^3; this form 105, of which the fractions take 68).
-constexpr int F2V_STRIP = 8;
-__global__ void __launch_bounds__(256) f2v_full_kernel(F2VArgs a) {
-    constexpr int R = TILE + 1, G = F2V_STRIP + 1;
-    __shared__ uint8_t s_col[R * R][G + 3];
-    __shared__ int s_off[R * R];
-    __shared__ uint8_t s_one[TILE * TILE][F2V_STRIP];
+// The band pass over every tile (8^3 tiles): a block takes 64 x 8 x 16 cells, a
+// thread a row of 64.  Node rows are kept as 64-bit words (node 64 in a second
+// one), read in groups of 8 colours, consecutive lanes along the rows; fractions go
+// out 16 bytes per lane along the rows.  HBM bound by the fractions (a tile at a
+// time, a lane per row, 152 us at 384^3; eight tiles along x, bytes of colours per
+// tile row, 105; this form about 85, of which the fractions take 68).
+constexpr int F2V_TX = 8, F2V_TZ = 2;                // a block's tiles along x and z
+constexpr int F2V_THREADS = TILE * TILE * F2V_TZ;    // a thread per row of cells
+inline long long f2v_blocks(const Grid &g) {
+    return (long long)((g.td[0] + F2V_TX - 1) / F2V_TX) * g.td[1] * ((g.td[2] + F2V_TZ - 1) / F2V_TZ);
+}
+__global__ void __launch_bounds__(F2V_THREADS) f2v_full_kernel(F2VArgs a) {
+    typedef unsigned long long u64;
+    constexpr int RY = TILE + 1, RZ = TILE * F2V_TZ + 1, G = F2V_TX + 1;
+    __shared__ ulonglong2 s_row[RY * RZ];  // nodes 0 .. 63 | nodes 64 .. 71 (byte 8)
+    __shared__ int s_off[RY * RZ];
+    __shared__ u64 s_one[F2V_THREADS];
     pdl_wait();
     if (a.zero && blockIdx.x == 0 && threadIdx.x == 0) *a.zero = 0;
     const unsigned full = 0xffffffffu;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nx = a.g.n[0], ny = a.g.n[1], nz = a.g.n[2];
     const long long n = (long long)nx * ny * nz;
     const bool even = nx % 2 == 0 && ((uintptr_t)a.C & 15) == 0;  // rows of C start on 16 bytes
-    const int sx = (a.g.td[0] + F2V_STRIP - 1) / F2V_STRIP;
-    const long long strips = (long long)sx * a.g.td[1] * a.g.td[2];
-    for (long long st = blockIdx.x; st < strips; st += gridDim.x) {
-        const int iyz = (int)((unsigned)st / (unsigned)sx), ix = (int)st - iyz * sx;
-        const int tz = iyz / a.g.td[1], ty = iyz - tz * a.g.td[1];
-        const int x0 = ix * F2V_STRIP * TILE, y0 = ty * TILE, z0 = tz * TILE;
-        if (threadIdx.x < R * R) {  // the rows' first nodes, once per row
-            const int r = threadIdx.x;
-            s_off[r] = (wrapc(z0 + r / R, nz) * ny + wrapc(y0 + r % R, ny)) * nx;
-        }
+    const unsigned bx = (a.g.td[0] + F2V_TX - 1) / F2V_TX;
+    const long long blocks = (long long)bx * a.g.td[1] * ((a.g.td[2] + F2V_TZ - 1) / F2V_TZ);
+    for (long long b = blockIdx.x; b < blocks; b += gridDim.x) {
+        const unsigned byz = (unsigned)b / bx, bz = byz / (unsigned)a.g.td[1];
+        const int tx0 = (int)((unsigned)b - byz * bx) * F2V_TX, ty = (int)(byz - bz * (unsigned)a.g.td[1]);
+        const int x0 = tx0 * TILE, y0 = ty * TILE, z0 = (int)bz * F2V_TZ * TILE;
+        // the rows' first nodes, once per row (rows past the last that a cell reads repeat it)
+        for (int r = tid; r < RY * RZ; r += F2V_THREADS)
+            s_off[r] = (wrapc(min(z0 + r / RY, nz), nz) * ny + wrapc(min(y0 + r % RY, ny), ny)) * nx + x0;
         __syncthreads();
-        // no group of the strip at the seam, and its rows start on 8 bytes
-        const bool inner = x0 + 8 * G <= nx && nx % 8 == 0 && a.cb_whole > 0;
-#pragma unroll
-        for (int q = 0; q < (R * R * G + 255) / 256; q++) {
-            const int k = threadIdx.x + 256 * q;
-            if (k >= R * R * G) continue;
-            const int r = k / G, gr = k - r * G, x = x0 + 8 * gr;
-            s_col[r][gr] = (uint8_t)(inner ? gather_bits(__ldg(reinterpret_cast<const unsigned long long *>(a.cb + (s_off[r] + x))))
-                                           : group_colours(a.cb, s_off[r], x, nx, a.cb_whole, n));
-        }
-        __syncthreads();
-        // warp w takes tile w of the strip, two rows of cells per lane
-        const int o0 = x0 + TILE * warp;
-        const unsigned vx = o0 >= nx ? 0u : (nx - o0 >= TILE ? 0xFFu : (1u << (nx - o0)) - 1u);
-        if (lane == 0 && o0 < nx) a.dirty[(tz * a.g.td[1] + ty) * a.g.td[0] + ix * F2V_STRIP + warp] = 0;
-        unsigned cut[2];
-#pragma unroll
-        for (int q = 0; q < 2; q++) {
-            const int r = lane + 32 * q, i = (r & 7) + R * (r >> 3);
-            auto row = [&](int k) -> unsigned {
-                const uint8_t *c = s_col[i + k] + warp;
-                return (unsigned)c[0] | ((unsigned)c[1] & 1u) << 8;
-            };
-            const unsigned c0 = row(0), c1 = row(1), c2 = row(R), c3 = row(R + 1);
-            const unsigned all = c0 & c1 & c2 & c3, any = c0 | c1 | c2 | c3;
-            const unsigned one = all & all >> 1 & 0xFFu;
-            s_one[r][warp] = (uint8_t)one;
-            cut[q] = y0 + (r & 7) < ny && z0 + (r >> 3) < nz ? (any | any >> 1) & ~one & vx : 0u;
-        }
-        unsigned total;
-        int pos = (int)warp_prefix(__popc(cut[0]) + __popc(cut[1]), &total);
-        if (total) {
-            int base = 0;
-            if (lane == 0) base = atomicAdd(a.ncut, (int)total);
-            pos += __shfl_sync(full, base, 0);
-#pragma unroll
-            for (int q = 0; q < 2; q++) {
-                const int r = lane + 32 * q;
-                const int id = ((z0 + (r >> 3)) * ny + y0 + (r & 7)) * nx + o0;
-                for (unsigned m = cut[q]; m; m &= m - 1) a.cut[pos++] = (unsigned)(id + __ffs((int)m) - 1);
+        uint8_t *bytes = reinterpret_cast<uint8_t *>(s_row);
+        constexpr int TASKS = RY * RZ * G;
+        if (x0 + 8 * G <= nx && nx % 8 == 0 && a.cb_whole > 0) {
+            // no group at the seam, and rows start on 8 bytes
+#pragma unroll 6
+            for (int k = tid; k < TASKS; k += F2V_THREADS) {
+                const int r = k / G, gr = k - r * G;
+                bytes[16 * r + gr] = (uint8_t)gather_bits(__ldg(reinterpret_cast<const u64 *>(a.cb + (s_off[r] + 8 * gr))));
+            }
+        } else {
+            for (int k = tid; k < TASKS; k += F2V_THREADS) {
+                const int r = k / G, gr = k - r * G;
+                bytes[16 * r + gr] = (uint8_t)group_colours(a.cb, s_off[r] - x0, x0 + 8 * gr, nx, a.cb_whole, n);
             }
         }
         __syncthreads();
-#pragma unroll
-        for (int q = 0; q < TILE * TILE * F2V_STRIP * TILE / 512; q++) {
-            const int k = threadIdx.x + 256 * q, r = k >> 5, xl = 2 * (k & 31);
-            const int y = y0 + (r & 7), z = z0 + (r >> 3), x = x0 + xl;
-            if (y >= ny || z >= nz || x >= nx) continue;
-            const unsigned w = s_one[r][xl >> 3] >> (xl & 7);
-            unsigned long long *p = reinterpret_cast<unsigned long long *>(a.C) + ((long long)z * ny + y) * nx + x;
-            const unsigned long long v0 = (w & 1u) ? 0x3FF0000000000000ull : 0ull,
-                                     v1 = (w & 2u) ? 0x3FF0000000000000ull : 0ull;
-            if (even) {
-                *reinterpret_cast<ulonglong2 *>(p) = make_ulonglong2(v0, v1);
-            } else {
-                p[0] = v0;
-                if (x + 1 < nx) p[1] = v1;
+        const int y = tid & 7, z = tid >> 3;
+        u64 one, cut;
+        {
+            const ulonglong2 *q = s_row + y + RY * z;
+            const ulonglong2 c0 = q[0], c1 = q[1], c2 = q[RY], c3 = q[RY + 1];
+            const u64 all = c0.x & c1.x & c2.x & c3.x, any = c0.x | c1.x | c2.x | c3.x;
+            one = all & (all >> 1 | (c0.y & c1.y & c2.y & c3.y) << 63);
+            cut = (any | any >> 1 | (c0.y | c1.y | c2.y | c3.y) << 63) & ~one;
+            if (nx - x0 < 64) cut &= (1ull << (nx - x0)) - 1ull;
+            if (y0 + y >= ny || z0 + z >= nz) cut = 0;
+        }
+        s_one[tid] = one;
+        // the cut cells, tile by tile (entries next to each other on the list share
+        // neighbourhoods)
+        if (__any_sync(full, cut != 0)) {
+            const int id = ((z0 + z) * ny + y0 + y) * nx + x0;
+            for (int k = 0; k < F2V_TX; k++) {
+                const unsigned m8 = (unsigned)(cut >> (8 * k)) & 0xFFu;
+                if (!__any_sync(full, m8)) continue;
+                unsigned total;
+                int pos = (int)warp_prefix((unsigned)__popc(m8), &total);
+                int base = 0;
+                if (lane == 0) base = atomicAdd(a.ncut, (int)total);
+                pos += __shfl_sync(full, base, 0);
+                for (unsigned m = m8; m; m &= m - 1) a.cut[pos++] = (unsigned)(id + 8 * k + __ffs((int)m) - 1);
             }
         }
+        if (tid < F2V_TX * F2V_TZ) {
+            const int tx = tx0 + tid % F2V_TX, tz = (int)bz * F2V_TZ + tid / F2V_TX;
+            if (tx < a.g.td[0] && tz < a.g.td[2]) a.dirty[(tz * a.g.td[1] + ty) * a.g.td[0] + tx] = 0;
+        }
         __syncthreads();
+        const int x = x0 + 2 * lane;
+        if (x < nx) {
+#pragma unroll 8
+            for (int r = warp; r < F2V_THREADS; r += F2V_THREADS / 32) {
+                const int yy = y0 + (r & 7), zz = z0 + (r >> 3);
+                if (yy >= ny || zz >= nz) continue;
+                const unsigned w = (unsigned)(s_one[r] >> (2 * lane));
+                u64 *p = reinterpret_cast<u64 *>(a.C) + ((long long)zz * ny + yy) * nx + x;
+                const u64 v0 = (w & 1u) ? 0x3FF0000000000000ull : 0ull, v1 = (w & 2u) ? 0x3FF0000000000000ull : 0ull;
+                if (even) {
+                    *reinterpret_cast<ulonglong2 *>(p) = make_ulonglong2(v0, v1);
+                } else {
+                    p[0] = v0;
+                    if (x + 1 < nx) p[1] = v1;
+                }
+            }
+        }
+        __syncthreads();  // the staging is rewritten by the next round
     }
 }
 
