@@ -639,6 +639,7 @@ int ebit_one_fluid(ebit_ctx *ctx, const double *C, const double *kappa_h, const 
     a.mu1 = mu1;
     a.mu2 = mu2;
     a.h = ctx->h;
+    a.inv_h = 1.0 / ctx->h;
     a.rho = rho;
     a.mu = mu;
     for (int d = 0; d < 3; d++) a.f[d] = force ? force + d * ctx->N : nullptr;
