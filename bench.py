@@ -47,15 +47,16 @@ SWEEP_BYTES_PER_CELL = 62.75
 F2V_BYTES_PER_CELL = 36.4
 # DRAM bytes (read + write) of one split sweep (list advection + band pass +
 # FP64 lists) per band cell, from one ncu capture of each kernel on the
-# converging drops at 256^3 (18.1 MB for about 4.8e5 band cells;
+# converging drops at 256^3 (16.8 MB for about 4.8e5 band cells;
 # profiles/sweep_kernels_merging_drops_256.md); scaled by the band of the run.
-NCU_DRAM_BYTES_PER_BAND_CELL = 18.12e6 / 4.807e5
+NCU_DRAM_BYTES_PER_BAND_CELL = 16.81e6 / 4.807e5
 # The FP64-list kernel's second roofline.  Peak: GB300's FP64 FMA rate
 # (6.2e11 thread operations per second, 2 per clock per SM; a probe of
 # independent FMA chains over every SM; the ncu counters give the same 304 per
 # clock).  Work: FP64 adds, multiplies and FMAs per marker of the sweep, from
 # the ncu capture of the kernel at 256^3 (3.49e6 per launch for 3.57e4
-# markers: 23.3 + 19.8 + 20.6 per elapsed cycle over 54 730 cycles).
+# markers: 23.3 + 19.8 + 20.6 per elapsed cycle over 54 730 cycles; the method's
+# count, before quotients shared reciprocals).
 FP64_PEAK_OPS_PER_S = 6.245e11
 FP64_OPS_PER_MARKER = 3.49e6 / 3.567e4
 
