@@ -382,7 +382,8 @@ int ebit_batch_launch_shape(const ebit_batch *b, int *ctas_per_sm, int *max_ctas
 int ebit_batch_set_launch_shape(ebit_batch *b, int ctas_per_sm);
 /* Tile shape: the cells per tile edge along x, y, z of the band tiles that the
  * batched sweep works on (512 cells each; every edge at least 4 cells, so the
- * tile proximity rule of the band still reaches only adjacent tiles).  The
+ * tile proximity rule of the band still reaches only adjacent tiles, and past
+ * a clipped last tile the one before it).  The
  * shape changes how the work is cut and staged, never the result: tiles
  * outside the band are unchanged by a sweep whatever their shape.
  *   EBIT_TILE_8x8x8 (0, the initial shape and that of single contexts),

@@ -410,9 +410,11 @@ __device__ __forceinline__ void band_tile(const SweepArgs &a, const Grid &g, int
         store_row<TX>(a.cbo, rowid, n0, f[0], f[1], f[2], vx);
         // cells with a marker before or after
         const uint32_t m = ((v000 ^ v100) | (v000 ^ v010) | (v000 ^ v001) | pres | p1 | p2) & vx;
-        const unsigned xs = ((m & ((1u << NEAR) - 1u)) ? 1u : 0u) | (m ? 2u : 0u) | ((m >> (TX - NEAR)) ? 4u : 0u);
-        const unsigned ys = (ly < NEAR ? 1u : 0u) | 1u << 3 | (ly >= TY - NEAR ? 1u << 6 : 0u);
-        const unsigned zs = (lz < NEAR ? 1u : 0u) | 1u << 9 | (lz >= TZ - NEAR ? 1u << 18 : 0u);
+        // (the layers next to the following tile, from the last cell inside the grid)
+        const unsigned xs = ((m & ((1u << NEAR) - 1u)) ? 1u : 0u) | (m ? 2u : 0u) |
+                            ((m >> max(min(TX, nx - o[0]) - NEAR, 0)) ? 4u : 0u);
+        const unsigned ys = (ly < NEAR ? 1u : 0u) | 1u << 3 | (ly >= min(TY, ny - o[1]) - NEAR ? 1u << 6 : 0u);
+        const unsigned zs = (lz < NEAR ? 1u : 0u) | 1u << 9 | (lz >= min(TZ, nz - o[2]) - NEAR ? 1u << 18 : 0u);
         near |= xs * ys * zs;
     }
     near = __reduce_or_sync(full, near);

@@ -88,7 +88,9 @@ constexpr int TILE_CELLS = TILE * TILE * TILE;          // cells of every tile s
 // Tile shapes (cells per tile edge along x, y, z; 512 cells each).  A single
 // grid uses shape 0; a batch may use any (chosen by its autotuner).  Every
 // edge is at least 4 cells, more than the NEAR = 3 layers of the proximity
-// mask, so a marker can only touch its own tile and the 26 adjacent ones.
+// mask, so a marker touches its own tile and the 26 adjacent ones; across a last
+// tile clipped to fewer than NEAR cells it also touches the tile before that one
+// (see narrow_last).
 constexpr int N_TILE_SHAPES = 3;
 __host__ __device__ constexpr int tile_log2(int sh, int a) {
     return sh == 0 ? 3 : (sh == 1 ? (a == 0 ? 4 : (a == 1 ? 3 : 2)) : (a == 0 ? 5 : 2));
@@ -111,7 +113,8 @@ struct TileShape {
 // Tile proximity mask: bit near_bit(dx, dy, dz) is set when a marker owned by a
 // node of the tile lies within NEAR cells of the neighbour tile in direction
 // (dx, dy, dz) (the owner node in the NEAR layers next to that neighbour, along
-// every axis with a non-zero step); bit near_bit(0, 0, 0) whenever the tile
+// every axis with a non-zero step, counted from the tile's last cell inside the
+// grid where it is clipped); bit near_bit(0, 0, 0) whenever the tile
 // owns a marker.  A sweep changes a node's byte or edges only if a marker is
 // owned by a node within one cell behind or two cells ahead of it (the window of
 // the band pass), and Front2VOF reads a cell's corners one cell ahead, so a
@@ -119,21 +122,6 @@ struct TileShape {
 // neighbour owns a marker within three cells of it.
 constexpr int NEAR = 3;
 __host__ __device__ inline int near_bit(int dx, int dy, int dz) { return 9 * (dz + 1) + 3 * (dy + 1) + (dx + 1); }
-// (lx, ly, lz: the node's place in a tile of tx x ty x tz cells)
-__host__ __device__ inline unsigned near_bits(int lx, int ly, int lz, int tx = TILE, int ty = TILE, int tz = TILE) {
-    unsigned m = 0;
-    for (int dz = -1; dz <= 1; dz++) {
-        if ((dz < 0 && lz >= NEAR) || (dz > 0 && lz < tz - NEAR)) continue;
-        for (int dy = -1; dy <= 1; dy++) {
-            if ((dy < 0 && ly >= NEAR) || (dy > 0 && ly < ty - NEAR)) continue;
-            for (int dx = -1; dx <= 1; dx++) {
-                if ((dx < 0 && lx >= NEAR) || (dx > 0 && lx < tx - NEAR)) continue;
-                m |= 1u << near_bit(dx, dy, dz);
-            }
-        }
-    }
-    return m;
-}
 
 enum Counter { C_MARKERS = 0, C_ANNIHILATE = 1, C_MULTI = 2, C_INCONSISTENT = 3, C_CFL = 4, C_N = 5 };
 // extra device counters after the event counters (C_NONFINITE: markers whose
@@ -157,13 +145,13 @@ __host__ __device__ inline void grid_tiles(Grid &g, int sh) {
     }
 }
 
-// Does a tile reach past the grid on some axis?  The proximity masks measure from
-// the tile's edges, so across the seam behind such a clipped tile they can miss
-// the neighbour of a marker: that tile stays out of the band and keeps its old
-// colours, and an edge it owns may then carry a marker that no list names and
-// whose offset was written by no sweep.
-__host__ __device__ inline bool has_clipped_tiles(const Grid &g) {
-    return ((g.n[0] & ((1 << g.tl[0]) - 1)) | (g.n[1] & ((1 << g.tl[1]) - 1)) | (g.n[2] & ((1 << g.tl[2]) - 1))) != 0;
+// Is the last tile of axis a clipped to fewer than NEAR cells?  A marker in the
+// first layers of tile 0 then touches, behind it across the periodic seam, both
+// the last tile and the one before that: tile 0's step -1 stands for both.  (Ahead
+// a marker touches no node further than the next one, so step +1 names one tile
+// whatever its width.)
+__host__ __device__ inline bool narrow_last(const Grid &g, int a) {
+    return g.n[a] - ((g.td[a] - 1) << g.tl[a]) < NEAR;
 }
 
 __host__ __device__ inline int wrapc(int v, int n) {
@@ -206,17 +194,17 @@ __device__ __forceinline__ void warp_count(unsigned long long *ctr, unsigned v) 
 
 // Is tile (tx, ty, tz) in the band: does it own a marker, or does a neighbour
 // own one within NEAR cells of it (that neighbour's proximity bit toward it)?
-// (the 27 loads are independent: no early exit)
+// (the loads are independent: no early exit)
 __device__ __forceinline__ bool in_band(const Grid &g, const uint32_t *__restrict__ mask, int tx, int ty, int tz) {
+    // step 2: from the tile before a narrow last one to tile 0, whose step -1 names both
+    const int ex = narrow_last(g, 0) && tx == g.td[0] - 2 ? 2 : 1, ey = narrow_last(g, 1) && ty == g.td[1] - 2 ? 2 : 1,
+              ez = narrow_last(g, 2) && tz == g.td[2] - 2 ? 2 : 1;
     unsigned on = 0;
-#pragma unroll
-    for (int dz = -1; dz <= 1; dz++)
-#pragma unroll
-        for (int dy = -1; dy <= 1; dy++)
-#pragma unroll
-            for (int dx = -1; dx <= 1; dx++) {
+    for (int dz = -1; dz <= ez; dz++)
+        for (int dy = -1; dy <= ey; dy++)
+            for (int dx = -1; dx <= ex; dx++) {
                 const int nx = wrapc(tx + dx, g.td[0]), ny = wrapc(ty + dy, g.td[1]), nz = wrapc(tz + dz, g.td[2]);
-                on |= mask[(nz * g.td[1] + ny) * g.td[0] + nx] >> near_bit(-dx, -dy, -dz);
+                on |= mask[(nz * g.td[1] + ny) * g.td[0] + nx] >> near_bit(dx < 2 ? -dx : -1, dy < 2 ? -dy : -1, dz < 2 ? -dz : -1);
             }
     return on & 1u;
 }

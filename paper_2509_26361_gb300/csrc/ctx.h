@@ -77,7 +77,6 @@ struct ebit_ctx {
     unsigned *work2[NWORK];
     int *scan_count;          // [3] lengths of the marker lists of a whole-grid scan
     int scan_done;            // those lists describe the current state
-    int sparse_s;             // offsets of unmarked edges not taken in: 1 no sweep since, 2 one sweep, 0 all there
     int *wcount2;
     unsigned *mk_al[2];       // aligned edges that carry a marker, per set
     int *mk_count;            // [2] their lengths

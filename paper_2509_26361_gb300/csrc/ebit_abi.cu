@@ -79,7 +79,6 @@ int mark_all(ebit_ctx *ctx) {
     // the next sweep processes every tile and lists the markers and band anew
     ctx->mk_valid = 0;
     ctx->scan_done = 0;
-    ctx->sparse_s = 0;
     ctx->last_C = nullptr;
     ctx->last_kh = nullptr;
     ctx->last_st = nullptr;
@@ -119,15 +118,11 @@ int call_stream(ebit_ctx *ctx, int flags, cudaStream_t *st) {
 }
 
 // The colours into the other buffer: a sweep leaves the tiles outside its band
-// unwritten.  Offsets need no copy where tiles divide the grid: they are read
-// only on edges with a marker, and a sweep writes every marker's.  With clipped
-// tiles an edge outside the band may be read (has_clipped_tiles), so there both
-// buffers hold the state's.
+// unwritten.  Offsets need no copy: they are read only on edges with a marker,
+// and a sweep writes every marker's.
 int copy_other(ebit_ctx *ctx) {
     const int c = ctx->cur, o = c ^ 1;
     CU(cudaMemcpyAsync(ctx->cb[o], ctx->cb[c], ctx->N, cudaMemcpyDeviceToDevice, ctx->stream));
-    for (int a = 0; a < 3 && has_clipped_tiles(ctx->g); a++)
-        CU(cudaMemcpyAsync(ctx->s[o][a], ctx->s[c][a], ctx->N * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
     return EBIT_OK;
 }
 
@@ -260,7 +255,6 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
     ctx->mk_dir = 0;
     ctx->mk_valid = 0;
     ctx->scan_done = 0;
-    ctx->sparse_s = 0;
     ctx->iface[0] = ctx->iface[1] = nullptr;
     ctx->wcount = ctx->ncut = ctx->niface = ctx->nscan = ctx->zero = nullptr;
     ctx->cut = ctx->scan = nullptr;
@@ -504,7 +498,6 @@ int ebit_set_state(ebit_ctx *ctx, const uint8_t *cb, const double *s) {
         mark_scan_kernel<<<scan_grid(ctx), 256, 0, ctx->stream>>>(a);
         if (int r = launch_check(ctx, "mark_scan_kernel")) return r;
         ctx->scan_done = 1;
-        ctx->sparse_s = !ctx->dense && has_clipped_tiles(ctx->g) ? 1 : 0;
         return EBIT_OK;
     }
     CU(cudaMemcpyAsync(ctx->cb[c], cb, ctx->N, cudaMemcpyDefault, ctx->stream));
@@ -616,9 +609,7 @@ int ebit_unpack_bricks(ebit_ctx *ctx, int nbricks, const int *tiles, const uint8
                     ctx->stream>>>(ctx->g, ctx->amr_slot, cb, s, bg, ctx->cb[c], ctx->cb[c ^ 1], ctx->s[c][0],
                                    ctx->s[c][1], ctx->s[c][2]);
     if (int r = launch_check(ctx, "unpack_kernel")) return r;
-    if (int r = mark_all(ctx)) return r;
-    ctx->sparse_s = !ctx->dense && has_clipped_tiles(ctx->g) ? 1 : 0;
-    return EBIT_OK;
+    return mark_all(ctx);
 }
 
 int ebit_one_fluid(ebit_ctx *ctx, const double *C, const double *kappa_h, const uint8_t *status, double sigma,
@@ -695,19 +686,6 @@ int ebit_advect_sweep(ebit_ctx *ctx, int dir, const double *u_face, double dt) {
     if (ctx->f2v_pending && (ctx->cur ^ 1) == ctx->f2v_buf) {
         CU(cudaStreamWaitEvent(ctx->stream, ctx->ev_f2v, 0));
         ctx->f2v_pending = 0;
-    }
-    // After a state taken in with its markers' offsets only, the first sweep (over
-    // every tile) reads no other; before the second, on a grid with clipped tiles,
-    // both buffers get what a whole state has there.
-    if (ctx->sparse_s == 2) {
-        const int now = ctx->cur, was = now ^ 1;
-        settle_offsets_kernel<<<scan_grid(ctx), 256, 0, ctx->stream>>>(
-            ctx->g, ctx->cb[was], ctx->cb[now], (ctx->N + 7) & ~7LL, ctx->s[was][0], ctx->s[was][1], ctx->s[was][2],
-            ctx->s[now][0], ctx->s[now][1], ctx->s[now][2]);
-        if (int r = launch_check(ctx, "settle_offsets_kernel")) return r;
-        ctx->sparse_s = 0;
-    } else if (ctx->sparse_s == 1) {
-        ctx->sparse_s = 2;
     }
     const int rd = ctx->mk_par, wr = rd ^ 1;
     const bool lists = !ctx->dense && ctx->mk_valid;

@@ -13,9 +13,7 @@
 // A sweep is one cooperative launch that runs these phases over all instances,
 // separated by grid barriers:
 //   advect  -- each listed marker moved once (velocity interpolated); the band
-//              built from the previous sweep's list of tiles with markers nearby
-//              (instances with clipped tiles: the markers of their band tiles,
-//              found from the colours in a phase of its own);
+//              built from the previous sweep's list of tiles with markers nearby;
 //   sweep   -- per band tile: integer colour/aligned-edge pass (band.cuh), FP64
 //              lists, the marker and tile lists of the next sweep;
 //   fp64    -- the FP64 lists.
@@ -61,7 +59,6 @@ struct BatchParams {
     const int *coff;          // [n + 1] first cell of each instance
     const int *toff;          // [n + 1] first tile of each instance
     int n;
-    int clipped;              // some instance has clipped tiles
     const double *const *u;   // [n] velocity component of the sweep direction
     const double *lam;        // [n] dt / h
     unsigned long long *ctr;  // [n][C_TOTAL]
@@ -117,55 +114,6 @@ __device__ __forceinline__ int find_inst(const int *off, int n, int i) {
     return lo;
 }
 
-// The markers of a band tile from its colours, each moved once (64 threads).
-template <int D, int SH>
-__device__ __forceinline__ void move_tile_markers(const BatchParams &p, const Grid &g, int i, int base, int tile,
-                                                  BandSmem<D, SH> &sm, int bar) {
-    using R = BandRegion<D, SH>;
-    using M = typename BandSmem<D, SH>::M;
-    constexpr int TX = R::TX, TY = R::TY, RY = TY + 1, ROWS = RY * (R::TZ + 1);
-    static_assert(ROWS <= R::ROWS, "the rows fit the band pass's");
-    constexpr uint32_t MT = TX == 32 ? 0xFFFFFFFFu : (1u << (TX & 31)) - 1u;
-    const int tid = threadIdx.x & (BAND_THREADS - 1), lane = tid & 31, warp = tid >> 5;
-    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    const long long n = (long long)nx * ny * nz;
-    uint16_t *list = sm.list + (warp ? BandSmem<D, SH>::LIST1 : 0);
-    int o[3];
-    tile_origin(g, tile, o);
-    for (int r = tid; r < ROWS; r += BAND_THREADS) {
-        uint32_t f;
-        sm.C[r] = load_row<M, TX, 0, TX + 1>(p.a.cb + base, (wrapc(o[2] + r / RY, nz) * ny + wrapc(o[1] + r % RY, ny)) * nx,
-                                            o[0], nx, (n + 7) & ~7LL, n, 1, &f);
-    }
-    band_sync(bar);
-    const int ly = tid % TY, lz = tid / TY, y = o[1] + ly, z = o[2] + lz;
-    uint32_t m[3] = {0, 0, 0};
-    if (tid < R::CELL_ROWS && y < ny && z < nz) {
-        const uint32_t vx = nx - o[0] >= TX ? MT : (1u << (nx - o[0])) - 1u;
-        const M *c = sm.C + ly + RY * lz;
-        m[0] = (uint32_t)(c[0] ^ c[0] >> 1) & vx;
-        m[1] = (uint32_t)(c[0] ^ c[1]) & vx;
-        m[2] = (uint32_t)(c[0] ^ c[RY]) & vx;
-    }
-    unsigned hits = 0, bad = 0;
-#pragma unroll
-    for (int e = 0; e < 3; e++) {
-        unsigned total;
-        int at = (int)warp_prefix(__popc(m[e]), &total);
-        for (uint32_t w = m[e]; w; w &= w - 1) list[at++] = (uint16_t)(tid * 32 + __ffs((int)w) - 1);
-        __syncwarp();
-        for (int k = lane; k < (int)total; k += 32) {
-            const int c = list[k], r = c >> 5;
-            const int gid = base + ((o[2] + r / TY) * ny + o[1] + r % TY) * nx + o[0] + (c & 31);
-            move_marker<D>(p.a, g, base, p.u[i], p.lam[i], e, gid, hits, bad);
-        }
-        __syncwarp();
-    }
-    unsigned long long *ctr = p.ctr + (size_t)i * C_TOTAL;
-    if (hits) atomicAdd(ctr + C_CFL, (unsigned long long)hits);
-    if (bad) atomicAdd(ctr + C_NONFINITE, (unsigned long long)bad);
-}
-
 template <int D, int SH>
 __global__ void __launch_bounds__(BATCH_THREADS, 4) batch_sweep_kernel(BatchParams p) {
     constexpr int GROUPS = BATCH_THREADS / BAND_THREADS;
@@ -202,7 +150,6 @@ __global__ void __launch_bounds__(BATCH_THREADS, 4) batch_sweep_kernel(BatchPara
             const int j = t - (k == 0 ? 0 : (k == 1 ? n0 : n0 + n1));
             const int gid = (int)__ldg((k == 0 ? p.al : (k == 1 ? p.un0 : p.un1)) + j);
             const int i = find_inst(s_coff, p.n, gid);
-            if (p.clipped && has_clipped_tiles(p.grid[i])) continue;  // moved below
             unsigned hits = 0, bad = 0;
             move_marker<D>(p.a, p.grid[i], s_coff[i], p.u[i], p.lam[i], pd + k < 3 ? pd + k : pd + k - 3, gid, hits, bad);
             if (hits) atomicAdd(p.ctr + (size_t)i * C_TOTAL + C_CFL, 1ull);
@@ -211,21 +158,6 @@ __global__ void __launch_bounds__(BATCH_THREADS, 4) batch_sweep_kernel(BatchPara
     }
     if (!grid_barrier(p, &s_ok)) return;
     const int grp = threadIdx.x / BAND_THREADS;
-
-    // ---- instances with clipped tiles move what their band tiles' colours show,
-    // edges that no list names among them (has_clipped_tiles)
-    if (p.clipped) {
-        const int nb = __ldcg(p.rd + B_BAND);
-        for (int li = grp * gridDim.x + blockIdx.x; li < nb; li += gridDim.x * GROUPS) {
-            const int gt = __ldcg(p.band + li);
-            const int i = find_inst(s_toff, p.n, gt);
-            const Grid g = p.grid[i];
-            if (!has_clipped_tiles(g)) continue;
-            move_tile_markers<D, SH>(p, g, i, s_coff[i], gt - s_toff[i], s_band[grp], 1 + grp);
-            band_sync(1 + grp);
-        }
-        if (!grid_barrier(p, &s_ok)) return;
-    }
 
     // ---- integer band pass
     {
@@ -470,8 +402,6 @@ BatchParams sweep_params(const ebit_batch *b, int d, int parity) {
     p.coff = off_cells(b);
     p.toff = off_tiles(b);
     p.n = b->n;
-    p.clipped = 0;
-    for (const ebit_ctx *c : b->inst) p.clipped |= has_clipped_tiles(c->g) ? 1 : 0;
     p.u = b->u[d];
     p.lam = b->lam;
     p.ctr = b->ctr;

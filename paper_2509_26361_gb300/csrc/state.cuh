@@ -209,30 +209,6 @@ static __global__ void __launch_bounds__(256) state_out_kernel(Grid g, const uin
     }
 }
 
-// After the first sweep since a state was taken in with its markers' offsets
-// only (colours and offsets `was`; the sweep wrote those of its markers, `now`):
-// the other offsets of both buffers as if the whole state had been taken into
-// both, 0 on its unmarked edges.
-static __global__ void __launch_bounds__(256) settle_offsets_kernel(Grid g, const uint8_t *__restrict__ was,
-                                                                    const uint8_t *__restrict__ now, long long whole,
-                                                                    double *w0, double *w1, double *w2, double *n0,
-                                                                    double *n1, double *n2) {
-    const int gx = (g.n[0] + 7) / 8;
-    const long long groups = (long long)gx * g.n[1] * g.n[2], stride = (long long)gridDim.x * blockDim.x;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < groups; t += stride) {
-        const RowGroup a = row_group(g, was, whole, gx, t), b = row_group(g, now, whole, gx, t);
-#pragma unroll
-        for (int k = 0; k < 3; k++) {
-            double *w = (k == 0 ? w0 : (k == 1 ? w1 : w2)) + a.id, *v = (k == 0 ? n0 : (k == 1 ? n1 : n2)) + a.id;
-            for (int j = 0; j < a.cnt; j++) {
-                const bool old = (a.m[k] >> j) & 1u;
-                if (!((b.m[k] >> j) & 1u)) v[j] = old ? w[j] : 0.0;
-                if (!old) w[j] = 0.0;
-            }
-        }
-    }
-}
-
 // Every tile marked for the next sweep and Front2VOF, the lists of the sweeps
 // empty: the tables of a context after a state change (null where it has none).
 struct MarkAllArgs {

@@ -291,15 +291,25 @@ __device__ __forceinline__ void move_marker(const SweepArgs &a, const Grid &g, i
 
 // Band item b (a direction) of a listed tile of grid g (its tiles start at
 // tbase): the neighbour the tile's mask points to that way (bit
-// near_bit(dx, dy, dz)), listed once.
+// near_bit(dx, dy, dz)), listed once; from tile 0 backwards, past a narrow last
+// tile, also the one before it (along each such axis: up to eight tiles).
 __device__ __forceinline__ void band_item(const Grid &g, int tbase, int tile, int b, const uint32_t *__restrict__ mask,
                                           uint32_t *band_flag, int *band, int *band_count) {
     if (!((__ldg(mask + tbase + tile) >> b) & 1u)) return;
     const int tx = tile % g.td[0], ty = (tile / g.td[0]) % g.td[1], tz = tile / (g.td[0] * g.td[1]);
-    const int bx = wrapc(tx + b % 3 - 1, g.td[0]), by = wrapc(ty + (b / 3) % 3 - 1, g.td[1]),
-              bz = wrapc(tz + b / 9 - 1, g.td[2]);
-    const int nt = tbase + (bz * g.td[1] + by) * g.td[0] + bx;
-    if (atomicExch(band_flag + nt, 1u) == 0u) band[atomicAdd(band_count, 1)] = nt;
+    const int dx = b % 3 - 1, dy = (b / 3) % 3 - 1, dz = b / 9 - 1;
+    const int bx = wrapc(tx + dx, g.td[0]), by = wrapc(ty + dy, g.td[1]), bz = wrapc(tz + dz, g.td[2]);
+    const int ex = dx < 0 && tx == 0 && narrow_last(g, 0), ey = dy < 0 && ty == 0 && narrow_last(g, 1),
+              ez = dz < 0 && tz == 0 && narrow_last(g, 2);
+    auto take = [&](int x, int y, int z) {
+        const int nt = tbase + (z * g.td[1] + y) * g.td[0] + x;
+        if (atomicExch(band_flag + nt, 1u) == 0u) band[atomicAdd(band_count, 1)] = nt;
+    };
+    take(bx, by, bz);
+    if (ex | ey | ez)
+#pragma unroll 1
+        for (int k = 1; k < 8; k++)
+            if ((k & 1) <= ex && (k >> 1 & 1) <= ey && (k >> 2) <= ez) take(bx - (k & 1), by - (k >> 1 & 1), bz - (k >> 2));
 }
 
 // Advection from the marker lists (Eq. 2): one thread per marker, no tile
