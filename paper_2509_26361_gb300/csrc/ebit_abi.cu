@@ -2,8 +2,8 @@
 //
 // The context owns a double-buffered EBIT state (colour bytes + three FP64
 // offset arrays) and per-tile tables that keep every call on the active band:
-// a sweep processes the tiles whose 3x3x3 tile neighbourhood held a marker
-// before or after the previous sweep, Front2VOF the tiles swept since its last
+// a sweep processes the tiles within reach of a marker that was there before or
+// after the previous sweep (common.cuh), Front2VOF the tiles swept since its last
 // call, curvature the tiles around cells whose volume fraction was rewritten.
 // A tile outside the band provably holds no marker and is not changed by the
 // call, and both state buffers agree on it, so band processing gives the same
