@@ -241,12 +241,17 @@ __global__ void brick_slots_kernel(const int *__restrict__ tiles, int n, int nt,
 // The state from a brick store: bricks copied in, every other tile filled with
 // its colour (bg: bit 0), face colours equal to it.  Both state buffers get the
 // colours (a sweep leaves tiles outside its band unwritten); the offsets go to
-// the first only, and only the bricks' (an offset is read where its edge
-// carries a marker, and a sweep writes every marker's).  A warp takes 32 groups
+// the first only, and only where an edge may carry a marker (an offset is read
+// there only, and a sweep writes every marker's): the bricks', and 0 on the edges
+// into a brick from a tile outside the store whose colour differs (a packed store has
+// none: that tile would hold a refined cell; but any store may be unpacked, and the
+// context's old offsets must not show; background_seams has the edges between two
+// tiles outside it).  A warp takes 32 groups
 // of up to 8 cells in a row: a lane writes its group's colours, and the bricks'
 // offsets go in 16-byte pieces, lane after lane.  HBM bound: two bytes per cell
 // and the bricks.  (A lane per row of a brick, value by value: 68 us at 384^3;
-// this form 54.)
+// this form 54, with the edges into a brick 57.  A background lane's look at the next
+// tiles, or a kernel of its own for them, cost 12 us in place of 3.)
 __global__ void __launch_bounds__(256) unpack_kernel(Grid g, const int *__restrict__ slot, const uint8_t *__restrict__ in_cb,
                                                      const double *__restrict__ in_s, const uint8_t *__restrict__ bg,
                                                      uint8_t *__restrict__ cb, uint8_t *__restrict__ cb2,
@@ -269,6 +274,11 @@ __global__ void __launch_bounds__(256) unpack_kernel(Grid g, const int *__restri
             unsigned long long v = (bg[tile] & 1) ? 0x0F0F0F0F0F0F0F0Full : 0ull;
             if (k >= 0) {
                 const int c = (y & 7) + 8 * (z & 7);
+                // the tile behind along each axis in which this is its first layer
+                const int bx = tx ? tile - 1 : tile + g.td[0] - 1,
+                          by = (y & 7) ? tile : (y ? tile : tile + g.td[1] * g.td[0]) - g.td[0],
+                          bz = (z & 7) ? tile : (z ? tile : tile + g.ntiles) - g.td[1] * g.td[0];
+                const int kx = slot[bx], ky = slot[by], kz = slot[bz], cx = bg[bx], cy = bg[by], cz = bg[bz];
                 const uint8_t *bc = in_cb + (size_t)k * TILE_CELLS + c * 8;
                 row8 = k * 3 * (TILE_CELLS / 8) + c;
                 if (((uintptr_t)bc & 7) == 0) {
@@ -276,6 +286,12 @@ __global__ void __launch_bounds__(256) unpack_kernel(Grid g, const int *__restri
                 } else {
                     v = 0;
                     for (int j = 0; j < 8; j++) v |= (unsigned long long)__ldg(bc + j) << (8 * j);
+                }
+                if (kx < 0 && ((v ^ cx) & 1)) s0[id + (tx ? -1 : nx - 1)] = 0.0;
+                for (int j = 0; j < cnt && min(ky, kz) < 0; j++) {
+                    const int colour = (int)(v >> (8 * j));
+                    if (ky < 0 && ((colour ^ cy) & 1)) s1[id + j + (y ? -nx : (ny - 1) * nx)] = 0.0;
+                    if (kz < 0 && ((colour ^ cz) & 1)) s2[id + j + (z ? -ny * nx : (nz - 1) * ny * nx)] = 0.0;
                 }
             }
             if (cnt == 8 && (((uintptr_t)(cb + id) | (uintptr_t)(cb2 + id)) & 7) == 0) {

@@ -64,9 +64,16 @@ int blocks_for(long long n, int threads, int sms) {
     return (int)b;
 }
 
-int mark_all(ebit_ctx *ctx) {
+// bg: the background colours of a brick store just unpacked (null: none was)
+int mark_all(ebit_ctx *ctx, const uint8_t *bg = nullptr) {
     ctx->sweeps_since_f2v = 1;
     MarkAllArgs m;
+    if (bg) {
+        m.slot = ctx->amr_slot;
+        m.bg = bg;
+        m.g = ctx->g;
+        for (int k = 0; k < 3; k++) m.s[k] = ctx->s[ctx->cur][k];
+    }
     m.ntiles = ctx->g.ntiles;
     m.tile_marker = ctx->tile_marker;
     m.dirty = ctx->dirty_set ? ctx->tile_dirty2 : ctx->tile_dirty;
@@ -609,7 +616,7 @@ int ebit_unpack_bricks(ebit_ctx *ctx, int nbricks, const int *tiles, const uint8
                     ctx->stream>>>(ctx->g, ctx->amr_slot, cb, s, bg, ctx->cb[c], ctx->cb[c ^ 1], ctx->s[c][0],
                                    ctx->s[c][1], ctx->s[c][2]);
     if (int r = launch_check(ctx, "unpack_kernel")) return r;
-    return mark_all(ctx);
+    return mark_all(ctx, bg);
 }
 
 int ebit_one_fluid(ebit_ctx *ctx, const double *C, const double *kappa_h, const uint8_t *status, double sigma,

@@ -217,10 +217,38 @@ struct MarkAllArgs {
     uint8_t *dirty, *clean;  // the tile flags the next Front2VOF takes, and the other set
     uint32_t *band_flag;
     int *band_count, *scan_count;
+    // a brick store just unpacked (see background_seams; null otherwise)
+    const int *slot = nullptr;
+    const uint8_t *bg = nullptr;
+    Grid g;
+    double *s[3] = {nullptr, nullptr, nullptr};
 };
+
+// Offset 0 on the edges between tile t and the next tiles where neither is in the
+// brick store and their colours differ.
+static __device__ __noinline__ void background_seams(const MarkAllArgs &a, int t) {
+    const Grid &g = a.g;
+    int o[3];
+    tile_origin(g, t, o);
+    for (int d = 0; d < 3; d++) {
+        const int step = d == 0 ? 1 : (d == 1 ? g.td[0] : g.td[0] * g.td[1]);
+        const int td = d == 0 ? g.td[0] : (d == 1 ? g.td[1] : g.td[2]);
+        const int l = min(d == 0 ? o[0] + TILE : (d == 1 ? o[1] + TILE : o[2] + TILE), d == 0 ? g.n[0] : (d == 1 ? g.n[1] : g.n[2])) - 1;
+        const int nt = l + 1 == (d == 0 ? g.n[0] : (d == 1 ? g.n[1] : g.n[2])) ? t - (td - 1) * step : t + step;
+        if (a.slot[nt] >= 0 || ((a.bg[nt] ^ a.bg[t]) & 1) == 0) continue;
+        for (int k = 0; k < TILE * TILE; k++) {
+            const int i = k & 7, j = k >> 3;
+            const int x = d == 0 ? l : o[0] + i, y = d == 1 ? l : o[1] + (d == 0 ? i : j), z = d == 2 ? l : o[2] + j;
+            if (x >= g.n[0] || y >= g.n[1] || z >= g.n[2]) continue;
+            (d == 0 ? a.s[0] : d == 1 ? a.s[1] : a.s[2])[((long long)z * g.n[1] + y) * g.n[0] + x] = 0.0;
+        }
+    }
+}
+
 static __global__ void mark_all_kernel(MarkAllArgs a) {
     const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
     for (int t = t0; t < a.ntiles; t += gridDim.x * blockDim.x) {
+        if (a.slot && a.slot[t] < 0) background_seams(a, t);
         a.tile_marker[t] = 0xFFFFFFFFu;
         a.dirty[t] = 1;
         if (a.clean) a.clean[t] = 0;
