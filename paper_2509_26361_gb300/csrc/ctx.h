@@ -77,6 +77,8 @@ struct ebit_ctx {
     unsigned *work2[NWORK];
     int *scan_count;          // [3] lengths of the marker lists of a whole-grid scan
     int scan_done;            // those lists describe the current state
+    unsigned long long scan_capture;  // the capture that the scan was recorded into (0: it ran)
+    int scan_clear;           // a replay may have left their lengths: cleared before every scan
     int *wcount2;
     unsigned *mk_al[2];       // aligned edges that carry a marker, per set
     int *mk_count;            // [2] their lengths

@@ -262,6 +262,8 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
     ctx->mk_dir = 0;
     ctx->mk_valid = 0;
     ctx->scan_done = 0;
+    ctx->scan_capture = 0;
+    ctx->scan_clear = 0;
     ctx->iface[0] = ctx->iface[1] = nullptr;
     ctx->wcount = ctx->ncut = ctx->niface = ctx->nscan = ctx->zero = nullptr;
     ctx->cut = ctx->scan = nullptr;
@@ -505,6 +507,8 @@ int ebit_set_state(ebit_ctx *ctx, const uint8_t *cb, const double *s) {
         mark_scan_kernel<<<scan_grid(ctx), 256, 0, ctx->stream>>>(a);
         if (int r = launch_check(ctx, "mark_scan_kernel")) return r;
         ctx->scan_done = 1;
+        ctx->scan_capture = capture_id(ctx->stream);
+        if (ctx->scan_capture) ctx->scan_clear = 1;
         return EBIT_OK;
     }
     CU(cudaMemcpyAsync(ctx->cb[c], cb, ctx->N, cudaMemcpyDefault, ctx->stream));
@@ -756,7 +760,14 @@ int ebit_advect_sweep(ebit_ctx *ctx, int dir, const double *u_face, double dt) {
         ml.band = nullptr;
         ml.band_count = nullptr;
         a.scan_count = ctx->scan_count;
+        if (ctx->scan_done && ctx->scan_capture != capture_id(ctx->stream)) {
+            // ebit_set_state listed the markers outside the graph this sweep goes
+            // into (or inside one this sweep is not part of): a replay needs its own
+            ctx->scan_done = 0;
+            ctx->scan_clear = 1;
+        }
         if (!ctx->scan_done) {
+            if (ctx->scan_clear) CU(cudaMemsetAsync(ctx->scan_count, 0, 3 * sizeof(int), ctx->stream));
             ProfScope ps(ctx, EBIT_PROF_ADVECT);
             int r = launched(ctx, launch_pdl(mark_scan_kernel, scan_grid(ctx), 256, 0, ctx->stream, scan_args(ctx)),
                              "mark_scan_kernel");

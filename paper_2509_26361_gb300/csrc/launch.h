@@ -24,4 +24,13 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t sme
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// The id of the capture that a stream's work is recorded into (0: it runs).  Work
+// that a replay repeats must not lean on lists that were made outside its graph.
+inline unsigned long long capture_id(cudaStream_t st) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) cudaGetLastError();
+    return status == cudaStreamCaptureStatusActive ? id : 0;
+}
+
 }  // namespace ebit

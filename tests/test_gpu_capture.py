@@ -1,0 +1,73 @@
+"""Sweeps a caller captures into a CUDA graph of its own: every replay advances
+the state that is there when it runs, also where a state was taken in before the
+capture or is replaced between replays; compared to the last bit with the same
+calls made directly."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2509_26361_gb300 import ebit
+from paper_2509_26361_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def problem(n3, seed):
+    """A state of spheres (taken from an initialised context) and a velocity field."""
+    rng = np.random.default_rng(seed)
+    sp = [W.Sphere(tuple(rng.uniform(0.2, 0.8, 3)), rng.uniform(0.12, 0.22)) for _ in range(3)]
+    phi, faces = W.sphere_phi_nodes_faces(n3, sp)
+    g = ebit.Grid(*n3)
+    g.init(dev(phi), dev(faces))
+    st = g.get_state()
+    g.close()
+    return st, tuple(dev(a) for a in W.fourier_velocity(n3, rng))
+
+
+def direct(n3, st, u, pairs):
+    g = ebit.Grid(*n3, dense=True)
+    g.set_state(*st)
+    for n in range(2 * pairs):
+        g.step(n, u, 0.4 * g.h)
+    out = g.get_state()
+    g.close()
+    return out
+
+
+@pytest.mark.parametrize("within", [False, True])
+@pytest.mark.parametrize("dense", [False, True])
+def test_steps_captured_after_a_state_was_taken_in(dense, within):
+    """The state set on the device before the capture (each replay goes on from
+    the one before), or within it (each replay starts from it again)."""
+    n3 = (24, 33, 40)
+    st, u = problem(n3, 3)
+    ref = [direct(n3, st, u, k) for k in (1, 2, 3)]
+    side = torch.cuda.Stream()
+    g = ebit.Grid(*n3, stream=side, dense=dense)
+    g.set_state(*st)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        if within:
+            g.set_state(*st)
+        g.step(0, u, 0.4 * g.h)
+        g.step(1, u, 0.4 * g.h)
+    for k in range(3):
+        with torch.cuda.stream(side):
+            graph.replay()
+        torch.cuda.synchronize()
+        cb, s = g.get_state()
+        want = ref[0 if within else k]
+        assert torch.equal(cb, want[0]) and torch.equal(s, want[1]), k
+    # and directly again, the state set anew
+    g.set_state(*st)
+    g.step(0, u, 0.4 * g.h)
+    g.step(1, u, 0.4 * g.h)
+    cb, s = g.get_state()
+    assert torch.equal(cb, ref[0][0]) and torch.equal(s, ref[0][1])
+    del graph
+    g.close()
