@@ -40,6 +40,7 @@
 #include "../../include/ebit.h"
 #include "common.cuh"
 #include "ctx.h"
+#include "launch.h"
 #include "state.cuh"
 #include "sweep.cuh"
 #include "tc.cuh"
@@ -328,6 +329,8 @@ struct ebit_batch {
     int occ[N_TILE_SHAPES][3] = {};  // co-resident blocks per SM of each shape's and direction's kernel
     int ctas_per_sm = 1;           // chosen launch shape (autotuned)
     int shape = 0;                 // tile shape (autotuned)
+    unsigned long long lists_capture = 0;  // the capture that the lists were last made or used in (0: none)
+    int own_capture = 0;           // ebit_batch_run is capturing its graph
     int tiles_cap = 0;             // tiles the tile tables hold (the largest total over the shapes)
     // CUDA graph of two steps (even: x y z, odd: z y x)
     cudaGraph_t graph = nullptr;
@@ -435,9 +438,14 @@ int upload_layout(ebit_batch *b) {
 }
 
 // Before a sweep (or a graph of them): if any instance's state was changed
-// since the last one, the lists of the current set from the state.
+// since the last one, the lists of the current set from the state.  Also before the
+// first sweep that a caller captures, whose replays may follow a change, and before
+// the first one after that (what was captured did not run).
 int ensure_lists(ebit_batch *b) {
-    bool valid = true;
+    if (b->own_capture) return EBIT_OK;  // made before it
+    const unsigned long long id = capture_id(b->stream);
+    bool valid = id == b->lists_capture;
+    b->lists_capture = id;
     for (const ebit_ctx *c : b->inst) valid = valid && c->mk_valid;
     if (valid) return EBIT_OK;
     const int rd = b->parity;
@@ -832,8 +840,10 @@ int ebit_batch_run(ebit_batch *b, int first_step, int steps, int use_graph) {
             std::string why;
             cudaGraph_t g = nullptr;
             if (cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+                b->own_capture = 1;
                 int r = one_step(0);
                 if (r == EBIT_OK) r = one_step(1);
+                b->own_capture = 0;
                 cudaError_t e = cudaStreamEndCapture(b->stream, &g);
                 if (r != EBIT_OK || e != cudaSuccess) {
                     why = "capture: " + (r != EBIT_OK ? b->errmsg : std::string(cudaGetErrorString(e)));

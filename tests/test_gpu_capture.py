@@ -71,3 +71,48 @@ def test_steps_captured_after_a_state_was_taken_in(dense, within):
     assert torch.equal(cb, ref[0][0]) and torch.equal(s, ref[0][1])
     del graph
     g.close()
+
+
+def test_batch_sweeps_captured_by_the_caller():
+    sizes = [(24, 16, 32), (32, 24, 16)]
+    first, second = [problem(n3, 5 + i) for i, n3 in enumerate(sizes)], [problem(n3, 15 + i) for i, n3 in enumerate(sizes)]
+    side = torch.cuda.Stream()
+    b = ebit.Batch(sizes, stream=side)
+    for i in range(2):
+        b.instance(i).set_state(*first[i][0])
+    b.set_velocity([u for _, u in first], [0.4 / n3[0] for n3 in sizes])
+    b.run(0, 2, graph=False)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        for d in (0, 1, 2, 2, 1, 0):
+            b.sweep(d)
+
+    def replay(times):
+        with torch.cuda.stream(side):
+            for _ in range(times):
+                graph.replay()
+        b.sync()
+
+    replay(2)
+    start = [first[0][0], first[1][0]]
+    pairs = [3, 3]
+    for turn in range(2):
+        for i, n3 in enumerate(sizes):
+            cb, s = b.instance(i).get_state()
+            want = direct(n3, start[i], first[i][1], pairs[i])
+            assert torch.equal(cb, want[0]) and torch.equal(s, want[1]), (turn, i)
+        if turn == 0:  # one instance's state replaced, the same graph again
+            start[1], pairs = second[1][0], [4, 1]
+            b.instance(1).set_state(*start[1])
+            torch.cuda.synchronize()
+            replay(1)
+    # and directly from there
+    b.run(0, 2, graph=False)
+    b.sync()
+    for i, n3 in enumerate(sizes):
+        cb, s = b.instance(i).get_state()
+        want = direct(n3, start[i], first[i][1], pairs[i] + 1)
+        assert torch.equal(cb, want[0]) and torch.equal(s, want[1]), i
+    del graph
+    b.close()
