@@ -133,6 +133,17 @@ int copy_other(ebit_ctx *ctx) {
     return EBIT_OK;
 }
 
+// The list length a Front2VOF or curvature call appends to is 0: the call before
+// cleared it.  In a graph the calls before are those of the replay before, which need
+// not have used the other slots, and the list would grow past its end replay by
+// replay: a captured call clears its own, and so does every later one of the context.
+int clear_length(ebit_ctx *ctx, int *length, cudaStream_t st) {
+    if (!ctx->captured && !capture_id(st)) return EBIT_OK;
+    ctx->captured = 1;
+    CU(cudaMemsetAsync(length, 0, sizeof(int), st));
+    return EBIT_OK;
+}
+
 // Is p memory that this device's kernels may access as T?
 template <typename T>
 bool on_device(const T *p) {
@@ -267,6 +278,7 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
     ctx->iface[0] = ctx->iface[1] = nullptr;
     ctx->wcount = ctx->ncut = ctx->niface = ctx->nscan = ctx->zero = nullptr;
     ctx->cut = ctx->scan = nullptr;
+    ctx->captured = 0;
     ctx->cur_if = 0;
     ctx->if_slot = 0;
     ctx->band_last = -1;
@@ -817,6 +829,7 @@ int ebit_front2vof(ebit_ctx *ctx, double *C, int flags) {
     // ncut[fp] is 0: the previous call cleared it (the readers of that slot, the
     // Front2VOF before and its curvature, were complete then)
     const int fp = ctx->f2v_par ^ 1;
+    if (int r = clear_length(ctx, ctx->ncut + fp, st)) return r;
     a.ncut = ctx->ncut + fp;
     a.zero = ctx->ncut + (fp ^ 1);
     a.bad = ctx->ctr + C_F2V_BAD;
@@ -866,6 +879,7 @@ int ebit_curvature(ebit_ctx *ctx, const double *C, double *kappa_h, uint8_t *sta
     // slot cprev, and clears slot cnext (last read by the previous call) for
     // the next call
     const int cs = ctx->if_slot, cnext = (cs + 1) % 3, cprev = (cs + 2) % 3;
+    if (int r = clear_length(ctx, ctx->niface + cs, st)) return r;
     HFArgs a;
     a.g = ctx->g;
     a.C = C;

@@ -116,3 +116,61 @@ def test_batch_sweeps_captured_by_the_caller():
         assert torch.equal(cb, want[0]) and torch.equal(s, want[1]), i
     del graph
     b.close()
+
+
+@pytest.mark.parametrize("flags", [ebit.EBIT_FULL, ebit.EBIT_INCREMENTAL])
+@pytest.mark.parametrize("density", [0.02, 0.5])
+def test_fractions_and_curvature_captured_once(density, flags):
+    """One Front2VOF and one curvature call in a graph, replayed: the lists of cut
+    and interface cells are the replay's own (with random colours nearly every cell
+    is cut, so that two replays' cells would not fit them)."""
+    n3 = (24, 16, 40)
+    rng = np.random.default_rng(2)
+    c = (rng.uniform(size=n3[::-1]) < density).astype(np.uint8)
+    cb, s = dev(15 * c), dev(rng.uniform(size=(3,) + c.shape))
+    u = tuple(dev(a) for a in W.fourier_velocity(n3, rng))
+
+    def arrays():
+        C = torch.zeros(c.shape, dtype=torch.float64, device="cuda")
+        return C, torch.zeros_like(C), torch.zeros(c.shape, dtype=torch.uint8, device="cuda")
+
+    d = ebit.Grid(*n3)
+    d.set_state(cb, s)
+    want, refs = arrays(), []
+    for k in range(5):
+        d.step(0, u, 0.2 * d.h)
+        d.step(1, u, 0.2 * d.h)
+        d.front2vof(want[0], ebit.EBIT_FULL)
+        d.curvature(*want, flags=ebit.EBIT_FULL)
+        refs.append([t.clone() for t in want])
+    side = torch.cuda.Stream()
+    g = ebit.Grid(*n3, stream=side)
+    g.set_state(cb, s)
+    out = arrays()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        g.step(0, u, 0.2 * g.h)
+        g.step(1, u, 0.2 * g.h)
+        g.front2vof(out[0])
+        g.curvature(*out)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        g.step(0, u, 0.2 * g.h)
+        g.step(1, u, 0.2 * g.h)
+        g.front2vof(out[0], flags)
+        g.curvature(*out, flags=ebit.EBIT_FULL)
+    for k in range(5):
+        if k in (1, 2, 3):
+            with torch.cuda.stream(side):
+                graph.replay()
+        elif k == 4:  # and directly again
+            g.step(0, u, 0.2 * g.h)
+            g.step(1, u, 0.2 * g.h)
+            g.front2vof(out[0])
+            g.curvature(*out)
+        torch.cuda.synchronize()
+        for a, b in zip(out, refs[k]):
+            assert torch.equal(a, b), k
+    del graph
+    d.close()
+    g.close()
