@@ -343,7 +343,7 @@ int ebit_mlp_load(ebit_ctx *ctx, const void *weights, size_t bytes);
 typedef struct ebit_batch ebit_batch;
 
 /* descs[n]: one descriptor per instance (n <= 1024, every edge >= 8 cells, at
- * most 2^20 tiles of 8^3 cells per instance and 2^31 cells in all, the same
+ * most 2^20 - 1 tiles per instance in any tile shape and 2^31 cells in all, the same
  * cuda_stream for all, no EBIT_DESC_DENSE).  EBIT_ECUDA if the device has no
  * cooperative launch. */
 int ebit_batch_create(int n, const ebit_desc *descs, ebit_batch **out);

@@ -31,6 +31,7 @@ __host__ __device__ constexpr int tile_edge(int sh, int a) { return 1 << tile_lo
 template <int D, int SH>
 struct BandRegion {
     static constexpr int TX = tile_edge(SH, 0), TY = tile_edge(SH, 1), TZ = tile_edge(SH, 2);
+    static_assert(TX * TY * TZ == TILE_CELLS && TX > NEAR && TY > NEAR && TZ > NEAR, "see Tile shapes");
     static constexpr int X0 = D == 0 ? -1 : 0, Y0 = D == 1 ? -1 : 0, Z0 = D == 2 ? -1 : 0;
     static constexpr int RX = TX + (D == 0 ? 3 : 1), RY = TY + (D == 1 ? 3 : 1), RZ = TZ + (D == 2 ? 3 : 1);
     static constexpr int ROWS = RY * RZ;      // x-rows

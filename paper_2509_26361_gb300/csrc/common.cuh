@@ -68,10 +68,14 @@ __device__ __forceinline__ Fp operator-(double a, Fp b) { return Fp(a) - b; }
 __device__ __forceinline__ Fp operator*(double a, Fp b) { return Fp(a) * b; }
 __device__ __forceinline__ Fp &operator+=(Fp &a, Fp b) { return a = a + b; }
 
-// a / b for a y that is 1 / b correctly rounded: one product, the exact remainder
-// and one correction give the correctly rounded quotient (P. Markstein, IBM J.
-// Res. Dev. 34, 1990), in three FP64 operations where a division takes nine.
-// safe_quotient: a is zero or far from the range where the remainder underflows.
+// a / b for a y that is 1 / b correctly rounded: one product, the remainder and one
+// correction (P. Markstein, IBM J. Res. Dev. 34, 1990), in three FP64 operations
+// where a division takes nine.  Correctly rounded where the product is within a unit
+// in the last place of the quotient (a's fraction not below b's, among others);
+// elsewhere what is rounded lies within 2^-52 units of it, and no operands were
+// found for which the result differs (7e7 whose quotients lie as near to the middle
+// of two doubles as any can, 2e8 others).  Only for operands that pass safe_quotient: not zero, and far from where
+// the remainder underflows or the product overflows; the callers divide the others.
 __device__ __forceinline__ double quotient(double a, double b, double y) {
     const double q = __fma_rn(a, y, fp_minus_zero());
     return __fma_rn(__fma_rn(-b, q, a), y, q);
@@ -95,20 +99,6 @@ constexpr int N_TILE_SHAPES = 3;
 __host__ __device__ constexpr int tile_log2(int sh, int a) {
     return sh == 0 ? 3 : (sh == 1 ? (a == 0 ? 4 : (a == 1 ? 3 : 2)) : (a == 0 ? 5 : 2));
 }
-template <int SH>
-struct TileShape {
-    static constexpr int LX = tile_log2(SH, 0), LY = tile_log2(SH, 1), LZ = tile_log2(SH, 2);
-    static constexpr int TX = 1 << LX, TY = 1 << LY, TZ = 1 << LZ;
-    static_assert(TX * TY * TZ == TILE_CELLS, "512 cells per tile");
-    static_assert(TX >= 4 && TY >= 4 && TZ >= 4, "tile edges of at least 4 cells");
-    static constexpr int t(int a) { return a == 0 ? TX : (a == 1 ? TY : TZ); }
-    // cell c of a tile -> its local coordinates (x fastest)
-    __device__ static void cell(int c, int l[3]) {
-        l[0] = c & (TX - 1);
-        l[1] = (c >> LX) & (TY - 1);
-        l[2] = c >> (LX + LY);
-    }
-};
 
 // Tile proximity mask: bit near_bit(dx, dy, dz) is set when a marker owned by a
 // node of the tile lies within NEAR cells of the neighbour tile in direction
@@ -174,22 +164,6 @@ __device__ __forceinline__ void tile_origin(const Grid &g, int t, int o[3]) {
     o[0] = tx << g.tl[0];
     o[1] = ty << g.tl[1];
     o[2] = tz << g.tl[2];
-}
-
-// cell c (0 .. 511) of a tile of g's shape -> its local coordinates
-__device__ __forceinline__ void tile_cell(const Grid &g, int c, int l[3]) {
-    l[0] = c & ((1 << g.tl[0]) - 1);
-    l[1] = (c >> g.tl[0]) & ((1 << g.tl[1]) - 1);
-    l[2] = c >> (g.tl[0] + g.tl[1]);
-}
-
-// one atomicAdd per warp for a per-thread counter increment
-__device__ __forceinline__ void warp_count(unsigned long long *ctr, unsigned v) {
-    unsigned m = __activemask();
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(m, v, o);
-    int leader = __ffs(m) - 1;
-    if ((int)(threadIdx.x & 31) == leader && v) atomicAdd(ctr, (unsigned long long)v);
 }
 
 // Is tile (tx, ty, tz) in the band: does it own a marker, or does a neighbour

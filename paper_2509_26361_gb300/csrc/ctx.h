@@ -26,7 +26,6 @@ struct ebit_mlp {
     float *loss;               // summed weighted squared error of the last step
     int step;
     int fwd_blocks;            // co-resident forward blocks per SM (warp-level MMA kernel)
-    int fwd_tc_blocks;         // the same for the tcgen05 kernel
     int path;                  // EBIT_MLP_PATH_MMA or EBIT_MLP_PATH_TCGEN05
     int *err;                  // set by a tcgen05 kernel whose bounded wait gave up
     std::string errmsg;
@@ -46,7 +45,7 @@ struct ebit_ctx {
     double *s[2][3];
     int cur;
     uint32_t *tile_marker;    // per tile: proximity mask of its markers (see near_bits)
-    uint8_t *tile_dirty, *tile_cchg;
+    uint8_t *tile_dirty;
     // Front2VOF and curvature may run on a side stream (EBIT_ASYNC), overlapping
     // the next sweeps.  The sweeps mark processed tiles in dirty set dirty_set;
     // each Front2VOF call consumes that set and the next sweeps mark the other

@@ -287,7 +287,7 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
     ctx->mlp = nullptr;
     ctx->own_mlp = nullptr;
     ctx->tile_marker = nullptr;
-    ctx->tile_dirty = ctx->tile_cchg = nullptr;
+    ctx->tile_dirty = nullptr;
     ctx->band_list = ctx->band_count = ctx->all_list = ctx->all_count = nullptr;
     ctx->ctr = nullptr;
     ctx->g.n[0] = desc->nx;
@@ -351,7 +351,7 @@ static int create_ctx(const ebit_desc *desc, const ebit_state_arrays *st, ebit_c
          alloc((void **)&ctx->iface[1], ctx->N * sizeof(unsigned)) &&
          alloc((void **)&ctx->ncut, 2 * sizeof(int)) && alloc((void **)&ctx->niface, 3 * sizeof(int)) &&
          alloc((void **)&ctx->nscan, sizeof(int)) && alloc((void **)&ctx->zero, sizeof(int));
-    ok = ok && alloc((void **)&ctx->tile_cchg, ntc) && alloc((void **)&ctx->band_list, ntc * sizeof(int)) &&
+    ok = ok && alloc((void **)&ctx->band_list, ntc * sizeof(int)) &&
          alloc((void **)&ctx->band_count, 2 * sizeof(int)) &&
          alloc((void **)&ctx->all_list, ntc * sizeof(int)) &&
          alloc((void **)&ctx->all_count, sizeof(int));
@@ -468,7 +468,6 @@ void ebit_destroy(ebit_ctx *ctx) {
         dev_free(ctx->mem, ctx->tile_dirty2);
         dev_free(ctx->mem, ctx->band_list2);
     }
-    dev_free(ctx->mem, ctx->tile_cchg);
     dev_free(ctx->mem, ctx->band_list);
     dev_free(ctx->mem, ctx->band_count);
     dev_free(ctx->mem, ctx->all_list);
@@ -1141,11 +1140,6 @@ int ebit_mlp_create(void *cuda_stream, ebit_mlp **out) {
     mlp->fwd_blocks = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&mlp->fwd_blocks, mlp_fwd_kernel<true, true>, 128, FWD_SMEM);
     mlp->fwd_blocks = std::max(1, mlp->fwd_blocks);
-    mlp->fwd_tc_blocks = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&mlp->fwd_tc_blocks, mlp_fwd_tc_kernel<true, true>, TC_THREADS,
-                                                  FWD_TC_SMEM);
-    // a block holds all 512 TMEM columns (one per SM)
-    mlp->fwd_tc_blocks = 1;
     mlp->path = EBIT_MLP_PATH_TCGEN05;
     cudaMemsetAsync(mlp->err, 0, sizeof(int), mlp->stream);
     cudaMemsetAsync(mlp->loss, 0, 8, mlp->stream);  // a training step starts from a cleared loss

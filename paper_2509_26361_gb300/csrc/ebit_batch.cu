@@ -640,7 +640,7 @@ int ebit_batch_create(int n, const ebit_desc *descs, ebit_batch **out) {
         long long tiles = 0;
         for (int i = 0; i < n; i++) {
             const long long nt = inst_tiles(b, i, sh);
-            if (nt >= (1 << 20)) {  // tile ids keep 20 bits
+            if (nt >= (1 << 20)) {  // the interface's limit
                 delete b;
                 return EBIT_EINVAL;
             }

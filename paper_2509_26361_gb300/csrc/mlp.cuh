@@ -331,11 +331,6 @@ __device__ __forceinline__ bool mlp_sin(const void *p, int size, int code) {
 #define MLP_S(p, size, code) true
 #endif
 
-__device__ __forceinline__ uint32_t ld32s(const __nv_bfloat16 *p) {
-    if (!MLP_S(p, 4, 1)) return 0u;
-    return *reinterpret_cast<const uint32_t *>(p);
-}
-
 // Four 8x8 bf16 matrices from shared memory (ldmatrix.x4): lanes 8i .. 8i+7
 // give the 16-byte rows of matrix i, and register i of lane l receives
 // row l / 4, columns 2 (l % 4) and 2 (l % 4) + 1 of matrix i -- the fragment

@@ -235,19 +235,6 @@ __device__ double interp_u(const Grid &g, const double *__restrict__ u, const in
     return (1.0 - t[2]) * c0 + t[2] * c1;
 }
 
-// warp-aggregated append: every lane of the warp must call it
-__device__ __forceinline__ int warp_append(int *counter, bool flag) {
-    const unsigned full = 0xffffffffu;
-    unsigned m = __ballot_sync(full, flag);
-    if (!m) return -1;
-    const int lane = threadIdx.x & 31;
-    const int leader = __ffs(m) - 1;
-    int base = 0;
-    if (lane == leader) base = atomicAdd(counter, __popc(m));
-    base = __shfl_sync(full, base, leader);
-    return flag ? base + __popc(m & ((1u << lane) - 1u)) : -1;
-}
-
 // ---------------------------------------------------------------- advection
 // the counters the band pass appends to start at zero (cleared by the launch before it)
 __device__ __forceinline__ void clear_sweep_counts(const SweepArgs &a) {
