@@ -288,11 +288,11 @@ __global__ void __launch_bounds__(256) unpack_kernel(Grid g, const int *__restri
                     for (int j = 0; j < 8; j++) v |= (unsigned long long)__ldg(bc + j) << (8 * j);
                 }
                 if (kx < 0 && ((v ^ cx) & 1)) s0[id + (tx ? -1 : nx - 1)] = 0.0;
-                for (int j = 0; j < cnt && min(ky, kz) < 0; j++) {
-                    const int colour = (int)(v >> (8 * j));
-                    if (ky < 0 && ((colour ^ cy) & 1)) s1[id + j + (y ? -nx : (ny - 1) * nx)] = 0.0;
-                    if (kz < 0 && ((colour ^ cz) & 1)) s2[id + j + (z ? -ny * nx : (nz - 1) * ny * nx)] = 0.0;
-                }
+                const unsigned colours = gather_bits(v), ok = (1u << cnt) - 1u;
+                for (unsigned m = ky < 0 ? (colours ^ (cy & 1 ? 0xFFu : 0u)) & ok : 0u; m; m &= m - 1)
+                    s1[id + __ffs((int)m) - 1 + (y ? -nx : (ny - 1) * nx)] = 0.0;
+                for (unsigned m = kz < 0 ? (colours ^ (cz & 1 ? 0xFFu : 0u)) & ok : 0u; m; m &= m - 1)
+                    s2[id + __ffs((int)m) - 1 + (z ? -ny * nx : (nz - 1) * ny * nx)] = 0.0;
             }
             if (cnt == 8 && (((uintptr_t)(cb + id) | (uintptr_t)(cb2 + id)) & 7) == 0) {
                 *reinterpret_cast<unsigned long long *>(cb + id) = v;

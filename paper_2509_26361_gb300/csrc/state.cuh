@@ -224,31 +224,39 @@ struct MarkAllArgs {
     double *s[3] = {nullptr, nullptr, nullptr};
 };
 
-// Offset 0 on the edges between tile t and the next tiles where neither is in the
-// brick store and their colours differ.
-static __device__ __noinline__ void background_seams(const MarkAllArgs &a, int t) {
-    const Grid &g = a.g;
+// Offset 0 on the edges between tile t and the next one along axis d (neither in the
+// brick store, their colours differ).
+static __device__ __noinline__ void background_seam(const Grid &g, int t, int d, double *s) {
     int o[3];
     tile_origin(g, t, o);
-    for (int d = 0; d < 3; d++) {
-        const int step = d == 0 ? 1 : (d == 1 ? g.td[0] : g.td[0] * g.td[1]);
-        const int td = d == 0 ? g.td[0] : (d == 1 ? g.td[1] : g.td[2]);
-        const int l = min(d == 0 ? o[0] + TILE : (d == 1 ? o[1] + TILE : o[2] + TILE), d == 0 ? g.n[0] : (d == 1 ? g.n[1] : g.n[2])) - 1;
-        const int nt = l + 1 == (d == 0 ? g.n[0] : (d == 1 ? g.n[1] : g.n[2])) ? t - (td - 1) * step : t + step;
-        if (a.slot[nt] >= 0 || ((a.bg[nt] ^ a.bg[t]) & 1) == 0) continue;
-        for (int k = 0; k < TILE * TILE; k++) {
-            const int i = k & 7, j = k >> 3;
-            const int x = d == 0 ? l : o[0] + i, y = d == 1 ? l : o[1] + (d == 0 ? i : j), z = d == 2 ? l : o[2] + j;
-            if (x >= g.n[0] || y >= g.n[1] || z >= g.n[2]) continue;
-            (d == 0 ? a.s[0] : d == 1 ? a.s[1] : a.s[2])[((long long)z * g.n[1] + y) * g.n[0] + x] = 0.0;
-        }
+    const int l0 = min(o[0] + TILE, g.n[0]) - 1, l1 = min(o[1] + TILE, g.n[1]) - 1, l2 = min(o[2] + TILE, g.n[2]) - 1;
+    for (int k = 0; k < TILE * TILE; k++) {
+        const int i = k & 7, j = k >> 3;
+        const int x = d == 0 ? l0 : o[0] + i, y = d == 1 ? l1 : o[1] + (d == 0 ? i : j), z = d == 2 ? l2 : o[2] + j;
+        if (x <= l0 && y <= l1 && z <= l2) s[((long long)z * g.n[1] + y) * g.n[0] + x] = 0.0;
     }
+}
+static __device__ __forceinline__ void background_seams(const MarkAllArgs &a, int t) {
+    const int sy = a.g.td[0], sz = a.g.td[0] * a.g.td[1];
+    const int tx = t % sy, r = t / sy, ty = r % a.g.td[1], tz = r / a.g.td[1];
+    const int next[3] = {tx + 1 < a.g.td[0] ? t + 1 : t - tx, ty + 1 < a.g.td[1] ? t + sy : t - ty * sy,
+                         tz + 1 < a.g.td[2] ? t + sz : t - tz * sz};
+    const int own = a.slot[t], colour = a.bg[t];
+    bool seam[3];
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        const int k = a.slot[next[d]], c = a.bg[next[d]];  // (one round of loads)
+        seam[d] = (own & k) < 0 && ((c ^ colour) & 1);
+    }
+#pragma unroll
+    for (int d = 0; d < 3; d++)
+        if (seam[d]) background_seam(a.g, t, d, a.s[d]);
 }
 
 static __global__ void mark_all_kernel(MarkAllArgs a) {
     const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
     for (int t = t0; t < a.ntiles; t += gridDim.x * blockDim.x) {
-        if (a.slot && a.slot[t] < 0) background_seams(a, t);
+        if (a.slot) background_seams(a, t);
         a.tile_marker[t] = 0xFFFFFFFFu;
         a.dirty[t] = 1;
         if (a.clean) a.clean[t] = 0;
