@@ -47,18 +47,18 @@ SWEEP_BYTES_PER_CELL = 62.75
 F2V_BYTES_PER_CELL = 36.4
 # DRAM bytes (read + write) of one split sweep (list advection + band pass +
 # FP64 lists) per band cell, from one ncu capture of each kernel on the
-# converging drops at 256^3 (16.8 MB for about 4.8e5 band cells;
+# converging drops at 256^3 (16.81 MB for about 4.8e5 band cells;
 # profiles/sweep_kernels_merging_drops_256.md); scaled by the band of the run.
 NCU_DRAM_BYTES_PER_BAND_CELL = 16.81e6 / 4.807e5
 # The FP64-list kernel's second roofline.  Peak: GB300's FP64 FMA rate
 # (6.2e11 thread operations per second, 2 per clock per SM; a probe of
 # independent FMA chains over every SM; the ncu counters give the same 304 per
-# clock).  Work: FP64 adds, multiplies and FMAs per marker of the sweep, from
-# the ncu capture of the kernel at 256^3 (3.49e6 per launch for 3.57e4
-# markers: 23.3 + 19.8 + 20.6 per elapsed cycle over 54 730 cycles; the method's
-# count, before quotients shared reciprocals).
+# clock).  Work: warp instructions of the FP64 pipe x 32 lanes per marker of the
+# sweep, from a one-pass capture of the kernel in this command at 512^3 (3.80e5
+# per launch for 1.425e5 markers; short lists, whose edges take two lanes each,
+# issue 100 per marker: 256^3).
 FP64_PEAK_OPS_PER_S = 6.245e11
-FP64_OPS_PER_MARKER = 3.49e6 / 3.567e4
+FP64_OPS_PER_MARKER = 3.80e5 * 32 / 1.425e5
 
 
 def peaks():
@@ -667,8 +667,8 @@ def roofline_block(res, prof):
         fp64 = {"kernel": "fp64_kernel (circle fits, face phases, crossing counts)", "bound": "alu",
                 "unit": "FP64 ops/s", "achieved": ops / t_fp64, "peak": FP64_PEAK_OPS_PER_S,
                 "frac": ops / t_fp64 / FP64_PEAK_OPS_PER_S, "ops_per_launch": ops, "avg_launch_us": t_fp64 * 1e6,
-                "rule": "ncu FP64 add/mul/FMA count per marker at 256^3 x markers per sweep; launch time from the "
-                        "instrumented pass (an event pair per launch)"}
+                "rule": "ncu count of FP64 pipe instructions x 32 lanes per marker at 512^3 x markers per sweep; "
+                        "launch time from the instrumented pass (an event pair per launch)"}
     return {"bound": "hbm", "kernel": "split sweep (advect + integer pass + FP64 lists)",
             "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm, "traffic": traffic,
             "peak_source": src, "alg_bytes_per_launch": alg, "alg_bytes_rule": "62.75 B per band cell per sweep",

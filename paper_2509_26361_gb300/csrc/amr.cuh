@@ -248,8 +248,8 @@ __global__ void brick_slots_kernel(const int *__restrict__ tiles, int n, int nt,
 // context's old offsets must not show; background_seams has the edges between two
 // tiles outside it).  A warp takes 32 groups
 // of up to 8 cells in a row: a lane writes its group's colours, and the bricks'
-// offsets go in 16-byte pieces, lane after lane.  HBM bound: two bytes per cell
-// and the bricks.  (A lane per row of a brick, value by value: 68 us at 384^3;
+// offsets go in 16-byte pieces, lane after lane.  Two bytes per cell and the bricks
+// are 17 us of traffic at 384^3; bound by issue (61 % of the slots) and latency.  (A lane per row of a brick, value by value: 68 us at 384^3;
 // this form 54, with the edges into a brick 57.  A background lane's look at the next
 // tiles, or a kernel of its own for them, cost 12 us in place of 3.)
 __global__ void __launch_bounds__(256) unpack_kernel(Grid g, const int *__restrict__ slot, const uint8_t *__restrict__ in_cb,

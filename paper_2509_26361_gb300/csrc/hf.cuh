@@ -133,10 +133,11 @@ __device__ __forceinline__ double fixed_double(long long v, int s) {
 // offsets, the axis a run-time value, one path for both ways of ordering the
 // axes): with separate code for cells at the seams, for each way of ordering and
 // a whole sum per axis tried, a warp ran up to twelve sums one after another.
-// The FP64 units (2 lanes per clock and SM) bound long lists: about 32 operations
-// for the formula per cell with heights; its columns' 72 additions and
-// their differences run as integers.  4.2e5 cells at 256^3 took 286 us, with
-// the additions in FP64 88, and take 62; the error against 64-bit references fell
+// The FP64 units (2 lanes per clock and SM) take about 32 operations per cell with
+// heights, for the formula; its columns' 72 additions and their differences run as
+// integers.  3.0e5 cells at 256^3 took 286 us, with the additions in FP64 88, and
+// take 62, bound by integer issue and the gathers (issue slots 42 % busy, the FP64
+// pipe 26 %); the error against 64-bit references fell
 // from 8.3e-15 to 7e-15.
 __device__ __forceinline__ int hf_cell(const HFCell &c, double *out) {
     int ox[3], oy[3], oz[3];
