@@ -92,7 +92,7 @@ struct ebit_ctx {
     int *ncut;                // [2] its length, one slot per Front2VOF call modulo 2
     unsigned *iface[2];       // interface cells of the last two curvature calls
     int *niface;              // [3] list lengths, one slot per curvature call modulo 3
-    int captured;             // a Front2VOF or curvature call was captured: see clear_length
+    int captured;             // a call was captured: see clear_length
     int cur_if;               // list buffer of the last curvature call
     int if_slot;              // length slot of the next call (0 on entry)
     unsigned *scan;           // interface cells found by a full curvature scan

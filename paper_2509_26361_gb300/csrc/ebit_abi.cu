@@ -133,10 +133,11 @@ int copy_other(ebit_ctx *ctx) {
     return EBIT_OK;
 }
 
-// The list length a Front2VOF or curvature call appends to is 0: the call before
-// cleared it.  In a graph the calls before are those of the replay before, which need
-// not have used the other slots, and the list would grow past its end replay by
-// replay: a captured call clears its own, and so does every later one of the context.
+// The list length a Front2VOF or curvature call or a sweep's band appends to is 0: the
+// call before cleared it.  In a graph the calls before are those of the replay
+// before, which need not have used the other slots, and the list would grow past its
+// end replay by replay: a captured call clears its own, and so does every later one
+// of the context.
 int clear_length(ebit_ctx *ctx, int *length, cudaStream_t st) {
     if (!ctx->captured && !capture_id(st)) return EBIT_OK;
     ctx->captured = 1;
@@ -761,6 +762,7 @@ int ebit_advect_sweep(ebit_ctx *ctx, int dir, const double *u_face, double dt) {
         ml.mtiles_count = ctx->mt_count + rd;
         ml.band = rd ? ctx->band_list2 : ctx->band_list;
         ml.band_count = ctx->band_count + rd;
+        if (int r = clear_length(ctx, ml.band_count, ctx->stream)) return r;
     } else {
         for (int k = 0; k < 3; k++) {
             ml.count[k] = ctx->scan_count + k;
